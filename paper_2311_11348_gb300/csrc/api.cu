@@ -742,8 +742,8 @@ static int usolve_all(swe_ctx* ctx, StateDev in) {
 // beside elem_base instead:
 //   B: usolve_corr (+ rc) -->      edge_corr ----> elem_corr(q >= 3) --> (join)
 //   A:                        ... edge_base --^--> elem_base ------------^
-// The tensor-core mode runs edge_corr -> vol_tc -> elem_corr(every q) on B
-// before the join.  Profiling runs everything on A.
+// The tensor-core mode runs edge_corr -> vol_tc -> elem_corr on B before the
+// join.  Profiling runs everything on A.
 static int run_stage(swe_ctx* ctx, StateDev in, StateDev nst, StateDev out, const Stage& stg, bool cfl_dt,
                      double dt_fixed) {
   const Phys ph = phys(ctx);
@@ -778,8 +778,7 @@ static int run_stage(swe_ctx* ctx, StateDev in, StateDev nst, StateDev out, cons
     unsigned long long* dmin = cfl_dt ? ctx->d_dmin : nullptr;
     CK(launch_usolve_base(A, ctx->dm, ctx->G, ph, in.cb, ctx->vel.ub, ub32_out(ctx), ctx->d_status, dmin));
     CK(fork_groups());
-    // the CUDA-core modes form rc in the velocity solve; the tensor-core mode in elem_corr (from vol)
-    if (ctx->tc) CK(corrtc::launch_usolve_corr(gs, ctx->dm, ctx->G, ph, in, ctx->vel, ctx->d_status, dmin, nullptr));
+    if (ctx->tc) CK(corrtc::launch_usolve_corr(gs, ctx->dm, ctx->G, ph, in, ctx->vel, ctx->d_status, dmin, ctx->rc));
     else if (ctx->corr32)
       CK(corr32::launch_usolve_corr(gs, ctx->dm, ctx->G, ph, in, ctx->vel, ctx->d_status, dmin, ctx->rc));
     else CK(corr64::launch_usolve_corr(gs, ctx->dm, ctx->G, ph, in, ctx->vel, ctx->d_status, dmin, ctx->rc));
@@ -803,18 +802,13 @@ static int run_stage(swe_ctx* ctx, StateDev in, StateDev nst, StateDev out, cons
     ProfScope ps(ctx, F_EDGEB);
     CK(launch_edge_base(A, ctx->dm, ph, stg, in.cb, ctx->vel.ub, ctx->fx, ctx->d_work));
   }
-  auto elem_corr = [&](int part) -> int {
+  auto elem_corr = [&]() -> int {
     ProfScope ps(ctx, F_ELEMC);
     CK(fork_groups());
     if (ctx->tc)
-      CK(corrtc::launch_elem_corr(gs, ctx->dm, ctx->ce, ctx->G, ph, stg, in, nst, out, ctx->vel, ctx->fx, ctx->rc,
-                                  part, ctx->vol));
-    else if (ctx->corr32)
-      CK(corr32::launch_elem_corr(gs, ctx->dm, ctx->ce, ctx->G, ph, stg, in, nst, out, ctx->vel, ctx->fx, ctx->rc,
-                                  part));
-    else
-      CK(corr64::launch_elem_corr(gs, ctx->dm, ctx->ce, ctx->G, ph, stg, in, nst, out, ctx->vel, ctx->fx, ctx->rc,
-                                  part));
+      CK(corrtc::launch_elem_corr(gs, ctx->dm, ctx->G, ph, stg, in, nst, out, ctx->vel, ctx->fx, ctx->vol));
+    else if (ctx->corr32) CK(corr32::launch_elem_corr(gs, ctx->dm, ctx->G, ph, stg, in, nst, out, ctx->vel, ctx->fx));
+    else CK(corr64::launch_elem_corr(gs, ctx->dm, ctx->G, ph, stg, in, nst, out, ctx->vel, ctx->fx));
     CK(join_groups());
     return 0;
   };
@@ -827,21 +821,17 @@ static int run_stage(swe_ctx* ctx, StateDev in, StateDev nst, StateDev out, cons
       else CK(corr64::launch_edge_corr(gs, ctx->dm, ctx->ce, ctx->G, ph, stg, in, ctx->vel, ctx->fx));
       CK(join_groups());
     }
-    if (ctx->tc) {  // every test mode (rc comes from the tensor-core volume terms)
-      {
-        ProfScope ps(ctx, F_VOLTC);
-        CK(corrtc::launch_vol_tc(B, ctx->dm, ctx->G, ph, in, ctx->vel, ctx->vol, ctx->d_status));
-      }
-      CK(elem_corr(0));
-    } else if (!split) {
-      CK(elem_corr(1));  // the higher test modes (the velocity solve formed rc)
+    if (ctx->tc) {
+      ProfScope ps(ctx, F_VOLTC);
+      CK(corrtc::launch_vol_tc(B, ctx->dm, ctx->G, ph, in, ctx->vel, ctx->vol, ctx->d_status));
     }
+    if (!split) CK(elem_corr());
   }
   if (conc) {
     CU(cudaEventRecord(ctx->ev_c, B));
     CU(cudaStreamWaitEvent(A, ctx->ev_c, 0));
   }
-  if (split) CK(elem_corr(1));  // the higher test modes, beside elem_base
+  if (split) CK(elem_corr());  // beside elem_base
   {
     ProfScope ps(ctx, F_ELEMB);
     CK(launch_elem_base(A, ctx->dm, ctx->G, ph, stg, in.cb, nst.cb, out.cb, cb32_out(ctx, out), ctx->vel.ub, ctx->fx,

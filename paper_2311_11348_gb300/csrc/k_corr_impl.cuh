@@ -7,8 +7,8 @@
 //                      (K x K symmetric, LDL^T), also writes the degree-1
 //                      modes, the element's trace record for the edge kernel,
 //                      in the first stage of a CFL step its CFL bound, and
-//                      (FP64 and mixed modes) the correction of the base
-//                      modes rc (volume terms of the degree-1 test modes)
+//                      the correction of the base modes rc (volume terms of
+//                      the degree-1 test modes)
 //   k_edge_corr<PM>    edges with max(p_L, p_R) = PM >= 2: traces of the P1
 //                      and higher parts at npts_for(PM) Gauss points, the LF
 //                      flux of the higher part written as a sum of products
@@ -17,14 +17,13 @@
 //                      two-point equivalent of the correction flux for the
 //                      base modes (Fbc)
 //   k_elem_corr<K>     volume terms as contractions with the reference
-//                      tensors D and G of Eq. (13) (compile-time sparsity),
-//                      source, the edges' projected fluxes and the SSP-RK
-//                      update of the higher modes (test modes q >= 3); in the
-//                      tensor-core mode also the test modes 1, 2 (rc)
+//                      tensors of Eq. (13) (compile-time sparsity), source,
+//                      the edges' projected fluxes and the SSP-RK update of
+//                      the higher modes (test modes q >= 3)
 //
 // With CORR_TC defined (k_corr_tc.cu) the volume terms of the momentum rows
-// come from a buffer that the tensor-core contraction k_vol_tc<K> wrote;
-// k_elem_corr then computes only the elevation row's volume term itself.
+// of the orders 3 and 4 come from a buffer that the tensor-core contraction
+// k_vol_tc<K> wrote; k_elem_vol then adds the elevation row's and the rest.
 #include <cfloat>
 #include <cstdio>
 
@@ -55,24 +54,44 @@ __device__ __forceinline__ const T* egeo_t(const DevMesh& m) {
 
 __host__ __device__ constexpr int pk(int i, int j) { return i <= j ? j * (j + 1) / 2 + i : i * (i + 1) / 2 + j; }
 __host__ __device__ constexpr int imax(int a, int b) { return a > b ? a : b; }
-// orthogonality zeros: phi_i is orthogonal to every polynomial of degree < deg i
+// Structural zeros of the reference tensors.  Mode i is phihat_(a,b), a + b =
+// deg i, b = i - K(deg i - 1): a Legendre polynomial P_a in the collapsed
+// coordinate across the triangle times a Jacobi polynomial in the other one.
+// T[n][i][j] vanishes unless the degrees satisfy the triangle inequality
+// (phi_i is orthogonal to every polynomial of lower degree), the Legendre
+// indices satisfy it too and have an even sum (the integral of P_a P_a' P_a''),
+// and for a constant factor unless the other two agree (orthonormality): 546
+// of the 2250 entries T[m < 10][i][j] remain for K = 15.
+// d_x phihat_q has only the modes of lower degree with a smaller Legendre index of
+// the other parity; (d_y - d_x / 2) phihat_q, the derivative along the line of
+// constant collapsed coordinate, those with a_m <= a_q of the same parity.
+__host__ __device__ constexpr int leg_of(int i) {
+  const int d = deg_of(i);
+  return d - (i - (d == 0 ? 0 : Kof(d - 1)));
+}
+__host__ __device__ constexpr bool tri_ok(int a, int b, int c) { return a <= b + c && b <= a + c && c <= a + b; }
 __host__ __device__ constexpr bool tnz(int n, int i, int j) {
-  return deg_of(n) <= deg_of(i) + deg_of(j) && deg_of(i) <= deg_of(n) + deg_of(j) && deg_of(j) <= deg_of(n) + deg_of(i);
+  if (n == 0) return i == j;
+  if (i == 0) return n == j;
+  if (j == 0) return n == i;
+  return tri_ok(deg_of(n), deg_of(i), deg_of(j)) && tri_ok(leg_of(n), leg_of(i), leg_of(j)) &&
+         (leg_of(n) + leg_of(i) + leg_of(j)) % 2 == 0;
 }
-__host__ __device__ constexpr bool gnz(int q, int i, int j) {
-  return deg_of(q) == 0 ? false
-         : deg_of(q) == 1 ? i == j
-                          : (deg_of(i) <= deg_of(j) + deg_of(q) - 1 && deg_of(j) <= deg_of(i) + deg_of(q) - 1);
+__host__ __device__ constexpr bool dxnz(int q, int m) {
+  return deg_of(m) < deg_of(q) && leg_of(m) < leg_of(q) && (leg_of(q) - leg_of(m)) % 2 == 1;
 }
-__host__ __device__ constexpr bool dnz(int q, int i) { return deg_of(i) < deg_of(q) && (deg_of(q) != 1 || i == 0); }
-__host__ __device__ constexpr bool base2(int q, int i) { return q < 3 && i < 3; }
-__host__ __device__ constexpr bool base3(int q, int i, int j) { return q < 3 && i < 3 && j < 3; }
+__host__ __device__ constexpr bool dsnz(int q, int m) {
+  return deg_of(m) < deg_of(q) && leg_of(m) <= leg_of(q) && (leg_of(q) - leg_of(m)) % 2 == 0;
+}
 // truncation of the auxiliary system (Sect. 3): K(max(deg i, deg j))
 __host__ __device__ constexpr int ktr(int i, int j) { return Kof(imax(deg_of(i), deg_of(j))); }
 
 __constant__ T cT[KMAX][120];       // T[n][i][j], (i, j) packed symmetric
+#ifdef CORR_TC
 __constant__ T cG[2][KMAX][120];    // G_k[q][i][j], (i, j) packed symmetric
-__constant__ T cD[2][KMAX][KMAX];   // D_k[q][i]
+#endif
+__constant__ T cDx[KMAX][10];       // D_x[q][m]: d_x phihat_q = sum_m D_x[q][m] phihat_m, deg m < 4
+__constant__ T cDs[KMAX][10];       // D_y[q][m] - D_x[q][m] / 2, alike
 __constant__ T cEB[3][3][KMAX][8];  // per PM-2: phihat_i(gamma_k(s_g)) at npts_for(PM) points
 __constant__ T cEW[3][8];           // weights on [0,1]
 __constant__ T cES[3][8];           // points on [0,1]
@@ -83,17 +102,23 @@ __constant__ double cEV[3][2][3];   // phihat_i(gamma_k(a)), i < 3, at the edge 
 
 void upload_tables() {
   const RefTables& R = tables();
-  static T t[KMAX][120], g[2][KMAX][120], d[2][KMAX][KMAX], eb[3][3][KMAX][8], ew[3][8], es[3][8];
+  static T t[KMAX][120], dx[KMAX][10], ds[KMAX][10], eb[3][3][KMAX][8], ew[3][8], es[3][8];
   for (int n = 0; n < KMAX; ++n)
     for (int j = 0; j < KMAX; ++j)
-      for (int i = 0; i <= j; ++i) {
-        t[n][pk(i, j)] = (T)R.T[n][i][j];
-        g[0][n][pk(i, j)] = (T)R.G[0][n][i][j];
-        g[1][n][pk(i, j)] = (T)R.G[1][n][i][j];
-      }
+      for (int i = 0; i <= j; ++i) t[n][pk(i, j)] = (T)R.T[n][i][j];
+  for (int q = 0; q < KMAX; ++q)
+    for (int m = 0; m < 10; ++m) {
+      dx[q][m] = (T)R.D[0][q][m];
+      ds[q][m] = (T)(R.D[1][q][m] - 0.5 * R.D[0][q][m]);
+    }
+#ifdef CORR_TC
+  static T g[2][KMAX][120];
   for (int k = 0; k < 2; ++k)
-    for (int q = 0; q < KMAX; ++q)
-      for (int i = 0; i < KMAX; ++i) d[k][q][i] = (T)R.D[k][q][i];
+    for (int n = 0; n < KMAX; ++n)
+      for (int j = 0; j < KMAX; ++j)
+        for (int i = 0; i <= j; ++i) g[k][n][pk(i, j)] = (T)R.G[k][n][i][j];
+  cudaMemcpyToSymbol(cG, g, sizeof g);
+#endif
   for (int pm = 2; pm <= 4; ++pm) {
     const int N = npts_for(pm);
     for (int gg = 0; gg < 8; ++gg) {
@@ -109,8 +134,8 @@ void upload_tables() {
   cudaMemcpyToSymbol(cRS2b, &rs2b, sizeof rs2b);
   const T phi0 = (T)R.phi0;
   cudaMemcpyToSymbol(cT, t, sizeof t);
-  cudaMemcpyToSymbol(cG, g, sizeof g);
-  cudaMemcpyToSymbol(cD, d, sizeof d);
+  cudaMemcpyToSymbol(cDx, dx, sizeof dx);
+  cudaMemcpyToSymbol(cDs, ds, sizeof ds);
   cudaMemcpyToSymbol(cEB, eb, sizeof eb);
   cudaMemcpyToSymbol(cEW, ew, sizeof ew);
   cudaMemcpyToSymbol(cES, es, sizeof es);
@@ -154,99 +179,71 @@ __device__ __forceinline__ void load_modes(T (&out)[K], const T* __restrict__ ba
 }
 
 // ---------------------------------------------------------------------------
-// Volume terms of Eq. (13) for one test mode Q (non-base index triples only),
-// with J^{-1} folded into the contravariant coefficients
-//   Uc_i = (J^-1 q_i)_xhat, Vc_i = (J^-1 q_i)_yhat, uc_j, vc_j likewise, pp_j = xi_j/2:
-//   r_xi = sum_i Uc_i D_x[Q][i] + Vc_i D_y[Q][i]
-//   r_U  = (1/s) [ sum_ij U_i (uc_j G_x[Q][i][j] + vc_j G_y[Q][i][j]) + g (J00 P_x + J10 P_y) ]
-//   r_V  = (1/s) [ sum_ij V_i (...) + g (J01 P_x + J11 P_y) ]
-//   P_k  = sum_ij xi_i pp_j G_k[Q][i][j] + sum_{i >= 3, j < 3} xi_i hb_j G_k[Q][i][j]
+// Volume terms of Eq. (13) of the higher test modes, in two steps.  The
+// derivative of a basis function is a combination of the modes of lower degree,
+// d_k phihat_q = sum_m D_k[q][m] phihat_m, so G_k[q][i][j] = sum_m D_k[q][m]
+// T[m][i][j]: instead of one contraction with G per test mode, the products
+//   Zuu_m = sum_ij T[m][i][j] U_i u_j,  Zuv, Zvu, Zvv likewise,
+//   P_m   = sum_ij T[m][i][j] xi_i (xi_j / 2 + [i >= 3, j < 3] hb_j)
+// are formed once for the K(p - 1) modes m below the element's degree, and
+// every test mode combines them with its two rows of D.  With J^{-1} applied to
+// the products (La = J0 + J2 / 2, Lb = J1 + J3 / 2 belong to D_x, J2, J3 to
+// D_s = D_y - D_x / 2) and E1 = Zuu + g P, E4 = Zvv + g P,
+//   r_xi[q] = sum_m D_x[q][m] (La U_m + Lb V_m) + D_s[q][m] (J2 U_m + J3 V_m)
+//   r_U [q] = (1/s) sum_m D_x[q][m] (La E1 + Lb Zuv) + D_s[q][m] (J2 E1 + J3 Zuv)
+//   r_V [q] = (1/s) sum_m D_x[q][m] (La Zvu + Lb E4) + D_s[q][m] (J2 Zvu + J3 E4)
+// This is 2,300 multiply-adds for K = 15 (10: 760, 6: 200) where the G tensors
+// of every test mode took 10,200 (2,900, 540).
 // The bottom term g xi h_b keeps only the products with a higher elevation
-// mode i >= 3.  For Q < 3 the rest are base triples.  For Q >= 3 the rest,
-// g (xi_lin h_b) with xi_lin the degree-1 part of xi, integrates by parts to
-// its own boundary integral (the gradient of xi_lin h_b is linear, so phi_Q
-// of degree >= 2 is orthogonal to it): the correction edge kernel moves that
-// integral into the edge flux, where it meets the flux's own g xi_lin h_b
-// term and leaves g h_b times the jump of xi_lin, formed in FP64.  In FP32
-// the two O(g |xi| h_b) integrals otherwise cancel to a residual several
-// orders of magnitude smaller and carry their rounding error into it.
+// mode i >= 3: the rest, g (xi_lin h_b) with xi_lin the degree-1 part of xi,
+// integrates by parts to its own boundary integral (the gradient of
+// xi_lin h_b is linear, so phi_q of degree >= 2 is orthogonal to it): the
+// correction edge kernel moves that integral into the edge flux, where it
+// meets the flux's own g xi_lin h_b term and leaves g h_b times the jump of
+// xi_lin, formed in FP64.  In FP32 the two O(g |xi| h_b) integrals otherwise
+// cancel to a residual several orders of magnitude smaller and carry their
+// rounding error into it.
 // ---------------------------------------------------------------------------
-// The structural zeros depend on the degrees of q, i, j only, so one body
-// serves every test mode of degree DQ (q a run-time value: the tensors are
-// read with a block-uniform index, and K = 15 needs 4 code bodies instead of
-// 14, which the instruction cache holds); QR stands for the degree class in
-// the compile-time predicates.
-template <int DQ>
-__host__ __device__ constexpr int qrep() { return DQ <= 1 ? DQ : Kof(DQ - 1); }
-
-template <int K, int DQ, int KL>
-__device__ __forceinline__ void volume_c(T (&r)[3], int q, const T (&xi)[K], const T (&U)[K], const T (&V)[K],
-                                         const T (&uc)[K], const T (&vc)[K], const T (&pp)[K], const T (&hb)[3],
-                                         const T (&Uc)[KL], const T (&Vc)[KL], T rs, T J0, T J1, T J2, T J3,
-                                         T g) {
-  constexpr int QR = qrep<DQ>();
-  T am = 0;
-  sfor<0, KL>([&](auto i) {
-    if constexpr (dnz(QR, i) && !base2(QR, i)) am += Uc[i] * cD[0][q][i] + Vc[i] * cD[1][q][i];
-  });
-  T aU = 0, aV = 0, Px = 0, Py = 0;
+// the products of one mode M: z = {Zuu + g P, Zuv, Zvu, Zvv + g P}
+template <int K, int M>
+__device__ __forceinline__ void products(T (&z)[4], const T (&xi)[K], const T (&U)[K], const T (&V)[K],
+                                         const T (&u)[K], const T (&v)[K], const T (&xh)[3], T g) {
+  T z0 = 0, z1 = 0, z2 = 0, z3 = 0, P = 0;
   sfor<0, K>([&](auto i) {
     constexpr bool any = [] {
       for (int j = 0; j < K; ++j)
-        if (gnz(QR, decltype(i)::value, j) && !base3(QR, decltype(i)::value, j)) return true;
+        if (tnz(M, decltype(i)::value, j)) return true;
       return false;
     }();
     if constexpr (any) {
-      T w = 0, px = 0, py = 0;
+      T a = 0, b = 0, w = 0;
       sfor<0, K>([&](auto j) {
-        if constexpr (gnz(QR, i, j) && !base3(QR, i, j)) {
-          const T gx = cG[0][q][pk(i, j)], gy = cG[1][q][pk(i, j)];
-          w += uc[j] * gx + vc[j] * gy;
-          T pj = pp[j];
-          if constexpr (i >= 3 && j < 3) pj += hb[j];
-          px += pj * gx;
-          py += pj * gy;
+        if constexpr (tnz(M, i, j)) {
+          const T t = cT[M][pk(i, j)];
+          a += u[j] * t;
+          b += v[j] * t;
+          // each unordered pair of P once: xi_i xi_j, on the diagonal half of it
+          if constexpr (j < i) w += (i >= 3 && j < 3 ? xh[j < 3 ? j : 0] : xi[j]) * t;
+          if constexpr (j == i) w += ((T)0.5 * xi[i]) * t;
         }
       });
-      aU += U[i] * w; aV += V[i] * w;
-      Px += xi[i] * px; Py += xi[i] * py;
+      z0 += U[i] * a; z1 += U[i] * b;
+      z2 += V[i] * a; z3 += V[i] * b;
+      P += xi[i] * w;
     }
   });
-  r[0] = am;
-  r[1] = rs * (aU + g * (J0 * Px + J2 * Py));
-  r[2] = rs * (aV + g * (J1 * Px + J3 * Py));
-}
-
-// one test mode Q known at compile time
-template <int K, int Q, int KL>
-__device__ __forceinline__ void volume_q(T (&r)[3], const T (&xi)[K], const T (&U)[K], const T (&V)[K],
-                                         const T (&uc)[K], const T (&vc)[K], const T (&pp)[K], const T (&hb)[3],
-                                         const T (&Uc)[KL], const T (&Vc)[KL], T rs, T J0, T J1, T J2, T J3,
-                                         T g) {
-  volume_c<K, deg_of(Q), KL>(r, Q, xi, U, V, uc, vc, pp, hb, Uc, Vc, rs, J0, J1, J2, J3, g);
-}
-
-// the elevation row of volume_c alone
-template <int K, int DQ, int KL>
-__device__ __forceinline__ T volume_xi(int q, const T (&Uc)[KL], const T (&Vc)[KL]) {
-  constexpr int QR = qrep<DQ>();
-  T am = 0;
-  sfor<0, KL>([&](auto i) {
-    if constexpr (dnz(QR, i) && !base2(QR, i)) am += Uc[i] * cD[0][q][i] + Vc[i] * cD[1][q][i];
-  });
-  return am;
+  z[0] = z0 + g * P;
+  z[1] = z1;
+  z[2] = z2;
+  z[3] = z3 + g * P;
 }
 
 #ifdef CORR_TC
-#define CORR_VOL_PARAM , const float* __restrict__ vol
-#define CORR_VOL_ARG , vol
 // orders whose momentum volume terms come from the tensor cores; for K = 6
 // the CUDA-core contraction measured as fast as the tensor-core kernel plus
 // the buffer round trip, so it stays here
 __host__ __device__ constexpr bool tc_vol(int K) { return K >= 10; }
 #else
-#define CORR_VOL_PARAM
-#define CORR_VOL_ARG
 __host__ __device__ constexpr bool tc_vol(int K) { return false; }
 #endif
 
@@ -296,16 +293,21 @@ __device__ __forceinline__ void usolve_corr_body(const DevMesh& m, int64_t g0, i
         A[pk(i, j)] = acc;
       });
     });
-    // LDL^T: A[pk(i,j)] (i > j) <- L_ij;  dg[j] = d_j, rd[j] = 1/d_j
+    // LDL^T: A[pk(i,j)] (i > j) <- L_ij, rd[j] = 1/d_j (row j's products L_jk d_k
+    // are shared by every row below it: one multiply-add per (i, j, k))
     T dg[K], rd[K];
     sfor<0, K>([&](auto j) {
+      T ld[K];
       T dj = A[pk(j, j)];
-      sfor<0, j>([&](auto k) { dj -= A[pk(j, k)] * A[pk(j, k)] * dg[k]; });
+      sfor<0, j>([&](auto k) {
+        ld[k] = A[pk(j, k)] * dg[k];
+        dj -= A[pk(j, k)] * ld[k];
+      });
       dg[j] = dj;
       rd[j] = (T)1 / dj;
       sfor<j + 1, K>([&](auto i) {
         T w = A[pk(i, j)];
-        sfor<0, j>([&](auto k) { w -= A[pk(i, k)] * A[pk(j, k)] * dg[k]; });
+        sfor<0, j>([&](auto k) { w -= A[pk(i, k)] * ld[k]; });
         A[pk(i, j)] = w * rd[j];
       });
     });
@@ -348,29 +350,24 @@ __device__ __forceinline__ void usolve_corr_body(const DevMesh& m, int64_t g0, i
       trv[l * K + i] = x[1][i] * s;
     });
     if (rc) {
-      constexpr int KL = Kof(deg_of(K - 1) - 1);  // modes of degree < p (the only ones D couples)
-      T uc[K], vc[K], pp[K], Uc[KL], Vc[KL];
-      const T J0 = geo[G_JI0 * ne + e], J1 = geo[G_JI1 * ne + e];
-      const T J2 = geo[G_JI2 * ne + e], J3 = geo[G_JI3 * ne + e];
-      const T hb[3] = {geo[G_HB0 * ne + e], geo[G_HB1 * ne + e], geo[G_HB2 * ne + e]};
-      sfor<0, K>([&](auto j) {
+      // test modes of degree 1 have a constant gradient, so by orthonormality
+      // their volume terms are sums over the modes alone (i >= 3 here)
+      T e1 = 0, e2 = 0, e3 = 0, e4 = 0, px = 0;
+      sfor<3, K>([&](auto j) {
         const T uu = x[0][j] * s, vv = x[1][j] * s;  // the velocity modes as stored above
-        uc[j] = J0 * uu + J1 * vv;
-        vc[j] = J2 * uu + J3 * vv;
-        pp[j] = (T)0.5 * xi[j];
-        if constexpr (j < KL) {
-          Uc[j] = J0 * U[j] + J1 * V[j];
-          Vc[j] = J2 * U[j] + J3 * V[j];
-        }
+        e1 += U[j] * uu; e2 += U[j] * vv;
+        e3 += V[j] * uu; e4 += V[j] * vv;
+        px += xi[j] * xi[j];
       });
-      const T rs = geo[G_RS * ne + e], g = (T)ph.g;
-      T r1[3], r2[3];
-      volume_q<K, 1, KL>(r1, xi, U, V, uc, vc, pp, hb, Uc, Vc, rs, J0, J1, J2, J3, g);
-      volume_q<K, 2, KL>(r2, xi, U, V, uc, vc, pp, hb, Uc, Vc, rs, J0, J1, J2, J3, g);
-      rc[0 * nrc + rc_off + l] = (double)r1[1];
-      rc[1 * nrc + rc_off + l] = (double)r2[1];
-      rc[2 * nrc + rc_off + l] = (double)r1[2];
-      rc[3 * nrc + rc_off + l] = (double)r2[2];
+      const T gp = (T)0.5 * (T)ph.g * px;
+      e1 += gp;
+      e4 += gp;
+      const T x1 = geo[G_GQ1X * ne + e], y1 = geo[G_GQ1Y * ne + e];
+      const T x2 = geo[G_GQ2X * ne + e], y2 = geo[G_GQ2Y * ne + e];
+      rc[0 * nrc + rc_off + l] = (double)(x1 * e1 + y1 * e2);
+      rc[1 * nrc + rc_off + l] = (double)(x2 * e1 + y2 * e2);
+      rc[2 * nrc + rc_off + l] = (double)(x1 * e3 + y1 * e4);
+      rc[3 * nrc + rc_off + l] = (double)(x2 * e3 + y2 * e4);
     }
   }
   if (dmin) cfl_min_store(dmin, mem, dcfl);  // uniform over the grid: every lane of the warp is here
@@ -435,7 +432,7 @@ int launch_usolve_corr(GroupStreams gs, const DevMesh& m, const Groups& G, const
 // carries no cancellation against the base flux.  F_f = F_b + F_h is the LF
 // flux the test modes of degree >= 2 see, except that the g xi_lin h_b terms
 // of F_b give way to g h_b times the jump of xi_lin (the volume term's share,
-// see volume_q).  Both are stored pre-weighted by |E| w_g at the points of
+// see products).  Both are stored pre-weighted by |E| w_g at the points of
 // the left element's direction.
 // ---------------------------------------------------------------------------
 struct Tr { T xb, Ub, Vb, ub, vb, xh, Uh, Vh, uh, vh; };
@@ -536,7 +533,7 @@ __device__ __forceinline__ void edge_corr_body(const DevMesh& m, const int32_t* 
   // jump xi_lin,R - xi_lin,L of the degree-1 elevations at the edge ends
   // (s = 0, 1 of the left element's parameter; the right element runs the
   // edge the other way) from the FP64 base modes: it carries the volume
-  // term g xi_lin h_b of the higher test modes (moved here, see volume_q),
+  // term g xi_lin h_b of the higher test modes (moved here, see products),
   // zero on land, where the mirror state has the same elevation
   double JA = 0.0, JB = 0.0;
   if (R >= 0 || bc == 2) {
@@ -688,122 +685,46 @@ int launch_edge_corr(GroupStreams gs, const DevMesh& m, const CorrEdges& ce, con
 
 
 // ---------------------------------------------------------------------------
-// correction element update of one order group (K = K(p), p >= 2).
-// Block = 128 elements of one test mode q: the grid is ordered q-major
-// (blocks 0..nb-1 compute q = 1, the next nb q = 2, ...), so the blocks that
-// run at the same time on an SM mostly share one branch of the specialised
-// code, and there is one branch per degree of q (volume_c), not per test
-// mode: the branches of all test modes do not fit the instruction cache
-// (ncu: no_instruction stalls).  q = 1, 2: the correction of the base
-// modes (volume terms with a higher coefficient index) -> rc;  q >= 3: the
-// full volume term, the source g grad h_b xi_q, the projections of the full
-// edge fluxes, and the SSP-RK combination of that higher mode.  One launch
-// covers the test modes qlo .. qlo + gridDim.x / nb - 1.
+// correction element update of one order group (K = K(p), p >= 2), test modes
+// q >= 3: volume terms, source g grad h_b xi_q, bottom friction and Coriolis, the
+// projections of the full edge fluxes (which the correction edge kernel left in
+// the element's slots) and the SSP-RK combination.
+//
+//
+// k_elem_corr_split: a block of KL = K(p - 1) warps works on 32 elements, warp m
+// forming the products of mode m and, from shared memory, the test modes 3 + m,
+// 3 + m + KL, ....  The form of every FP64 group: one FP64 instruction takes a warp
+// 64 cycles whatever its parallelism inside the warp and four warps fill an
+// SM's pipe (19 cycles each), so what counts is the instruction count and
+// that few elements still give every scheduler a warp.  FP64, 165,888 elements
+// alone: K = 6, 10, 15 118, 382, 1131 us (GB300), 75 - 85 % of what the pipe
+// can issue; the contraction per test mode took about 250, 1260, 4450.
+// k_elem_corr (FP32, large groups): one thread per element, each coefficient
+// loaded once, the 3 (K - 3) results in registers.  It is straight-line code (55
+// KB for K = 15) and waits for instruction fetches: 19, 42, 90 us for 165,888
+// elements of K = 6, 10, 15 (the split form 20, 52, 319: ten code bodies at once
+// on an SM), but 20 us for 512 of K = 15 (split 10).  The forms cross where the
+// split form's threads fill the device about once (n KL = 60,000: K = 15
+// between 5,000 and 10,000 elements, K = 10 between 10,000 and 20,000).
 // ---------------------------------------------------------------------------
+// source, edges and RK combination of one higher test mode: r = volume terms
 template <int K>
-__global__ void __launch_bounds__(128, kF32 ? 4 : 2) k_elem_corr(DevMesh m, CorrEdges ce, int64_t g0, int64_t n,
-                                                            int64_t rc_off, int64_t nrc, int qlo, Phys ph, Stage stg,
-                                                            const T* __restrict__ cbS,
-                                                            const T* __restrict__ chS, const T* __restrict__ chN,
-                                                            T* __restrict__ chO, const T* __restrict__ ub,
-                                                            const T* __restrict__ uh, const T* __restrict__ pe,
-                                                            double* __restrict__ rc CORR_VOL_PARAM) {
-  const int64_t nb = (n + 127) / 128;
-  const int q = qlo + (int)(blockIdx.x / nb);
-  const int64_t l = (blockIdx.x % nb) * 128 + threadIdx.x;
-  if (l >= n) return;
-  const int64_t e = g0 + l, ne = m.ne;
+__device__ __forceinline__ void finish_mode(const Stage& stg, const Phys& ph, int64_t n, int64_t l, int q, T (&r)[3], T xq, T Uq, T Vq, T uq, T vq, T gdx, T gdy, T tau,
+                                            T dt, const T* __restrict__ pe, const T* __restrict__ chN,
+                                            T* __restrict__ chO) {
   constexpr int KH = K - 3;
-  constexpr int KL = Kof(deg_of(K - 1) - 1);  // modes of degree < p (the only ones D couples)
-  const T* geo = geo_t(m);
-  const T J0 = geo[G_JI0 * ne + e], J1 = geo[G_JI1 * ne + e];
-  const T J2 = geo[G_JI2 * ne + e], J3 = geo[G_JI3 * ne + e];
-  const T rs = geo[G_RS * ne + e];
-  const T g = (T)ph.g;
-  T r[3] = {0, 0, 0};
-  // the test mode's own coefficients and the element's mean elevation
-  T xq = 0, Uq = 0, Vq = 0, xi0 = 0;
-  if constexpr (tc_vol(K)) {
-#ifdef CORR_TC
-    // the momentum volume terms come from the tensor cores: only the xi row's
-    // contravariant momenta (modes of degree < p) are needed here
-    T Uc[KL], Vc[KL];
-    sfor<0, KL>([&](auto j) {
-      T Uj, Vj;
-      if constexpr (j < 3) {
-        Uj = cbS[(1 * 3 + j) * ne + e];
-        Vj = cbS[(2 * 3 + j) * ne + e];
-      } else {
-        Uj = chS[(1 * KH + (j - 3)) * n + l];
-        Vj = chS[(2 * KH + (j - 3)) * n + l];
-      }
-      Uc[j] = J0 * Uj + J1 * Vj;
-      Vc[j] = J2 * Uj + J3 * Vj;
-    });
-    sfor<1, deg_of(K - 1) + 1>([&](auto DQ) {
-      if (deg_of(q) == DQ) r[0] = volume_xi<K, DQ, KL>(q, Uc, Vc);
-    });
-    r[1] = (T)vol[q * nrc + rc_off + l];
-    r[2] = (T)vol[(16 + q) * nrc + rc_off + l];
-    if (q >= 3) {
-      xq = chS[(0 * KH + (q - 3)) * n + l];
-      Uq = chS[(1 * KH + (q - 3)) * n + l];
-      Vq = chS[(2 * KH + (q - 3)) * n + l];
-    }
-    xi0 = cbS[e];
-#endif
-  } else {
-    T xi[K], U[K], V[K], uc[K], vc[K], pp[K], Uc[KL], Vc[KL];
-    T uu[K], vv[K];
-    load_modes<K>(xi, cbS, ne, e, chS, n, l, 0);
-    load_modes<K>(U, cbS, ne, e, chS, n, l, 1);
-    load_modes<K>(V, cbS, ne, e, chS, n, l, 2);
-    load_modes<K>(uu, ub, ne, e, uh, n, l, 0);
-    load_modes<K>(vv, ub, ne, e, uh, n, l, 1);
-    const T hb[3] = {geo[G_HB0 * ne + e], geo[G_HB1 * ne + e], geo[G_HB2 * ne + e]};
-    sfor<0, K>([&](auto j) {
-      uc[j] = J0 * uu[j] + J1 * vv[j];
-      vc[j] = J2 * uu[j] + J3 * vv[j];
-      pp[j] = (T)0.5 * xi[j];
-      if constexpr (j < KL) {
-        Uc[j] = J0 * U[j] + J1 * V[j];
-        Vc[j] = J2 * U[j] + J3 * V[j];
-      }
-    });
-    sfor<1, deg_of(K - 1) + 1>([&](auto DQ) {
-      if (deg_of(q) == DQ) volume_c<K, DQ, KL>(r, q, xi, U, V, uc, vc, pp, hb, Uc, Vc, rs, J0, J1, J2, J3, g);
-    });
-    sfor<3, K>([&](auto Q) {
-      if (q == Q) { xq = xi[Q]; Uq = U[Q]; Vq = V[Q]; }
-    });
-    xi0 = xi[0];
-  }
-  if (q < 3) {
-    rc[(0 * 2 + (q - 1)) * nrc + rc_off + l] = (double)r[1];
-    rc[(1 * 2 + (q - 1)) * nrc + rc_off + l] = (double)r[2];
-    return;
-  }
-  r[1] += geo[G_GDHX * ne + e] * xq;
-  r[2] += geo[G_GDHY * ne + e] * xq;
-  if (ph.src) {  // bottom friction (tau from the element means, Sect. 3) and Coriolis of Eq. (5)
-    const T ra = (T)1.4142135623730951 * rs;
-    const T Hm = (xi0 + geo[G_HB0 * ne + e]) * ra;
-    const T um = ub[0 * ne + e] * ra, vm = ub[3 * ne + e] * ra;  // mode 0 of u, v (layout [2][3][ne])
-    const T tau = (T)ph.fric_lin * Hm + (T)ph.fric_quad * sqrt(um * um + vm * vm);
-    const T uq = uh[(0 * KH + (q - 3)) * n + l], vq = uh[(1 * KH + (q - 3)) * n + l];
+  r[1] += gdx * xq;
+  r[2] += gdy * xq;
+  if (ph.src) {
     r[1] += (T)ph.f_c * Vq - tau * uq;
     r[2] -= (T)ph.f_c * Uq + tau * vq;
   }
-  // edges: every edge of a p >= 2 element is a correction edge, whose kernel
-  // left the projections in this element's slots
-  {
-    const T* P = pe + (q - 3) * n + l;
+  const T* P = pe + (q - 3) * n + l;
 #pragma unroll
-    for (int k = 0; k < 3; ++k)
+  for (int k = 0; k < 3; ++k)
 #pragma unroll
-      for (int f = 0; f < 3; ++f) r[f] += P[(k * 3 + f) * KH * n];
-  }
-  const T dt = (T)stage_dt(stg, m.mem[e]), a = (T)stg.a, b = (T)stg.b;
+    for (int f = 0; f < 3; ++f) r[f] += P[(k * 3 + f) * KH * n];
+  const T a = (T)stg.a, b = (T)stg.b;
   const T cs3[3] = {xq, Uq, Vq};
 #pragma unroll
   for (int f = 0; f < 3; ++f) {
@@ -811,6 +732,167 @@ __global__ void __launch_bounds__(128, kF32 ? 4 : 2) k_elem_corr(DevMesh m, Corr
     chO[ix] = stg.rhs_only ? r[f] : (stg.a != 0.0 ? a * chN[ix] : (T)0) + b * (cs3[f] + dt * r[f]);
   }
 }
+
+// bottom friction coefficient tau from the element means (Sect. 3), 0 without source terms
+__device__ __forceinline__ T friction(const DevMesh& m, const Phys& ph, int64_t e, T rs, T xi0, T u0, T v0) {
+  if (!ph.src) return 0;
+  const T ra = (T)1.4142135623730951 * rs;
+  const T Hm = (xi0 + geo_t(m)[G_HB0 * m.ne + e]) * ra;
+  const T um = u0 * ra, vm = v0 * ra;
+  return (T)ph.fric_lin * Hm + (T)ph.fric_quad * sqrt(um * um + vm * vm);
+}
+
+#define ELEM_CORR_PARAMS                                                                                          \
+  DevMesh m, int64_t g0, int64_t n, Phys ph, Stage stg, const T *__restrict__ cbS, const T *__restrict__ chS,       \
+      const T *__restrict__ chN, T *__restrict__ chO, const T *__restrict__ ub, const T *__restrict__ uh,           \
+      const T *__restrict__ pe
+
+template <int K>
+__global__ void __launch_bounds__(128, K == 6 ? 5 : K == 10 ? 4 : 3) k_elem_corr(ELEM_CORR_PARAMS) {
+  const int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (l >= n) return;
+  const int64_t e = g0 + l, ne = m.ne;
+  constexpr int KL = Kof(deg_of(K - 1) - 1);
+  const T* geo = geo_t(m);
+  T xi[K], U[K], V[K], u[K], v[K];
+  load_modes<K>(xi, cbS, ne, e, chS, n, l, 0);
+  load_modes<K>(U, cbS, ne, e, chS, n, l, 1);
+  load_modes<K>(V, cbS, ne, e, chS, n, l, 2);
+  load_modes<K>(u, ub, ne, e, uh, n, l, 0);
+  load_modes<K>(v, ub, ne, e, uh, n, l, 1);
+  const T J2 = geo[G_JI2 * ne + e], J3 = geo[G_JI3 * ne + e];
+  const T La = geo[G_JI0 * ne + e] + (T)0.5 * J2, Lb = geo[G_JI1 * ne + e] + (T)0.5 * J3;
+  const T rs = geo[G_RS * ne + e], g = (T)ph.g;
+  const T xh[3] = {xi[0] + geo[G_HB0 * ne + e], xi[1] + geo[G_HB1 * ne + e], xi[2] + geo[G_HB2 * ne + e]};
+  T r[3][K];
+  sfor<3, K>([&](auto q) { r[0][q] = r[1][q] = r[2][q] = 0; });
+  sfor<0, KL>([&](auto M) {
+    T z[4];
+    products<K, M>(z, xi, U, V, u, v, xh, g);
+    const T x0 = La * U[M] + Lb * V[M], s0 = J2 * U[M] + J3 * V[M];
+    const T x1 = rs * (La * z[0] + Lb * z[1]), s1 = rs * (J2 * z[0] + J3 * z[1]);
+    const T x2 = rs * (La * z[2] + Lb * z[3]), s2 = rs * (J2 * z[2] + J3 * z[3]);
+    sfor<3, K>([&](auto q) {
+      if constexpr (dxnz(q, M)) {
+        r[0][q] += cDx[q][M] * x0;
+        r[1][q] += cDx[q][M] * x1;
+        r[2][q] += cDx[q][M] * x2;
+      }
+      if constexpr (dsnz(q, M)) {
+        r[0][q] += cDs[q][M] * s0;
+        r[1][q] += cDs[q][M] * s1;
+        r[2][q] += cDs[q][M] * s2;
+      }
+    });
+  });
+  const T gdx = geo[G_GDHX * ne + e], gdy = geo[G_GDHY * ne + e];
+  const T tau = friction(m, ph, e, rs, xi[0], u[0], v[0]);
+  const T dt = (T)stage_dt(stg, m.mem[e]);
+  sfor<3, K>([&](auto q) {
+    T rq[3] = {r[0][q], r[1][q], r[2][q]};
+    finish_mode<K>(stg, ph, n, l, q, rq, xi[q], U[q], V[q], u[q], v[q], gdx, gdy, tau, dt, pe, chN, chO);
+  });
+}
+
+template <int K>
+__global__ void __launch_bounds__(32 * Kof(deg_of(K - 1) - 1)) k_elem_corr_split(ELEM_CORR_PARAMS) {
+  constexpr int KL = Kof(deg_of(K - 1) - 1), KH = K - 3;
+  __shared__ T B[KL][6][32];  // per mode m: the factors of D_x and D_s in the three equations
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t l = blockIdx.x * (int64_t)32 + lane;
+  const bool live = l < n;
+  const int64_t e = g0 + (live ? l : 0), ne = m.ne;
+  const T* geo = geo_t(m);
+  const T rs = geo[G_RS * ne + e];
+  if (live) {
+    T xi[K], U[K], V[K], u[K], v[K];
+    load_modes<K>(xi, cbS, ne, e, chS, n, l, 0);
+    load_modes<K>(U, cbS, ne, e, chS, n, l, 1);
+    load_modes<K>(V, cbS, ne, e, chS, n, l, 2);
+    load_modes<K>(u, ub, ne, e, uh, n, l, 0);
+    load_modes<K>(v, ub, ne, e, uh, n, l, 1);
+    const T J2 = geo[G_JI2 * ne + e], J3 = geo[G_JI3 * ne + e];
+    const T La = geo[G_JI0 * ne + e] + (T)0.5 * J2, Lb = geo[G_JI1 * ne + e] + (T)0.5 * J3;
+    const T xh[3] = {xi[0] + geo[G_HB0 * ne + e], xi[1] + geo[G_HB1 * ne + e], xi[2] + geo[G_HB2 * ne + e]};
+    sfor<0, KL>([&](auto M) {
+      if (w == M) {  // uniform over the warp
+        T z[4];
+        products<K, M>(z, xi, U, V, u, v, xh, (T)ph.g);
+        B[M][0][lane] = La * U[M] + Lb * V[M];
+        B[M][1][lane] = J2 * U[M] + J3 * V[M];
+        B[M][2][lane] = La * z[0] + Lb * z[1];
+        B[M][3][lane] = J2 * z[0] + J3 * z[1];
+        B[M][4][lane] = La * z[2] + Lb * z[3];
+        B[M][5][lane] = J2 * z[2] + J3 * z[3];
+      }
+    });
+  }
+  __syncthreads();
+  if (!live) return;
+  const T gdx = geo[G_GDHX * ne + e], gdy = geo[G_GDHY * ne + e];
+  const T tau = friction(m, ph, e, rs, cbS[e], ub[e], ub[3 * ne + e]);
+  const T dt = (T)stage_dt(stg, m.mem[e]);
+  sfor<3, K>([&](auto q) {
+    if ((q - 3) % KL == w) {  // uniform over the warp
+      T r[3];
+#pragma unroll
+      for (int f = 0; f < 3; ++f) {
+        T acc = 0;
+        sfor<0, KL>([&](auto M) {
+          if constexpr (dxnz(q, M)) acc += cDx[q][M] * B[M][2 * f][lane];
+          if constexpr (dsnz(q, M)) acc += cDs[q][M] * B[M][2 * f + 1][lane];
+        });
+        r[f] = f == 0 ? acc : rs * acc;
+      }
+      T uq = 0, vq = 0;
+      if (ph.src) {
+        uq = uh[(0 * KH + (q - 3)) * n + l];
+        vq = uh[(1 * KH + (q - 3)) * n + l];
+      }
+      finish_mode<K>(stg, ph, n, l, q, r, chS[(0 * KH + (q - 3)) * n + l], chS[(1 * KH + (q - 3)) * n + l],
+                     chS[(2 * KH + (q - 3)) * n + l], uq, vq, gdx, gdy, tau, dt, pe, chN, chO);
+    }
+  });
+}
+
+#ifdef CORR_TC
+// tensor-core mode, orders 3 and 4: block = 128 elements of one test mode (the
+// grid is ordered q-major); the momentum volume terms come from vol
+template <int K>
+__global__ void __launch_bounds__(128, 4) k_elem_vol(ELEM_CORR_PARAMS, const float* __restrict__ vol, int64_t rc_off,
+                                                     int64_t nrc) {
+  const int64_t nb = (n + 127) / 128;
+  const int q = 3 + (int)(blockIdx.x / nb);
+  const int64_t l = (blockIdx.x % nb) * 128 + threadIdx.x;
+  if (l >= n) return;
+  const int64_t e = g0 + l, ne = m.ne;
+  constexpr int KH = K - 3, KL = Kof(deg_of(K - 1) - 1);
+  const T* geo = geo_t(m);
+  const T J2 = geo[G_JI2 * ne + e], J3 = geo[G_JI3 * ne + e];
+  const T La = geo[G_JI0 * ne + e] + (T)0.5 * J2, Lb = geo[G_JI1 * ne + e] + (T)0.5 * J3;
+  T U[KL], V[KL];
+  load_modes<KL>(U, cbS, ne, e, chS + (1 * KH - (KL - 3)) * n, n, l, 1);
+  load_modes<KL>(V, cbS, ne, e, chS + 2 * (KH - (KL - 3)) * n, n, l, 2);
+  T r[3] = {0, vol[q * nrc + rc_off + l], vol[(16 + q) * nrc + rc_off + l]};
+  sfor<3, K>([&](auto Q) {
+    if (q == Q)
+      sfor<0, KL>([&](auto M) {
+        if constexpr (dxnz(Q, M)) r[0] += cDx[Q][M] * (La * U[M] + Lb * V[M]);
+        if constexpr (dsnz(Q, M)) r[0] += cDs[Q][M] * (J2 * U[M] + J3 * V[M]);
+      });
+  });
+  const T tau = friction(m, ph, e, geo[G_RS * ne + e], cbS[e], ub[e], ub[3 * ne + e]);
+  finish_mode<K>(stg, ph, n, l, q, r, chS[(0 * KH + (q - 3)) * n + l], chS[(1 * KH + (q - 3)) * n + l],
+                 chS[(2 * KH + (q - 3)) * n + l], ph.src ? uh[(0 * KH + (q - 3)) * n + l] : 0,
+                 ph.src ? uh[(1 * KH + (q - 3)) * n + l] : 0, geo[G_GDHX * ne + e], geo[G_GDHY * ne + e], tau,
+                 (T)stage_dt(stg, m.mem[e]), pe, chN, chO);
+}
+#define CORR_VOL_PARAM , const float* __restrict__ vol
+#define CORR_VOL_ARG , vol
+#else
+#define CORR_VOL_PARAM
+#define CORR_VOL_ARG
+#endif
 
 static const T* base_c_host(const StateDev& s) {
   if constexpr (kF32) return (const T*)s.cb32; else return (const T*)s.cb;
@@ -820,29 +902,37 @@ static const T* base_u_host(const VelDev& u) {
 }
 
 template <int K>
-static int elem_group(cudaStream_t st, const DevMesh& m, const CorrEdges& ce, const Groups& G, int p, const Phys& ph,
-                      const Stage& stg, StateDev cS, StateDev cN, StateDev cO, VelDev u, EdgeFlux fx,
-                      void* rc, int part CORR_VOL_PARAM) {
+static int elem_group(cudaStream_t st, const DevMesh& m, const Groups& G, int p, const Phys& ph, const Stage& stg,
+                      StateDev cS, StateDev cN, StateDev cO, VelDev u, EdgeFlux fx CORR_VOL_PARAM) {
   const int64_t g0 = G.start[p], n = G.start[p + 1] - g0;
   if (n == 0) return 0;
-  const int64_t nrc = G.start[5] - G.start[2], rc_off = g0 - G.start[2];
-  // part 0: every test mode 1 .. K - 1 (rc included); part 1: the higher test modes 3 .. K - 1
-  const int qlo = part == 0 ? 1 : 3, nq = part == 0 ? K - 1 : K - 3;
-  k_elem_corr<K><<<(unsigned)(((n + 127) / 128) * nq), 128, 0, st>>>(m, ce, g0, n, rc_off, nrc, qlo, ph, stg, base_c_host(cS),
-                                                           (const T*)cS.ch[p], (const T*)cN.ch[p], (T*)cO.ch[p],
-                                                           base_u_host(u), (const T*)u.uh[p], (const T*)fx.Pf[p],
-                                                           (double*)rc CORR_VOL_ARG);
+  const T *cb = base_c_host(cS), *ub = base_u_host(u), *chS = (const T*)cS.ch[p], *chN = (const T*)cN.ch[p];
+  const T *uh = (const T*)u.uh[p], *pe = (const T*)fx.Pf[p];
+  T* chO = (T*)cO.ch[p];
+  if constexpr (!tc_vol(K)) {
+    constexpr int KL = Kof(deg_of(K - 1) - 1);
+    if (!kF32 || n * KL <= 60000) {
+      k_elem_corr_split<K><<<nblocks(n, 32), 32 * KL, 0, st>>>(m, g0, n, ph, stg, cb, chS, chN, chO, ub, uh, pe);
+    } else if constexpr (kF32) {
+      const int t = launch_shape().corr_threads;
+      k_elem_corr<K><<<nblocks(n, t), t, 0, st>>>(m, g0, n, ph, stg, cb, chS, chN, chO, ub, uh, pe);
+    }
+  } else {
+#ifdef CORR_TC
+    k_elem_vol<K><<<(unsigned)(((n + 127) / 128) * (K - 3)), 128, 0, st>>>(
+        m, g0, n, ph, stg, cb, chS, chN, chO, ub, uh, pe, vol, g0 - G.start[2], G.start[5] - G.start[2]);
+#endif
+  }
   count_launch();
   SWE_CUDA_OK(cudaGetLastError());
   return 0;
 }
 
-int launch_elem_corr(GroupStreams gs, const DevMesh& m, const CorrEdges& ce, const Groups& G, const Phys& ph,
-                     const Stage& stg, StateDev cS, StateDev cN, StateDev cO, VelDev u, EdgeFlux fx,
-                     void* rc, int part CORR_VOL_PARAM) {
-  int r = elem_group<6>(gs.s[0], m, ce, G, 2, ph, stg, cS, cN, cO, u, fx, rc, part CORR_VOL_ARG);
-  if (!r) r = elem_group<10>(gs.s[1], m, ce, G, 3, ph, stg, cS, cN, cO, u, fx, rc, part CORR_VOL_ARG);
-  if (!r) r = elem_group<15>(gs.s[2], m, ce, G, 4, ph, stg, cS, cN, cO, u, fx, rc, part CORR_VOL_ARG);
+int launch_elem_corr(GroupStreams gs, const DevMesh& m, const Groups& G, const Phys& ph, const Stage& stg,
+                     StateDev cS, StateDev cN, StateDev cO, VelDev u, EdgeFlux fx CORR_VOL_PARAM) {
+  int r = elem_group<6>(gs.s[0], m, G, 2, ph, stg, cS, cN, cO, u, fx CORR_VOL_ARG);
+  if (!r) r = elem_group<10>(gs.s[1], m, G, 3, ph, stg, cS, cN, cO, u, fx CORR_VOL_ARG);
+  if (!r) r = elem_group<15>(gs.s[2], m, G, 4, ph, stg, cS, cN, cO, u, fx CORR_VOL_ARG);
   return r;
 }
 

@@ -66,6 +66,14 @@
 namespace swedg {
 namespace corrtc {
 
+// orthogonality zeros of G_k[q][i][j], and the base triples
+__host__ __device__ constexpr bool gnz(int q, int i, int j) {
+  return deg_of(q) == 0 ? false
+         : deg_of(q) == 1 ? i == j
+                          : (deg_of(i) <= deg_of(j) + deg_of(q) - 1 && deg_of(j) <= deg_of(i) + deg_of(q) - 1);
+}
+__host__ __device__ constexpr bool base3(int q, int i, int j) { return q < 3 && i < 3 && j < 3; }
+
 constexpr int TC_M = 128;     // elements per tile = MMA M
 constexpr int TC_KD = 32;     // reduction columns of a row (2 K, padded)
 constexpr int TC_COLS = 512;  // TMEM columns per CTA

@@ -155,9 +155,8 @@ struct GroupStreams {
                          unsigned* status, unsigned long long* dmin, void* rc);                                  \
   int launch_edge_corr(GroupStreams gs, const DevMesh& m, const CorrEdges& ce, const Groups& G, const Phys& ph,   \
                        const Stage& stg, StateDev c, VelDev u, EdgeFlux fx);                                      \
-  int launch_elem_corr(GroupStreams gs, const DevMesh& m, const CorrEdges& ce, const Groups& G, const Phys& ph,   \
-                       const Stage& stg, StateDev cS, StateDev cN, StateDev cO, VelDev u, EdgeFlux fx, void* rc,  \
-                       int part);                                                                                 \
+  int launch_elem_corr(GroupStreams gs, const DevMesh& m, const Groups& G, const Phys& ph, const Stage& stg,       \
+                       StateDev cS, StateDev cN, StateDev cO, VelDev u, EdgeFlux fx);                             \
   }
 SWE_CORR_DECL(corr64)
 SWE_CORR_DECL(corr32)
@@ -172,9 +171,8 @@ int launch_usolve_corr(GroupStreams gs, const DevMesh& m, const Groups& G, const
                        unsigned* status, unsigned long long* dmin, void* rc);
 int launch_edge_corr(GroupStreams gs, const DevMesh& m, const CorrEdges& ce, const Groups& G, const Phys& ph,
                      const Stage& stg, StateDev c, VelDev u, EdgeFlux fx);
-int launch_elem_corr(GroupStreams gs, const DevMesh& m, const CorrEdges& ce, const Groups& G, const Phys& ph,
-                     const Stage& stg, StateDev cS, StateDev cN, StateDev cO, VelDev u, EdgeFlux fx, void* rc,
-                     int part, const float* vol);
+int launch_elem_corr(GroupStreams gs, const DevMesh& m, const Groups& G, const Phys& ph, const Stage& stg,
+                     StateDev cS, StateDev cN, StateDev cO, VelDev u, EdgeFlux fx, const float* vol);
 int launch_vol_tc(cudaStream_t st, const DevMesh& m, const Groups& G, const Phys& ph, StateDev c, VelDev u,
                   float* vol, unsigned* status);
 // host: the shared-memory image of the B operands for K = 6, 10, 15 (floats written, or needed when out is NULL)

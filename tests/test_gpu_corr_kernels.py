@@ -1,0 +1,59 @@
+"""GPU tests of the correction kernels' dispatch at the sizes where it changes
+(rule on the group size) and at ragged ends, against the FP64 oracle.
+
+Tolerances, of the largest entry of each field: FP64 1e-12 (the bound of the
+other right-hand side tests); FP32 100 * 2^-24, i.e. one rounding for each of
+the about 100 terms an entry sums over its volume and edge parts."""
+import os
+import sys
+
+import numpy as np
+import pytest
+
+sys.path.insert(0, os.path.join(os.path.dirname(__file__), "..", "oracle"))
+import oracle as O  # noqa: E402
+from paper_2311_11348_gb300 import inputs, swedg  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+TOL = {swedg.PREC_FP64: 1e-12, swedg.PREC_MIXED_FP32: 100 * 2.0**-24, swedg.PREC_MIXED_TF32: 100 * 2.0**-24}
+
+
+def rect(nx, ny):
+    """the triangles of nx x ny squares out of a larger split-square mesh, so that any count can be made"""
+    n = max(nx, ny)
+    xy, tri = inputs.split_square_mesh(n, 1e3, jitter=0.2, seed=7)
+    return xy, tri.reshape(n, n, 2, 3)[:nx, :ny].reshape(-1, 3)
+
+
+def rhs_errors(orders_of, nx, ny, prec, **kw):
+    xy, tri = rect(nx, ny)
+    hv = inputs.fourier_bathymetry(xy, 1e3, lo=10.0, hi=50.0, seed=2)
+    orders = orders_of(len(tri))
+    m = O.Mesh(xy, tri, hv, orders)
+    c = m.project_state(lambda x, y: (0.3 * np.exp(-((x - 400) ** 2 + (y - 600) ** 2) / 4e4),
+                                      2.0 + np.sin(x / 150), 1.0 + np.cos(y / 130)))
+    ref = m.rhs(O.Params(g=9.81, **kw), c)
+    s = swedg.Solver(g=9.81, precision=prec, friction=(kw.get("fric_lin", 0.0), kw.get("fric_quad", 0.0)),
+                     f_c=kw.get("f_c", 0.0))
+    s.set_mesh(xy, tri)
+    s.set_bathymetry(hv)
+    s.set_orders(orders)
+    out = s.rhs(c)
+    s.close()
+    return [float(np.abs(out[f] - ref[f]).max() / np.abs(ref[f]).max()) for f in range(3)]
+
+
+@pytest.mark.parametrize("p,nx,ny", [(4, 50, 60), (4, 51, 59), (3, 64, 78), (3, 70, 72), (2, 100, 100), (2, 99, 102)])
+def test_element_kernel_forms_meet_at_the_size_rule(p, nx, ny):
+    """groups just below and above K(p-1) n = 60,000, where the FP32 element update changes its form"""
+    for prec in (swedg.PREC_MIXED_FP32, swedg.PREC_MIXED_TF32):
+        err = rhs_errors(lambda n: np.full(n, p, np.int8), nx, ny, prec)
+        assert max(err) < TOL[prec], err
+
+
+@pytest.mark.parametrize("prec", [swedg.PREC_FP64, swedg.PREC_MIXED_FP32, swedg.PREC_MIXED_TF32])
+@pytest.mark.parametrize("nx,ny", [(1, 1), (3, 5), (4, 4), (11, 3)])
+def test_correction_kernels_on_ragged_groups(prec, nx, ny):
+    """every order at once, groups of a few elements and around a warp, all source terms"""
+    err = rhs_errors(lambda n: (np.arange(n) % 5).astype(np.int8), nx, ny, prec, fric_lin=1e-4, fric_quad=0.009, f_c=1e-2)
+    assert max(err) < TOL[prec], err
