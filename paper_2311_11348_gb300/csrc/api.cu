@@ -458,15 +458,17 @@ static int regroup(swe_ctx* ctx, bool keep_state) {
   if (keep_state)  // the state in the old internal order, out to the caller layout
     CK(launch_to_user(ctx->stream, ctx->dm, ctx->G, ctx->d_perm, nullptr, ctx->corr32, ctx->st[0], ctx->d_user));
   CK(launch_regroup(ctx->stream, ctx->ms, ctx->d_newp, ctx->dout, ctx->rw));
-  int64_t info[11] = {};
+  int64_t info[12] = {};
   CU(cudaMemcpyAsync(info, ctx->rw.info, sizeof info, cudaMemcpyDeviceToHost, ctx->stream));
   CU(cudaStreamSynchronize(ctx->stream));
   for (int p = 0; p <= 5; ++p) ctx->G.start[p] = info[p];
   for (int pm = 0; pm < 5; ++pm) ctx->ce.n[pm] = (pm >= 2 && ctx->nedge > 0) ? info[6 + pm - 1] - info[6 + pm - 2] : 0;
-  ctx->packed_n = info[10];
+  ctx->ce.n[1] = ctx->nedge > 0 ? info[10] - info[9] : 0;
+  ctx->packed_n = info[11];
   CK(alloc_group_buffers(ctx));
   // edges that no longer touch a p >= 2 element carry no correction flux
-  CU(cudaMemsetAsync(ctx->fx.Fbc, 0, sizeof(double) * 6 * (size_t)std::max<int64_t>(ctx->nedge, 1), ctx->stream));
+  if (ctx->fx.Fbc)
+    CU(cudaMemsetAsync(ctx->fx.Fbc, 0, sizeof(double) * 6 * (size_t)std::max<int64_t>(ctx->nedge, 1), ctx->stream));
   if (keep_state)
     CK(launch_from_user(ctx->stream, ctx->dm, ctx->G, ctx->d_perm, nullptr, ctx->corr32, ctx->d_user, ctx->st[0]));
   if (ctx->packed_n != packed_before)  // the asynchronous staging buffers follow the packed size
@@ -636,14 +638,14 @@ static int build_device(swe_ctx* ctx) {
       (rc = dalloc(ctx, &D.geo32, 4 * (size_t)NGEO * ne)) || (rc = dalloc(ctx, &D.etb, 96 * (size_t)ne)) ||
       (rc = dalloc(ctx, &D.mem, 4 * (size_t)ne)) || (rc = dalloc(ctx, &D.eedge, 12 * (size_t)ne)) ||
       (rc = dalloc(ctx, &D.eL, 4 * (size_t)nE)) || (rc = dalloc(ctx, &D.eR, 4 * (size_t)nE)) ||
-      (rc = dalloc(ctx, &D.slot, 4 * (size_t)nE)) || (rc = dalloc(ctx, &D.lists, 12 * (size_t)nE)) ||
+      (rc = dalloc(ctx, &D.slot, 4 * (size_t)nE)) || (rc = dalloc(ctx, &D.lists, 16 * (size_t)nE)) ||
       (rc = dalloc(ctx, &D.off, 8 * (size_t)ne)))
     return cuda_err(ctx, rc);
   {
     const int64_t be = regroup_blocks(ne), bg = regroup_blocks(nE);
     RegroupScratch& W = ctx->rw;
     if ((rc = dalloc(ctx, &W.ecnt, 4 * 5 * (size_t)be)) || (rc = dalloc(ctx, &W.eoff, 8 * 5 * (size_t)be)) ||
-        (rc = dalloc(ctx, &W.gcnt, 4 * 3 * (size_t)bg)) || (rc = dalloc(ctx, &W.goff, 8 * 3 * (size_t)bg)) ||
+        (rc = dalloc(ctx, &W.gcnt, 4 * 4 * (size_t)bg)) || (rc = dalloc(ctx, &W.goff, 8 * 4 * (size_t)bg)) ||
         (rc = dalloc(ctx, &W.psum, 8 * (size_t)be)) || (rc = dalloc(ctx, &W.poff, 8 * (size_t)(be + 1))) ||
         (rc = dalloc(ctx, &W.info, 8 * 16)))
       return cuda_err(ctx, rc);
@@ -655,6 +657,7 @@ static int build_device(swe_ctx* ctx) {
                     D.mem, d_emem, ctx->nmem, nullptr};
   ctx->ce.slot = D.slot;
   for (int pm = 2; pm <= 4; ++pm) ctx->ce.list[pm] = D.lists + (size_t)(pm - 2) * nE;
+  ctx->ce.list[1] = D.lists + (size_t)3 * nE;
   // base state, velocity and fluxes (sized by the mesh)
   for (int s = 0; s < 3; ++s) {
     if ((rc = dalloc(ctx, &ctx->st[s].cb, sizeof(double) * 9 * ne))) return cuda_err(ctx, rc);
@@ -668,7 +671,9 @@ static int build_device(swe_ctx* ctx) {
   if ((rc = dalloc(ctx, &ctx->vel.ub, sizeof(double) * 6 * ne))) return cuda_err(ctx, rc);
   ctx->vel.ub32 = nullptr;
   if (ctx->corr32 && (rc = dalloc(ctx, &ctx->vel.ub32, sizeof(float) * 6 * ne))) return cuda_err(ctx, rc);
-  if ((rc = dalloc(ctx, &ctx->fx.Fb, sizeof(double) * 6 * nE)) || (rc = dalloc(ctx, &ctx->fx.Fbc, sizeof(double) * 6 * nE)))
+  ctx->fx.Fbc = nullptr;
+  if ((rc = dalloc(ctx, &ctx->fx.Fb, sizeof(double) * 6 * nE)) ||
+      (ctx->corr32 && (rc = dalloc(ctx, &ctx->fx.Fbc, sizeof(double) * 6 * nE))))
     return cuda_err(ctx, rc);
   if ((rc = dalloc(ctx, &ctx->d_user, sizeof(double) * 3 * KMAX * ne)) ||
       (rc = dalloc(ctx, &ctx->d_user2, sizeof(double) * 3 * KMAX * ne)))
@@ -800,7 +805,10 @@ static int run_stage(swe_ctx* ctx, StateDev in, StateDev nst, StateDev out, cons
   }
   {
     ProfScope ps(ctx, F_EDGEB);
-    CK(launch_edge_base(A, ctx->dm, ph, stg, in.cb, ctx->vel.ub, ctx->fx, ctx->d_work));
+    // in FP64 the correction edge kernel computes the whole flux of its edges
+    const bool part = !ctx->corr32 && !stg.base_only && ctx->ce.n[1] < ctx->nedge;
+    CK(launch_edge_base(A, ctx->dm, part ? ctx->ce.list[1] : nullptr, part ? ctx->ce.n[1] : ctx->nedge, ph, stg, in.cb,
+                        ctx->vel.ub, ctx->fx, ctx->d_work));
   }
   auto elem_corr = [&]() -> int {
     ProfScope ps(ctx, F_ELEMC);

@@ -124,7 +124,7 @@ struct DevMesh {
   unsigned* mstatus;      // [nmem] status bits per member (ST_DEPTH, ST_NONFINITE), set beside the global word
 };
 
-// Correction edges grouped by pmax = max(p_L, p_R) in 2..4.
+// Edges grouped by pmax = max(p_L, p_R): 2..4 the correction edges, [1] the others.
 struct CorrEdges {
   int64_t n[5];           // per pmax
   const int32_t* list[5]; // edge ids

@@ -358,10 +358,13 @@ __device__ __forceinline__ void p1_traces(const DevMesh& m, const double* __rest
   t.w[1] = t.w0 + w[1] * b11 + w[2] * b21;
 }
 
-__global__ void __launch_bounds__(128) k_edge_base(DevMesh m, Phys ph, Stage stg, const double* __restrict__ cb,
+// The edges of list[n], or all of them (list == nullptr, n = nedge).
+__global__ void __launch_bounds__(128) k_edge_base(DevMesh m, Phys ph, Stage stg, const int32_t* __restrict__ list,
+                                                   int64_t n, const double* __restrict__ cb,
                                                    const double* __restrict__ ub, double* __restrict__ Fb, int chunk,
                                                    unsigned* work) {
-  for_units(m.nedge, chunk, work, [&](int64_t ed) {
+  for_units(n, chunk, work, [&](int64_t unit) {
+  const int64_t ed = list ? list[unit] : unit;
   const int64_t ne = m.ne, nE = m.nedge;
   const int L = m.eL[ed], R = m.eR[ed], info = m.einfo[ed];
   const int kL = info & 3, kR = (info >> 2) & 3, bc = info >> 4;
@@ -418,12 +421,12 @@ __global__ void __launch_bounds__(128) k_edge_base(DevMesh m, Phys ph, Stage stg
 // grid of one block per base_threads units needs no schedule)
 static inline int base_chunk(const LaunchShape& L) { return L.base_bpsm > 0 ? L.base_chunk : 0; }
 
-int launch_edge_base(cudaStream_t s, const DevMesh& m, const Phys& ph, const Stage& stg, const double* cb,
-                     const double* ub, EdgeFlux fx, unsigned* work) {
-  if (m.nedge == 0) return 0;
+int launch_edge_base(cudaStream_t s, const DevMesh& m, const int32_t* list, int64_t n, const Phys& ph,
+                     const Stage& stg, const double* cb, const double* ub, EdgeFlux fx, unsigned* work) {
+  if (n == 0) return 0;
   const LaunchShape& L = launch_shape();
-  k_edge_base<<<capped_blocks(m.nedge, L.base_threads, L.base_bpsm), L.base_threads, 0, s>>>(m, ph, stg, cb, ub, fx.Fb,
-                                                                                             base_chunk(L), work);
+  k_edge_base<<<capped_blocks(n, L.base_threads, L.base_bpsm), L.base_threads, 0, s>>>(m, ph, stg, list, n, cb, ub,
+                                                                                       fx.Fb, base_chunk(L), work);
   count_launch();
   SWE_CUDA_OK(cudaGetLastError());
   return 0;
@@ -511,7 +514,7 @@ __global__ void __launch_bounds__(128, MINB) k_elem_base(DevMesh m, Phys ph, Sta
     for (int f = 0; f < 3; ++f) {
       F[f][0] = Fb[(f * 2 + 0) * nE + ed];
       F[f][1] = Fb[(f * 2 + 1) * nE + ed];
-      if (!stg.base_only) {
+      if (Fbc) {
         F[f][0] += Fbc[(f * 2 + 0) * nE + ed];
         F[f][1] += Fbc[(f * 2 + 1) * nE + ed];
       }
@@ -567,11 +570,12 @@ int launch_elem_base(cudaStream_t s, const DevMesh& m, const Groups& G, const Ph
   if (m.ne == 0) return 0;
   const LaunchShape& L = launch_shape();
   const int nb = capped_blocks(m.ne, L.base_threads, L.base_bpsm);
+  const double* Fbc = stg.base_only ? nullptr : fx.Fbc;
   if (L.base_bpsm == 0 || L.base_bpsm >= 4)
-    k_elem_base<4><<<nb, L.base_threads, 0, s>>>(m, ph, stg, cbS, cbN, cbO, cbO32, ub, fx.Fb, fx.Fbc,
+    k_elem_base<4><<<nb, L.base_threads, 0, s>>>(m, ph, stg, cbS, cbN, cbO, cbO32, ub, fx.Fb, Fbc,
                                                  (const double*)rc, G.start[2], base_chunk(L), work);
   else
-    k_elem_base<3><<<nb, L.base_threads, 0, s>>>(m, ph, stg, cbS, cbN, cbO, cbO32, ub, fx.Fb, fx.Fbc,
+    k_elem_base<3><<<nb, L.base_threads, 0, s>>>(m, ph, stg, cbS, cbN, cbO, cbO32, ub, fx.Fb, Fbc,
                                                  (const double*)rc, G.start[2], base_chunk(L), work);
   count_launch();
   SWE_CUDA_OK(cudaGetLastError());

@@ -9,13 +9,12 @@
 //                      in the first stage of a CFL step its CFL bound, and
 //                      the correction of the base modes rc (volume terms of
 //                      the degree-1 test modes)
-//   k_edge_corr<PM>    edges with max(p_L, p_R) = PM >= 2: traces of the P1
-//                      and higher parts at npts_for(PM) Gauss points, the LF
-//                      flux of the higher part written as a sum of products
-//                      (no cancellation against the base flux), the full flux
-//                      projected onto both sides' higher test modes, and the
-//                      two-point equivalent of the correction flux for the
-//                      base modes (Fbc)
+//   k_edge_corr<PM>    edges with max(p_L, p_R) = PM >= 2: traces as Legendre
+//                      coefficients along the edge, the moments of the LF
+//                      flux, projected onto both sides' higher test modes,
+//                      and the two-point equivalent for the base modes of
+//                      the correction flux (FP32, Fbc: no cancellation against
+//                      the base flux) or of the whole flux (FP64, Fb)
 //   k_elem_corr<K>     volume terms as contractions with the reference
 //                      tensors of Eq. (13) (compile-time sparsity), source,
 //                      the edges' projected fluxes and the SSP-RK update of
@@ -92,17 +91,22 @@ __constant__ T cG[2][KMAX][120];    // G_k[q][i][j], (i, j) packed symmetric
 #endif
 __constant__ T cDx[KMAX][10];       // D_x[q][m]: d_x phihat_q = sum_m D_x[q][m] phihat_m, deg m < 4
 __constant__ T cDs[KMAX][10];       // D_y[q][m] - D_x[q][m] / 2, alike
-__constant__ T cEB[3][3][KMAX][8];  // per PM-2: phihat_i(gamma_k(s_g)) at npts_for(PM) points
-__constant__ T cEW[3][8];           // weights on [0,1]
-__constant__ T cES[3][8];           // points on [0,1]
-__constant__ T cPhi0;
-__constant__ T cS2b[2];             // points of the two-point base rule on [0,1]
-__constant__ T cRS2b;               // 1 / (s_1 - s_0)
-__constant__ double cEV[3][2][3];   // phihat_i(gamma_k(a)), i < 3, at the edge ends a = 0, 1 (FP64 in every mode)
+__constant__ T cEL[3][KMAX][5];     // phihat_i(gamma_k(s)) = sum_l cEL[k][i][l] P_l(2 s - 1), l <= deg i
+__constant__ double cEJ[3][3][2];    // the P1 rows of cEL in FP64 in every mode (the jump of xi_lin)
+__constant__ T cGP[3][4][5];        // per PM-2: P_l at the points t > 0 (then the middle one) of the npts_for(PM) rule on [-1,1]
+__constant__ T cGW[3][4];           // their weights (the rule's weights on [0,1])
+
+// P_0 .. P_4 at t
+static void legendre5(double t, double (&P)[5]) {
+  P[0] = 1.0;
+  P[1] = t;
+  for (int l = 1; l < 4; ++l) P[l + 1] = ((2 * l + 1) * t * P[l] - l * P[l - 1]) / (l + 1);
+}
 
 void upload_tables() {
   const RefTables& R = tables();
-  static T t[KMAX][120], dx[KMAX][10], ds[KMAX][10], eb[3][3][KMAX][8], ew[3][8], es[3][8];
+  static double ej[3][3][2];
+  static T t[KMAX][120], dx[KMAX][10], ds[KMAX][10], el[3][KMAX][5], gp[3][4][5], gw[3][4];
   for (int n = 0; n < KMAX; ++n)
     for (int j = 0; j < KMAX; ++j)
       for (int i = 0; i <= j; ++i) t[n][pk(i, j)] = (T)R.T[n][i][j];
@@ -119,28 +123,34 @@ void upload_tables() {
         for (int i = 0; i <= j; ++i) g[k][n][pk(i, j)] = (T)R.G[k][n][i][j];
   cudaMemcpyToSymbol(cG, g, sizeof g);
 #endif
+  for (int k = 0; k < 3; ++k)
+    for (int i = 0; i < KMAX; ++i)
+      for (int l = 0; l < 5; ++l) {  // (2 l + 1) int_0^1 phihat_i(gamma_k(s)) P_l(2 s - 1) ds, exact with 8 points
+        double acc = 0.0, P[5];
+        for (int gg = 0; gg < 8; ++gg) {
+          legendre5(2.0 * R.es[8][gg] - 1.0, P);
+          acc += R.ew[8][gg] * R.EB[8][k][i][gg] * P[l];
+        }
+        el[k][i][l] = (T)((2 * l + 1) * acc);
+        if (i < 3 && l < 2) ej[k][i][l] = (2 * l + 1) * acc;
+      }
   for (int pm = 2; pm <= 4; ++pm) {
-    const int N = npts_for(pm);
-    for (int gg = 0; gg < 8; ++gg) {
-      ew[pm - 2][gg] = gg < N ? (T)R.ew[N][gg] : (T)0;
-      es[pm - 2][gg] = gg < N ? (T)R.es[N][gg] : (T)0;
-      for (int k = 0; k < 3; ++k)
-        for (int i = 0; i < KMAX; ++i) eb[pm - 2][k][i][gg] = gg < N ? (T)R.EB[N][k][i][gg] : (T)0;
+    const int N = npts_for(pm), H = N / 2;
+    for (int j = 0; j < 4; ++j) {
+      double P[5] = {0, 0, 0, 0, 0};
+      const bool mid = j == H && N % 2;
+      if (j < H || mid) legendre5(mid ? 0.0 : 2.0 * R.es[N][N - 1 - j] - 1.0, P);
+      for (int l = 0; l < 5; ++l) gp[pm - 2][j][l] = (T)P[l];
+      gw[pm - 2][j] = j < H || mid ? (T)R.ew[N][N - 1 - j] : (T)0;
     }
   }
-  const T s2b[2] = {(T)R.es[2][0], (T)R.es[2][1]};
-  const T rs2b = (T)(1.0 / (R.es[2][1] - R.es[2][0]));
-  cudaMemcpyToSymbol(cS2b, s2b, sizeof s2b);
-  cudaMemcpyToSymbol(cRS2b, &rs2b, sizeof rs2b);
-  const T phi0 = (T)R.phi0;
   cudaMemcpyToSymbol(cT, t, sizeof t);
   cudaMemcpyToSymbol(cDx, dx, sizeof dx);
   cudaMemcpyToSymbol(cDs, ds, sizeof ds);
-  cudaMemcpyToSymbol(cEB, eb, sizeof eb);
-  cudaMemcpyToSymbol(cEW, ew, sizeof ew);
-  cudaMemcpyToSymbol(cES, es, sizeof es);
-  cudaMemcpyToSymbol(cPhi0, &phi0, sizeof phi0);
-  cudaMemcpyToSymbol(cEV, R.EV, sizeof R.EV);
+  cudaMemcpyToSymbol(cEL, el, sizeof el);
+  cudaMemcpyToSymbol(cEJ, ej, sizeof ej);
+  cudaMemcpyToSymbol(cGP, gp, sizeof gp);
+  cudaMemcpyToSymbol(cGW, gw, sizeof gw);
 }
 
 static inline int nblocks(int64_t n, int t) { return (int)((n + t - 1) / t); }
@@ -423,24 +433,48 @@ int launch_usolve_corr(GroupStreams gs, const DevMesh& m, const Groups& G, const
 }
 
 // ---------------------------------------------------------------------------
-// correction edge flux.  Per side the traces are split into the P1 part (b)
-// and the higher part (h).  With w = u.n, P = g xi (xi/2 + h_b):
-//   A.n(b+h) - A.n(b) = ( U_h nx + V_h ny,
-//                         U_h w + U_b w_h + g nx xi_h (xi_b + xi_h/2 + h_b),
-//                         V_h w + V_b w_h + g ny xi_h (xi_b + xi_h/2 + h_b) )
-// so the correction flux  F_h = 1/2 (A_h(L) + A_h(R) + lambda (c_h(L) - c_h(R)))
-// carries no cancellation against the base flux.  F_f = F_b + F_h is the LF
-// flux the test modes of degree >= 2 see, except that the g xi_lin h_b terms
-// of F_b give way to g h_b times the jump of xi_lin (the volume term's share,
-// see products).  Both are stored pre-weighted by |E| w_g at the points of
-// the left element's direction.
+// correction edge flux.  Along an edge every trace is a polynomial of the
+// side's degree; with t = 2 s - 1 in the left element's parameter s it is held as
+// Legendre coefficients (the right side runs the edge the other way: its odd
+// coefficients change sign), and the test functions see a flux only through its
+// moments m_l = int_0^1 F P_l(t) ds, l <= the side's degree.  Linear terms of the
+// flux go from coefficients to moments directly (m_l = F_l / (2 l + 1)), so do
+// the products with the linear h_b; only the products U w, V w and xi^2 are
+// formed at the npts_for(PM) Gauss points, in pairs +-t whose even and odd
+// parts are shared.  With w = u.n and lambda added to the constant coefficient of w
+// (w + lambda on the left, w - lambda on the right) the momentum flux is
+//   F_U = U_L w_L + U_R w_R + g nx (xi_L^2 / 2 + xi_R^2 / 2 + h_b (xi_L + xi_R)).
+// The test modes of degree >= 2 see this flux with its g xi_lin h_b terms
+// replaced by g h_b times the jump of xi_lin (the volume term's share, see
+// products).
+// FP64 writes the moments of degree <= 1 of the whole flux as the edge's
+// two-point flux; the base edge kernel leaves these edges out.
+// FP32 splits every trace into its P1 part (b) and the higher part (h): the
+// correction's share of the base modes, from
+//   U w - U_b w_b = U_h w + U_b w_h,  xi^2 / 2 - xi_b^2 / 2 = xi_h (xi_b + xi_h / 2),
+// carries no cancellation against the base flux that the base edge kernel
+// computes in FP64, and goes to Fbc; the products of two P1 parts reach the
+// higher test modes through their three moments in closed form.
+// All fluxes are weighted by |E| / 4 (the weight of the two-point base rule)
+// through the normal.
+// FP64 is bound by its instruction count (about 340, 620, 1,080 per edge of
+// pmax = 2, 3, 4 with one side an order lower, against 700, 1,450, 3,000 and the base
+// flux for traces and projections mode by mode at every point): 226, 371, 601 us for
+// 249,000 edges between elements of order 2, 3, 4 (GB300, alone), 0.9, 1.5, 2.4 ns
+// per edge where the other form took 1.6, 2.9, 5.8.  FP32 waits on the gathers of
+// the two trace records; 37, 50, 79 us for the same edges, and 106, 115, 123
+// registers instead of 124, 168, 210, so that every pmax runs 4 blocks per SM.
 // ---------------------------------------------------------------------------
-struct Tr { T xb, Ub, Vb, ub, vb, xh, Uh, Vh, uh, vh; };
+template <int PM>
+struct SideC {
+  T x[PM + 1], U[PM + 1], V[PM + 1], w[PM + 1];  // FP64: the whole trace; FP32: its higher part
+  T xl[2], Ul[2], Vl[2], wl[2];                  // the P1 part (FP64: only xl is kept apart)
+  T un, xm;                                      // mean normal velocity and mean elevation
+};
 
 template <int PM>
-__device__ __forceinline__ void side_traces(const DevMesh& m, const Groups& G, StateDev c, VelDev u, int64_t e,
-                                            int p, int k, bool reverse, Tr (&tr)[npts_for(PM)]) {
-  constexpr int N = npts_for(PM), KM = Kof(PM), GI = PM - 2;
+__device__ __forceinline__ void side_coefs(const DevMesh& m, const Groups& G, const StateDev& c, const VelDev& u,
+                                           int64_t e, int p, int k, bool reverse, T nxw, T nyw, SideC<PM>& S) {
   const int64_t ne = m.ne;
   const int K = Kof(p);
   const T rs = geo_t(m)[G_RS * ne + e];
@@ -456,9 +490,10 @@ __device__ __forceinline__ void side_traces(const DevMesh& m, const Groups& G, S
     r4 = (const T*)(p == 2 ? u.tr[2] : p == 3 ? u.tr[3] : u.tr[4]) + l * K * 4;
     rv = (const T*)(p == 2 ? u.trv[2] : p == 3 ? u.trv[3] : u.trv[4]) + l * K;
   }
-  sfor<0, N>([&](auto g) { tr[g] = Tr{0, 0, 0, 0, 0, 0, 0, 0, 0, 0}; });
-  sfor<0, KM>([&](auto i) {
-    if (i >= K) return;
+  sfor<0, PM + 1>([&](auto l) { S.x[l] = S.U[l] = S.V[l] = S.w[l] = 0; });
+  S.xl[1] = S.Ul[1] = S.Vl[1] = S.wl[1] = 0;
+  sfor<0, Kof(PM)>([&](auto i) {
+    if (i >= K && i >= 3) return;
     T cx, cU, cV, cu, cv;
     if (p >= 2) {
       ld4(r4 + i * 4, cx, cU, cV, cu);
@@ -467,22 +502,71 @@ __device__ __forceinline__ void side_traces(const DevMesh& m, const Groups& G, S
       cx = cbt[(0 * 3 + i) * ne + e]; cU = cbt[(1 * 3 + i) * ne + e]; cV = cbt[(2 * 3 + i) * ne + e];
       cu = ubt[(0 * 3 + i) * ne + e]; cv = ubt[(1 * 3 + i) * ne + e];
     }
-    sfor<0, N>([&](auto g) {
-      const T b = rs * (reverse ? cEB[GI][k][i][N - 1 - g] : cEB[GI][k][i][g]);
-      if constexpr (i < 3) {
-        tr[g].xb += cx * b; tr[g].Ub += cU * b; tr[g].Vb += cV * b; tr[g].ub += cu * b; tr[g].vb += cv * b;
-      } else {
-        tr[g].xh += cx * b; tr[g].Uh += cU * b; tr[g].Vh += cV * b; tr[g].uh += cu * b; tr[g].vh += cv * b;
-      }
-    });
+    const T cw = cu * nxw + cv * nyw;
+    if constexpr (i == 0) {
+      const T b = cEL[0][0][0];  // the constant mode, the same on every edge
+      S.xl[0] = cx * b; S.Ul[0] = cU * b; S.Vl[0] = cV * b; S.wl[0] = cw * b;
+      S.xm = S.xl[0] * rs;
+      S.un = S.wl[0] * rs;
+    } else {
+      sfor<0, deg_of(i) + 1>([&](auto l) {
+        const T b = cEL[k][i][l];
+        if constexpr (i < 3) {
+          S.xl[l] += cx * b; S.Ul[l] += cU * b; S.Vl[l] += cV * b; S.wl[l] += cw * b;
+        } else {
+          S.x[l] += cx * b; S.U[l] += cU * b; S.V[l] += cV * b; S.w[l] += cw * b;
+        }
+      });
+    }
   });
+  const T rso = reverse ? -rs : rs;  // odd coefficients change sign on the reversed edge
+  if constexpr (!kF32) {
+    sfor<0, 2>([&](auto l) { S.x[l] += S.xl[l]; S.U[l] += S.Ul[l]; S.V[l] += S.Vl[l]; S.w[l] += S.wl[l]; });
+  }
+  sfor<0, PM + 1>([&](auto l) {
+    const T f = l % 2 ? rso : rs;
+    S.x[l] *= f; S.U[l] *= f; S.V[l] *= f; S.w[l] *= f;
+  });
+  S.xl[0] *= rs;
+  S.xl[1] *= rso;
+  if constexpr (kF32) {
+    S.Ul[0] *= rs; S.Vl[0] *= rs; S.wl[0] *= rs;
+    S.Ul[1] *= rso; S.Vl[1] *= rso; S.wl[1] *= rso;
+  }
+}
+
+// values at the points +t and -t of pair j (the middle point: j = N / 2, N odd, in vp) of sum_l c[l] P_l
+template <int PM, int J>
+__device__ __forceinline__ void at_pair(const T (&c)[PM + 1], T& vp, T& vm) {
+  constexpr int GI = PM - 2;
+  T ev = c[0] + c[2] * cGP[GI][J][2];
+  if constexpr (PM >= 4) ev += c[4] * cGP[GI][J][4];
+  if constexpr (2 * J + 1 == npts_for(PM)) {
+    vp = vm = ev;
+  } else if constexpr (PM >= 3) {
+    const T od = c[1] * cGP[GI][J][1] + c[3] * cGP[GI][J][3];
+    vp = ev + od;
+    vm = ev - od;
+  } else {
+    vp = ev + c[1] * cGP[GI][J][1];
+    vm = ev - c[1] * cGP[GI][J][1];
+  }
+}
+
+// r += the three moments (l = 0, 1, 2) of the product of two linear functions
+__device__ __forceinline__ void add_lin2(T& r0, T& r1, T& r2, const T (&a)[2], const T (&b)[2]) {
+  const T p = a[1] * b[1];
+  r0 += a[0] * b[0] + p * (T)(1.0 / 3.0);
+  r1 += (a[0] * b[1] + a[1] * b[0]) * (T)(1.0 / 3.0);
+  r2 += p * (T)(2.0 / 15.0);
 }
 
 template <int PM>
 __device__ __forceinline__ void edge_corr_body(const DevMesh& m, const int32_t* __restrict__ list, int64_t nl,
                                                const Groups& G, const Phys& ph, const Stage& stg, const StateDev& c,
-                                               const VelDev& u, double* __restrict__ Fbc, const EdgeFlux& fx) {
+                                               const VelDev& u, const EdgeFlux& fx) {
   constexpr int N = npts_for(PM), GI = PM - 2;
+  double* F2 = kF32 ? fx.Fbc : fx.Fb;
   void* const* Pf = fx.Pf;
   const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (idx >= nl) return;
@@ -491,171 +575,243 @@ __device__ __forceinline__ void edge_corr_body(const DevMesh& m, const int32_t* 
   const int kL = info & 3, kR = (info >> 2) & 3, bc = info >> 4;
   const int pL = m.p[L], pR = R >= 0 ? m.p[R] : 0;
   const T* eg = egeo_t(m);
-  const T len = eg[E_LEN * nE + ed], nx = eg[E_NX * nE + ed], ny = eg[E_NY * nE + ed];
-  const T hA = eg[E_HA * nE + ed], hB = eg[E_HB * nE + ed];
+  const T nxw = eg[E_NXW * nE + ed], nyw = eg[E_NYW * nE + ed], wl = eg[E_WLEN * nE + ed];
+  const T h0 = eg[E_HMID * nE + ed], h1 = (T)0.5 * (eg[E_HB * nE + ed] - eg[E_HA * nE + ed]);
   const T g = (T)ph.g;
-  const T hmid = eg[E_HMID * nE + ed];
-  // lambda of Eq. (10) from the element means (Sect. 3), as in the base flux
-  const T* cbt = base_c(c);
-  const T* ubt = base_u(u);
-  const T* geo = geo_t(m);
-  const int64_t ne = m.ne;
-  const T mL = (T)1.4142135623730951 * geo[G_RS * ne + L];
-  const T unL = (ubt[L] * nx + ubt[3 * ne + L] * ny) * mL;
-  const T HL = cbt[L] * mL + hmid;
-  T unR, HR;
-  double xt = 0.0;  // open sea elevation
-  Tr a[N], b[N];
-  side_traces<PM>(m, G, c, u, L, pL, kL, false, a);
+  SideC<PM> a, b;
+  side_coefs<PM>(m, G, c, u, L, pL, kL, false, nxw, nyw, a);
+  // the right state, and the jump of the degree-1 elevation (zero on land)
+  T j0 = 0, j1 = 0;
   if (R >= 0) {
-    side_traces<PM>(m, G, c, u, R, pR, kR, true, b);
-    const T mR = (T)1.4142135623730951 * geo[G_RS * ne + R];
-    unR = (ubt[R] * nx + ubt[3 * ne + R] * ny) * mR;
-    HR = cbt[R] * mR + hmid;
+    side_coefs<PM>(m, G, c, u, R, pR, kR, true, nxw, nyw, b);
   } else if (bc == 2) {
-    xt = tide_value(ph, stage_time(stg, m.emem[ed]));
-    const T xh = (T)xt;
-    sfor<0, N>([&](auto q) { b[q] = a[q]; b[q].xb = xh; b[q].xh = 0; });
-    unR = unL;
-    HR = xh + hmid;
+    const T xh = (T)tide_value(ph, stage_time(stg, m.emem[ed]));
+    b = a;
+    sfor<0, PM + 1>([&](auto l) { b.x[l] = 0; });
+    b.xl[0] = xh;
+    b.xl[1] = 0;
+    if constexpr (!kF32) b.x[0] = xh;
+    b.xm = xh;
   } else {
-    unR = -unL;
-    HR = HL;
-    sfor<0, N>([&](auto q) {
-      const Tr& t = a[q];
-      const T qb = t.Ub * nx + t.Vb * ny, qh = t.Uh * nx + t.Vh * ny;
-      const T wb = t.ub * nx + t.vb * ny, wh = t.uh * nx + t.vh * ny;
-      b[q] = Tr{t.xb, t.Ub - 2 * qb * nx, t.Vb - 2 * qb * ny, t.ub - 2 * wb * nx, t.vb - 2 * wb * ny,
-                t.xh, t.Uh - 2 * qh * nx, t.Vh - 2 * qh * ny, t.uh - 2 * wh * nx, t.vh - 2 * wh * ny};
+    const T nx = eg[E_NX * nE + ed], ny = eg[E_NY * nE + ed];
+    b = a;
+    sfor<0, PM + 1>([&](auto l) {
+      const T qn = 2 * (a.U[l] * nx + a.V[l] * ny);
+      b.U[l] = a.U[l] - qn * nx;
+      b.V[l] = a.V[l] - qn * ny;
+      b.w[l] = -a.w[l];
+    });
+    sfor<0, 2>([&](auto l) {
+      const T qn = 2 * (a.Ul[l] * nx + a.Vl[l] * ny);
+      b.Ul[l] = a.Ul[l] - qn * nx;
+      b.Vl[l] = a.Vl[l] - qn * ny;
+      b.wl[l] = -a.wl[l];
+    });
+    b.un = -a.un;
+  }
+  if constexpr (kF32) {
+    // the jump of xi_lin from the FP64 base modes: it carries the volume term
+    // g xi_lin h_b of the higher test modes (moved here, see products)
+    if (R >= 0 || bc == 2) {
+      const double rl = m.geo[G_RS * m.ne + L];
+      double l0 = c.cb[L] * cEJ[0][0][0], l1 = 0.0;
+#pragma unroll
+      for (int i = 1; i < 3; ++i) {
+        l0 += c.cb[i * m.ne + L] * cEJ[kL][i][0];
+        l1 += c.cb[i * m.ne + L] * cEJ[kL][i][1];
+      }
+      double r0 = 0.0, r1 = 0.0;
+      if (R >= 0) {
+        const double rr = m.geo[G_RS * m.ne + R];
+        r0 = c.cb[R] * cEJ[0][0][0];
+#pragma unroll
+        for (int i = 1; i < 3; ++i) {
+          r0 += c.cb[i * m.ne + R] * cEJ[kR][i][0];
+          r1 -= c.cb[i * m.ne + R] * cEJ[kR][i][1];
+        }
+        r0 *= rr;
+        r1 *= rr;
+      } else {
+        r0 = tide_value(ph, stage_time(stg, m.emem[ed]));
+      }
+      j0 = (T)(r0 - rl * l0);
+      j1 = (T)(r1 - rl * l1);
+    }
+  } else if (R >= 0 || bc == 2) {
+    j0 = b.xl[0] - a.xl[0];
+    j1 = b.xl[1] - a.xl[1];
+  }
+  // lambda of Eq. (10) from the element means (Sect. 3), weighted like w
+  const T lam = fmax(fabs(a.un), fabs(b.un)) + wl * sqrt(g * fmax(a.xm + h0, b.xm + h0));
+  // the elevation row is linear; lambda then joins w
+  T m0[PM + 1], m1[PM + 1], m2[PM + 1];
+  sfor<0, PM + 1>([&](auto l) {
+    m0[l] = ((a.U[l] + b.U[l]) * nxw + (a.V[l] + b.V[l]) * nyw + lam * (a.x[l] - b.x[l])) * (T)(1.0 / (2 * l + 1));
+    m1[l] = m2[l] = 0;
+  });
+  T z0[2], z1[3], z2[3];  // FP32: moments of the P1 parts' flux (elevation row; momentum rows)
+  if constexpr (kF32) {
+    sfor<0, 2>([&](auto l) {
+      z0[l] = ((a.Ul[l] + b.Ul[l]) * nxw + (a.Vl[l] + b.Vl[l]) * nyw + lam * (a.xl[l] - b.xl[l])) * (T)(1.0 / (2 * l + 1));
+    });
+    a.wl[0] += lam;
+    b.wl[0] -= lam;
+  } else {
+    a.w[0] += lam;
+    b.w[0] -= lam;
+  }
+  // the products, at the Gauss points
+  const T gnx = g * nxw, gny = g * nyw;
+  sfor<0, (N + 1) / 2>([&](auto J) {
+    constexpr bool mid = 2 * J + 1 == N;
+    T f1[2] = {0, 0}, f2[2] = {0, 0}, pp[2] = {0, 0};
+    auto side = [&](const SideC<PM>& S) {
+      T x[2], U[2], V[2], w[2];
+      at_pair<PM, J>(S.x, x[0], x[1]);
+      at_pair<PM, J>(S.U, U[0], U[1]);
+      at_pair<PM, J>(S.V, V[0], V[1]);
+      at_pair<PM, J>(S.w, w[0], w[1]);
+      sfor<0, mid ? 1 : 2>([&](auto s) {
+        if constexpr (kF32) {
+          const T t = s == 0 ? cGP[GI][J][1] : -cGP[GI][J][1];
+          const T xb = S.xl[0] + S.xl[1] * t, Ub = S.Ul[0] + S.Ul[1] * t, Vb = S.Vl[0] + S.Vl[1] * t;
+          const T wf = S.wl[0] + S.wl[1] * t + w[s];
+          f1[s] += U[s] * wf + Ub * w[s];
+          f2[s] += V[s] * wf + Vb * w[s];
+          pp[s] += x[s] * (xb + (T)0.5 * x[s]);
+        } else {
+          f1[s] += U[s] * w[s];
+          f2[s] += V[s] * w[s];
+          pp[s] += x[s] * x[s];
+        }
+      });
+    };
+    side(a);
+    side(b);
+    sfor<0, mid ? 1 : 2>([&](auto s) {
+      const T P = kF32 ? pp[s] : (T)0.5 * pp[s];
+      f1[s] += P * gnx;
+      f2[s] += P * gny;
+    });
+    const T wgt = cGW[GI][J];
+    if constexpr (mid) {
+      f1[0] *= wgt;
+      f2[0] *= wgt;
+      sfor<0, PM + 1>([&](auto l) {
+        if constexpr (l % 2 == 0) {
+          m1[l] += f1[0] * cGP[GI][J][l];
+          m2[l] += f2[0] * cGP[GI][J][l];
+        }
+      });
+    } else {
+      const T e1 = wgt * (f1[0] + f1[1]), o1 = wgt * (f1[0] - f1[1]);
+      const T e2 = wgt * (f2[0] + f2[1]), o2 = wgt * (f2[0] - f2[1]);
+      sfor<0, PM + 1>([&](auto l) {
+        m1[l] += (l % 2 ? o1 : e1) * cGP[GI][J][l];
+        m2[l] += (l % 2 ? o2 : e2) * cGP[GI][J][l];
+      });
+    }
+  });
+  // h_b (xi_h,L + xi_h,R): the product with the linear h_b shifts the moments by one
+  {
+    T S[PM + 1];
+    sfor<0, PM + 1>([&](auto l) {
+      S[l] = a.x[l] + b.x[l];
+      if constexpr (!kF32 && l < 2) S[l] -= a.xl[l] + b.xl[l];
+    });
+    sfor<0, PM + 1>([&](auto l) {
+      T s1 = 0;
+      if constexpr (l > 0) s1 += S[l > 0 ? l - 1 : 0] * (T)((double)l / (2 * l - 1));
+      if constexpr (l < PM) s1 += S[l < PM ? l + 1 : 0] * (T)((double)(l + 1) / (2 * l + 3));
+      const T hs = (h0 * S[l] + h1 * s1) * (T)(1.0 / (2 * l + 1));
+      m1[l] += gnx * hs;
+      m2[l] += gny * hs;
     });
   }
-  const T lam = fmax(fabs(unL), fabs(unR)) + sqrt(g * fmax(HL, HR));
-  // jump xi_lin,R - xi_lin,L of the degree-1 elevations at the edge ends
-  // (s = 0, 1 of the left element's parameter; the right element runs the
-  // edge the other way) from the FP64 base modes: it carries the volume
-  // term g xi_lin h_b of the higher test modes (moved here, see products),
-  // zero on land, where the mirror state has the same elevation
-  double JA = 0.0, JB = 0.0;
-  if (R >= 0 || bc == 2) {
-    const double rl = m.geo[G_RS * ne + L];
-    double lA = 0.0, lB = 0.0;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      lA += c.cb[i * ne + L] * cEV[kL][0][i];
-      lB += c.cb[i * ne + L] * cEV[kL][1][i];
+  // the base modes' two-point flux: in FP64 with the g xi_lin h_b terms
+  {
+    T q1[2] = {m1[0], m1[1]}, q2[2] = {m2[0], m2[1]};
+    if constexpr (!kF32) {
+      const T s0 = a.xl[0] + b.xl[0], s1 = a.xl[1] + b.xl[1];
+      const T y0 = h0 * s0 + h1 * s1 * (T)(1.0 / 3.0), y1 = (h0 * s1 + h1 * s0) * (T)(1.0 / 3.0);
+      q1[0] += gnx * y0; q1[1] += gnx * y1;
+      q2[0] += gny * y0; q2[1] += gny * y1;
     }
-    double rA = xt, rB = xt;
-    if (R >= 0) {
-      const double rr = m.geo[G_RS * ne + R];
-      rA = rB = 0.0;
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        rA += c.cb[i * ne + R] * cEV[kR][1][i];
-        rB += c.cb[i * ne + R] * cEV[kR][0][i];
-      }
-      rA *= rr;
-      rB *= rr;
-    }
-    JA = rA - rl * lA;
-    JB = rB - rl * lB;
+    const T r3 = (T)1.7320508075688772;  // the points of the two-point rule are +-1 / sqrt 3
+    F2[0 * nE + ed] = (double)(m0[0] - r3 * m0[1]);
+    F2[1 * nE + ed] = (double)(m0[0] + r3 * m0[1]);
+    F2[2 * nE + ed] = (double)(q1[0] - r3 * q1[1]);
+    F2[3 * nE + ed] = (double)(q1[0] + r3 * q1[1]);
+    F2[4 * nE + ed] = (double)(q2[0] - r3 * q2[1]);
+    F2[5 * nE + ed] = (double)(q2[0] + r3 * q2[1]);
   }
-  const T JA_ = (T)JA, dJ = (T)(JB - JA);
-  // zeroth and first moments (in the left element's edge parameter s) of the
-  // weighted correction flux: they are all the test modes of degree <= 1 see
-  T M0[3] = {0, 0, 0}, M1[3] = {0, 0, 0};
-  T Ffull[3][N], FJ[N];
-  sfor<0, N>([&](auto q) {
-    const T hb = hA + cES[GI][q] * (hB - hA);
-    const Tr& x = a[q];
-    const Tr& y = b[q];
-    // base flux (P1 parts, which the base modes take from the base edge
-    // kernel): for the higher modes g h_b J replaces its g xi_lin h_b terms
-    const T wxb = x.ub * nx + x.vb * ny, wyb = y.ub * nx + y.vb * ny;
-    const T pxb = g * x.xb * ((T)0.5 * x.xb), pyb = g * y.xb * ((T)0.5 * y.xb);
-    const T Fb0 = (x.Ub + y.Ub) * nx + (x.Vb + y.Vb) * ny + lam * (x.xb - y.xb);
-    const T Fb1 = x.Ub * wxb + y.Ub * wyb + (pxb + pyb) * nx + lam * (x.Ub - y.Ub);
-    const T Fb2 = x.Vb * wxb + y.Vb * wyb + (pxb + pyb) * ny + lam * (x.Vb - y.Vb);
-    // higher part as a sum of products
-    const T wxh = x.uh * nx + x.vh * ny, wyh = y.uh * nx + y.vh * ny;
-    const T pxh = g * x.xh * (x.xb + (T)0.5 * x.xh + hb), pyh = g * y.xh * (y.xb + (T)0.5 * y.xh + hb);
-    const T Fh0 = (x.Uh + y.Uh) * nx + (x.Vh + y.Vh) * ny + lam * (x.xh - y.xh);
-    const T Fh1 = x.Uh * (wxb + wxh) + x.Ub * wxh + y.Uh * (wyb + wyh) + y.Ub * wyh + (pxh + pyh) * nx +
-                  lam * (x.Uh - y.Uh);
-    const T Fh2 = x.Vh * (wxb + wxh) + x.Vb * wxh + y.Vh * (wyb + wyh) + y.Vb * wyh + (pxh + pyh) * ny +
-                  lam * (x.Vh - y.Vh);
-    const T wgt = (T)0.5 * len * cEW[GI][q];
-    const T h0 = wgt * Fh0, h1 = wgt * Fh1, h2 = wgt * Fh2;
-    M0[0] += h0; M0[1] += h1; M0[2] += h2;
-    M1[0] += h0 * cES[GI][q]; M1[1] += h1 * cES[GI][q]; M1[2] += h2 * cES[GI][q];
-    Ffull[0][q] = wgt * (Fb0 + Fh0);
-    Ffull[1][q] = wgt * (Fb1 + Fh1);
-    Ffull[2][q] = wgt * (Fb2 + Fh2);
-    FJ[q] = wgt * g * hb * (JA_ + cES[GI][q] * dJ);
-  });
-  // the full flux projected onto the higher test modes of each side once here,
-  //   P[k][f][q] = -+ (1/s) sum_g (F_f(s_g) +- n_f FJ(s_g)) phihat_q(gamma_k(s_g)),
-  // (left: minus, points in its own direction, +J; right: plus, points
-  // reversed, -J), stored in the element's own slot of its order group (local
-  // edge k), so that the element kernel reads one value per edge, field and
-  // mode, consecutive elements contiguous
+  if constexpr (kF32) {  // the P1 parts' share of the higher test modes
+    sfor<0, 3>([&](auto l) { z1[l] = z2[l] = 0; });
+    T zp[3] = {0, 0, 0};
+    add_lin2(z1[0], z1[1], z1[2], a.Ul, a.wl);
+    add_lin2(z1[0], z1[1], z1[2], b.Ul, b.wl);
+    add_lin2(z2[0], z2[1], z2[2], a.Vl, a.wl);
+    add_lin2(z2[0], z2[1], z2[2], b.Vl, b.wl);
+    add_lin2(zp[0], zp[1], zp[2], a.xl, a.xl);
+    add_lin2(zp[0], zp[1], zp[2], b.xl, b.xl);
+    m0[0] += z0[0];
+    m0[1] += z0[1];
+    sfor<0, 3>([&](auto l) {
+      m1[l] += z1[l] + (T)0.5 * gnx * zp[l];
+      m2[l] += z2[l] + (T)0.5 * gny * zp[l];
+    });
+  }
+  // moments of h_b times the jump (a quadratic)
+  const T mj[3] = {h0 * j0 + h1 * j1 * (T)(1.0 / 3.0), (h0 * j1 + h1 * j0) * (T)(1.0 / 3.0), h1 * j1 * (T)(2.0 / 15.0)};
+  // the flux projected onto the higher test modes of each side once here,
+  //   P[k][f][q] = -+ (2/s) sum_l cEL[k][q][l] (+-1)^l (m_l +- n_f g mj_l)
+  // (left: minus, +J; right: plus, odd l reversed, -J; the 2 undoes the weight
+  // |E| / 4), stored in the element's own slot of its order group (local edge
+  // k), so that the element kernel reads one value per edge, field and mode,
+  // consecutive elements contiguous
   auto project = [&](int side, int64_t el, int k, int pside, T sg) {
     const int Kside = Kof(pside), KH = Kside - 3;
     const int64_t s0 = pside == 2 ? G.start[2] : pside == 3 ? G.start[3] : G.start[4];
     const int64_t ns = (pside == 2 ? G.start[3] : pside == 3 ? G.start[4] : G.start[5]) - s0;
     T* P = (T*)(pside == 2 ? Pf[2] : pside == 3 ? Pf[3] : Pf[4]) + (el - s0);
-    const T jx = side ? -nx : nx, jy = side ? -ny : ny;
+    const T jx = side ? -gnx : gnx, jy = side ? -gny : gny;
+    const T sgo = side ? -sg : sg;
+    T y0[PM + 1], y1[PM + 1], y2[PM + 1];
+    sfor<0, PM + 1>([&](auto l) {
+      const T f = l % 2 ? sgo : sg;
+      y0[l] = f * m0[l];
+      if constexpr (l < 3) {
+        y1[l] = f * (m1[l] + jx * mj[l]);
+        y2[l] = f * (m2[l] + jy * mj[l]);
+      } else {
+        y1[l] = f * m1[l];
+        y2[l] = f * m2[l];
+      }
+    });
     sfor<3, Kof(PM)>([&](auto q) {
       if (q < Kside) {
-        T acc[3] = {0, 0, 0}, aj = 0;
-        sfor<0, N>([&](auto g) {
-          const T bq = side ? cEB[GI][k][q][N - 1 - g] : cEB[GI][k][q][g];
-          acc[0] += Ffull[0][g] * bq;
-          acc[1] += Ffull[1][g] * bq;
-          acc[2] += Ffull[2][g] * bq;
-          aj += FJ[g] * bq;
+        T acc[3] = {0, 0, 0};
+        sfor<0, deg_of(q) + 1>([&](auto l) {
+          const T bq = cEL[k][q][l];
+          acc[0] += y0[l] * bq;
+          acc[1] += y1[l] * bq;
+          acc[2] += y2[l] * bq;
         });
-        P[((k * 3 + 0) * KH + (q - 3)) * ns] = sg * acc[0];
-        P[((k * 3 + 1) * KH + (q - 3)) * ns] = sg * (acc[1] + jx * aj);
-        P[((k * 3 + 2) * KH + (q - 3)) * ns] = sg * (acc[2] + jy * aj);
+        P[((k * 3 + 0) * KH + (q - 3)) * ns] = acc[0];
+        P[((k * 3 + 1) * KH + (q - 3)) * ns] = acc[1];
+        P[((k * 3 + 2) * KH + (q - 3)) * ns] = acc[2];
       }
     });
   };
-  if (pL >= 2) project(0, L, kL, pL, -geo[G_RS * ne + L]);
-  if (R >= 0 && pR >= 2) project(1, R, kR, pR, geo[G_RS * ne + R]);
-  // Degree-<=1 test functions are linear along the edge, so the correction's
-  // share of the base modes is fixed by (M0, M1); the two-point flux with the
-  // same moments is stored next to the base flux of this edge, and both sides
-  // project their sum in FP64 (one value per edge: conservative in every mode).
-  sfor<0, 3>([&](auto f) {
-    const T f1 = (M1[f] - cS2b[0] * M0[f]) * cRS2b;
-    const T f0 = M0[f] - f1;
-    Fbc[(f * 2 + 0) * nE + ed] = (double)f0;
-    Fbc[(f * 2 + 1) * nE + ed] = (double)f1;
-  });
+  const T* geo = geo_t(m);
+  if (pL >= 2) project(0, L, kL, pL, (T)-2 * geo[G_RS * m.ne + L]);
+  if (R >= 0 && pR >= 2) project(1, R, kR, pR, (T)2 * geo[G_RS * m.ne + R]);
 }
 
-// Register budgets: the compiler's allocation (FP32: 124, 168, 210 registers
-// for pmax = 2, 3, 4), and in FP32 second builds for pmax = 3 in 128 and for
-// pmax = 4 in 168 registers (4 and 3 blocks per SM) for launch shapes that
-// cap the base grids: where the correction kernels share the SMs with a few
-// base blocks, the extra warps pay (with the K = 15 velocity solve in 168
-// registers, measured on the p 1-4 shelf: -2.6 % per step); beside uncapped
-// base grids they do not.
 template <int PM>
 __global__ void __launch_bounds__(128) k_edge_corr(DevMesh m, const int32_t* __restrict__ list, int64_t nl, Groups G,
-                                                   Phys ph, Stage stg, StateDev c, VelDev u,
-                                                   double* __restrict__ Fbc, EdgeFlux fx) {
-  edge_corr_body<PM>(m, list, nl, G, ph, stg, c, u, Fbc, fx);
-}
-__global__ void __launch_bounds__(128, 3) k_edge_corr4(DevMesh m, const int32_t* __restrict__ list, int64_t nl,
-                                                       Groups G, Phys ph, Stage stg, StateDev c, VelDev u,
-                                                       double* __restrict__ Fbc, EdgeFlux fx) {
-  edge_corr_body<4>(m, list, nl, G, ph, stg, c, u, Fbc, fx);
-}
-__global__ void __launch_bounds__(128, 4) k_edge_corr3(DevMesh m, const int32_t* __restrict__ list, int64_t nl,
-                                                       Groups G, Phys ph, Stage stg, StateDev c, VelDev u,
-                                                       double* __restrict__ Fbc, EdgeFlux fx) {
-  edge_corr_body<3>(m, list, nl, G, ph, stg, c, u, Fbc, fx);
+                                                   Phys ph, Stage stg, StateDev c, VelDev u, EdgeFlux fx) {
+  edge_corr_body<PM>(m, list, nl, G, ph, stg, c, u, fx);
 }
 
 template <int PM>
@@ -664,12 +820,7 @@ static int edge_group(cudaStream_t st, const DevMesh& m, const CorrEdges& ce, co
   const int64_t nl = ce.n[PM];
   if (nl == 0) return 0;
   const int ct = launch_shape().corr_threads;
-  if (PM == 3 && kF32 && launch_shape().base_bpsm > 0)
-    k_edge_corr3<<<nblocks(nl, ct), ct, 0, st>>>(m, ce.list[PM], nl, G, ph, stg, c, u, fx.Fbc, fx);
-  else if (PM == 4 && kF32 && launch_shape().base_bpsm > 0)
-    k_edge_corr4<<<nblocks(nl, ct), ct, 0, st>>>(m, ce.list[PM], nl, G, ph, stg, c, u, fx.Fbc, fx);
-  else
-    k_edge_corr<PM><<<nblocks(nl, ct), ct, 0, st>>>(m, ce.list[PM], nl, G, ph, stg, c, u, fx.Fbc, fx);
+  k_edge_corr<PM><<<nblocks(nl, ct), ct, 0, st>>>(m, ce.list[PM], nl, G, ph, stg, c, u, fx);
   count_launch();
   SWE_CUDA_OK(cudaGetLastError());
   return 0;

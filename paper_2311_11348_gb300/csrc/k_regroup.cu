@@ -25,7 +25,7 @@ constexpr int RG_W = RG_T / 32;
 constexpr int RG_MAXC = 5;  // categories at most (orders 0..4)
 
 // category of a unit: element u -> its order; edge i -> pmax - 2 for a
-// correction edge (pmax = the larger order of its elements >= 2), else -1
+// correction edge (pmax = the larger order of its elements >= 2), else 3
 struct ElemCat {
   const int8_t* p;
   __device__ int operator()(int64_t u) const { return p[u]; }
@@ -38,7 +38,7 @@ struct EdgeCat {
     int pm = p[eLu[i]];
     const int r = eRu[i];
     if (r >= 0) pm = max(pm, (int)p[r]);
-    return pm >= 2 ? pm - 2 : -1;
+    return pm >= 2 ? pm - 2 : 3;
   }
 };
 
@@ -133,22 +133,18 @@ __global__ void __launch_bounds__(RG_T) k_elem_scatter(const int8_t* p_user, int
 }
 
 // edges: slot[i] = (pmax << 28) | position in its correction group, or -1;
-// lists[(pmax - 2) * nedge + position] = i.  off includes the group starts
-// (start3), which the positions are taken relative to.
+// lists[category * nedge + position] = i.  off includes the group starts
+// (start), which the positions are taken relative to.
 __global__ void __launch_bounds__(RG_T) k_edge_scatter(EdgeCat cat, int64_t nedge, const int64_t* off,
-                                                      const int64_t* start3, int32_t* slot, int32_t* lists) {
+                                                      const int64_t* start, int32_t* slot, int32_t* lists) {
   __shared__ int cnt_s[RG_W][RG_MAXC];
   const int64_t i = blockIdx.x * (int64_t)RG_T + threadIdx.x;
   const int c = i < nedge ? cat(i) : -1;
-  const int r = block_rank<3>(c, cnt_s);
+  const int r = block_rank<4>(c, cnt_s);
   if (i < nedge) {
-    if (c < 0) {
-      slot[i] = -1;
-    } else {
-      const int64_t pos = off[(int64_t)blockIdx.x * 3 + c] + r - start3[c];
-      slot[i] = ((c + 2) << 28) | (int32_t)pos;
-      lists[(int64_t)c * nedge + pos] = (int32_t)i;
-    }
+    const int64_t pos = off[(int64_t)blockIdx.x * 4 + c] + r - start[c];
+    slot[i] = c < 3 ? ((c + 2) << 28) | (int32_t)pos : -1;
+    lists[(int64_t)c * nedge + pos] = (int32_t)i;
   }
 }
 
@@ -245,15 +241,15 @@ int64_t regroup_blocks(int64_t n) { return nb(n, RG_T); }
 int launch_regroup(cudaStream_t s, const MeshStatic& S, const int8_t* p_user, DevMeshOut D, RegroupScratch W) {
   const int64_t ne = S.ne, nE = S.nedge;
   const int64_t be = nb(ne, RG_T), bg = nb(nE, RG_T);
-  // W.info: [0..5] order group starts, [6..9] correction edge group starts, [10] packed size
+  // W.info: [0..5] order group starts, [6..10] edge group starts, [11] packed size
   k_part_counts<5><<<(unsigned)be, RG_T, 0, s>>>(ElemCat{p_user}, ne, W.ecnt);
   k_part_scan<5><<<1, 1024, 0, s>>>(W.ecnt, be, W.eoff, W.info);
   k_elem_scatter<<<(unsigned)be, RG_T, 0, s>>>(p_user, ne, W.eoff, D.perm, D.inv, D.p);
   count_launch(3);
   if (nE > 0) {
     const EdgeCat ec{p_user, S.eLu, S.eRu};
-    k_part_counts<3><<<(unsigned)bg, RG_T, 0, s>>>(ec, nE, W.gcnt);
-    k_part_scan<3><<<1, 1024, 0, s>>>(W.gcnt, bg, W.goff, W.info + 6);
+    k_part_counts<4><<<(unsigned)bg, RG_T, 0, s>>>(ec, nE, W.gcnt);
+    k_part_scan<4><<<1, 1024, 0, s>>>(W.gcnt, bg, W.goff, W.info + 6);
     k_edge_scatter<<<(unsigned)bg, RG_T, 0, s>>>(ec, nE, W.goff, W.info + 6, D.slot, D.lists);
     k_gather_edges<<<nb(nE, 256), 256, 0, s>>>(S, D.inv, D);
     count_launch(4);
@@ -265,7 +261,7 @@ int launch_regroup(cudaStream_t s, const MeshStatic& S, const int8_t* p_user, De
   count_launch(4);
   SWE_CUDA_OK(cudaGetLastError());
   // the packed total (poff[be]) next to the group starts
-  SWE_CUDA_OK(cudaMemcpyAsync(W.info + 10, W.poff + be, sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
+  SWE_CUDA_OK(cudaMemcpyAsync(W.info + 11, W.poff + be, sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
   return 0;
 }
 

@@ -29,9 +29,10 @@ struct Groups {
 };
 
 struct EdgeFlux {
-  double* Fb;        // [3][2][nedge] base flux (weighted by |E| w_g) at the 2-point rule
-  double* Fbc;       // [3][2][nedge] two-point equivalent of the correction flux's share of the
-                     // base modes (zero on edges without a p >= 2 side)
+  double* Fb;        // [3][2][nedge] base flux (weighted by |E| w_g) at the 2-point rule; in FP64 mode the
+                     // whole flux on the edges with a p >= 2 side (from the correction edge kernel)
+  double* Fbc;       // mixed modes: [3][2][nedge] two-point equivalent of the correction flux's share of
+                     // the base modes (zero on edges without a p >= 2 side); nullptr in FP64 mode
   void* Pf[5];       // per element order p = 2..4: [3 local edges][3 fields][K(p)-3][n_p]: the full flux of
                      // each of the element's (correction) edges projected onto its higher test modes (q >= 3),
                      // written by the correction edge kernel, read contiguously by the element kernel
@@ -64,18 +65,18 @@ struct DevMeshOut {
   int32_t* eL;     // [nedge] internal index of the left element
   int32_t* eR;     // [nedge] internal index of the right element or -1
   int32_t* slot;   // [nedge] (pmax << 28) | position in the correction group, or -1
-  int32_t* lists;  // [3][nedge] correction edge ids per pmax = 2, 3, 4
+  int32_t* lists;  // [4][nedge] edge ids per pmax = 2, 3, 4 (correction edges), then those with pmax <= 1
   int64_t* off;    // [ne] packed caller layout offsets (caller order)
 };
 // scratch of the partitions (sizes from regroup_blocks of ne and nedge)
 struct RegroupScratch {
   int32_t* ecnt;  // [be][5]
   int64_t* eoff;  // [be][5]
-  int32_t* gcnt;  // [bg][3]
-  int64_t* goff;  // [bg][3]
+  int32_t* gcnt;  // [bg][4]
+  int64_t* goff;  // [bg][4]
   int64_t* psum;  // [be]
   int64_t* poff;  // [be + 1]
-  int64_t* info;  // [16]: order group starts [0..5], correction group starts [6..9], packed size [10]
+  int64_t* info;  // [16]: order group starts [0..5], edge group starts [6..10], packed size [11]
 };
 int64_t regroup_blocks(int64_t n);
 // the internal arrays for the orders p_user (device, caller order); the
@@ -121,8 +122,9 @@ int launch_usolve_base(cudaStream_t s, const DevMesh& m, const Groups& G, const 
                        double* ub, float* ub32, unsigned* status, unsigned long long* dmin);
 // work: two zero-initialised counters per kernel for the dynamic schedule
 // (left at zero when the launch ends), used by one launch at a time
-int launch_edge_base(cudaStream_t s, const DevMesh& m, const Phys& ph, const Stage& stg, const double* cb,
-                     const double* ub, EdgeFlux fx, unsigned* work);
+// list[n]: the edges to compute (nullptr: all, n = nedge)
+int launch_edge_base(cudaStream_t s, const DevMesh& m, const int32_t* list, int64_t n, const Phys& ph,
+                     const Stage& stg, const double* cb, const double* ub, EdgeFlux fx, unsigned* work);
 int launch_elem_base(cudaStream_t s, const DevMesh& m, const Groups& G, const Phys& ph, const Stage& stg,
                      const double* cbS, const double* cbN, double* cbO, float* cbO32, const double* ub, EdgeFlux fx,
                      const void* rc, unsigned* work);
