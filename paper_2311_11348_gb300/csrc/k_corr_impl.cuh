@@ -230,22 +230,22 @@ __device__ __forceinline__ void products(T (&z)[4], const T (&xi)[K], const T (&
       sfor<0, K>([&](auto j) {
         if constexpr (tnz(M, i, j)) {
           const T t = cT[M][pk(i, j)];
-          a += u[j] * t;
-          b += v[j] * t;
+          a = fma(u[j], t, a);
+          b = fma(v[j], t, b);
           // each unordered pair of P once: xi_i xi_j, on the diagonal half of it
-          if constexpr (j < i) w += (i >= 3 && j < 3 ? xh[j < 3 ? j : 0] : xi[j]) * t;
-          if constexpr (j == i) w += ((T)0.5 * xi[i]) * t;
+          if constexpr (j < i) w = fma(i >= 3 && j < 3 ? xh[j < 3 ? j : 0] : xi[j], t, w);
+          if constexpr (j == i) w = fma((T)0.5 * xi[i], t, w);
         }
       });
-      z0 += U[i] * a; z1 += U[i] * b;
-      z2 += V[i] * a; z3 += V[i] * b;
-      P += xi[i] * w;
+      z0 = fma(U[i], a, z0); z1 = fma(U[i], b, z1);
+      z2 = fma(V[i], a, z2); z3 = fma(V[i], b, z3);
+      P = fma(xi[i], w, P);
     }
   });
-  z[0] = z0 + g * P;
+  z[0] = fma(g, P, z0);
   z[1] = z1;
   z[2] = z2;
-  z[3] = z3 + g * P;
+  z[3] = fma(g, P, z3);
 }
 
 #ifdef CORR_TC
@@ -860,15 +860,16 @@ int launch_edge_corr(GroupStreams gs, const DevMesh& m, const CorrEdges& ce, con
 // ---------------------------------------------------------------------------
 // source, edges and RK combination of one higher test mode: r = volume terms
 template <int K>
-__device__ __forceinline__ void finish_mode(const Stage& stg, const Phys& ph, int64_t n, int64_t l, int q, T (&r)[3], T xq, T Uq, T Vq, T uq, T vq, T gdx, T gdy, T tau,
-                                            T dt, const T* __restrict__ pe, const T* __restrict__ chN,
+__device__ __forceinline__ void finish_mode(const Stage& stg, const Phys& ph, int64_t n, int64_t l, int q,
+                                            T (&r)[3], T xq, T Uq, T Vq, T uq, T vq, T gdx, T gdy, T tau, T dt,
+                                            const T* __restrict__ pe, const T* __restrict__ chN,
                                             T* __restrict__ chO) {
   constexpr int KH = K - 3;
-  r[1] += gdx * xq;
-  r[2] += gdy * xq;
+  r[1] = fma(gdx, xq, r[1]);
+  r[2] = fma(gdy, xq, r[2]);
   if (ph.src) {
-    r[1] += (T)ph.f_c * Vq - tau * uq;
-    r[2] -= (T)ph.f_c * Uq + tau * vq;
+    r[1] += fma((T)ph.f_c, Vq, -(tau * uq));
+    r[2] -= fma((T)ph.f_c, Uq, tau * vq);
   }
   const T* P = pe + (q - 3) * n + l;
 #pragma unroll
@@ -880,7 +881,8 @@ __device__ __forceinline__ void finish_mode(const Stage& stg, const Phys& ph, in
 #pragma unroll
   for (int f = 0; f < 3; ++f) {
     const int64_t ix = (f * KH + (q - 3)) * n + l;
-    chO[ix] = stg.rhs_only ? r[f] : (stg.a != 0.0 ? a * chN[ix] : (T)0) + b * (cs3[f] + dt * r[f]);
+    const T y = fma(dt, r[f], cs3[f]);
+    chO[ix] = stg.rhs_only ? r[f] : fma(b, y, stg.a != 0.0 ? a * chN[ix] : (T)0);
   }
 }
 
@@ -897,6 +899,19 @@ __device__ __forceinline__ T friction(const DevMesh& m, const Phys& ph, int64_t 
   DevMesh m, int64_t g0, int64_t n, Phys ph, Stage stg, const T *__restrict__ cbS, const T *__restrict__ chS,       \
       const T *__restrict__ chN, T *__restrict__ chO, const T *__restrict__ ub, const T *__restrict__ uh,           \
       const T *__restrict__ pe
+
+// The factors of D_x and D_s in the three equations (without the 1/s of the
+// momentum rows) from mode m's momenta and products.  Spelled out in fma, like the
+// sums that use them: a group takes one kernel form or the other by its size,
+// and an element's result must not depend on it.
+__device__ __forceinline__ void row_factors(T (&x)[3], T (&s)[3], T La, T Lb, T J2, T J3, T U, T V, const T (&z)[4]) {
+  x[0] = fma(La, U, Lb * V);
+  s[0] = fma(J2, U, J3 * V);
+  x[1] = fma(La, z[0], Lb * z[1]);
+  s[1] = fma(J2, z[0], J3 * z[1]);
+  x[2] = fma(La, z[2], Lb * z[3]);
+  s[2] = fma(J2, z[2], J3 * z[3]);
+}
 
 template <int K>
 __global__ void __launch_bounds__(128, K == 6 ? 5 : K == 10 ? 4 : 3) k_elem_corr(ELEM_CORR_PARAMS) {
@@ -920,27 +935,20 @@ __global__ void __launch_bounds__(128, K == 6 ? 5 : K == 10 ? 4 : 3) k_elem_corr
   sfor<0, KL>([&](auto M) {
     T z[4];
     products<K, M>(z, xi, U, V, u, v, xh, g);
-    const T x0 = La * U[M] + Lb * V[M], s0 = J2 * U[M] + J3 * V[M];
-    const T x1 = rs * (La * z[0] + Lb * z[1]), s1 = rs * (J2 * z[0] + J3 * z[1]);
-    const T x2 = rs * (La * z[2] + Lb * z[3]), s2 = rs * (J2 * z[2] + J3 * z[3]);
+    T x[3], s[3];
+    row_factors(x, s, La, Lb, J2, J3, U[M], V[M], z);
     sfor<3, K>([&](auto q) {
-      if constexpr (dxnz(q, M)) {
-        r[0][q] += cDx[q][M] * x0;
-        r[1][q] += cDx[q][M] * x1;
-        r[2][q] += cDx[q][M] * x2;
-      }
-      if constexpr (dsnz(q, M)) {
-        r[0][q] += cDs[q][M] * s0;
-        r[1][q] += cDs[q][M] * s1;
-        r[2][q] += cDs[q][M] * s2;
-      }
+      sfor<0, 3>([&](auto f) {
+        if constexpr (dxnz(q, M)) r[f][q] = fma(cDx[q][M], x[f], r[f][q]);
+        if constexpr (dsnz(q, M)) r[f][q] = fma(cDs[q][M], s[f], r[f][q]);
+      });
     });
   });
   const T gdx = geo[G_GDHX * ne + e], gdy = geo[G_GDHY * ne + e];
   const T tau = friction(m, ph, e, rs, xi[0], u[0], v[0]);
   const T dt = (T)stage_dt(stg, m.mem[e]);
   sfor<3, K>([&](auto q) {
-    T rq[3] = {r[0][q], r[1][q], r[2][q]};
+    T rq[3] = {r[0][q], rs * r[1][q], rs * r[2][q]};
     finish_mode<K>(stg, ph, n, l, q, rq, xi[q], U[q], V[q], u[q], v[q], gdx, gdy, tau, dt, pe, chN, chO);
   });
 }
@@ -969,12 +977,13 @@ __global__ void __launch_bounds__(32 * Kof(deg_of(K - 1) - 1)) k_elem_corr_split
       if (w == M) {  // uniform over the warp
         T z[4];
         products<K, M>(z, xi, U, V, u, v, xh, (T)ph.g);
-        B[M][0][lane] = La * U[M] + Lb * V[M];
-        B[M][1][lane] = J2 * U[M] + J3 * V[M];
-        B[M][2][lane] = La * z[0] + Lb * z[1];
-        B[M][3][lane] = J2 * z[0] + J3 * z[1];
-        B[M][4][lane] = La * z[2] + Lb * z[3];
-        B[M][5][lane] = J2 * z[2] + J3 * z[3];
+        T x[3], s[3];
+        row_factors(x, s, La, Lb, J2, J3, U[M], V[M], z);
+#pragma unroll
+        for (int f = 0; f < 3; ++f) {
+          B[M][2 * f][lane] = x[f];
+          B[M][2 * f + 1][lane] = s[f];
+        }
       }
     });
   }
@@ -990,8 +999,8 @@ __global__ void __launch_bounds__(32 * Kof(deg_of(K - 1) - 1)) k_elem_corr_split
       for (int f = 0; f < 3; ++f) {
         T acc = 0;
         sfor<0, KL>([&](auto M) {
-          if constexpr (dxnz(q, M)) acc += cDx[q][M] * B[M][2 * f][lane];
-          if constexpr (dsnz(q, M)) acc += cDs[q][M] * B[M][2 * f + 1][lane];
+          if constexpr (dxnz(q, M)) acc = fma(cDx[q][M], B[M][2 * f][lane], acc);
+          if constexpr (dsnz(q, M)) acc = fma(cDs[q][M], B[M][2 * f + 1][lane], acc);
         });
         r[f] = f == 0 ? acc : rs * acc;
       }

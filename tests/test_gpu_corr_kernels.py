@@ -57,3 +57,29 @@ def test_correction_kernels_on_ragged_groups(prec, nx, ny):
     """every order at once, groups of a few elements and around a warp, all source terms"""
     err = rhs_errors(lambda n: (np.arange(n) % 5).astype(np.int8), nx, ny, prec, fric_lin=1e-4, fric_quad=0.009, f_c=1e-2)
     assert max(err) < TOL[prec], err
+
+
+@pytest.mark.parametrize("p,sizes", [(4, [(50, 60), (40, 50)]), (3, [(64, 78), (50, 60)]), (2, [(100, 100), (60, 70)])])
+def test_member_alone_and_in_a_union_across_the_size_rule_bitwise(p, sizes):
+    """alone the first member's group is at most 60,000 / K(p-1) elements, in the union it is more"""
+    from paper_2311_11348_gb300.ensemble import Ensemble
+    members, states = [], []
+    for k, (nx, ny) in enumerate(sizes):
+        n = max(nx, ny)
+        xy, tri = inputs.split_square_mesh(n, 1e3, jitter=0.2, seed=7 + k)
+        tri = np.ascontiguousarray(tri.reshape(n, n, 2, 3)[:nx, :ny].reshape(-1, 3))
+        members.append(dict(xy=xy, tri=tri, hv=inputs.fourier_bathymetry(xy, 1e3, lo=10.0, hi=50.0, seed=2 + k),
+                            orders=np.full(len(tri), p, np.int8)))
+        rng = np.random.default_rng(5 + k)
+        K = (p + 1) * (p + 2) // 2
+        c = np.zeros((3, swedg.KMAX, len(tri)))
+        c[:, :K] = rng.standard_normal((3, K, len(tri))) * 0.1
+        states.append(c)
+    out = []
+    for ms, cs in ((members[:1], states[:1]), (members, states)):
+        e = Ensemble(ms, g=9.81, rk_order=3, precision=swedg.PREC_MIXED_FP32)
+        e.set_states(cs)
+        e.run(2)
+        out.append(e.states()[0])
+        e.close()
+    assert np.isfinite(out[0]).all() and np.array_equal(out[0], out[1])
