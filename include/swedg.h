@@ -372,10 +372,11 @@ int swe_profile_read(swe_ctx* ctx, int n, const char** names, double* ms, int64_
  *   nbr[ne][3]  element across the edge opposite vertex k, or -1 (land)
  *   c[3][3][ne] modes 1..3 of xi, U, V (the basis of the context layout)
  *   rhs_out[3][3][ne]  the right-hand side of those modes
- * The intermediate values -- the auxiliary velocity u and the flux of every
- * edge at its two Gauss points -- live in one file-scope __device__ array
- * sized for SWE_NOALLOC_MAX_ELEMENTS elements (24 doubles each, 12.6 MB),
- * which every GPU that loads the library holds until the process exits.
+ * The intermediate values -- the auxiliary velocity u and the flux moments of
+ * every edge -- live in file-scope __device__ arrays sized for
+ * SWE_NOALLOC_MAX_ELEMENTS elements (24 doubles and a byte each, 12.6 MB),
+ * which every GPU that loads the library holds until the process exits;
+ * rhs_out holds intermediate values too until the call's last kernel has run.
  * Errors: SWE_EINVAL for ne < 1, ne > SWE_NOALLOC_MAX_ELEMENTS, nv < 3,
  * g not in (0, inf) or a NULL array; SWE_ECUDA when a launch fails, or when
  * the calling thread already had a CUDA error pending on entry (it is
@@ -387,10 +388,9 @@ int swe_profile_read(swe_ctx* ctx, int n, const char** names, double* ms, int64_
  *    with n in [0, ne), n usable, and e in n's own list; otherwise (an id
  *    outside [0, ne), a one-sided entry) the edge is land for e.
  * No depth or finiteness status is reported (there is no context to hold it).
- * The first call on a device context copies the reference tables to constant
- * memory and looks up the device address of the scratch array
- * (cudaMemcpyToSymbol, cudaGetSymbolAddress; no allocation); make that first
- * call before any stream capture.  The set-up is serialised across host
+ * The first call on a device context looks up the device addresses of the
+ * scratch arrays (cudaGetSymbolAddress; no allocation); make that first call
+ * before any stream capture.  The set-up is serialised across host
  * threads and repeated when the device's context is re-created (for
  * instance after cudaDeviceReset).  Every call shares the one scratch array
  * and leaves its contents behind; nothing in it needs to start at zero (each

@@ -12,43 +12,46 @@
 // process exits.  The caller passes inputs and outputs; nothing else is
 // allocated, by this file or by any library it calls.
 //
-// The same arithmetic as the context path (k_usolve_base, k_edge_base,
-// k_elem_base): Sect. 2-3 of the paper for p = 1 with land walls.
+// Sect. 2-3 of the paper for p = 1 with land walls, in the vertex values of the
+// linear fields (equal to the modal form in exact arithmetic): with every
+// quantity at the vertices the traces on an edge are its two ends' values, the
+// element's gradients and the edge normals are coordinate differences, and
+// the areas cancel, so that the only square roots are one per element (the scale
+// of its orthonormal basis) and one per edge (lambda), and there is no division
+// but the solve's.  FP64 instructions bound these kernels (GB300: 19 cycles of
+// an SM each, 64 of the warp): about 95 per element in k_na_usolve, 97 per edge,
+// 130 per element in k_na_elem, where the modal form with its geometry formed at
+// every visit took 1,900 per element; 72 -> 40 us for 20,000 elements (GB300).
 #include <cuda.h>
 
 #include <cmath>
-#include <cstring>
 #include <mutex>
 
 #include "../../include/swedg.h"
 #include "common.h"
-#include "kernels.h"
-#include "tables.h"
 
 namespace swedg {
 namespace na {
 
 constexpr int64_t NMAX = SWE_NOALLOC_MAX_ELEMENTS;
-// per element: u [2][3] and edge flux [3 fields][2 points][3 local edges]
+// per element: u, v at the three vertices, then the edge flux's moments
+// [3 fields][2 ends][3 local edges]
 constexpr int64_t PER_ELEM = 6 + 18;
 static __device__ __align__(256) double g_na_scratch[PER_ELEM * NMAX];
+static __device__ __align__(256) unsigned char g_na_ok[NMAX];  // 1: a usable element (see elem_ok)
 
-__constant__ double nB2[3][3][2];  // phihat_i(gamma_k(s_g)), i < 3, two-point rule
-__constant__ double nW2[2], nS2[2];
-__constant__ double nT1[3][3][3];  // T[n][i][j], n, i, j < 3
-__constant__ double nLv[3][3];     // int lambda_v phihat_i
-__constant__ double nGrad[3][2];   // grad phihat_q, q < 3
-__constant__ double nPhi0;
-
-// Set-up once per device context (with that device current): tables into
-// constant memory and the device address of the scratch array.  The context
-// is identified by its driver id, so a context re-created after
-// cudaDeviceReset (whose constant memory starts zeroed) is set up again; a
-// mutex serialises the set-up of host threads that call at the same time.
+// Set-up once per device context (with that device current): the device
+// addresses of the scratch arrays.  The context is identified by its driver
+// id, so a context re-created after cudaDeviceReset is set up again; a mutex
+// serialises the set-up of host threads that call at the same time.
+struct Scratch {
+  double* v = nullptr;
+  unsigned char* ok = nullptr;
+};
 struct DevState {
   bool ready = false;
   unsigned long long ctx_id = 0;
-  double* scratch = nullptr;
+  Scratch scratch;
 };
 static DevState g_dev[64];
 static std::mutex g_setup_mutex;
@@ -80,7 +83,7 @@ static unsigned long long current_ctx_id() {
   return id;
 }
 
-static int setup(int dev, double** scratch) {
+static int setup(int dev, Scratch* scratch) {
   if (dev < 0 || dev >= 64) return SWE_EINVAL;
   std::lock_guard<std::mutex> lock(g_setup_mutex);
   const unsigned long long id0 = current_ctx_id();
@@ -89,71 +92,33 @@ static int setup(int dev, double** scratch) {
     return 0;
   }
   // the symbol lookup also makes the device's primary context current
-  void* p = nullptr;
-  if (cudaGetSymbolAddress(&p, g_na_scratch) != cudaSuccess || p == nullptr) return SWE_ECUDA;
-  const unsigned long long id = current_ctx_id();
-  if (g_dev[dev].ready && id != 0 && id == g_dev[dev].ctx_id) {
-    *scratch = g_dev[dev].scratch;
-    return 0;
-  }
+  void *p = nullptr, *q = nullptr;
   g_dev[dev].ready = false;
-  const RefTables& R = tables();
-  double B[3][3][2], T1[3][3][3], Lv[3][3], Gr[3][2];
-  for (int k = 0; k < 3; ++k)
-    for (int i = 0; i < 3; ++i)
-      for (int g = 0; g < 2; ++g) B[k][i][g] = R.EB[2][k][i][g];
-  for (int n = 0; n < 3; ++n)
-    for (int i = 0; i < 3; ++i)
-      for (int j = 0; j < 3; ++j) T1[n][i][j] = R.T[n][i][j];
-  std::memcpy(Lv, R.Lv, sizeof Lv);
-  std::memcpy(Gr, R.grad1, sizeof Gr);
-  if (cudaMemcpyToSymbol(nB2, B, sizeof B) != cudaSuccess ||
-      cudaMemcpyToSymbol(nW2, R.ew[2], sizeof(double) * 2) != cudaSuccess ||
-      cudaMemcpyToSymbol(nS2, R.es[2], sizeof(double) * 2) != cudaSuccess ||
-      cudaMemcpyToSymbol(nT1, T1, sizeof T1) != cudaSuccess || cudaMemcpyToSymbol(nLv, Lv, sizeof Lv) != cudaSuccess ||
-      cudaMemcpyToSymbol(nGrad, Gr, sizeof Gr) != cudaSuccess ||
-      cudaMemcpyToSymbol(nPhi0, &R.phi0, sizeof(double)) != cudaSuccess)
-    return SWE_ECUDA;
-  g_dev[dev].scratch = (double*)p;
-  g_dev[dev].ctx_id = id;
+  if (cudaGetSymbolAddress(&p, g_na_scratch) != cudaSuccess || p == nullptr) return SWE_ECUDA;
+  if (cudaGetSymbolAddress(&q, g_na_ok) != cudaSuccess || q == nullptr) return SWE_ECUDA;
+  g_dev[dev].scratch.v = (double*)p;
+  g_dev[dev].scratch.ok = (unsigned char*)q;
+  g_dev[dev].ctx_id = current_ctx_id();
   g_dev[dev].ready = true;
-  *scratch = (double*)p;
+  *scratch = g_dev[dev].scratch;
   return 0;
 }
 
-struct Geo {
-  double rs, s, Ji[4];
+struct P2 {
+  double x, y;
 };
 
-__device__ __forceinline__ Geo element_geo(const double* __restrict__ xy, const int32_t* __restrict__ tri, int64_t e) {
-  const int32_t v0 = tri[3 * e], v1 = tri[3 * e + 1], v2 = tri[3 * e + 2];
-  const double x0 = xy[2 * v0], y0 = xy[2 * v0 + 1];
-  const double J00 = xy[2 * v1] - x0, J01 = xy[2 * v2] - x0;
-  const double J10 = xy[2 * v1 + 1] - y0, J11 = xy[2 * v2 + 1] - y0;
-  const double det = J00 * J11 - J01 * J10;
-  Geo G;
-  G.s = sqrt(det);
-  G.rs = 1.0 / G.s;
-  G.Ji[0] = J11 / det; G.Ji[1] = -J01 / det; G.Ji[2] = -J10 / det; G.Ji[3] = J00 / det;
-  return G;
-}
-
-__device__ __forceinline__ void hb_modes(const double* __restrict__ hv, const int32_t* __restrict__ tri, int64_t e,
-                                         double s, double (&hb)[3]) {
-  const double h[3] = {hv[tri[3 * e]], hv[tri[3 * e + 1]], hv[tri[3 * e + 2]]};
-#pragma unroll
-  for (int i = 0; i < 3; ++i) hb[i] = s * (h[0] * nLv[0][i] + h[1] * nLv[1][i] + h[2] * nLv[2][i]);
+__device__ __forceinline__ P2 vertex(const double* __restrict__ xy, int64_t v) {
+  return P2{xy[2 * v], xy[2 * v + 1]};  // 8-byte loads: the caller's array may start anywhere
 }
 
 // An element is used only when its vertex ids lie in [0, nv) and it is
 // counter-clockwise with positive area (det J_e > 0); any other element gets
 // NaN rows and is a land edge to its neighbours.
-__device__ __forceinline__ bool elem_ok(const double* __restrict__ xy, const int32_t* __restrict__ tri, int64_t nv,
-                                        int64_t e) {
-  const int32_t a = tri[3 * e], b = tri[3 * e + 1], c = tri[3 * e + 2];
-  if (!(a >= 0 && b >= 0 && c >= 0 && a < nv && b < nv && c < nv)) return false;
-  const double x0 = xy[2 * a], y0 = xy[2 * a + 1];
-  const double det = (xy[2 * b] - x0) * (xy[2 * c + 1] - y0) - (xy[2 * c] - x0) * (xy[2 * b + 1] - y0);
+__device__ __forceinline__ bool elem_ok(const double* __restrict__ xy, const int32_t (&v)[3], int64_t nv, double& det) {
+  if (!(v[0] >= 0 && v[1] >= 0 && v[2] >= 0 && v[0] < nv && v[1] < nv && v[2] < nv)) return false;
+  const P2 a = vertex(xy, v[0]), b = vertex(xy, v[1]), c = vertex(xy, v[2]);
+  det = (b.x - a.x) * (c.y - a.y) - (c.x - a.x) * (b.y - a.y);
   return det > 0.0;
 }
 
@@ -162,190 +127,277 @@ __device__ __forceinline__ bool elem_ok(const double* __restrict__ xy, const int
 // neighbour, or one whose own list does not name e.  Both the edge and the
 // element kernel decide through this one function, so every flux slot an
 // element reads was written by the same call.
-__device__ __forceinline__ int64_t mutual_nbr(const double* __restrict__ xy, const int32_t* __restrict__ tri,
-                                              const int32_t* __restrict__ nbr, int64_t nv, int64_t ne, int64_t e,
-                                              int k, int& kn) {
+__device__ __forceinline__ int64_t mutual_nbr(const int32_t* __restrict__ nbr, const unsigned char* __restrict__ ok,
+                                              int64_t ne, int64_t e, int k, int& kn) {
   const int64_t n = nbr[3 * e + k];
-  if (n < 0 || n >= ne || n == e || !elem_ok(xy, tri, nv, n)) return -1;
+  if (n < 0 || n >= ne || n == e || !ok[n]) return -1;
   for (int j = 0; j < 3; ++j)
     if (nbr[3 * n + j] == e) { kn = j; return n; }
   return -1;
 }
 
-// auxiliary system of Sect. 3 for p = 1 (3 x 3, adjugate)
-__global__ void k_na_usolve(int64_t nv, int64_t ne, const double* __restrict__ xy, const double* __restrict__ hv,
-                            const int32_t* __restrict__ tri, const double* __restrict__ c, double* __restrict__ scr) {
-  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (e >= ne || !elem_ok(xy, tri, nv, e)) return;
-  const Geo G = element_geo(xy, tri, e);
-  double hb[3];
-  hb_modes(hv, tri, e, G.s, hb);
-  double H[3], U[3], V[3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) { H[i] = c[i * ne + e] + hb[i]; U[i] = c[(3 + i) * ne + e]; V[i] = c[(6 + i) * ne + e]; }
-  const double a = H[0] * nT1[0][0][0];
-  const double b = H[0] * nT1[0][0][1] + H[1] * nT1[1][0][1] + H[2] * nT1[2][0][1];
-  const double cc = H[0] * nT1[0][0][2] + H[1] * nT1[1][0][2] + H[2] * nT1[2][0][2];
-  const double d = H[0] * nT1[0][1][1] + H[1] * nT1[1][1][1] + H[2] * nT1[2][1][1];
-  const double f = H[0] * nT1[0][1][2] + H[1] * nT1[1][1][2] + H[2] * nT1[2][1][2];
-  const double h = H[0] * nT1[0][2][2] + H[1] * nT1[1][2][2] + H[2] * nT1[2][2][2];
-  const double C00 = d * h - f * f, C01 = cc * f - b * h, C02 = b * f - cc * d;
-  const double C11 = a * h - cc * cc, C12 = b * cc - a * f, C22 = a * d - b * b;
-  const double r = G.s / (a * C00 + b * C01 + cc * C02);
-  scr[0 * NMAX + e] = (C00 * U[0] + C01 * U[1] + C02 * U[2]) * r;
-  scr[1 * NMAX + e] = (C01 * U[0] + C11 * U[1] + C12 * U[2]) * r;
-  scr[2 * NMAX + e] = (C02 * U[0] + C12 * U[1] + C22 * U[2]) * r;
-  scr[3 * NMAX + e] = (C00 * V[0] + C01 * V[1] + C02 * V[2]) * r;
-  scr[4 * NMAX + e] = (C01 * V[0] + C11 * V[1] + C12 * V[2]) * r;
-  scr[5 * NMAX + e] = (C02 * V[0] + C12 * V[1] + C22 * V[2]) * r;
+// The degree-1 modes at the vertices are (sqrt 2, -+sqrt 12, -2), (.., +sqrt 12,
+// -2), (sqrt 2, 0, 4) over s = sqrt det: vertex values of one field's modes.
+constexpr double kR2 = 1.4142135623730951, kR12 = 3.4641016151377544;
+__device__ __forceinline__ void to_vertices(const double* c, int64_t ne, double rs, double (&n)[3]) {
+  const double c2 = (2.0 * rs) * c[2 * ne], c1 = (kR12 * rs) * c[ne];
+  const double a = (kR2 * rs) * c[0], b = a - c2;
+  n[0] = b - c1;
+  n[1] = b + c1;
+  n[2] = fma(2.0, c2, a);
 }
 
-// P1 traces of xi, U, V, u, v of element e on its local edge k at the two points
-__device__ __forceinline__ void traces(const double* __restrict__ c, const double* __restrict__ scr, int64_t ne,
-                                       int64_t e, int k, bool reverse, double rs, double (&t)[5][2]) {
-#pragma unroll
-  for (int g = 0; g < 2; ++g) {
-    const int gg = reverse ? 1 - g : g;
-#pragma unroll
-    for (int f = 0; f < 5; ++f) {
-      double acc = 0.0;
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        const double coef = f < 3 ? c[(f * 3 + i) * ne + e] : scr[((f - 3) * 3 + i) * NMAX + e];
-        acc += coef * nB2[k][i][gg];
-      }
-      t[f][g] = rs * acc;
-    }
-  }
-}
-
-// LF flux (Sect. 2) of every edge at its two Gauss points, stored once in the
-// slot of its lower-numbered element, pre-weighted by |E| w_g / 2
-__global__ void k_na_edge(int64_t nv, int64_t ne, const double* __restrict__ xy, const double* __restrict__ hv,
-                          const int32_t* __restrict__ tri, const int32_t* __restrict__ nbr,
-                          const double* __restrict__ c, double g, double* __restrict__ scr) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= 3 * ne) return;
-  const int64_t e = t / 3;
-  const int k = (int)(t % 3);
-  if (!elem_ok(xy, tri, nv, e)) return;
-  int kn = 0;
-  const int64_t n = mutual_nbr(xy, tri, nbr, nv, ne, e, k, kn);
-  if (n >= 0 && n < e) return;  // owned by the neighbour
-  const int32_t va = tri[3 * e + (k + 1) % 3], vb = tri[3 * e + (k + 2) % 3];
-  const double dx = xy[2 * vb] - xy[2 * va], dy = xy[2 * vb + 1] - xy[2 * va + 1];
-  const double len = sqrt(dx * dx + dy * dy), nx = dy / len, ny = -dx / len;
-  const double hA = hv[va], hB = hv[vb], hmid = 0.5 * (hA + hB);
-  const Geo GL = element_geo(xy, tri, e);
-  double a[5][2], b[5][2];
-  traces(c, scr, ne, e, k, false, GL.rs, a);
-  const double mL = nPhi0 * GL.rs;
-  const double unL = (scr[0 * NMAX + e] * nx + scr[3 * NMAX + e] * ny) * mL;
-  const double HL = c[e] * mL + hmid;
-  double unR, HR;
-  if (n >= 0) {
-    const Geo GR = element_geo(xy, tri, n);
-    traces(c, scr, ne, n, kn, true, GR.rs, b);
-    const double mR = nPhi0 * GR.rs;
-    unR = (scr[0 * NMAX + n] * nx + scr[3 * NMAX + n] * ny) * mR;
-    HR = c[n] * mR + hmid;
-  } else {  // land: mirror state
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const double qn = a[1][q] * nx + a[2][q] * ny, wn = a[3][q] * nx + a[4][q] * ny;
-      b[0][q] = a[0][q];
-      b[1][q] = a[1][q] - 2.0 * qn * nx; b[2][q] = a[2][q] - 2.0 * qn * ny;
-      b[3][q] = a[3][q] - 2.0 * wn * nx; b[4][q] = a[4][q] - 2.0 * wn * ny;
-    }
-    unR = -unL;
-    HR = HL;
-  }
-  const double lam = fmax(fabs(unL), fabs(unR)) + fmax(sqrt(g * HL), sqrt(g * HR));
-  double* F = scr + 6 * NMAX;
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const double hb = hA + nS2[q] * (hB - hA);
-    const double wa = a[3][q] * nx + a[4][q] * ny, wb = b[3][q] * nx + b[4][q] * ny;
-    const double pa = g * a[0][q] * (0.5 * a[0][q] + hb), pb = g * b[0][q] * (0.5 * b[0][q] + hb);
-    const double F0 = (a[1][q] + b[1][q]) * nx + (a[2][q] + b[2][q]) * ny + lam * (a[0][q] - b[0][q]);
-    const double F1 = a[1][q] * wa + b[1][q] * wb + (pa + pb) * nx + lam * (a[1][q] - b[1][q]);
-    const double F2 = a[2][q] * wa + b[2][q] * wb + (pa + pb) * ny + lam * (a[2][q] - b[2][q]);
-    const double wgt = 0.5 * len * nW2[q];
-    F[((0 * 2 + q) * 3 + k) * NMAX + e] = wgt * F0;
-    F[((1 * 2 + q) * 3 + k) * NMAX + e] = wgt * F1;
-    F[((2 * 2 + q) * 3 + k) * NMAX + e] = wgt * F2;
-  }
-}
-
-// volume, source and edge terms of the degree <= 1 test modes (closed form)
-__global__ void k_na_elem(int64_t nv, int64_t ne, const double* __restrict__ xy, const double* __restrict__ hv,
-                          const int32_t* __restrict__ tri, const int32_t* __restrict__ nbr,
-                          const double* __restrict__ c, double g, const double* __restrict__ scr,
-                          double* __restrict__ rhs) {
+// The element's fields at its vertices, into rhs (the caller's output array serves
+// as their buffer until k_na_elem overwrites it; a call with rhs == c works
+// too, k_na_elem reads nothing else of c), and the auxiliary system of Sect. 3:
+// sum_k u_k int H lambda_j lambda_k = int U lambda_j with H linear, a 3 x 3
+// symmetric system with entries 2 S + 4 H_j and 2 S - H_l (times det / 120) for
+// S = H_0 + H_1 + H_2, solved with its adjugate.
+__global__ void __launch_bounds__(64) k_na_usolve(int64_t nv, int64_t ne, const double* __restrict__ xy,
+                                                  const double* __restrict__ hv, const int32_t* __restrict__ tri,
+                                                  const double* c, double* rhs, double* __restrict__ scr,
+                                                  unsigned char* __restrict__ ok) {
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= ne) return;
-  if (!elem_ok(xy, tri, nv, e)) {  // unusable element: NaN rows, nothing read
+  const int32_t v[3] = {tri[3 * e], tri[3 * e + 1], tri[3 * e + 2]};
+  double det = 0.0;
+  const bool good = elem_ok(xy, v, nv, det);
+  ok[e] = good;
+  if (!good) return;
+  const double rs = rsqrt(det);
+  double f[3][3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) to_vertices(c + 3 * i * ne + e, ne, rs, f[i]);
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) rhs[(3 * i + j) * ne + e] = f[i][j];
+  const double H0 = hv[v[0]] + f[0][0], H1 = hv[v[1]] + f[0][1], H2 = hv[v[2]] + f[0][2];
+  const double S2 = 2.0 * (H0 + H1 + H2);
+  const double a = fma(4.0, H0, S2), d = fma(4.0, H1, S2), h = fma(4.0, H2, S2);
+  const double b = S2 - H2, cc = S2 - H1, g = S2 - H0;  // entries (0,1), (0,2), (1,2)
+  const double C00 = d * h - g * g, C01 = cc * g - b * h, C02 = b * g - cc * d;
+  const double C11 = a * h - cc * cc, C12 = b * cc - a * g, C22 = a * d - b * b;
+  const double r = 5.0 / (a * C00 + b * C01 + cc * C02);
+#pragma unroll
+  for (int i = 1; i < 3; ++i) {  // int U lambda_j = det / 24 (U_0 + U_1 + U_2 + U_j)
+    const double s = f[i][0] + f[i][1] + f[i][2];
+    const double b0 = (s + f[i][0]) * r, b1 = (s + f[i][1]) * r, b2 = (s + f[i][2]) * r;
+    scr[(3 * (i - 1) + 0) * NMAX + e] = C00 * b0 + C01 * b1 + C02 * b2;
+    scr[(3 * (i - 1) + 1) * NMAX + e] = C01 * b0 + C11 * b1 + C12 * b2;
+    scr[(3 * (i - 1) + 2) * NMAX + e] = C02 * b0 + C12 * b1 + C22 * b2;
+  }
+}
+
+// One side of an edge: xi, U, V, w = u.N at its two ends A, B (N the scaled
+// normal), and the element means of w and xi.
+struct Side {
+  double x[2], U[2], V[2], w[2], wm, xm;
+};
+__device__ __forceinline__ Side side(const double* f, const double* __restrict__ scr, int64_t ne, int64_t e, int ia,
+                                     int ib, int ic, double Nx, double Ny) {
+  Side s;
+  const int i[2] = {ia, ib};
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    s.x[a] = f[i[a] * ne + e];
+    s.U[a] = f[(3 + i[a]) * ne + e];
+    s.V[a] = f[(6 + i[a]) * ne + e];
+    s.w[a] = scr[i[a] * NMAX + e] * Nx + scr[(3 + i[a]) * NMAX + e] * Ny;
+  }
+  const double wc = scr[ic * NMAX + e] * Nx + scr[(3 + ic) * NMAX + e] * Ny;
+  s.wm = (s.w[0] + s.w[1] + wc) * (1.0 / 3.0);
+  s.xm = (s.x[0] + s.x[1] + f[ic * ne + e]) * (1.0 / 3.0);
+  return s;
+}
+
+// LF flux (Sect. 2) of every edge, as its moments with the two linear functions
+// that are 1 at one end: for products of two linear functions a b these are
+// |E| / 12 (2 a_A b_A + (a_A + a_B)(b_A + b_B)) and alike for B, for a linear F
+// |E| / 6 (2 F_A + F_B); a half of each is taken for the flux average.  Stored
+// once in the slot of the lower-numbered element.  A block takes the 3 ET edges
+// of ET elements and first packs those it owns (half of them on average): an
+// FP64 instruction takes its 64 cycles for one active lane as for 32.
+constexpr int ET = 40, BT = 64;
+__global__ void __launch_bounds__(BT) k_na_edge(int64_t ne, const double* __restrict__ xy,
+                                                const double* __restrict__ hv, const int32_t* __restrict__ tri,
+                                                const int32_t* __restrict__ nbr, const double* f, double g,
+                                                double* __restrict__ scr, const unsigned char* __restrict__ ok) {
+  __shared__ int32_t own[3 * ET], own_n[3 * ET];  // local edge of the block << 2 | neighbour's local edge; neighbour
+  __shared__ int count[(3 * ET + 31) / 32 + 1];
+  const int64_t e0 = blockIdx.x * (int64_t)ET;
+  const int lane = threadIdx.x & 31;
+  constexpr int NC = (3 * ET + BT - 1) / BT;
+  int kn[NC], mine[NC], rank[NC];
+  int64_t nn[NC];
+#pragma unroll
+  for (int r = 0; r < NC; ++r) {
+    const int t = r * BT + threadIdx.x;
+    const int64_t e = e0 + t / 3;
+    kn[r] = 0;
+    nn[r] = -1;
+    mine[r] = 0;
+    if (t < 3 * ET && e < ne && ok[e]) {
+      nn[r] = mutual_nbr(nbr, ok, ne, e, t % 3, kn[r]);
+      mine[r] = nn[r] < 0 || nn[r] > e;  // else owned by the neighbour
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, mine[r]);
+    rank[r] = __popc(m & ((1u << lane) - 1u));
+    if (lane == 0 && t / 32 < (3 * ET + 31) / 32) count[t / 32] = __popc(m);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int s = 0;
+    for (int i = 0; i < (3 * ET + 31) / 32; ++i) {
+      const int x = count[i];
+      count[i] = s;
+      s += x;
+    }
+    count[(3 * ET + 31) / 32] = s;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < NC; ++r)
+    if (mine[r]) {
+      const int t = r * BT + threadIdx.x, p = count[t / 32] + rank[r];
+      own[p] = t << 2 | kn[r];
+      own_n[p] = (int32_t)nn[r];
+    }
+  __syncthreads();
+  const int total = count[(3 * ET + 31) / 32];
+  for (int p = threadIdx.x; p < total; p += BT) {
+    const int t = own[p] >> 2, kr = own[p] & 3, k = t % 3;
+    const int64_t e = e0 + t / 3, n = own_n[p];
+    const int ia = k == 2 ? 0 : k + 1, ib = k == 0 ? 2 : k - 1;
+    const int32_t va = tri[3 * e + ia], vb = tri[3 * e + ib];
+    const P2 A = vertex(xy, va), B = vertex(xy, vb);
+    // |E| / 24 times the unit normal carries the weights of the momentum rows
+    const double Nx = (B.y - A.y) * (1.0 / 24.0), Ny = (A.x - B.x) * (1.0 / 24.0);
+    const double hA = hv[va], hB = hv[vb], hm = 0.5 * (hA + hB), N2 = Nx * Nx + Ny * Ny;
+    Side a = side(f, scr, ne, e, ia, ib, k, Nx, Ny), b;
+    if (n >= 0) {  // the neighbour runs the edge the other way
+      b = side(f, scr, ne, n, kr == 0 ? 2 : kr - 1, kr == 2 ? 0 : kr + 1, kr, Nx, Ny);
+    } else {  // land: mirror state
+      const double r = 2.0 / N2;
+      b = a;
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const double qn = (a.U[q] * Nx + a.V[q] * Ny) * r;
+        b.U[q] = a.U[q] - qn * Nx;
+        b.V[q] = a.V[q] - qn * Ny;
+        b.w[q] = -a.w[q];
+      }
+      b.wm = -a.wm;
+    }
+    const double lam = fmax(fabs(a.wm), fabs(b.wm)) + sqrt(N2 * (g * (fmax(a.xm, b.xm) + hm)));
+    double* F = scr + 6 * NMAX + e;
+    // elevation row: linear
+    double FA = (a.U[0] + b.U[0]) * Nx + (a.V[0] + b.V[0]) * Ny + lam * (a.x[0] - b.x[0]);
+    double FB = (a.U[1] + b.U[1]) * Nx + (a.V[1] + b.V[1]) * Ny + lam * (a.x[1] - b.x[1]);
+    F[(0 * 3 + k) * NMAX] = 2.0 * fma(2.0, FA, FB);
+    F[(1 * 3 + k) * NMAX] = 2.0 * fma(2.0, FB, FA);
+    // momentum rows: U (w + lambda) + U+ (w+ - lambda) + (P + P+) N
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      a.w[q] += lam;
+      b.w[q] -= lam;
+    }
+    const double wa = a.w[0] + a.w[1], wb = b.w[0] + b.w[1];
+    const double xa = a.x[0] + a.x[1], xb = b.x[0] + b.x[1];
+    const double gNx = g * Nx, gNy = g * Ny, hs = hA + hB;
+    const double PA = a.x[0] * fma(0.5, a.x[0], hA) + b.x[0] * fma(0.5, b.x[0], hA);
+    const double PB = a.x[1] * fma(0.5, a.x[1], hB) + b.x[1] * fma(0.5, b.x[1], hB);
+    const double PS = xa * fma(0.5, xa, hs) + xb * fma(0.5, xb, hs);
+    const double XA = a.U[0] * a.w[0] + b.U[0] * b.w[0] + PA * gNx, XB = a.U[1] * a.w[1] + b.U[1] * b.w[1] + PB * gNx;
+    const double XS = (a.U[0] + a.U[1]) * wa + (b.U[0] + b.U[1]) * wb + PS * gNx;
+    F[(2 * 3 + k) * NMAX] = fma(2.0, XA, XS);
+    F[(3 * 3 + k) * NMAX] = fma(2.0, XB, XS);
+    const double YA = a.V[0] * a.w[0] + b.V[0] * b.w[0] + PA * gNy, YB = a.V[1] * a.w[1] + b.V[1] * b.w[1] + PB * gNy;
+    const double YS = (a.V[0] + a.V[1]) * wa + (b.V[0] + b.V[1]) * wb + PS * gNy;
+    F[(4 * 3 + k) * NMAX] = fma(2.0, YA, YS);
+    F[(5 * 3 + k) * NMAX] = fma(2.0, YB, YS);
+  }
+}
+
+// Volume, source and edge terms as loads R_j = (.., lambda_j) at the vertices, then
+// the modal rows sum_j phi_q(v_j) R_j.  With d_j = det grad lambda_j (coordinate
+// differences) and the vertex sums the areas cancel: int a b = det / 24
+// (sum a sum b + sum a_j b_j), grad h_b = sum h_j d_j / det.
+__global__ void __launch_bounds__(64) k_na_elem(int64_t ne, const double* __restrict__ xy,
+                                                const double* __restrict__ hv, const int32_t* __restrict__ tri,
+                                                const int32_t* __restrict__ nbr, double g,
+                                                const double* __restrict__ scr, const unsigned char* __restrict__ ok,
+                                                double* rhs) {
+  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (e >= ne) return;
+  if (!ok[e]) {  // unusable element: NaN rows, nothing read
     for (int i = 0; i < 9; ++i) rhs[i * ne + e] = __longlong_as_double(0x7ff8000000000000LL);
     return;
   }
-  const Geo G = element_geo(xy, tri, e);
-  double hb[3];
-  hb_modes(hv, tri, e, G.s, hb);
-  double cc[3][3], u[2][3];
+  const int32_t v[3] = {tri[3 * e], tri[3 * e + 1], tri[3 * e + 2]};
+  const P2 p[3] = {vertex(xy, v[0]), vertex(xy, v[1]), vertex(xy, v[2])};
+  const double dx[3] = {p[1].y - p[2].y, p[2].y - p[0].y, p[0].y - p[1].y};
+  const double dy[3] = {p[2].x - p[1].x, p[0].x - p[2].x, p[1].x - p[0].x};
+  const double h[3] = {hv[v[0]], hv[v[1]], hv[v[2]]};
+  double f[3][3], u[2][3];
 #pragma unroll
-  for (int f = 0; f < 3; ++f)
+  for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int i = 0; i < 3; ++i) cc[f][i] = c[(f * 3 + i) * ne + e];
+    for (int j = 0; j < 3; ++j) f[i][j] = rhs[(3 * i + j) * ne + e];
 #pragma unroll
-  for (int f = 0; f < 2; ++f)
+  for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int i = 0; i < 3; ++i) u[f][i] = scr[(f * 3 + i) * NMAX + e];
-  const int32_t v0 = tri[3 * e], v1 = tri[3 * e + 1], v2 = tri[3 * e + 2];
-  const double dh1 = hv[v1] - hv[v0], dh2 = hv[v2] - hv[v0];
-  const double dhx = dh1 * G.Ji[0] + dh2 * G.Ji[2], dhy = dh1 * G.Ji[1] + dh2 * G.Ji[3];
-  double Axx = 0.0, Axy = 0.0, Ayx = 0.0, Ayy = 0.0, P = 0.0;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    Axx += cc[1][i] * u[0][i]; Axy += cc[1][i] * u[1][i];
-    Ayx += cc[2][i] * u[0][i]; Ayy += cc[2][i] * u[1][i];
-    P += cc[0][i] * (0.5 * cc[0][i] + hb[i]);
-  }
-  P *= g;
-  const double m0 = G.s / nPhi0;
-  double r[3][3];
-  r[0][0] = 0.0;
-  r[1][0] = g * dhx * cc[0][0];
-  r[2][0] = g * dhy * cc[0][0];
-#pragma unroll
-  for (int q = 1; q < 3; ++q) {
-    const double gx = G.rs * (nGrad[q][0] * G.Ji[0] + nGrad[q][1] * G.Ji[2]);
-    const double gy = G.rs * (nGrad[q][0] * G.Ji[1] + nGrad[q][1] * G.Ji[3]);
-    r[0][q] = (gx * cc[1][0] + gy * cc[2][0]) * m0;
-    r[1][q] = gx * (Axx + P) + gy * Axy + g * dhx * cc[0][q];
-    r[2][q] = gx * Ayx + gy * (Ayy + P) + g * dhy * cc[0][q];
-  }
-  const double* F = scr + 6 * NMAX;
+    for (int j = 0; j < 3; ++j) u[i][j] = scr[(3 * i + j) * NMAX + e];
+  // the edges' moments, collected at the vertices (- for the flux's own direction)
+  double R[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     int kn = 0;
-    const int64_t n = mutual_nbr(xy, tri, nbr, nv, ne, e, k, kn);
+    const int64_t n = mutual_nbr(nbr, ok, ne, e, k, kn);
     const bool right = n >= 0 && n < e;  // the flux is stored by the neighbour, in its direction
-    const int64_t owner = right ? n : e;
+    const double* F = scr + 6 * NMAX + (right ? n : e);
     const int ko = right ? kn : k;
-    const double sg = right ? G.rs : -G.rs;
+    const unsigned long long neg = right ? 0ull : 0x8000000000000000ull;
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      const double b0 = right ? nB2[k][q][1] : nB2[k][q][0];
-      const double b1 = right ? nB2[k][q][0] : nB2[k][q][1];
-#pragma unroll
-      for (int f = 0; f < 3; ++f)
-        r[f][q] += sg * (F[((f * 2 + 0) * 3 + ko) * NMAX + owner] * b0 + F[((f * 2 + 1) * 3 + ko) * NMAX + owner] * b1);
+    for (int i = 0; i < 3; ++i) {
+      const double a = F[((2 * i + (right ? 1 : 0)) * 3 + ko) * NMAX], b = F[((2 * i + (right ? 0 : 1)) * 3 + ko) * NMAX];
+      R[i][(k + 1) % 3] += __longlong_as_double(__double_as_longlong(a) ^ neg);
+      R[i][(k + 2) % 3] += __longlong_as_double(__double_as_longlong(b) ^ neg);
     }
   }
+  const double xs = f[0][0] + f[0][1] + f[0][2], Us = f[1][0] + f[1][1] + f[1][2], Vs = f[2][0] + f[2][1] + f[2][2];
+  const double us = u[0][0] + u[0][1] + u[0][2], vs = u[1][0] + u[1][1] + u[1][2];
+  double Axx = Us * us, Axy = Us * vs, Ayx = Vs * us, Ayy = Vs * vs;
+  double q[3], P = 0.0;
 #pragma unroll
-  for (int f = 0; f < 3; ++f)
+  for (int j = 0; j < 3; ++j) {
+    Axx += f[1][j] * u[0][j]; Axy += f[1][j] * u[1][j];
+    Ayx += f[2][j] * u[0][j]; Ayy += f[2][j] * u[1][j];
+    q[j] = fma(0.5, f[0][j], h[j]);
+    P += f[0][j] * q[j];
+  }
+  P = g * fma(xs, q[0] + q[1] + q[2], P);
+  constexpr double r24 = 1.0 / 24.0;
+  Axx = (Axx + P) * r24; Axy *= r24; Ayx *= r24; Ayy = (Ayy + P) * r24;
+  const double g24 = g * r24, hx = g24 * (h[0] * dx[0] + h[1] * dx[1] + h[2] * dx[2]);
+  const double hy = g24 * (h[0] * dy[0] + h[1] * dy[1] + h[2] * dy[2]);
+  const double U6 = Us * (1.0 / 6.0), V6 = Vs * (1.0 / 6.0);
 #pragma unroll
-    for (int q = 0; q < 3; ++q) rhs[(f * 3 + q) * ne + e] = r[f][q];
+  for (int j = 0; j < 3; ++j) {
+    const double xj = xs + f[0][j];
+    R[0][j] += dx[j] * U6 + dy[j] * V6;
+    R[1][j] += dx[j] * Axx + dy[j] * Axy + hx * xj;
+    R[2][j] += dx[j] * Ayx + dy[j] * Ayy + hy * xj;
+  }
+  const double det = dy[2] * dx[1] - dy[1] * dx[2];
+  const double rs = rsqrt(det), t0 = kR2 * rs, t1 = kR12 * rs, t2 = 2.0 * rs;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const double s = R[i][0] + R[i][1];
+    rhs[(3 * i + 0) * ne + e] = t0 * (s + R[i][2]);
+    rhs[(3 * i + 1) * ne + e] = t1 * (R[i][1] - R[i][0]);
+    rhs[(3 * i + 2) * ne + e] = t2 * fma(2.0, R[i][2], -s);
+  }
 }
 
 }  // namespace na
@@ -362,15 +414,16 @@ extern "C" int swe_rhs_p1_noalloc(int64_t nv, const double* xy, const double* hv
   if (cudaGetLastError() != cudaSuccess) return SWE_ECUDA;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return SWE_ECUDA;
-  double* scr = nullptr;
+  na::Scratch scr;
   const int rc = na::setup(dev, &scr);
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
-  const int T = 128;
-  na::k_na_usolve<<<(unsigned)((ne + T - 1) / T), T, 0, s>>>(nv, ne, xy, hv, tri, c, scr);
+  const int T = 64;
+  const unsigned nb = (unsigned)((ne + T - 1) / T);
+  na::k_na_usolve<<<nb, T, 0, s>>>(nv, ne, xy, hv, tri, c, rhs_out, scr.v, scr.ok);
   if (cudaGetLastError() != cudaSuccess) return SWE_ECUDA;
-  na::k_na_edge<<<(unsigned)((3 * ne + T - 1) / T), T, 0, s>>>(nv, ne, xy, hv, tri, nbr, c, g, scr);
+  na::k_na_edge<<<(unsigned)((ne + na::ET - 1) / na::ET), na::BT, 0, s>>>(ne, xy, hv, tri, nbr, rhs_out, g, scr.v, scr.ok);
   if (cudaGetLastError() != cudaSuccess) return SWE_ECUDA;
-  na::k_na_elem<<<(unsigned)((ne + T - 1) / T), T, 0, s>>>(nv, ne, xy, hv, tri, nbr, c, g, scr, rhs_out);
+  na::k_na_elem<<<nb, T, 0, s>>>(ne, xy, hv, tri, nbr, g, scr.v, scr.ok, rhs_out);
   return cudaGetLastError() == cudaSuccess ? 0 : SWE_ECUDA;
 }
