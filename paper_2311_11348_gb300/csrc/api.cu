@@ -456,7 +456,7 @@ static int regroup(swe_ctx* ctx, bool keep_state) {
   nvtxRangePushA("regroup");
   const int64_t packed_before = ctx->packed_n;
   if (keep_state)  // the state in the old internal order, out to the caller layout
-    CK(launch_to_user(ctx->stream, ctx->dm, ctx->G, ctx->d_perm, nullptr, ctx->corr32, ctx->st[0], ctx->d_user));
+    CK(launch_to_user(ctx->stream, ctx->dm, ctx->G, ctx->dout.inv, nullptr, 0, ctx->corr32, ctx->st[0], ctx->d_user));
   CK(launch_regroup(ctx->stream, ctx->ms, ctx->d_newp, ctx->dout, ctx->rw));
   int64_t info[12] = {};
   CU(cudaMemcpyAsync(info, ctx->rw.info, sizeof info, cudaMemcpyDeviceToHost, ctx->stream));
@@ -470,7 +470,7 @@ static int regroup(swe_ctx* ctx, bool keep_state) {
   if (ctx->fx.Fbc)
     CU(cudaMemsetAsync(ctx->fx.Fbc, 0, sizeof(double) * 6 * (size_t)std::max<int64_t>(ctx->nedge, 1), ctx->stream));
   if (keep_state)
-    CK(launch_from_user(ctx->stream, ctx->dm, ctx->G, ctx->d_perm, nullptr, ctx->corr32, ctx->d_user, ctx->st[0]));
+    CK(launch_from_user(ctx->stream, ctx->dm, ctx->G, ctx->dout.inv, nullptr, 0, ctx->corr32, ctx->d_user, ctx->st[0]));
   if (ctx->packed_n != packed_before)  // the asynchronous staging buffers follow the packed size
     for (int k = 0; k < 2; ++k) {
       if (ctx->d_stage_in[k]) { CU(cudaStreamSynchronize(ctx->cin)); dfree(ctx, ctx->d_stage_in[k]); }
@@ -901,7 +901,7 @@ static int state_in(swe_ctx* ctx, const double* c, int s, bool packed = false) {
     CU(cudaMemcpyAsync(ctx->d_user, c, bytes, cudaMemcpyHostToDevice, ctx->stream));
     src = ctx->d_user;
   }
-  CK(launch_from_user(ctx->stream, ctx->dm, ctx->G, ctx->d_perm, packed ? ctx->d_off : nullptr, ctx->corr32, src,
+  CK(launch_from_user(ctx->stream, ctx->dm, ctx->G, ctx->dout.inv, packed ? ctx->d_off : nullptr, ctx->packed_n, ctx->corr32, src,
                       ctx->st[s]));
   if (s == 0)  // a new state: the members' status starts afresh
     CU(cudaMemsetAsync(ctx->d_mstatus, 0, sizeof(unsigned) * (size_t)ctx->nmem, ctx->stream));
@@ -912,7 +912,7 @@ static int state_out(swe_ctx* ctx, StateDev st, double* c, bool packed = false) 
   const size_t bytes = sizeof(double) * (packed ? (size_t)ctx->packed_n : (size_t)3 * KMAX * ctx->ne);
   const bool dev = is_device_ptr(c);
   double* dst = dev ? c : ctx->d_user2;
-  CK(launch_to_user(ctx->stream, ctx->dm, ctx->G, ctx->d_perm, packed ? ctx->d_off : nullptr, ctx->corr32, st,
+  CK(launch_to_user(ctx->stream, ctx->dm, ctx->G, ctx->dout.inv, packed ? ctx->d_off : nullptr, ctx->packed_n, ctx->corr32, st,
                     dst));
   if (!dev) CU(cudaMemcpyAsync(c, dst, bytes, cudaMemcpyDeviceToHost, ctx->stream));
   CU(cudaStreamSynchronize(ctx->stream));
@@ -1273,7 +1273,7 @@ static int rhs_impl(swe_ctx* ctx, const double* c_in, double* out0, double* out1
   if (!out1) return state_out(ctx, ctx->st[2], out0);
   // order separation: the whole rhs, then the base part alone; corr = whole - base
   const int64_t n = 3 * KMAX * ctx->ne;
-  CK(launch_to_user(ctx->stream, ctx->dm, ctx->G, ctx->d_perm, nullptr, ctx->corr32, ctx->st[2], ctx->d_user));
+  CK(launch_to_user(ctx->stream, ctx->dm, ctx->G, ctx->dout.inv, nullptr, 0, ctx->corr32, ctx->st[2], ctx->d_user));
   s.base_only = 1;
   CK(run_stage(ctx, ctx->st[1], ctx->st[1], ctx->st[2], s, false, 0.0));
   for (int p = 2; p < 5; ++p)  // the base part has no higher modes
@@ -1404,10 +1404,10 @@ int swe_set_state_packed_async(swe_ctx* ctx, const double* c, double t) {
     CU(cudaEventRecord(ctx->ev_in[k], ctx->cin));
     CU(cudaStreamWaitEvent(ctx->stream, ctx->ev_in[k], 0));
     src = ctx->d_stage_in[k];
-    CK(launch_from_user(ctx->stream, ctx->dm, ctx->G, ctx->d_perm, ctx->d_off, ctx->corr32, src, ctx->st[0]));
+    CK(launch_from_user(ctx->stream, ctx->dm, ctx->G, ctx->dout.inv, ctx->d_off, ctx->packed_n, ctx->corr32, src, ctx->st[0]));
     CU(cudaEventRecord(ctx->ev_conv[k], ctx->stream));
   } else {
-    CK(launch_from_user(ctx->stream, ctx->dm, ctx->G, ctx->d_perm, ctx->d_off, ctx->corr32, src, ctx->st[0]));
+    CK(launch_from_user(ctx->stream, ctx->dm, ctx->G, ctx->dout.inv, ctx->d_off, ctx->packed_n, ctx->corr32, src, ctx->st[0]));
   }
   CK(launch_fill(ctx->stream, ctx->d_t, t, ctx->nmem));
   CU(cudaMemsetAsync(ctx->d_mstatus, 0, sizeof(unsigned) * (size_t)ctx->nmem, ctx->stream));
@@ -1427,14 +1427,14 @@ int swe_get_state_packed_async(swe_ctx* ctx, double* c_out) {
   CK(ensure_async(ctx));
   LaunchScope ls(ctx);
   if (is_device_ptr(c_out)) {
-    CK(launch_to_user(ctx->stream, ctx->dm, ctx->G, ctx->d_perm, ctx->d_off, ctx->corr32, ctx->st[0], c_out));
+    CK(launch_to_user(ctx->stream, ctx->dm, ctx->G, ctx->dout.inv, ctx->d_off, ctx->packed_n, ctx->corr32, ctx->st[0], c_out));
     return 0;
   }
   const int k = ctx->out_slot;
   ctx->out_slot ^= 1;
   // the staging buffer is free once its previous copy to the host has run
   CU(cudaStreamWaitEvent(ctx->stream, ctx->ev_d2h[k], 0));
-  CK(launch_to_user(ctx->stream, ctx->dm, ctx->G, ctx->d_perm, ctx->d_off, ctx->corr32, ctx->st[0],
+  CK(launch_to_user(ctx->stream, ctx->dm, ctx->G, ctx->dout.inv, ctx->d_off, ctx->packed_n, ctx->corr32, ctx->st[0],
                     ctx->d_stage_out[k]));
   CU(cudaEventRecord(ctx->ev_oready[k], ctx->stream));
   CU(cudaStreamWaitEvent(ctx->cout, ctx->ev_oready[k], 0));

@@ -108,11 +108,12 @@ void upload_base_tables();
 void set_sm_count(int n);
 
 // off == nullptr: the caller layout c[3][15][ne]; else packed, element u's
-// 3 K(p_u) values (field-major) from off[u]
-int launch_from_user(cudaStream_t s, const DevMesh& m, const Groups& G, const int32_t* perm, const int64_t* off,
-                     int corr_fp32, const double* cu, StateDev st);
-int launch_to_user(cudaStream_t s, const DevMesh& m, const Groups& G, const int32_t* perm, const int64_t* off,
-                   int corr_fp32, StateDev st, double* cu);
+// 3 K(p_u) values (field-major) from off[u], packed_n in all; inv: caller
+// index -> internal
+int launch_from_user(cudaStream_t s, const DevMesh& m, const Groups& G, const int32_t* inv, const int64_t* off,
+                     int64_t packed_n, int corr_fp32, const double* cu, StateDev st);
+int launch_to_user(cudaStream_t s, const DevMesh& m, const Groups& G, const int32_t* inv, const int64_t* off,
+                   int64_t packed_n, int corr_fp32, StateDev st, double* cu);
 int launch_sub(cudaStream_t s, const double* a, const double* b, double* out, int64_t n);
 
 // dmin (or nullptr): per member, the running minimum of the elements' CFL
