@@ -307,19 +307,22 @@ int64_t swe_tc_operand_image(int K, float* out, int64_t cap);
 /* Launch shapes (the paper has no counterpart: they tune the GPU kernels to
  * the mesh, orders and device).  shape[6]:
  *   [0] resident blocks per SM of the grid-stride base edge and element
- *       kernels, 0..32 (0: no cap, one block per base_threads units of work)
+ *       kernels, 0..32 (0: no cap, one block per base_threads units of work;
+ *       a mesh of at most one unit per thread of the capped grid runs uncapped)
  *   [1] threads per block of those kernels, 32..128, a multiple of 32
  *   [2] threads per block of the base u-solve, 32..256, a multiple of 32
  *   [3] threads per block of the correction u-solve and edge kernels,
  *       32..128, a multiple of 32
+ *       ([1] to [3] are upper bounds: blocks of few units are made smaller, down
+ *       to a warp, so that they cover the SMs)
  *   [4] schedule of the correction element kernel (FP64 and mixed modes;
  *       ignored in SWE_PREC_MIXED_TF32): 0 = its higher test modes run
  *       before the base element kernel, 1 = beside it (on the correction
  *       stream, joined at the end of the stage)
  *   [5] work distribution of the capped base grids ([0] > 0), 0..16:
  *       0 = equal grid-stride shares per block; c > 0 = dynamic tiles: a
- *       block takes c * [1] consecutive edges (elements) at a time from a
- *       ticket counter until none are left, so blocks that share their SM
+ *       block takes up to c * [1] consecutive edges (elements) at a time from
+ *       a ticket counter until none are left, so blocks that share their SM
  *       with the concurrent correction kernels take fewer tiles
  * Defaults {2, 128, 256, 128, 0, 2}.  Results do not depend on the shape (every
  * unit of work is computed by one thread in the same order).  SWE_EINVAL for

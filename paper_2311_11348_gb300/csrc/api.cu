@@ -749,7 +749,7 @@ static int usolve_all(swe_ctx* ctx, StateDev in) {
 //   A:                        ... edge_base --^--> elem_base ------------^
 // The tensor-core mode runs edge_corr -> vol_tc -> elem_corr on B before the
 // join.  Profiling runs everything on A.
-static int run_stage(swe_ctx* ctx, StateDev in, StateDev nst, StateDev out, const Stage& stg, bool cfl_dt,
+static int run_stage(swe_ctx* ctx, StateDev in, StateDev nst, StateDev out, const Stage& stg, bool first, bool last,
                      double dt_fixed) {
   const Phys ph = phys(ctx);
   const bool conc = !ctx->prof;
@@ -780,7 +780,7 @@ static int run_stage(swe_ctx* ctx, StateDev in, StateDev nst, StateDev out, cons
   {
     // the first stage of a CFL step folds the elements' CFL bounds into d_dmin
     ProfScope ps(ctx, F_USOLVE);
-    unsigned long long* dmin = cfl_dt ? ctx->d_dmin : nullptr;
+    unsigned long long* dmin = first && dt_fixed <= 0.0 ? ctx->d_dmin : nullptr;
     CK(launch_usolve_base(A, ctx->dm, ctx->G, ph, in.cb, ctx->vel.ub, ub32_out(ctx), ctx->d_status, dmin));
     CK(fork_groups());
     if (ctx->tc) CK(corrtc::launch_usolve_corr(gs, ctx->dm, ctx->G, ph, in, ctx->vel, ctx->d_status, dmin, ctx->rc));
@@ -795,10 +795,10 @@ static int run_stage(swe_ctx* ctx, StateDev in, StateDev nst, StateDev out, cons
     CU(cudaStreamWaitEvent(A, ctx->ev_u2, 0));
     CU(cudaStreamWaitEvent(B, ctx->ev_u1, 0));
   }
-  if (cfl_dt) {
-    ProfScope ps(ctx, F_DT);  // dt = cfl * min, and the minimum reset for the next step
+  if (first) {
+    ProfScope ps(ctx, F_DT);  // dt = dt_fixed or cfl * min, and the minimum reset for the next step
     CK(launch_advance_time(A, nullptr, ctx->d_dmin, ctx->prm.cfl, dt_fixed, ctx->d_dt, ctx->nmem));
-    if (conc) {  // the correction branch reads dt (stage time, RK update)
+    if (conc) {  // the correction branch reads dt (RK update)
       CU(cudaEventRecord(ctx->ev_dt, A));
       CU(cudaStreamWaitEvent(B, ctx->ev_dt, 0));
     }
@@ -849,6 +849,10 @@ static int run_stage(swe_ctx* ctx, StateDev in, StateDev nst, StateDev out, cons
     CU(cudaEventRecord(ctx->ev_c2, B));
     CU(cudaStreamWaitEvent(A, ctx->ev_c2, 0));
   }
+  if (last) {
+    ProfScope ps(ctx, F_OTHER);
+    CK(launch_advance_time(A, ctx->d_t, nullptr, 0.0, 0.0, ctx->d_dt, ctx->nmem));
+  }
   return 0;
 }
 
@@ -858,26 +862,19 @@ static int enqueue_step(swe_ctx* ctx, double dt_fixed) {
   Stage s{};
   s.dt = ctx->d_dt;
   s.t_dev = ctx->d_t;
-  if (dt_fixed > 0.0) {
-    ProfScope ps(ctx, F_DT);
-    CK(launch_advance_time(ctx->stream, nullptr, ctx->d_dmin, ctx->prm.cfl, dt_fixed, ctx->d_dt, ctx->nmem));
-  }
-  const bool cfl = dt_fixed <= 0.0;
   if (ctx->prm.rk_order == 3) {
     s.a = 0.0; s.b = 1.0; s.tau = 0.0;
-    CK(run_stage(ctx, A, A, B, s, cfl, dt_fixed));
+    CK(run_stage(ctx, A, A, B, s, true, false, dt_fixed));
     s.a = 0.75; s.b = 0.25; s.tau = 1.0;
-    CK(run_stage(ctx, B, A, C, s, false, dt_fixed));
+    CK(run_stage(ctx, B, A, C, s, false, false, dt_fixed));
     s.a = 1.0 / 3.0; s.b = 2.0 / 3.0; s.tau = 0.5;
-    CK(run_stage(ctx, C, A, A, s, false, dt_fixed));
+    CK(run_stage(ctx, C, A, A, s, false, true, dt_fixed));
   } else {
     s.a = 0.0; s.b = 1.0; s.tau = 0.0;
-    CK(run_stage(ctx, A, A, B, s, cfl, dt_fixed));
+    CK(run_stage(ctx, A, A, B, s, true, false, dt_fixed));
     s.a = 0.5; s.b = 0.5; s.tau = 1.0;
-    CK(run_stage(ctx, B, A, A, s, false, dt_fixed));
+    CK(run_stage(ctx, B, A, A, s, false, true, dt_fixed));
   }
-  ProfScope ps(ctx, F_OTHER);
-  CK(launch_advance_time(ctx->stream, ctx->d_t, nullptr, 0.0, 0.0, ctx->d_dt, ctx->nmem));
   return 0;
 }
 
@@ -1267,7 +1264,7 @@ static int rhs_impl(swe_ctx* ctx, const double* c_in, double* out0, double* out1
   s.rhs_only = 1;
   s.dt = nullptr; s.dt_host = 0.0;
   s.t_dev = ctx->d_t; s.tau = 0.0;
-  CK(run_stage(ctx, ctx->st[1], ctx->st[1], ctx->st[2], s, false, 0.0));
+  CK(run_stage(ctx, ctx->st[1], ctx->st[1], ctx->st[2], s, false, false, 0.0));
   int rc = read_status(ctx, false);
   if (rc) return rc;
   if (!out1) return state_out(ctx, ctx->st[2], out0);
@@ -1275,7 +1272,7 @@ static int rhs_impl(swe_ctx* ctx, const double* c_in, double* out0, double* out1
   const int64_t n = 3 * KMAX * ctx->ne;
   CK(launch_to_user(ctx->stream, ctx->dm, ctx->G, ctx->dout.inv, nullptr, 0, ctx->corr32, ctx->st[2], ctx->d_user));
   s.base_only = 1;
-  CK(run_stage(ctx, ctx->st[1], ctx->st[1], ctx->st[2], s, false, 0.0));
+  CK(run_stage(ctx, ctx->st[1], ctx->st[1], ctx->st[2], s, false, false, 0.0));
   for (int p = 2; p < 5; ++p)  // the base part has no higher modes
     if (ctx->st[2].ch[p]) {
       const int64_t np = ctx->G.start[p + 1] - ctx->G.start[p];

@@ -31,28 +31,49 @@ void upload_base_tables() {
 
 static inline int nblocks(int64_t n, int t) { return (int)((n + t - 1) / t); }
 
-// Grid of the FP64-pipe-bound base kernels: `per_sm` resident blocks per SM,
-// grid-stride loops over the work.  A few warps per SM already keep the FP64
-// pipe busy; the rest of the SM stays free for the concurrent FP32 correction.
 static int g_sm_count = 152;
 void set_sm_count(int n) { g_sm_count = n > 0 ? n : 152; }
-static inline int capped_blocks(int64_t n, int t, int per_sm) {
-  const int64_t b = (n + t - 1) / t, cap = (int64_t)g_sm_count * per_sm;
-  return (int)(per_sm <= 0 || b < cap ? b : cap);
+
+// Threads per block of a kernel over n units: t, halved (down to a warp) while the
+// blocks would not cover the SMs twice.  An FP64 instruction takes a warp 64 cycles and
+// its SM 19, so four warps in one block run a kernel of few units at half
+// the speed of the same four on four SMs.
+int spread_threads(int64_t n, int t) {
+  while (t > 32 && nblocks(n, t) < 2 * g_sm_count) t = (t / 2 + 31) / 32 * 32;
+  return t;
+}
+
+// Grid of the FP64-pipe-bound base kernels.  `per_sm` > 0 resident blocks per SM
+// once the work is more than one unit per thread of that grid: a few warps
+// per SM keep the FP64 pipe busy, and the rest of the SM stays free for the
+// concurrent FP32 correction.
+struct BaseGrid {
+  int blocks, threads, chunk;
+};
+static BaseGrid base_grid(int64_t n, const LaunchShape& L) {
+  const int64_t blocks = (int64_t)g_sm_count * L.base_bpsm, threads = blocks * L.base_threads;
+  if (L.base_bpsm <= 0 || n <= threads) {
+    const int t = spread_threads(n, L.base_threads);
+    return {nblocks(n, t), t, 0};
+  }
+  // tiles of chunk * threads units, smaller ones where a block would take less than four
+  int c = L.base_chunk;
+  while (c > 1 && n < 4 * c * threads) c /= 2;
+  return {(int)blocks, L.base_threads, c};
 }
 
 template <typename T>
 __device__ __forceinline__ T* chp(void* p) { return reinterpret_cast<T*>(p); }
 
-// Work distribution of the persistent base kernels over n units (edges or
-// elements).  chunk == 0 or work == nullptr: equal grid-stride shares.
-// Otherwise every block takes tiles of chunk * blockDim.x consecutive units
-// from an atomic ticket counter (work[0]) until none are left -- the next
-// ticket is fetched while the current tile runs -- so a block on an SM that
-// the concurrent correction kernels keep busy simply takes fewer tiles; the
-// last block to finish (counted in work[1]) resets both counters for the next
-// launch on the stream.  Every unit is computed by one thread with the same
-// arithmetic whatever the schedule, so results do not depend on it.
+// Work distribution of the base kernels over n units (edges or elements).
+// chunk == 0 or work == nullptr: equal grid-stride shares.  Otherwise every block
+// takes tiles of chunk * blockDim.x consecutive units from an atomic ticket
+// counter (work[0]) until none are left -- the next ticket is fetched while the
+// current tile runs -- so a block on an SM that the concurrent correction
+// kernels keep busy simply takes fewer tiles; the last block to finish (counted
+// in work[1]) resets both counters for the next launch on the stream.  Every unit is
+// computed by one thread with the same arithmetic whatever the schedule, so
+// results do not depend on it.
 template <typename F>
 __device__ __forceinline__ void for_units(int64_t n, int chunk, unsigned* work, F&& f) {
   const bool dyn = chunk > 0 && work != nullptr;
@@ -336,7 +357,7 @@ int launch_usolve_base(cudaStream_t s, const DevMesh& m, const Groups& G, const 
                        double* ub, float* ub32, unsigned* status, unsigned long long* dmin) {
   const int64_t n = G.start[2];
   if (n == 0) return 0;
-  const int ut = launch_shape().usolve_threads;
+  const int ut = spread_threads(n, launch_shape().usolve_threads);
   k_usolve_base<<<nblocks(n, ut), ut, 0, s>>>(m, n, ph, cb, ub, ub32, status, dmin);
   count_launch();
   SWE_CUDA_OK(cudaGetLastError());
@@ -500,16 +521,11 @@ __global__ void __launch_bounds__(128) k_edge_base(DevMesh m, Phys ph, Stage stg
   });
 }
 
-// the tile size of the dynamic schedule, 0 for the static one (an uncapped
-// grid of one block per base_threads units needs no schedule)
-static inline int base_chunk(const LaunchShape& L) { return L.base_bpsm > 0 ? L.base_chunk : 0; }
-
 int launch_edge_base(cudaStream_t s, const DevMesh& m, const int32_t* list, int64_t n, const Phys& ph,
                      const Stage& stg, const double* cb, const double* ub, EdgeFlux fx, unsigned* work) {
   if (n == 0) return 0;
-  const LaunchShape& L = launch_shape();
-  k_edge_base<<<capped_blocks(n, L.base_threads, L.base_bpsm), L.base_threads, 0, s>>>(m, ph, stg, list, n, cb, ub,
-                                                                                       fx.Fb, base_chunk(L), work);
+  const BaseGrid g = base_grid(n, launch_shape());
+  k_edge_base<<<g.blocks, g.threads, 0, s>>>(m, ph, stg, list, n, cb, ub, fx.Fb, g.chunk, work);
   count_launch();
   SWE_CUDA_OK(cudaGetLastError());
   return 0;
@@ -652,14 +668,14 @@ int launch_elem_base(cudaStream_t s, const DevMesh& m, const Groups& G, const Ph
                      const void* rc, unsigned* work) {
   if (m.ne == 0) return 0;
   const LaunchShape& L = launch_shape();
-  const int nb = capped_blocks(m.ne, L.base_threads, L.base_bpsm);
+  const BaseGrid g = base_grid(m.ne, L);
   const double* Fbc = stg.base_only ? nullptr : fx.Fbc;
   if (L.base_bpsm == 0 || L.base_bpsm >= 4)
-    k_elem_base<4><<<nb, L.base_threads, 0, s>>>(m, ph, stg, cbS, cbN, cbO, cbO32, ub, fx.Fb, Fbc,
-                                                 (const double*)rc, G.start[2], base_chunk(L), work);
+    k_elem_base<4><<<g.blocks, g.threads, 0, s>>>(m, ph, stg, cbS, cbN, cbO, cbO32, ub, fx.Fb, Fbc, (const double*)rc,
+                                                  G.start[2], g.chunk, work);
   else
-    k_elem_base<3><<<nb, L.base_threads, 0, s>>>(m, ph, stg, cbS, cbN, cbO, cbO32, ub, fx.Fb, Fbc,
-                                                 (const double*)rc, G.start[2], base_chunk(L), work);
+    k_elem_base<3><<<g.blocks, g.threads, 0, s>>>(m, ph, stg, cbS, cbN, cbO, cbO32, ub, fx.Fb, Fbc, (const double*)rc,
+                                                  G.start[2], g.chunk, work);
   count_launch();
   SWE_CUDA_OK(cudaGetLastError());
   return 0;

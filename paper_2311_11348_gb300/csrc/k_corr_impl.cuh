@@ -410,7 +410,7 @@ static int usolve_group(cudaStream_t st, const DevMesh& m, const Groups& G, int 
   const int64_t g0 = G.start[p], n = G.start[p + 1] - g0;
   if (n == 0) return 0;
   const int64_t nrc = G.start[5] - G.start[2], rc_off = g0 - G.start[2];
-  const int ct = launch_shape().corr_threads;
+  const int ct = spread_threads(n, launch_shape().corr_threads);
   if (K == 15 && kF32 && launch_shape().base_bpsm > 0)
     k_usolve_corr15<<<nblocks(n, ct), ct, 0, st>>>(m, g0, n, ph, c, (const T*)c.ch[p], u.ub, u.ub32,
                                                    (T*)u.uh[p], (T*)u.tr[p], (T*)u.trv[p], status, dmin,
@@ -819,7 +819,7 @@ static int edge_group(cudaStream_t st, const DevMesh& m, const CorrEdges& ce, co
                       const Stage& stg, StateDev c, VelDev u, EdgeFlux fx) {
   const int64_t nl = ce.n[PM];
   if (nl == 0) return 0;
-  const int ct = launch_shape().corr_threads;
+  const int ct = spread_threads(nl, launch_shape().corr_threads);
   k_edge_corr<PM><<<nblocks(nl, ct), ct, 0, st>>>(m, ce.list[PM], nl, G, ph, stg, c, u, fx);
   count_launch();
   SWE_CUDA_OK(cudaGetLastError());

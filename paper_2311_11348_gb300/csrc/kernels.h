@@ -98,14 +98,15 @@ struct LaunchShape {
   int corr_threads;    // threads per block of the correction u-solve and edge kernels (32..128)
   int split;           // 1: the correction element kernel's higher test modes run beside the base
                        // element kernel instead of before it (FP64 and mixed modes)
-  int base_chunk;      // schedule of the capped base grids: 0 = equal grid-stride shares, c > 0 =
-                       // dynamic tiles of c * base_threads edges / elements taken from a ticket counter
+  int base_chunk;      // schedule of the capped base grids: 0 = equal grid-stride shares, c > 0 = dynamic
+                       // tiles of up to c * base_threads edges / elements taken from a ticket counter
 };
 const LaunchShape& launch_shape();
 
 // base-path tables (host -> constant memory of the base kernels)
 void upload_base_tables();
 void set_sm_count(int n);
+int spread_threads(int64_t n, int t);  // threads per block (at most t) so that n units cover the SMs
 
 // off == nullptr: the caller layout c[3][15][ne]; else packed, element u's
 // 3 K(p_u) values (field-major) from off[u], packed_n in all; inv: caller
