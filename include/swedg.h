@@ -57,7 +57,7 @@ extern "C" {
 #define SWE_PREC_MIXED_FP32 1 /* correction arithmetic and storage in FP32           */
 #define SWE_PREC_MIXED_TF32 2 /* as MIXED_FP32, but the momentum volume terms of the
                                * correction (the G contractions of Eq. 13) run on the
-                               * tensor cores: every FP32 operand split into two TF32
+                               * tensor cores for the orders 3 and 4: every FP32 operand split into two TF32
                                * parts, three partial products, FP32 accumulation   */
 
 typedef struct swe_ctx swe_ctx; /* opaque */
@@ -286,12 +286,14 @@ int swe_reference_tensors(double* D, double* G, double* T);
  * npts in 1..8; host pointers.  Needs no device. */
 int swe_edge_table(int npts, double* s, double* w, double* B);
 
-/* Shared-memory image of the constant tensor-core operand of the
- * SWE_PREC_MIXED_TF32 volume contraction for K = 6, 10 or 15 modes (the paper
- * has no counterpart: it is the GB300 layout of the G_k tensors of Eq. 13).
- * The contraction runs as GEMMs of per-element rows of 2 K values (the
- * velocities, or the pressure products, for k = x^ then y^) against one
- * operand B with 16 K rows and 32 columns:
+/* Shared-memory image of a tensor-core operand that contracts the G_k tensors of
+ * Eq. 13 for K = 6, 10 or 15 modes (the paper has no counterpart: it is a GB300
+ * layout for callers with contractions of their own; the library's
+ * SWE_PREC_MIXED_TF32 kernel contracts with T[m][i][j] instead, in rows of the same
+ * layout, because G_k[q][i][j] = sum_m D_k[q][m] T[m][i][j] shares the GEMM between
+ * the test modes).  GEMMs of per-element rows of 2 K values (the velocities, or
+ * the pressure products, for k = x^ then y^) run against one operand B with 16 K
+ * rows and 32 columns:
  *   B[16 i + q][k K + j] = G_k[q][i][j]
  * (zero for q >= K, for columns >= 2 K, for the base triples q, i, j < 3 and
  * for structural zeros).  The image holds two parts one after the other, each

@@ -96,7 +96,7 @@ struct swe_ctx {
   RegroupScratch rw{};
   // capacities (bytes) of the buffers sized by the order groups
   size_t cap_ch[3][5] = {}, cap_uh[5] = {}, cap_tr[5] = {}, cap_trv[5] = {}, cap_pf[5] = {};
-  size_t cap_rc = 0, cap_vol = 0;
+  size_t cap_rc = 0;
   // device
   std::vector<std::pair<void*, size_t>> allocs;
   DevMesh dm{};
@@ -106,7 +106,6 @@ struct swe_ctx {
   VelDev vel{};
   EdgeFlux fx{};
   void* rc = nullptr;
-  float* vol = nullptr;  // tensor-core volume terms [32][elements of order >= 2]
   double* d_user = nullptr;
   double* d_user2 = nullptr;
   int64_t* d_off = nullptr;  // packed caller layout: offset of each caller element's 3 K(p) values
@@ -419,8 +418,7 @@ static int build_topology(swe_ctx* ctx) {
 
 // Buffers whose sizes follow the order groups (the current G and ce.n): the
 // correction parts of the three RK states, of the velocity and of the trace
-// records, the correction edges' projections, rc, the tensor-core volume
-// terms and the per-element correction edge slots.  Grown as needed (a new
+// records, the correction edges' projections and rc.  Grown as needed (a new
 // buffer starts zeroed; the contents of a regrown one are not kept).
 static int alloc_group_buffers(swe_ctx* ctx) {
   const size_t ts = ctx->corr32 ? sizeof(float) : sizeof(double);
@@ -443,7 +441,6 @@ static int alloc_group_buffers(swe_ctx* ctx) {
   }
   const size_t nrc = (size_t)std::max<int64_t>(ctx->ne - ctx->G.start[2], 1);
   if (!rc) rc = grow(&ctx->rc, &ctx->cap_rc, sizeof(double) * 4 * nrc);
-  if (!rc && ctx->tc) rc = grow(&ctx->vol, &ctx->cap_vol, sizeof(float) * 32 * nrc);
   return rc ? cuda_err(ctx, rc) : 0;
 }
 
@@ -496,7 +493,7 @@ static int build_device(swe_ctx* ctx) {
     ctx->fx.Pf[p] = nullptr;
     ctx->cap_uh[p] = ctx->cap_tr[p] = ctx->cap_trv[p] = ctx->cap_pf[p] = 0;
   }
-  ctx->rc = nullptr; ctx->vol = nullptr; ctx->cap_rc = ctx->cap_vol = 0;
+  ctx->rc = nullptr; ctx->cap_rc = 0;
   std::memset(&ctx->ce, 0, sizeof ctx->ce);
   const int64_t ne = ctx->ne;
   const RefTables& R = tables();
@@ -747,8 +744,8 @@ static int usolve_all(swe_ctx* ctx, StateDev in) {
 // beside elem_base instead:
 //   B: usolve_corr (+ rc) -->      edge_corr ----> elem_corr(q >= 3) --> (join)
 //   A:                        ... edge_base --^--> elem_base ------------^
-// The tensor-core mode runs edge_corr -> vol_tc -> elem_corr on B before the
-// join.  Profiling runs everything on A.
+// The tensor-core mode runs edge_corr -> elem_corr (order 2) -> elem_tc on B before
+// the join.  Profiling runs everything on A.
 static int run_stage(swe_ctx* ctx, StateDev in, StateDev nst, StateDev out, const Stage& stg, bool first, bool last,
                      double dt_fixed) {
   const Phys ph = phys(ctx);
@@ -813,8 +810,7 @@ static int run_stage(swe_ctx* ctx, StateDev in, StateDev nst, StateDev out, cons
   auto elem_corr = [&]() -> int {
     ProfScope ps(ctx, F_ELEMC);
     CK(fork_groups());
-    if (ctx->tc)
-      CK(corrtc::launch_elem_corr(gs, ctx->dm, ctx->G, ph, stg, in, nst, out, ctx->vel, ctx->fx, ctx->vol));
+    if (ctx->tc) CK(corrtc::launch_elem_corr(gs, ctx->dm, ctx->G, ph, stg, in, nst, out, ctx->vel, ctx->fx));
     else if (ctx->corr32) CK(corr32::launch_elem_corr(gs, ctx->dm, ctx->G, ph, stg, in, nst, out, ctx->vel, ctx->fx));
     else CK(corr64::launch_elem_corr(gs, ctx->dm, ctx->G, ph, stg, in, nst, out, ctx->vel, ctx->fx));
     CK(join_groups());
@@ -829,11 +825,11 @@ static int run_stage(swe_ctx* ctx, StateDev in, StateDev nst, StateDev out, cons
       else CK(corr64::launch_edge_corr(gs, ctx->dm, ctx->ce, ctx->G, ph, stg, in, ctx->vel, ctx->fx));
       CK(join_groups());
     }
+    if (!split) CK(elem_corr());
     if (ctx->tc) {
       ProfScope ps(ctx, F_VOLTC);
-      CK(corrtc::launch_vol_tc(B, ctx->dm, ctx->G, ph, in, ctx->vel, ctx->vol, ctx->d_status));
+        CK(corrtc::launch_elem_tc(B, ctx->dm, ctx->G, ph, stg, in, nst, out, ctx->vel, ctx->fx, ctx->d_status));
     }
-    if (!split) CK(elem_corr());
   }
   if (conc) {
     CU(cudaEventRecord(ctx->ev_c, B));

@@ -20,9 +20,8 @@
 //                      the edges' projected fluxes and the SSP-RK update of
 //                      the higher modes (test modes q >= 3)
 //
-// With CORR_TC defined (k_corr_tc.cu) the volume terms of the momentum rows
-// of the orders 3 and 4 come from a buffer that the tensor-core contraction
-// k_vol_tc<K> wrote; k_elem_vol then adds the elevation row's and the rest.
+// With CORR_TC defined (k_corr_tc.cu) the element update of the orders 3 and 4
+// is that file's tensor-core kernel.
 #include <cfloat>
 #include <cstdio>
 
@@ -86,9 +85,6 @@ __host__ __device__ constexpr bool dsnz(int q, int m) {
 __host__ __device__ constexpr int ktr(int i, int j) { return Kof(imax(deg_of(i), deg_of(j))); }
 
 __constant__ T cT[KMAX][120];       // T[n][i][j], (i, j) packed symmetric
-#ifdef CORR_TC
-__constant__ T cG[2][KMAX][120];    // G_k[q][i][j], (i, j) packed symmetric
-#endif
 __constant__ T cDx[KMAX][10];       // D_x[q][m]: d_x phihat_q = sum_m D_x[q][m] phihat_m, deg m < 4
 __constant__ T cDs[KMAX][10];       // D_y[q][m] - D_x[q][m] / 2, alike
 __constant__ T cEL[3][KMAX][5];     // phihat_i(gamma_k(s)) = sum_l cEL[k][i][l] P_l(2 s - 1), l <= deg i
@@ -115,14 +111,6 @@ void upload_tables() {
       dx[q][m] = (T)R.D[0][q][m];
       ds[q][m] = (T)(R.D[1][q][m] - 0.5 * R.D[0][q][m]);
     }
-#ifdef CORR_TC
-  static T g[2][KMAX][120];
-  for (int k = 0; k < 2; ++k)
-    for (int n = 0; n < KMAX; ++n)
-      for (int j = 0; j < KMAX; ++j)
-        for (int i = 0; i <= j; ++i) g[k][n][pk(i, j)] = (T)R.G[k][n][i][j];
-  cudaMemcpyToSymbol(cG, g, sizeof g);
-#endif
   for (int k = 0; k < 3; ++k)
     for (int i = 0; i < KMAX; ++i)
       for (int l = 0; l < 5; ++l) {  // (2 l + 1) int_0^1 phihat_i(gamma_k(s)) P_l(2 s - 1) ds, exact with 8 points
@@ -248,13 +236,12 @@ __device__ __forceinline__ void products(T (&z)[4], const T (&xi)[K], const T (&
   z[3] = fma(g, P, z3);
 }
 
+// orders whose element update runs on the tensor cores (for K = 6 the GEMMs
+// would be a few columns)
 #ifdef CORR_TC
-// orders whose momentum volume terms come from the tensor cores; for K = 6
-// the CUDA-core contraction measured as fast as the tensor-core kernel plus
-// the buffer round trip, so it stays here
-__host__ __device__ constexpr bool tc_vol(int K) { return K >= 10; }
+__host__ __device__ constexpr bool on_tc(int K) { return K >= 10; }
 #else
-__host__ __device__ constexpr bool tc_vol(int K) { return false; }
+__host__ __device__ constexpr bool on_tc(int K) { return false; }
 #endif
 
 // ---------------------------------------------------------------------------
@@ -1015,45 +1002,6 @@ __global__ void __launch_bounds__(32 * Kof(deg_of(K - 1) - 1)) k_elem_corr_split
   });
 }
 
-#ifdef CORR_TC
-// tensor-core mode, orders 3 and 4: block = 128 elements of one test mode (the
-// grid is ordered q-major); the momentum volume terms come from vol
-template <int K>
-__global__ void __launch_bounds__(128, 4) k_elem_vol(ELEM_CORR_PARAMS, const float* __restrict__ vol, int64_t rc_off,
-                                                     int64_t nrc) {
-  const int64_t nb = (n + 127) / 128;
-  const int q = 3 + (int)(blockIdx.x / nb);
-  const int64_t l = (blockIdx.x % nb) * 128 + threadIdx.x;
-  if (l >= n) return;
-  const int64_t e = g0 + l, ne = m.ne;
-  constexpr int KH = K - 3, KL = Kof(deg_of(K - 1) - 1);
-  const T* geo = geo_t(m);
-  const T J2 = geo[G_JI2 * ne + e], J3 = geo[G_JI3 * ne + e];
-  const T La = geo[G_JI0 * ne + e] + (T)0.5 * J2, Lb = geo[G_JI1 * ne + e] + (T)0.5 * J3;
-  T U[KL], V[KL];
-  load_modes<KL>(U, cbS, ne, e, chS + (1 * KH - (KL - 3)) * n, n, l, 1);
-  load_modes<KL>(V, cbS, ne, e, chS + 2 * (KH - (KL - 3)) * n, n, l, 2);
-  T r[3] = {0, vol[q * nrc + rc_off + l], vol[(16 + q) * nrc + rc_off + l]};
-  sfor<3, K>([&](auto Q) {
-    if (q == Q)
-      sfor<0, KL>([&](auto M) {
-        if constexpr (dxnz(Q, M)) r[0] += cDx[Q][M] * (La * U[M] + Lb * V[M]);
-        if constexpr (dsnz(Q, M)) r[0] += cDs[Q][M] * (J2 * U[M] + J3 * V[M]);
-      });
-  });
-  const T tau = friction(m, ph, e, geo[G_RS * ne + e], cbS[e], ub[e], ub[3 * ne + e]);
-  finish_mode<K>(stg, ph, n, l, q, r, chS[(0 * KH + (q - 3)) * n + l], chS[(1 * KH + (q - 3)) * n + l],
-                 chS[(2 * KH + (q - 3)) * n + l], ph.src ? uh[(0 * KH + (q - 3)) * n + l] : 0,
-                 ph.src ? uh[(1 * KH + (q - 3)) * n + l] : 0, geo[G_GDHX * ne + e], geo[G_GDHY * ne + e], tau,
-                 (T)stage_dt(stg, m.mem[e]), pe, chN, chO);
-}
-#define CORR_VOL_PARAM , const float* __restrict__ vol
-#define CORR_VOL_ARG , vol
-#else
-#define CORR_VOL_PARAM
-#define CORR_VOL_ARG
-#endif
-
 static const T* base_c_host(const StateDev& s) {
   if constexpr (kF32) return (const T*)s.cb32; else return (const T*)s.cb;
 }
@@ -1063,25 +1011,18 @@ static const T* base_u_host(const VelDev& u) {
 
 template <int K>
 static int elem_group(cudaStream_t st, const DevMesh& m, const Groups& G, int p, const Phys& ph, const Stage& stg,
-                      StateDev cS, StateDev cN, StateDev cO, VelDev u, EdgeFlux fx CORR_VOL_PARAM) {
+                      StateDev cS, StateDev cN, StateDev cO, VelDev u, EdgeFlux fx) {
   const int64_t g0 = G.start[p], n = G.start[p + 1] - g0;
   if (n == 0) return 0;
   const T *cb = base_c_host(cS), *ub = base_u_host(u), *chS = (const T*)cS.ch[p], *chN = (const T*)cN.ch[p];
   const T *uh = (const T*)u.uh[p], *pe = (const T*)fx.Pf[p];
   T* chO = (T*)cO.ch[p];
-  if constexpr (!tc_vol(K)) {
-    constexpr int KL = Kof(deg_of(K - 1) - 1);
-    if (!kF32 || n * KL <= 60000) {
-      k_elem_corr_split<K><<<nblocks(n, 32), 32 * KL, 0, st>>>(m, g0, n, ph, stg, cb, chS, chN, chO, ub, uh, pe);
-    } else if constexpr (kF32) {
-      const int t = launch_shape().corr_threads;
-      k_elem_corr<K><<<nblocks(n, t), t, 0, st>>>(m, g0, n, ph, stg, cb, chS, chN, chO, ub, uh, pe);
-    }
-  } else {
-#ifdef CORR_TC
-    k_elem_vol<K><<<(unsigned)(((n + 127) / 128) * (K - 3)), 128, 0, st>>>(
-        m, g0, n, ph, stg, cb, chS, chN, chO, ub, uh, pe, vol, g0 - G.start[2], G.start[5] - G.start[2]);
-#endif
+  constexpr int KL = Kof(deg_of(K - 1) - 1);
+  if (!kF32 || n * KL <= 60000) {
+    k_elem_corr_split<K><<<nblocks(n, 32), 32 * KL, 0, st>>>(m, g0, n, ph, stg, cb, chS, chN, chO, ub, uh, pe);
+  } else if constexpr (kF32) {
+    const int t = launch_shape().corr_threads;
+    k_elem_corr<K><<<nblocks(n, t), t, 0, st>>>(m, g0, n, ph, stg, cb, chS, chN, chO, ub, uh, pe);
   }
   count_launch();
   SWE_CUDA_OK(cudaGetLastError());
@@ -1089,10 +1030,12 @@ static int elem_group(cudaStream_t st, const DevMesh& m, const Groups& G, int p,
 }
 
 int launch_elem_corr(GroupStreams gs, const DevMesh& m, const Groups& G, const Phys& ph, const Stage& stg,
-                     StateDev cS, StateDev cN, StateDev cO, VelDev u, EdgeFlux fx CORR_VOL_PARAM) {
-  int r = elem_group<6>(gs.s[0], m, G, 2, ph, stg, cS, cN, cO, u, fx CORR_VOL_ARG);
-  if (!r) r = elem_group<10>(gs.s[1], m, G, 3, ph, stg, cS, cN, cO, u, fx CORR_VOL_ARG);
-  if (!r) r = elem_group<15>(gs.s[2], m, G, 4, ph, stg, cS, cN, cO, u, fx CORR_VOL_ARG);
+                     StateDev cS, StateDev cN, StateDev cO, VelDev u, EdgeFlux fx) {
+  int r = elem_group<6>(gs.s[0], m, G, 2, ph, stg, cS, cN, cO, u, fx);
+  if constexpr (!on_tc(10)) {
+    if (!r) r = elem_group<10>(gs.s[1], m, G, 3, ph, stg, cS, cN, cO, u, fx);
+    if (!r) r = elem_group<15>(gs.s[2], m, G, 4, ph, stg, cS, cN, cO, u, fx);
+  }
   return r;
 }
 

@@ -166,20 +166,14 @@ SWE_CORR_DECL(corr64)
 SWE_CORR_DECL(corr32)
 
 // FP32 correction whose momentum volume terms run on the tensor cores
-// (k_corr_tc.cu): the same launchers as corr32, elem_corr reads the volume
-// terms that launch_vol_tc wrote to vol[32][elements of order >= 2].
+// (k_corr_tc.cu): the same launchers as corr32; launch_elem_corr updates the
+// order 2, launch_elem_tc the orders 3 and 4.
+SWE_CORR_DECL(corrtc)
 namespace corrtc {
-void upload_tables();
 int upload_tc_tables();
-int launch_usolve_corr(GroupStreams gs, const DevMesh& m, const Groups& G, const Phys& ph, StateDev c, VelDev u,
-                       unsigned* status, unsigned long long* dmin, void* rc);
-int launch_edge_corr(GroupStreams gs, const DevMesh& m, const CorrEdges& ce, const Groups& G, const Phys& ph,
-                     const Stage& stg, StateDev c, VelDev u, EdgeFlux fx);
-int launch_elem_corr(GroupStreams gs, const DevMesh& m, const Groups& G, const Phys& ph, const Stage& stg,
-                     StateDev cS, StateDev cN, StateDev cO, VelDev u, EdgeFlux fx, const float* vol);
-int launch_vol_tc(cudaStream_t st, const DevMesh& m, const Groups& G, const Phys& ph, StateDev c, VelDev u,
-                  float* vol, unsigned* status);
-// host: the shared-memory image of the B operands for K = 6, 10, 15 (floats written, or needed when out is NULL)
+int launch_elem_tc(cudaStream_t st, const DevMesh& m, const Groups& G, const Phys& ph, const Stage& stg, StateDev cS,
+                   StateDev cN, StateDev cO, VelDev u, EdgeFlux fx, unsigned* status);
+// host: the operand image of swe_tc_operand_image (floats written, or needed when out is NULL)
 int64_t tc_operand_image(int K, float* out, int64_t cap);
 // a bounded wait on an mbarrier that nothing arrives on: sets ST_TIMEOUT
 int launch_wait_selftest(cudaStream_t st, int64_t spins, unsigned* status);
