@@ -317,10 +317,9 @@ int64_t swe_tc_operand_image(int K, float* out, int64_t cap);
  *       32..128, a multiple of 32
  *       ([1] to [3] are upper bounds: blocks of few units are made smaller, down
  *       to a warp, so that they cover the SMs)
- *   [4] schedule of the correction element kernel (FP64 and mixed modes;
- *       ignored in SWE_PREC_MIXED_TF32): 0 = its higher test modes run
- *       before the base element kernel, 1 = beside it (on the correction
- *       stream, joined at the end of the stage)
+ *   [4] 0 or 1, without effect: the correction element kernel runs beside the
+ *       base element kernel (on the correction stream, joined at the end of
+ *       the stage)
  *   [5] work distribution of the capped base grids ([0] > 0), 0..16:
  *       0 = equal grid-stride shares per block; c > 0 = dynamic tiles: a
  *       block takes up to c * [1] consecutive edges (elements) at a time from
@@ -334,8 +333,8 @@ int swe_set_launch_shape(swe_ctx* ctx, const int32_t* shape);
 
 /* Autotuner: for candidate launch shapes (coordinate descent: blocks per SM
  * in {1,2,3,4,6,0}, then base threads {64,128}, u-solve threads {128,256},
- * correction threads {64,128}, schedule {0,1}, base tiles {0,1,2,4}), runs `steps` CFL steps of the context's own
- * mesh and state, times them with CUDA events on the context stream, keeps
+ * correction threads {64,128}, base tiles {0,1,2,4}), runs `steps` CFL steps of the
+ * context's own mesh and state, times them with CUDA events on the context stream, keeps
  * the fastest shape and restores the state and member times.  shape_out[6]
  * and ms_out (time per step of the choice) may be NULL.  Needs the state to
  * stay valid for the trial steps (errors of swe_run are returned). */
@@ -353,7 +352,7 @@ int swe_selftest_wait(swe_ctx* ctx, int64_t spins);
  * each family) accumulated while swe_profile(ctx, 1) is on; swe_run then
  * launches the steps directly instead of replaying its CUDA graph.  Families:
  * usolve, dt, edge_base, edge_corr, elem_corr, elem_base, other, vol_tc (the
- * tensor-core volume contraction of SWE_PREC_MIXED_TF32), and a last
+ * tensor-core element update of SWE_PREC_MIXED_TF32), and a last
  * entry "kernels" whose launch count is every kernel the library launched
  * since the last swe_profile call (graph replays included).  names (static
  * strings), ms and launches receive up to n entries; returns the number of

@@ -735,22 +735,18 @@ static int usolve_all(swe_ctx* ctx, StateDev in) {
 // The base kernels (FP64 pipe bound) run on stream A, the correction kernels
 // on stream B, concurrently on the same SMs -- the GB300 counterpart of the
 // paper's base/correction distribution over CPU and GPU (Sect. 3-5):
-//   A: usolve_base --------> [dt] edge_base -------------------------> elem_base
-//   B: usolve_corr (+ rc) -->      edge_corr -> elem_corr(q >= 3) ---^
-// (each edge kernel needs both u-solves; elem_base needs the rc of the base
-// test modes, which the velocity solve forms, and edge_corr's share of the
-// base-mode flux).  With the split schedule (a launch-shape choice) the
-// higher test modes, which write only the correction part of the state, run
-// beside elem_base instead:
-//   B: usolve_corr (+ rc) -->      edge_corr ----> elem_corr(q >= 3) --> (join)
-//   A:                        ... edge_base --^--> elem_base ------------^
-// The tensor-core mode runs edge_corr -> elem_corr (order 2) -> elem_tc on B before
-// the join.  Profiling runs everything on A.
+//   A: usolve_base --------> [dt] edge_base -> elem_base ---------------^
+//   B: usolve_corr (+ rc) -> edge_corr --^---> elem_corr(q >= 3) --> (join)
+// Each edge kernel needs both u-solves; elem_base needs the rc of the base test
+// modes, which the velocity solve forms, and edge_corr's share of the base-mode
+// flux; elem_corr writes only the correction part of the state, so it runs
+// beside elem_base.  (The element updates one after the other cost 3 to 8 % of a
+// step: elem_base then has the SMs alone and leaves the FP32 pipe idle.)
+// Profiling runs everything on A.
 static int run_stage(swe_ctx* ctx, StateDev in, StateDev nst, StateDev out, const Stage& stg, bool first, bool last,
                      double dt_fixed) {
   const Phys ph = phys(ctx);
   const bool conc = !ctx->prof;
-  const bool split = ctx->shape.split && !ctx->tc && !stg.base_only;
   cudaStream_t A = ctx->stream, B = conc ? ctx->stream2 : ctx->stream;
   // the order groups of each correction launch run concurrently: forked from
   // B onto the group streams and joined back before B's next launch
@@ -807,15 +803,6 @@ static int run_stage(swe_ctx* ctx, StateDev in, StateDev nst, StateDev out, cons
     CK(launch_edge_base(A, ctx->dm, part ? ctx->ce.list[1] : nullptr, part ? ctx->ce.n[1] : ctx->nedge, ph, stg, in.cb,
                         ctx->vel.ub, ctx->fx, ctx->d_work));
   }
-  auto elem_corr = [&]() -> int {
-    ProfScope ps(ctx, F_ELEMC);
-    CK(fork_groups());
-    if (ctx->tc) CK(corrtc::launch_elem_corr(gs, ctx->dm, ctx->G, ph, stg, in, nst, out, ctx->vel, ctx->fx));
-    else if (ctx->corr32) CK(corr32::launch_elem_corr(gs, ctx->dm, ctx->G, ph, stg, in, nst, out, ctx->vel, ctx->fx));
-    else CK(corr64::launch_elem_corr(gs, ctx->dm, ctx->G, ph, stg, in, nst, out, ctx->vel, ctx->fx));
-    CK(join_groups());
-    return 0;
-  };
   if (!stg.base_only) {
     {
       ProfScope ps(ctx, F_EDGEC);
@@ -825,23 +812,31 @@ static int run_stage(swe_ctx* ctx, StateDev in, StateDev nst, StateDev out, cons
       else CK(corr64::launch_edge_corr(gs, ctx->dm, ctx->ce, ctx->G, ph, stg, in, ctx->vel, ctx->fx));
       CK(join_groups());
     }
-    if (!split) CK(elem_corr());
-    if (ctx->tc) {
-      ProfScope ps(ctx, F_VOLTC);
-        CK(corrtc::launch_elem_tc(B, ctx->dm, ctx->G, ph, stg, in, nst, out, ctx->vel, ctx->fx, ctx->d_status));
-    }
   }
-  if (conc) {
+  if (conc) {  // edge_corr's share of the base modes' flux
     CU(cudaEventRecord(ctx->ev_c, B));
     CU(cudaStreamWaitEvent(A, ctx->ev_c, 0));
   }
-  if (split) CK(elem_corr());  // beside elem_base
+  if (!stg.base_only) {
+    {
+      ProfScope ps(ctx, F_ELEMC);
+      CK(fork_groups());
+      if (ctx->tc) CK(corrtc::launch_elem_corr(gs, ctx->dm, ctx->G, ph, stg, in, nst, out, ctx->vel, ctx->fx));
+      else if (ctx->corr32) CK(corr32::launch_elem_corr(gs, ctx->dm, ctx->G, ph, stg, in, nst, out, ctx->vel, ctx->fx));
+      else CK(corr64::launch_elem_corr(gs, ctx->dm, ctx->G, ph, stg, in, nst, out, ctx->vel, ctx->fx));
+    }
+    if (ctx->tc) {  // orders 3 and 4, beside order 2
+      ProfScope ps(ctx, F_VOLTC);
+      CK(corrtc::launch_elem_tc(gs.s[1], ctx->dm, ctx->G, ph, stg, in, nst, out, ctx->vel, ctx->fx, ctx->d_status));
+    }
+    CK(join_groups());
+  }
   {
     ProfScope ps(ctx, F_ELEMB);
     CK(launch_elem_base(A, ctx->dm, ctx->G, ph, stg, in.cb, nst.cb, out.cb, cb32_out(ctx, out), ctx->vel.ub, ctx->fx,
                         ctx->rc, ctx->d_work + 2));
   }
-  if (conc && split) {
+  if (conc) {
     CU(cudaEventRecord(ctx->ev_c2, B));
     CU(cudaStreamWaitEvent(A, ctx->ev_c2, 0));
   }
@@ -1648,14 +1643,13 @@ int swe_autotune(swe_ctx* ctx, int steps, int32_t* shape_out, double* ms_out) {
   LaunchShape best = ctx->shape;
   double best_ms = 0.0;
   if (!rc) rc = measure(best, &best_ms);
-  const std::vector<int> cand[6] = {{1, 2, 3, 4, 6, 0}, {64, 128}, {128, 256}, {64, 128}, {0, 1}, {0, 1, 2, 4}};
+  const std::vector<int> cand[6] = {{1, 2, 3, 4, 6, 0}, {64, 128}, {128, 256}, {64, 128}, {}, {0, 1, 2, 4}};
   for (int k = 0; k < 6 && !rc; ++k)
     for (int v : cand[k]) {
-      if (k == 4 && ctx->tc) break;   // the tensor-core mode has one schedule
       if (k == 5 && best.base_bpsm == 0) break;  // an uncapped grid has no tile schedule
       LaunchShape sh = best;
       int* f = k == 0 ? &sh.base_bpsm : k == 1 ? &sh.base_threads : k == 2 ? &sh.usolve_threads
-             : k == 3 ? &sh.corr_threads : k == 4 ? &sh.split : &sh.base_chunk;
+             : k == 3 ? &sh.corr_threads : &sh.base_chunk;
       if (*f == v) continue;
       *f = v;
       double ms = 0.0;

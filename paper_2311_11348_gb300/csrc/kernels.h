@@ -96,8 +96,7 @@ struct LaunchShape {
   int base_threads;    // threads per block of those kernels (32..128)
   int usolve_threads;  // threads per block of the base u-solve (32..256)
   int corr_threads;    // threads per block of the correction u-solve and edge kernels (32..128)
-  int split;           // 1: the correction element kernel's higher test modes run beside the base
-                       // element kernel instead of before it (FP64 and mixed modes)
+  int split;           // 0 or 1, without effect
   int base_chunk;      // schedule of the capped base grids: 0 = equal grid-stride shares, c > 0 = dynamic
                        // tiles of up to c * base_threads edges / elements taken from a ticket counter
 };
