@@ -58,8 +58,10 @@ struct swe_ctx {
   cudaStream_t stream = nullptr;   // the caller's (or our) stream: base branch and ordering
   cudaStream_t stream2 = nullptr;  // the correction branch runs here, concurrently with the base
   cudaStream_t sg[2] = {nullptr, nullptr};  // its order groups p = 3, 4 (p = 2 stays on stream2)
+  cudaStream_t sdt = nullptr;      // the step size and time updates, beside the edge and element kernels
   cudaEvent_t ev_gf = nullptr, ev_gj[2] = {nullptr, nullptr};
   cudaEvent_t ev_fork = nullptr, ev_u1 = nullptr, ev_u2 = nullptr, ev_c = nullptr, ev_dt = nullptr, ev_c2 = nullptr;
+  cudaEvent_t ev_e1 = nullptr, ev_t = nullptr;
   bool own_stream = false;
   // asynchronous packed transfers: one copy stream per direction, two staging
   // buffers per direction (allocated on first use), events that order them
@@ -206,7 +208,7 @@ static int device_pool(int dev, cudaMemPool_t* out) {
 
 // every stream of the context idle (before buffers are returned to the pool)
 static void sync_streams(swe_ctx* ctx) {
-  for (cudaStream_t s : {ctx->stream, ctx->stream2, ctx->sg[0], ctx->sg[1], ctx->cin, ctx->cout})
+  for (cudaStream_t s : {ctx->stream, ctx->stream2, ctx->sg[0], ctx->sg[1], ctx->sdt, ctx->cin, ctx->cout})
     if (s) cudaStreamSynchronize(s);
 }
 
@@ -463,9 +465,6 @@ static int regroup(swe_ctx* ctx, bool keep_state) {
   ctx->ce.n[1] = ctx->nedge > 0 ? info[10] - info[9] : 0;
   ctx->packed_n = info[11];
   CK(alloc_group_buffers(ctx));
-  // edges that no longer touch a p >= 2 element carry no correction flux
-  if (ctx->fx.Fbc)
-    CU(cudaMemsetAsync(ctx->fx.Fbc, 0, sizeof(double) * 6 * (size_t)std::max<int64_t>(ctx->nedge, 1), ctx->stream));
   if (keep_state)
     CK(launch_from_user(ctx->stream, ctx->dm, ctx->G, ctx->dout.inv, nullptr, 0, ctx->corr32, ctx->d_user, ctx->st[0]));
   if (ctx->packed_n != packed_before)  // the asynchronous staging buffers follow the packed size
@@ -668,10 +667,7 @@ static int build_device(swe_ctx* ctx) {
   if ((rc = dalloc(ctx, &ctx->vel.ub, sizeof(double) * 6 * ne))) return cuda_err(ctx, rc);
   ctx->vel.ub32 = nullptr;
   if (ctx->corr32 && (rc = dalloc(ctx, &ctx->vel.ub32, sizeof(float) * 6 * ne))) return cuda_err(ctx, rc);
-  ctx->fx.Fbc = nullptr;
-  if ((rc = dalloc(ctx, &ctx->fx.Fb, sizeof(double) * 6 * nE)) ||
-      (ctx->corr32 && (rc = dalloc(ctx, &ctx->fx.Fbc, sizeof(double) * 6 * nE))))
-    return cuda_err(ctx, rc);
+  if ((rc = dalloc(ctx, &ctx->fx.Fb, sizeof(double) * 6 * nE))) return cuda_err(ctx, rc);
   if ((rc = dalloc(ctx, &ctx->d_user, sizeof(double) * 3 * KMAX * ne)) ||
       (rc = dalloc(ctx, &ctx->d_user2, sizeof(double) * 3 * KMAX * ne)))
     return cuda_err(ctx, rc);
@@ -735,14 +731,17 @@ static int usolve_all(swe_ctx* ctx, StateDev in) {
 // The base kernels (FP64 pipe bound) run on stream A, the correction kernels
 // on stream B, concurrently on the same SMs -- the GB300 counterpart of the
 // paper's base/correction distribution over CPU and GPU (Sect. 3-5):
-//   A: usolve_base --------> [dt] edge_base -> elem_base ---------------^
-//   B: usolve_corr (+ rc) -> edge_corr --^---> elem_corr(q >= 3) --> (join)
-// Each edge kernel needs both u-solves; elem_base needs the rc of the base test
-// modes, which the velocity solve forms, and edge_corr's share of the base-mode
-// flux; elem_corr writes only the correction part of the state, so it runs
-// beside elem_base.  (The element updates one after the other cost 3 to 8 % of a
-// step: elem_base then has the SMs alone and leaves the FP32 pipe idle.)
-// Profiling runs everything on A.
+//   A: usolve_base ---------> edge_base (p <= 1 on both sides) --> elem_base ------^
+//   B: usolve_corr (+ rc) --> edge_corr (the other edges) ----^--> elem_corr --> (join)
+// edge_corr needs both u-solves, edge_base the first alone; elem_base needs the
+// rc of the base test modes, which the velocity solve forms, and every edge's
+// flux; elem_corr (test modes q >= 3) writes only the correction part of the state,
+// so it runs beside elem_base.  (The element updates one after the other cost 3 to 8 %
+// of a step: elem_base then has the SMs alone and leaves the FP32 pipe idle.)
+// The step size (first stage: needed by the element kernels, not by the edge
+// kernels, whose stage time is the step's start) and the time update (last
+// stage: after the edge kernels, which read the time) run on a stream of their
+// own beside the edge and element kernels.  Profiling runs everything on A.
 static int run_stage(swe_ctx* ctx, StateDev in, StateDev nst, StateDev out, const Stage& stg, bool first, bool last,
                      double dt_fixed) {
   const Phys ph = phys(ctx);
@@ -782,40 +781,56 @@ static int run_stage(swe_ctx* ctx, StateDev in, StateDev nst, StateDev out, cons
     else CK(corr64::launch_usolve_corr(gs, ctx->dm, ctx->G, ph, in, ctx->vel, ctx->d_status, dmin, ctx->rc));
     CK(join_groups());
   }
+  // the correction edge kernel computes the whole flux of its edges; both
+  // elements of the others have order <= 1, so they need usolve_base alone
+  const bool part = !stg.base_only && ctx->ce.n[1] < ctx->nedge;
   if (conc) {
     CU(cudaEventRecord(ctx->ev_u1, A));
     CU(cudaEventRecord(ctx->ev_u2, B));
-    CU(cudaStreamWaitEvent(A, ctx->ev_u2, 0));
+    if (!part) CU(cudaStreamWaitEvent(A, ctx->ev_u2, 0));
     CU(cudaStreamWaitEvent(B, ctx->ev_u1, 0));
   }
+  Stage es = stg;  // of the edge kernels
   if (first) {
     ProfScope ps(ctx, F_DT);  // dt = dt_fixed or cfl * min, and the minimum reset for the next step
-    CK(launch_advance_time(A, nullptr, ctx->d_dmin, ctx->prm.cfl, dt_fixed, ctx->d_dt, ctx->nmem));
-    if (conc) {  // the correction branch reads dt (RK update)
-      CU(cudaEventRecord(ctx->ev_dt, A));
-      CU(cudaStreamWaitEvent(B, ctx->ev_dt, 0));
+    if (conc) {
+      CU(cudaStreamWaitEvent(ctx->sdt, ctx->ev_u1, 0));
+      CU(cudaStreamWaitEvent(ctx->sdt, ctx->ev_u2, 0));
     }
+    CK(launch_advance_time(conc ? ctx->sdt : A, nullptr, ctx->d_dmin, ctx->prm.cfl, dt_fixed, ctx->d_dt, ctx->nmem));
+    if (conc) CU(cudaEventRecord(ctx->ev_dt, ctx->sdt));
+    es.dt = nullptr;
+    es.dt_host = 0.0;
   }
   {
     ProfScope ps(ctx, F_EDGEB);
-    // in FP64 the correction edge kernel computes the whole flux of its edges
-    const bool part = !ctx->corr32 && !stg.base_only && ctx->ce.n[1] < ctx->nedge;
-    CK(launch_edge_base(A, ctx->dm, part ? ctx->ce.list[1] : nullptr, part ? ctx->ce.n[1] : ctx->nedge, ph, stg, in.cb,
+    CK(launch_edge_base(A, ctx->dm, part ? ctx->ce.list[1] : nullptr, part ? ctx->ce.n[1] : ctx->nedge, ph, es, in.cb,
                         ctx->vel.ub, ctx->fx, ctx->d_work));
   }
+  if (conc && last) CU(cudaEventRecord(ctx->ev_e1, A));
   if (!stg.base_only) {
     {
       ProfScope ps(ctx, F_EDGEC);
       CK(fork_groups());
-      if (ctx->tc) CK(corrtc::launch_edge_corr(gs, ctx->dm, ctx->ce, ctx->G, ph, stg, in, ctx->vel, ctx->fx));
-      else if (ctx->corr32) CK(corr32::launch_edge_corr(gs, ctx->dm, ctx->ce, ctx->G, ph, stg, in, ctx->vel, ctx->fx));
-      else CK(corr64::launch_edge_corr(gs, ctx->dm, ctx->ce, ctx->G, ph, stg, in, ctx->vel, ctx->fx));
+      if (ctx->tc) CK(corrtc::launch_edge_corr(gs, ctx->dm, ctx->ce, ctx->G, ph, es, in, ctx->vel, ctx->fx));
+      else if (ctx->corr32) CK(corr32::launch_edge_corr(gs, ctx->dm, ctx->ce, ctx->G, ph, es, in, ctx->vel, ctx->fx));
+      else CK(corr64::launch_edge_corr(gs, ctx->dm, ctx->ce, ctx->G, ph, es, in, ctx->vel, ctx->fx));
       CK(join_groups());
     }
   }
-  if (conc) {  // edge_corr's share of the base modes' flux
+  if (conc) {  // the fluxes of edge_corr's edges
     CU(cudaEventRecord(ctx->ev_c, B));
     CU(cudaStreamWaitEvent(A, ctx->ev_c, 0));
+  }
+  if (conc && last) {  // t += dt once the edge kernels have read t
+    CU(cudaStreamWaitEvent(ctx->sdt, ctx->ev_e1, 0));
+    CU(cudaStreamWaitEvent(ctx->sdt, ctx->ev_c, 0));
+    CK(launch_advance_time(ctx->sdt, ctx->d_t, nullptr, 0.0, 0.0, ctx->d_dt, ctx->nmem));
+    CU(cudaEventRecord(ctx->ev_t, ctx->sdt));
+  }
+  if (conc && first) {
+    CU(cudaStreamWaitEvent(A, ctx->ev_dt, 0));
+    CU(cudaStreamWaitEvent(B, ctx->ev_dt, 0));
   }
   if (!stg.base_only) {
     {
@@ -841,8 +856,12 @@ static int run_stage(swe_ctx* ctx, StateDev in, StateDev nst, StateDev out, cons
     CU(cudaStreamWaitEvent(A, ctx->ev_c2, 0));
   }
   if (last) {
-    ProfScope ps(ctx, F_OTHER);
-    CK(launch_advance_time(A, ctx->d_t, nullptr, 0.0, 0.0, ctx->d_dt, ctx->nmem));
+    if (conc) {
+      CU(cudaStreamWaitEvent(A, ctx->ev_t, 0));
+    } else {
+      ProfScope ps(ctx, F_OTHER);
+      CK(launch_advance_time(A, ctx->d_t, nullptr, 0.0, 0.0, ctx->d_dt, ctx->nmem));
+    }
   }
   return 0;
 }
@@ -957,6 +976,7 @@ int swe_create(swe_ctx** out, const swe_params* params) {
     e = cudaStreamCreateWithPriority(&ctx->stream2, cudaStreamNonBlocking, hi);
     for (int i = 0; i < 2 && e == cudaSuccess; ++i)
       e = cudaStreamCreateWithPriority(&ctx->sg[i], cudaStreamNonBlocking, hi);
+    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&ctx->sdt, cudaStreamNonBlocking, hi);
   }
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_u1, cudaEventDisableTiming);
@@ -965,6 +985,8 @@ int swe_create(swe_ctx** out, const swe_params* params) {
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_dt, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_c2, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_gf, cudaEventDisableTiming);
+  for (cudaEvent_t* ev : {&ctx->ev_e1, &ctx->ev_t})
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
   for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&ctx->ev_gj[i], cudaEventDisableTiming);
   if (e != cudaSuccess) {
     g_create_err = "stream/event creation failed";
@@ -1022,7 +1044,7 @@ void swe_destroy(swe_ctx* ctx) {
   for (auto& ev : ctx->evs) { cudaEventDestroy(ev.a); cudaEventDestroy(ev.b); }
   for (auto ev : ctx->pool) cudaEventDestroy(ev);
   for (cudaEvent_t ev : {ctx->ev_fork, ctx->ev_u1, ctx->ev_u2, ctx->ev_c, ctx->ev_dt, ctx->ev_c2, ctx->ev_gf,
-                         ctx->ev_gj[0], ctx->ev_gj[1]})
+                         ctx->ev_gj[0], ctx->ev_gj[1], ctx->ev_e1, ctx->ev_t})
     if (ev) cudaEventDestroy(ev);
   if (ctx->stream2) { cudaStreamSynchronize(ctx->stream2); cudaStreamDestroy(ctx->stream2); }
   for (cudaStream_t cs : {ctx->cin, ctx->cout})
@@ -1030,7 +1052,7 @@ void swe_destroy(swe_ctx* ctx) {
   for (int k = 0; k < 2; ++k)
     for (cudaEvent_t ev : {ctx->ev_in[k], ctx->ev_conv[k], ctx->ev_oready[k], ctx->ev_d2h[k]})
       if (ev) cudaEventDestroy(ev);
-  for (cudaStream_t sgi : ctx->sg)
+  for (cudaStream_t sgi : {ctx->sg[0], ctx->sg[1], ctx->sdt})
     if (sgi) { cudaStreamSynchronize(sgi); cudaStreamDestroy(sgi); }
   if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
   delete ctx;

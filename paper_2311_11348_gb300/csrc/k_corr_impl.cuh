@@ -12,9 +12,9 @@
 //   k_edge_corr<PM>    edges with max(p_L, p_R) = PM >= 2: traces as Legendre
 //                      coefficients along the edge, the moments of the LF
 //                      flux, projected onto both sides' higher test modes,
-//                      and the two-point equivalent for the base modes of
-//                      the correction flux (FP32, Fbc: no cancellation against
-//                      the base flux) or of the whole flux (FP64, Fb)
+//                      and the whole two-point flux for the base modes (Fb;
+//                      FP32: the FP64 base flux plus the two-point equivalent
+//                      of the correction flux)
 //   k_elem_corr<K>     volume terms as contractions with the reference
 //                      tensors of Eq. (13) (compile-time sparsity), source,
 //                      the edges' projected fluxes and the SSP-RK update of
@@ -25,6 +25,7 @@
 #include <cfloat>
 #include <cstdio>
 
+#include "base_edge.cuh"
 #include "kernels.h"
 #include "tables.h"
 
@@ -88,7 +89,6 @@ __constant__ T cT[KMAX][120];       // T[n][i][j], (i, j) packed symmetric
 __constant__ T cDx[KMAX][10];       // D_x[q][m]: d_x phihat_q = sum_m D_x[q][m] phihat_m, deg m < 4
 __constant__ T cDs[KMAX][10];       // D_y[q][m] - D_x[q][m] / 2, alike
 __constant__ T cEL[3][KMAX][5];     // phihat_i(gamma_k(s)) = sum_l cEL[k][i][l] P_l(2 s - 1), l <= deg i
-__constant__ double cEJ[3][3][2];    // the P1 rows of cEL in FP64 in every mode (the jump of xi_lin)
 __constant__ T cGP[3][4][5];        // per PM-2: P_l at the points t > 0 (then the middle one) of the npts_for(PM) rule on [-1,1]
 __constant__ T cGW[3][4];           // their weights (the rule's weights on [0,1])
 
@@ -101,7 +101,6 @@ static void legendre5(double t, double (&P)[5]) {
 
 void upload_tables() {
   const RefTables& R = tables();
-  static double ej[3][3][2];
   static T t[KMAX][120], dx[KMAX][10], ds[KMAX][10], el[3][KMAX][5], gp[3][4][5], gw[3][4];
   for (int n = 0; n < KMAX; ++n)
     for (int j = 0; j < KMAX; ++j)
@@ -120,7 +119,6 @@ void upload_tables() {
           acc += R.ew[8][gg] * R.EB[8][k][i][gg] * P[l];
         }
         el[k][i][l] = (T)((2 * l + 1) * acc);
-        if (i < 3 && l < 2) ej[k][i][l] = (2 * l + 1) * acc;
       }
   for (int pm = 2; pm <= 4; ++pm) {
     const int N = npts_for(pm), H = N / 2;
@@ -136,17 +134,11 @@ void upload_tables() {
   cudaMemcpyToSymbol(cDx, dx, sizeof dx);
   cudaMemcpyToSymbol(cDs, ds, sizeof ds);
   cudaMemcpyToSymbol(cEL, el, sizeof el);
-  cudaMemcpyToSymbol(cEJ, ej, sizeof ej);
   cudaMemcpyToSymbol(cGP, gp, sizeof gp);
   cudaMemcpyToSymbol(cGW, gw, sizeof gw);
 }
 
 static inline int nblocks(int64_t n, int t) { return (int)((n + t - 1) / t); }
-
-__device__ __forceinline__ double tide_value(const Phys& ph, double t) {
-  if (ph.tide_period <= 0.0) return ph.tide_amp;
-  return ph.tide_amp * sin(2.0 * 3.14159265358979323846 * t / ph.tide_period + ph.tide_phase);
-}
 
 // 16-byte accesses to 4 consecutive values (FP64: two of them)
 __device__ __forceinline__ void st4(float* p, float a, float b, float c, float d) {
@@ -435,13 +427,15 @@ int launch_usolve_corr(GroupStreams gs, const DevMesh& m, const Groups& G, const
 // replaced by g h_b times the jump of xi_lin (the volume term's share, see
 // products).
 // FP64 writes the moments of degree <= 1 of the whole flux as the edge's
-// two-point flux; the base edge kernel leaves these edges out.
+// two-point flux.
 // FP32 splits every trace into its P1 part (b) and the higher part (h): the
 // correction's share of the base modes, from
 //   U w - U_b w_b = U_h w + U_b w_h,  xi^2 / 2 - xi_b^2 / 2 = xi_h (xi_b + xi_h / 2),
-// carries no cancellation against the base flux that the base edge kernel
-// computes in FP64, and goes to Fbc; the products of two P1 parts reach the
-// higher test modes through their three moments in closed form.
+// carries no cancellation against the base flux; the products of two P1 parts
+// reach the higher test modes through their three moments in closed form.  The
+// same thread computes the base flux in FP64 and stores the sum, one flux for
+// both sides of the edge: a separate array cost the base element kernel 18
+// FP64 additions and 18 loads per element.
 // All fluxes are weighted by |E| / 4 (the weight of the two-point base rule)
 // through the normal.
 // FP64 is bound by its instruction count (about 340, 620, 1,080 per edge of
@@ -553,7 +547,6 @@ __device__ __forceinline__ void edge_corr_body(const DevMesh& m, const int32_t* 
                                                const Groups& G, const Phys& ph, const Stage& stg, const StateDev& c,
                                                const VelDev& u, const EdgeFlux& fx) {
   constexpr int N = npts_for(PM), GI = PM - 2;
-  double* F2 = kF32 ? fx.Fbc : fx.Fb;
   void* const* Pf = fx.Pf;
   const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (idx >= nl) return;
@@ -565,10 +558,20 @@ __device__ __forceinline__ void edge_corr_body(const DevMesh& m, const int32_t* 
   const T nxw = eg[E_NXW * nE + ed], nyw = eg[E_NYW * nE + ed], wl = eg[E_WLEN * nE + ed];
   const T h0 = eg[E_HMID * nE + ed], h1 = (T)0.5 * (eg[E_HB * nE + ed] - eg[E_HA * nE + ed]);
   const T g = (T)ph.g;
+  // jump of the degree-1 elevation along the edge, j0 + j1 t (zero on land): it
+  // carries the volume term g xi_lin h_b of the higher test modes (moved here,
+  // see products)
+  T j0 = 0, j1 = 0;
+  double F[6];
+  if constexpr (kF32) {
+    // the base flux, in FP64, with the jump at its two points t = -+1 / sqrt 3
+    double jump[2];
+    base_flux(m, ph, stg, ed, L, R, info, c.cb, u.ub, F, jump);
+    j0 = (T)(0.5 * (jump[0] + jump[1]));
+    j1 = (T)(0.8660254037844386 * (jump[1] - jump[0]));
+  }
   SideC<PM> a, b;
   side_coefs<PM>(m, G, c, u, L, pL, kL, false, nxw, nyw, a);
-  // the right state, and the jump of the degree-1 elevation (zero on land)
-  T j0 = 0, j1 = 0;
   if (R >= 0) {
     side_coefs<PM>(m, G, c, u, R, pR, kR, true, nxw, nyw, b);
   } else if (bc == 2) {
@@ -596,37 +599,11 @@ __device__ __forceinline__ void edge_corr_body(const DevMesh& m, const int32_t* 
     });
     b.un = -a.un;
   }
-  if constexpr (kF32) {
-    // the jump of xi_lin from the FP64 base modes: it carries the volume term
-    // g xi_lin h_b of the higher test modes (moved here, see products)
+  if constexpr (!kF32) {
     if (R >= 0 || bc == 2) {
-      const double rl = m.geo[G_RS * m.ne + L];
-      double l0 = c.cb[L] * cEJ[0][0][0], l1 = 0.0;
-#pragma unroll
-      for (int i = 1; i < 3; ++i) {
-        l0 += c.cb[i * m.ne + L] * cEJ[kL][i][0];
-        l1 += c.cb[i * m.ne + L] * cEJ[kL][i][1];
-      }
-      double r0 = 0.0, r1 = 0.0;
-      if (R >= 0) {
-        const double rr = m.geo[G_RS * m.ne + R];
-        r0 = c.cb[R] * cEJ[0][0][0];
-#pragma unroll
-        for (int i = 1; i < 3; ++i) {
-          r0 += c.cb[i * m.ne + R] * cEJ[kR][i][0];
-          r1 -= c.cb[i * m.ne + R] * cEJ[kR][i][1];
-        }
-        r0 *= rr;
-        r1 *= rr;
-      } else {
-        r0 = tide_value(ph, stage_time(stg, m.emem[ed]));
-      }
-      j0 = (T)(r0 - rl * l0);
-      j1 = (T)(r1 - rl * l1);
+      j0 = b.xl[0] - a.xl[0];
+      j1 = b.xl[1] - a.xl[1];
     }
-  } else if (R >= 0 || bc == 2) {
-    j0 = b.xl[0] - a.xl[0];
-    j1 = b.xl[1] - a.xl[1];
   }
   // lambda of Eq. (10) from the element means (Sect. 3), weighted like w
   const T lam = fmax(fabs(a.un), fabs(b.un)) + wl * sqrt(g * fmax(a.xm + h0, b.xm + h0));
@@ -716,6 +693,7 @@ __device__ __forceinline__ void edge_corr_body(const DevMesh& m, const int32_t* 
     });
   }
   // the base modes' two-point flux: in FP64 with the g xi_lin h_b terms
+  T f2[6];
   {
     T q1[2] = {m1[0], m1[1]}, q2[2] = {m2[0], m2[1]};
     if constexpr (!kF32) {
@@ -725,12 +703,10 @@ __device__ __forceinline__ void edge_corr_body(const DevMesh& m, const int32_t* 
       q2[0] += gny * y0; q2[1] += gny * y1;
     }
     const T r3 = (T)1.7320508075688772;  // the points of the two-point rule are +-1 / sqrt 3
-    F2[0 * nE + ed] = (double)(m0[0] - r3 * m0[1]);
-    F2[1 * nE + ed] = (double)(m0[0] + r3 * m0[1]);
-    F2[2 * nE + ed] = (double)(q1[0] - r3 * q1[1]);
-    F2[3 * nE + ed] = (double)(q1[0] + r3 * q1[1]);
-    F2[4 * nE + ed] = (double)(q2[0] - r3 * q2[1]);
-    F2[5 * nE + ed] = (double)(q2[0] + r3 * q2[1]);
+    f2[0] = m0[0] - r3 * m0[1]; f2[1] = m0[0] + r3 * m0[1];
+    f2[2] = q1[0] - r3 * q1[1]; f2[3] = q1[0] + r3 * q1[1];
+    f2[4] = q2[0] - r3 * q2[1]; f2[5] = q2[0] + r3 * q2[1];
+    sfor<0, 6>([&](auto i) { fx.Fb[i * nE + ed] = kF32 ? F[i] + (double)f2[i] : (double)f2[i]; });
   }
   if constexpr (kF32) {  // the P1 parts' share of the higher test modes
     sfor<0, 3>([&](auto l) { z1[l] = z2[l] = 0; });

@@ -29,10 +29,8 @@ struct Groups {
 };
 
 struct EdgeFlux {
-  double* Fb;        // [3][2][nedge] base flux (weighted by |E| w_g) at the 2-point rule; in FP64 mode the
-                     // whole flux on the edges with a p >= 2 side (from the correction edge kernel)
-  double* Fbc;       // mixed modes: [3][2][nedge] two-point equivalent of the correction flux's share of
-                     // the base modes (zero on edges without a p >= 2 side); nullptr in FP64 mode
+  double* Fb;        // [3][2][nedge] the flux the base modes see (weighted by |E| w_g) at the 2-point rule:
+                     // base part and, on edges with a p >= 2 side, correction
   void* Pf[5];       // per element order p = 2..4: [3 local edges][3 fields][K(p)-3][n_p]: the full flux of
                      // each of the element's (correction) edges projected onto its higher test modes (q >= 3),
                      // written by the correction edge kernel, read contiguously by the element kernel

@@ -75,8 +75,7 @@ def device_bytes(meshes, precision):
               20 * be, 40 * be, 16 * bg, 32 * bg, 8 * be, 8 * (be + 1), 128]                # partition scratch
     allocs += [72 * ne] * 3 + ([36 * ne] * 3 if corr32 else [])                             # base RK states
     allocs += [48 * ne] + ([24 * ne] if corr32 else [])                                     # base velocity
-    allocs += [48 * nE] + ([48 * nE] if corr32 else [])                                     # fluxes
-    allocs += [8 * 3 * KMAX * ne, 8 * 3 * KMAX * ne, ne,                                    # staging, orders
+    allocs += [48 * nE, 8 * 3 * KMAX * ne, 8 * 3 * KMAX * ne, ne,                             # fluxes, staging, orders
                8 * nm, 8 * nm, 8 * nm, 4, 4 * nm,                                           # members, status words
                8 * min(1024, max(1, (ne + 255) // 256)), 16, 16]                           # sums, tickets
     for q in (2, 3, 4):                                                                     # order groups
