@@ -147,18 +147,53 @@ __device__ __forceinline__ double cfl_bound(double u0, double v0, double H0, dou
   return (dd > 0.0 && dd < 1.7976931348623157e308) ? dd : 1.7976931348623157e308;
 }
 
-// min of d into dmin[mem] over the whole grid: positive doubles order like
-// their bit patterns, so an integer atomicMin gives the exact minimum
-// independent of the order of the blocks.  Every lane of the warp calls it
-// (lanes without an element pass DBL_MAX); one atomic per warp when the
-// warp's elements share a member (the usual case).
-__device__ __forceinline__ void cfl_min_store(unsigned long long* dmin, int mem, double d) {
+// The elements' CFL bounds folded into dmin[mem], a minimum over the whole grid:
+// positive doubles order like their bit patterns, so an integer atomicMin
+// gives the exact minimum independent of the order of the blocks.  Every thread of
+// the block calls it (valid: it has an element).  The bound takes about 35 FP64
+// instructions (two square roots and a division); an FP32 estimate, good to
+// 1e-6, shows which elements can hold the minimum, and only warps with one --
+// within 1e-5 of the smallest estimate of the block's warps of the same member,
+// and of the minimum found so far -- compute it in FP64.  An estimate
+// outside FP32's range computes it as well.
+__device__ __forceinline__ void cfl_fold(unsigned long long* dmin, bool valid, int mem, double u0, double v0, double H0,
+                                         double rs, double g, double diam, int p) {
+  __shared__ float s_est[32];
+  __shared__ int s_mem[32];
   const unsigned full = 0xffffffffu;
-  const double dmax = 1.7976931348623157e308;
+  const float inf = __int_as_float(0x7f800000);
+  float est = inf;
+  bool odd = false;
+  unsigned long long cur = ~0ull >> 1;
+  if (valid) {
+    cur = __ldcg(dmin + mem);
+    const float r = 1.41421356f * (float)rs, ub = (float)u0 * r, vb = (float)v0 * r, Hb = (float)H0 * r;
+    est = (float)diam / ((sqrtf(ub * ub + vb * vb) + sqrtf((float)g * Hb)) * (2.0f * p + 1.0f));
+    odd = !(est > 1e-30f && est < 1e30f);
+  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int mem0 = __shfl_sync(full, mem, 0);
-  if (__all_sync(full, mem == mem0)) {
+  const bool any = __any_sync(full, valid), one = __all_sync(full, !valid || mem == mem0);
+  float e = odd || !valid ? inf : est;
+  for (int o = 16; o > 0; o >>= 1) e = fminf(e, __shfl_xor_sync(full, e, o));
+  if (lane == 0) {
+    s_est[warp] = e;
+    s_mem[warp] = any && one ? mem0 : -1;
+  }
+  __syncthreads();
+  if (one) {
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
+      if (s_mem[w] == mem0) e = fminf(e, s_est[w]);
+  } else {
+    e = inf;  // members mixed inside the warp: nothing to compare with
+  }
+  const bool cand = valid && (odd || (est <= e * 1.00001f && est * 0.99999f <= (float)__longlong_as_double((long long)cur)));
+  if (!__any_sync(full, cand)) return;
+  const double dmax = 1.7976931348623157e308;
+  double d = cand ? cfl_bound(u0, v0, H0, rs, g, diam, p) : dmax;
+  if (one) {  // one atomic per warp
     for (int o = 16; o > 0; o >>= 1) d = fmin(d, __shfl_xor_sync(full, d, o));
-    if ((threadIdx.x & 31) == 0 && d < dmax) atomicMin(dmin + mem0, (unsigned long long)__double_as_longlong(d));
+    if (lane == 0 && d < dmax) atomicMin(dmin + mem0, (unsigned long long)__double_as_longlong(d));
   } else if (d < dmax) {
     atomicMin(dmin + mem, (unsigned long long)__double_as_longlong(d));
   }

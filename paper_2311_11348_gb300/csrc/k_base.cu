@@ -305,12 +305,10 @@ __global__ void __launch_bounds__(256) k_usolve_base(DevMesh m, int64_t n_end, P
                                                      double* __restrict__ ub, float* __restrict__ ub32,
                                                      unsigned* status, unsigned long long* dmin) {
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  double dcfl = DBL_MAX;
-  int mem = 0;
+  double u0 = 0.0, v0 = 0.0, H0 = 0.0;
   if (e < n_end) {
     const int64_t ne = m.ne;
-    const double rs = m.geo[G_RS * ne + e];
-    const double H0 = cb[0 * ne + e] + m.geo[G_HB0 * ne + e];
+    H0 = cb[0 * ne + e] + m.geo[G_HB0 * ne + e];
     const double U0 = cb[3 * ne + e], V0 = cb[6 * ne + e];
     if (!(H0 * m.geo[G_M0 * ne + e] > ph.h_min)) {  // mean depth: mode 0 times phi_{e,1} = phihat_1 / s_e
       atomicOr(status, (unsigned)ST_DEPTH);
@@ -346,12 +344,14 @@ __global__ void __launch_bounds__(256) k_usolve_base(DevMesh m, int64_t n_end, P
       ub[i * ne + e] = v[i];
       if (ub32) ub32[i * ne + e] = (float)v[i];
     }
-    if (dmin) {
-      mem = m.mem[e];
-      dcfl = cfl_bound(v[0], v[3], H0, rs, ph.g, m.geo[G_DIAM * ne + e], m.p[e]);
-    }
+    u0 = v[0];
+    v0 = v[3];
   }
-  if (dmin) cfl_min_store(dmin, mem, dcfl);  // uniform over the grid: every lane of the warp is here
+  if (dmin) {  // uniform over the grid: every thread of the block is here
+    const bool in = e < n_end;
+    const int64_t x = in ? e : 0;
+    cfl_fold(dmin, in, m.mem[x], u0, v0, H0, m.geo[G_RS * m.ne + x], ph.g, m.geo[G_DIAM * m.ne + x], m.p[x]);
+  }
 }
 
 int launch_usolve_base(cudaStream_t s, const DevMesh& m, const Groups& G, const Phys& ph, const double* cb,

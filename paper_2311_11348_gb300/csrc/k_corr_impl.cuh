@@ -22,7 +22,6 @@
 //
 // With CORR_TC defined (k_corr_tc.cu) the element update of the orders 3 and 4
 // is that file's tensor-core kernel.
-#include <cfloat>
 #include <cstdio>
 
 #include "base_edge.cuh"
@@ -253,8 +252,7 @@ __device__ __forceinline__ void usolve_corr_body(const DevMesh& m, int64_t g0, i
                                                  unsigned* status, unsigned long long* dmin,
                                                  double* __restrict__ rc, int64_t rc_off, int64_t nrc) {
   const int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  double dcfl = DBL_MAX;
-  int mem = 0;
+  double u00 = 0.0, v00 = 0.0, H0d = 0.0;  // mode 0 of u and v as stored, and of the depth (FP64)
   if (l < n) {
     const int64_t e = g0 + l, ne = m.ne;
     constexpr int KH = K - 3, NP = K * (K + 1) / 2;
@@ -266,7 +264,7 @@ __device__ __forceinline__ void usolve_corr_body(const DevMesh& m, int64_t g0, i
     H[1] += geo[G_HB1 * ne + e];
     H[2] += geo[G_HB2 * ne + e];
     // depth check on the FP64 mean (base modes are FP64 in every mode)
-    const double H0d = c.cb[e] + m.geo[G_HB0 * ne + e];
+    H0d = c.cb[e] + m.geo[G_HB0 * ne + e];
     if (!(H0d * m.geo[G_RS * ne + e] * 1.4142135623730951 > ph.h_min)) {
       atomicOr(status, (unsigned)ST_DEPTH);
       atomicOr(m.mstatus + m.mem[e], (unsigned)ST_DEPTH);
@@ -282,29 +280,48 @@ __device__ __forceinline__ void usolve_corr_body(const DevMesh& m, int64_t g0, i
         A[pk(i, j)] = acc;
       });
     });
-    // LDL^T: A[pk(i,j)] (i > j) <- L_ij, rd[j] = 1/d_j (row j's products L_jk d_k
-    // are shared by every row below it: one multiply-add per (i, j, k))
-    T dg[K], rd[K];
-    sfor<0, K>([&](auto j) {
-      T ld[K];
-      T dj = A[pk(j, j)];
-      sfor<0, j>([&](auto k) {
-        ld[k] = A[pk(j, k)] * dg[k];
-        dj -= A[pk(j, k)] * ld[k];
+    T rd[K];  // 1/d_j
+    if constexpr (!kF32 && K == 15) {
+      // LDL^T: row j's products L_jk d_k are shared by every row below it
+      T dg[K];
+      sfor<0, K>([&](auto j) {
+        T ld[K];
+        T dj = A[pk(j, j)];
+        sfor<0, j>([&](auto k) {
+          ld[k] = A[pk(j, k)] * dg[k];
+          dj = fma(-A[pk(j, k)], ld[k], dj);
+        });
+        dg[j] = dj;
+        rd[j] = (T)1 / dj;
+        sfor<j + 1, K>([&](auto i) {
+          T w = A[pk(i, j)];
+          sfor<0, j>([&](auto k) { w = fma(-A[pk(i, k)], ld[k], w); });
+          A[pk(i, j)] = w * rd[j];
+        });
       });
-      dg[j] = dj;
-      rd[j] = (T)1 / dj;
-      sfor<j + 1, K>([&](auto i) {
-        T w = A[pk(i, j)];
-        sfor<0, j>([&](auto k) { w -= A[pk(i, k)] * ld[k]; });
-        A[pk(i, j)] = w * rd[j];
+    } else {
+      // row j holds W_jk = L_jk d_k until its turn, then L_jk: one product per
+      // entry fewer (FP64, K = 15 spills more registers this way: 95 against 77 us
+      // for up to 10,000 elements)
+      sfor<0, K>([&](auto j) {
+        T dj = A[pk(j, j)];
+        sfor<0, j>([&](auto k) {
+          const T L = A[pk(j, k)] * rd[k];
+          dj = fma(-A[pk(j, k)], L, dj);
+          A[pk(j, k)] = L;
+        });
+        rd[j] = (T)1 / dj;
+        sfor<j + 1, K>([&](auto i) {
+          T w = A[pk(i, j)];
+          sfor<0, j>([&](auto k) { w = fma(-A[pk(i, k)], A[pk(j, k)], w); });
+          A[pk(i, j)] = w;
+        });
       });
-    });
+    }
     T x[2][K];
     load_modes<K>(x[0], cb, ne, e, ch, n, l, 1);
     load_modes<K>(x[1], cb, ne, e, ch, n, l, 2);
     const T s = sv;
-    double u00 = 0.0, v00 = 0.0;  // mode 0 of u and v as stored (FP64)
     sfor<0, 2>([&](auto r) {
       sfor<0, K>([&](auto i) { sfor<0, i>([&](auto k) { x[r][i] -= A[pk(i, k)] * x[r][k]; }); });
       sfor<0, K>([&](auto i) { x[r][i] *= rd[i]; });
@@ -325,10 +342,6 @@ __device__ __forceinline__ void usolve_corr_body(const DevMesh& m, int64_t g0, i
         }
       });
     });
-    if (dmin) {
-      mem = m.mem[e];
-      dcfl = cfl_bound(u00, v00, H0d, m.geo[G_RS * ne + e], ph.g, m.geo[G_DIAM * ne + e], m.p[e]);
-    }
     T xi[K], U[K], V[K];
     load_modes<K>(xi, cb, ne, e, ch, n, l, 0);
     load_modes<K>(U, cb, ne, e, ch, n, l, 1);
@@ -359,7 +372,11 @@ __device__ __forceinline__ void usolve_corr_body(const DevMesh& m, int64_t g0, i
       rc[3 * nrc + rc_off + l] = (double)(x2 * e3 + y2 * e4);
     }
   }
-  if (dmin) cfl_min_store(dmin, mem, dcfl);  // uniform over the grid: every lane of the warp is here
+  if (dmin) {  // uniform over the grid: every thread of the block is here
+    const bool in = l < n;
+    const int64_t x = in ? g0 + l : 0;
+    cfl_fold(dmin, in, m.mem[x], u00, v00, H0d, m.geo[G_RS * m.ne + x], ph.g, m.geo[G_DIAM * m.ne + x], m.p[x]);
+  }
 }
 
 // The compiler's register allocation (FP32: 80, 127, 255 registers for K =
