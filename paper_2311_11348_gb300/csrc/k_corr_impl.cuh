@@ -22,7 +22,9 @@
 //
 // With CORR_TC defined (k_corr_tc.cu) the element update of the orders 3 and 4
 // is that file's tensor-core kernel.
+#include <algorithm>
 #include <cstdio>
+#include <vector>
 
 #include "base_edge.cuh"
 #include "kernels.h"
@@ -91,6 +93,47 @@ __constant__ T cEL[3][KMAX][5];     // phihat_i(gamma_k(s)) = sum_l cEL[k][i][l]
 __constant__ T cGP[3][4][5];        // per PM-2: P_l at the points t > 0 (then the middle one) of the npts_for(PM) rule on [-1,1]
 __constant__ T cGW[3][4];           // their weights (the rule's weights on [0,1])
 
+#ifdef CORR_LANES
+// Terms of the entries S_ij = sum_n H_n T[n][i][j] (j <= i < 15, n < ktr(i, j), structural
+// zeros left out; 390 of them) dealt to 16 lanes for k_usolve_lanes, the longest entries first,
+// each to the lane with the fewest terms so far: step s of lane t adds H_n t to
+// its running sum, and stores it at pk(i, j) after the entry's last term.
+constexpr int UL_STEPS = 32;
+struct UsolveTerms {
+  double t[UL_STEPS][16];
+  int code[UL_STEPS][16];  // n | (destination << 8, 255 while the sum goes on)
+  int steps;
+};
+__device__ UsolveTerms gUsolve;
+
+static void usolve_terms(UsolveTerms* U) {
+  constexpr int K = 15;
+  const RefTables& R = tables();
+  struct Entry { int i, j, nz; };
+  std::vector<Entry> es;
+  for (int i = 0; i < K; ++i)
+    for (int j = 0; j <= i; ++j) {
+      int nz = 0;
+      for (int n = 0; n < ktr(i, j); ++n) nz += tnz(n, i, j);
+      es.push_back({i, j, nz});
+    }
+  std::stable_sort(es.begin(), es.end(), [](const Entry& a, const Entry& b) { return a.nz > b.nz; });
+  for (int s = 0; s < UL_STEPS; ++s)
+    for (int t = 0; t < 16; ++t) { U->t[s][t] = 0; U->code[s][t] = 255 << 8; }
+  int used[16] = {};
+  for (const Entry& e : es) {
+    const int t = (int)(std::min_element(used, used + 16) - used);
+    int left = e.nz;
+    for (int n = 0; n < ktr(e.i, e.j); ++n) {
+      if (!tnz(n, e.i, e.j)) continue;
+      U->t[used[t]][t] = R.T[n][e.i][e.j];
+      U->code[used[t]++][t] = n | (--left == 0 ? pk(e.i, e.j) : 255) << 8;
+    }
+  }
+  U->steps = *std::max_element(used, used + 16);  // 25
+}
+#endif
+
 // P_0 .. P_4 at t
 static void legendre5(double t, double (&P)[5]) {
   P[0] = 1.0;
@@ -129,6 +172,11 @@ void upload_tables() {
       gw[pm - 2][j] = j < H || mid ? (T)R.ew[N][N - 1 - j] : (T)0;
     }
   }
+#ifdef CORR_LANES
+  static UsolveTerms ut;
+  usolve_terms(&ut);
+  cudaMemcpyToSymbol(gUsolve, &ut, sizeof ut);
+#endif
   cudaMemcpyToSymbol(cT, t, sizeof t);
   cudaMemcpyToSymbol(cDx, dx, sizeof dx);
   cudaMemcpyToSymbol(cDs, ds, sizeof ds);
@@ -275,7 +323,7 @@ __device__ __forceinline__ void usolve_corr_body(const DevMesh& m, int64_t g0, i
       sfor<0, j + 1>([&](auto i) {
         T acc = 0;
         sfor<0, ktr(i, j)>([&](auto nn) {
-          if constexpr (tnz(nn, i, j)) acc += H[nn] * cT[nn][pk(i, j)];
+          if constexpr (tnz(nn, i, j)) acc = fma(H[nn], cT[nn][pk(i, j)], acc);
         });
         A[pk(i, j)] = acc;
       });
@@ -323,11 +371,14 @@ __device__ __forceinline__ void usolve_corr_body(const DevMesh& m, int64_t g0, i
     load_modes<K>(x[1], cb, ne, e, ch, n, l, 2);
     const T s = sv;
     sfor<0, 2>([&](auto r) {
-      sfor<0, K>([&](auto i) { sfor<0, i>([&](auto k) { x[r][i] -= A[pk(i, k)] * x[r][k]; }); });
+      sfor<0, K>([&](auto i) { sfor<0, i>([&](auto k) { x[r][i] = fma(-A[pk(i, k)], x[r][k], x[r][i]); }); });
       sfor<0, K>([&](auto i) { x[r][i] *= rd[i]; });
       sfor<0, K>([&](auto ii) {
         constexpr int i = K - 1 - ii;
-        sfor<i + 1, K>([&](auto k) { x[r][i] -= A[pk(k, i)] * x[r][k]; });
+        sfor<0, ii>([&](auto kk) {
+          constexpr int k = K - 1 - kk;
+          x[r][i] = fma(-A[pk(k, i)], x[r][k], x[r][i]);
+        });
       });
       sfor<0, K>([&](auto i) {
         const T v = x[r][i] * s;
@@ -357,19 +408,19 @@ __device__ __forceinline__ void usolve_corr_body(const DevMesh& m, int64_t g0, i
       T e1 = 0, e2 = 0, e3 = 0, e4 = 0, px = 0;
       sfor<3, K>([&](auto j) {
         const T uu = x[0][j] * s, vv = x[1][j] * s;  // the velocity modes as stored above
-        e1 += U[j] * uu; e2 += U[j] * vv;
-        e3 += V[j] * uu; e4 += V[j] * vv;
-        px += xi[j] * xi[j];
+        e1 = fma(U[j], uu, e1); e2 = fma(U[j], vv, e2);
+        e3 = fma(V[j], uu, e3); e4 = fma(V[j], vv, e4);
+        px = fma(xi[j], xi[j], px);
       });
-      const T gp = (T)0.5 * (T)ph.g * px;
-      e1 += gp;
-      e4 += gp;
+      const T hg = (T)0.5 * (T)ph.g;
+      e1 = fma(hg, px, e1);
+      e4 = fma(hg, px, e4);
       const T x1 = geo[G_GQ1X * ne + e], y1 = geo[G_GQ1Y * ne + e];
       const T x2 = geo[G_GQ2X * ne + e], y2 = geo[G_GQ2Y * ne + e];
-      rc[0 * nrc + rc_off + l] = (double)(x1 * e1 + y1 * e2);
-      rc[1 * nrc + rc_off + l] = (double)(x2 * e1 + y2 * e2);
-      rc[2 * nrc + rc_off + l] = (double)(x1 * e3 + y1 * e4);
-      rc[3 * nrc + rc_off + l] = (double)(x2 * e3 + y2 * e4);
+      rc[0 * nrc + rc_off + l] = (double)fma(x1, e1, y1 * e2);
+      rc[1 * nrc + rc_off + l] = (double)fma(x2, e1, y2 * e2);
+      rc[2 * nrc + rc_off + l] = (double)fma(x1, e3, y1 * e4);
+      rc[3 * nrc + rc_off + l] = (double)fma(x2, e3, y2 * e4);
     }
   }
   if (dmin) {  // uniform over the grid: every thread of the block is here
@@ -400,6 +451,132 @@ __global__ void __launch_bounds__(128, 3) k_usolve_corr15(DevMesh m, int64_t g0,
   usolve_corr_body<15>(m, g0, n, ph, c, ch, ub, ub32, uh, tr, trv, status, dmin, rc, rc_off, nrc);
 }
 
+// The solve of FP64 groups of order 4 with 16 lanes per element, for small groups:
+// one thread runs 1,700 FP64 instructions one after the other, 64 cycles each.
+// Lane i holds row i; the entries are summed by the lanes in shares of equal
+// length and the elimination broadcasts L_kj d_j from lane to lane, about 300
+// instructions per warp of two elements (twice the total).  Every operation on an
+// element is the same, in the same order, as in the one-thread form, so the
+// results are too.  77 us for any group up to 10,000 elements on one thread; 24 us
+// here for 512, 70 for 5,000 (GB300); beside the other groups' kernels, which share
+// the FP64 pipe, it pays up to about 3,000.
+#ifdef CORR_LANES
+constexpr int64_t UL_MAX = 3000;
+constexpr int UL_BLOCK = 128, UL_EL = UL_BLOCK / 16;
+__global__ void __launch_bounds__(UL_BLOCK) k_usolve_lanes(DevMesh m, int64_t g0, int64_t n, Phys ph, StateDev c,
+                                                           const T* __restrict__ ch, double* __restrict__ ub,
+                                                           T* __restrict__ uh,
+                                                           T* __restrict__ tr, T* __restrict__ trv, unsigned* status,
+                                                           unsigned long long* dmin, double* __restrict__ rc,
+                                                           int64_t rc_off, int64_t nrc) {
+  constexpr int K = 15, KH = K - 3, NP = K * (K + 1) / 2;
+  __shared__ T sA[UL_EL][NP], sH[UL_EL][16], sx[UL_EL][5][16];
+  const unsigned full = 0xffffffffu;
+  const int g = threadIdx.x >> 4, i = threadIdx.x & 15;
+  const int64_t l = blockIdx.x * (int64_t)UL_EL + g, ne = m.ne;
+  const bool live = l < n, row = live && i < K;
+  const int64_t e = g0 + (live ? l : 0);
+  const T* cb = base_c(c);
+  const T* geo = geo_t(m);
+  T xi = 0, x[2] = {0, 0};
+  if (row) {
+    if (i < 3) {
+      xi = cb[i * ne + e]; x[0] = cb[(3 + i) * ne + e]; x[1] = cb[(6 + i) * ne + e];
+    } else {
+      xi = ch[(i - 3) * n + l]; x[0] = ch[(KH + i - 3) * n + l]; x[1] = ch[(2 * KH + i - 3) * n + l];
+    }
+  }
+  const T U = x[0], V = x[1];
+  double H0d = 0.0;
+  if (live && i == 0) {  // depth check on the FP64 mean
+    H0d = c.cb[e] + m.geo[G_HB0 * ne + e];
+    if (!(H0d * m.geo[G_RS * ne + e] * 1.4142135623730951 > ph.h_min)) {
+      atomicOr(status, (unsigned)ST_DEPTH);
+      atomicOr(m.mstatus + m.mem[e], (unsigned)ST_DEPTH);
+    }
+  }
+  sH[g][i] = row && i < 3 ? xi + geo[(G_HB0 + i) * ne + e] : xi;
+  __syncwarp();
+  {
+    const UsolveTerms& tb = gUsolve;
+    const int steps = tb.steps;
+    T acc = 0;
+    for (int s = 0; s < steps; ++s) {
+      const int code = tb.code[s][i], dst = code >> 8;
+      acc = fma(sH[g][code & 255], tb.t[s][i], acc);
+      if (dst != 255) {
+        sA[g][dst] = acc;
+        acc = 0;
+      }
+    }
+  }
+  __syncwarp();
+  // row i of the lower triangle (lanes without a row: the identity)
+  T a[K], rdi = 1;
+  sfor<0, K>([&](auto j) { a[j] = row && j <= i ? sA[g][pk(i < K ? i : 0, j)] : (T)(j == i); });
+  sfor<0, K>([&](auto j) {
+    const T d = __shfl_sync(full, a[j], j, 16), rd = (T)1 / d;
+    if (i == j) rdi = rd;
+    const T lij = a[j] * rd, ld = lij * d;  // L_ij, L_ij d_j (i > j)
+    sfor<j + 1, K>([&](auto k) {
+      const T ldk = __shfl_sync(full, ld, k, 16);
+      if (i >= k) a[k] = fma(-lij, ldk, a[k]);
+    });
+    if (i > j) a[j] = lij;
+  });
+  sfor<0, K>([&](auto j) {
+    if (row && j < i) sA[g][pk(i < K ? i : 0, j)] = a[j];
+  });
+  __syncwarp();
+  sfor<0, 2>([&](auto r) {
+    sfor<0, K>([&](auto j) {
+      const T xj = __shfl_sync(full, x[r], j, 16);
+      if (i > j) x[r] = fma(-a[j], xj, x[r]);
+    });
+    x[r] *= rdi;
+  });
+  sfor<0, K>([&](auto k) { a[k] = row && i < k ? sA[g][pk(i < K ? i : 0, k)] : (T)0; });  // column i of L
+  sfor<0, 2>([&](auto r) {
+    sfor<0, K>([&](auto kk) {
+      constexpr int k = K - 1 - kk;
+      const T xk = __shfl_sync(full, x[r], k, 16);
+      if (i < k) x[r] = fma(-a[k], xk, x[r]);
+    });
+  });
+  const T s = geo[G_S * ne + e];
+  const T uu = x[0] * s, vv = x[1] * s;
+  if (row) {
+    if (i < 3) {
+      ub[i * ne + e] = (double)uu;
+      ub[(3 + i) * ne + e] = (double)vv;
+    } else {
+      uh[(i - 3) * n + l] = uu;
+      uh[(KH + i - 3) * n + l] = vv;
+    }
+    st4(tr + (l * K + i) * 4, xi, U, V, uu);
+    trv[l * K + i] = vv;
+  }
+  if (rc) {  // see usolve_corr_body; lane q < 4 forms rc[q], lanes 0 .. 4 the five sums
+    sx[g][0][i] = U; sx[g][1][i] = V; sx[g][2][i] = uu; sx[g][3][i] = vv; sx[g][4][i] = xi;
+    __syncwarp();
+    const int pa = i == 4 ? 4 : i >> 1 & 1, pb = i == 4 ? 4 : 2 + (i & 1);  // U u, U v, V u, V v, xi xi
+    T sum = 0;
+    if (i < 5)
+      for (int j = 3; j < K; ++j) sum = fma(sx[g][pa][j], sx[g][pb][j], sum);
+    const T px = __shfl_sync(full, sum, 4, 16);
+    if (i == 0 || i == 3) sum = fma((T)0.5 * (T)ph.g, px, sum);
+    const T ea = __shfl_sync(full, sum, i >> 1 << 1 & 15, 16), eb = __shfl_sync(full, sum, (i >> 1 << 1 | 1) & 15, 16);
+    if (live && i < 4) {
+      const T gx = geo[(i & 1 ? G_GQ2X : G_GQ1X) * ne + e], gy = geo[(i & 1 ? G_GQ2Y : G_GQ1Y) * ne + e];
+      rc[i * nrc + rc_off + l] = (double)fma(gx, ea, gy * eb);
+    }
+  }
+  if (dmin)  // uniform over the grid
+    cfl_fold(dmin, live && i == 0, m.mem[e], (double)uu, (double)vv, H0d, m.geo[G_RS * ne + e], ph.g,
+             m.geo[G_DIAM * ne + e], m.p[e]);
+}
+#endif
+
 template <int K>
 static int usolve_group(cudaStream_t st, const DevMesh& m, const Groups& G, int p, const Phys& ph, StateDev c,
                         VelDev u, unsigned* status, unsigned long long* dmin, void* rc) {
@@ -407,6 +584,16 @@ static int usolve_group(cudaStream_t st, const DevMesh& m, const Groups& G, int 
   if (n == 0) return 0;
   const int64_t nrc = G.start[5] - G.start[2], rc_off = g0 - G.start[2];
   const int ct = spread_threads(n, launch_shape().corr_threads);
+#ifdef CORR_LANES
+  if (K == 15 && n <= UL_MAX) {
+    k_usolve_lanes<<<nblocks(n, UL_EL), UL_BLOCK, 0, st>>>(m, g0, n, ph, c, (const T*)c.ch[p], u.ub, (T*)u.uh[p],
+                                                           (T*)u.tr[p], (T*)u.trv[p], status, dmin, (double*)rc,
+                                                           rc_off, nrc);
+    count_launch();
+    SWE_CUDA_OK(cudaGetLastError());
+    return 0;
+  }
+#endif
   if (K == 15 && kF32 && launch_shape().base_bpsm > 0)
     k_usolve_corr15<<<nblocks(n, ct), ct, 0, st>>>(m, g0, n, ph, c, (const T*)c.ch[p], u.ub, u.ub32,
                                                    (T*)u.uh[p], (T*)u.tr[p], (T*)u.trv[p], status, dmin,

@@ -59,9 +59,14 @@ def test_correction_kernels_on_ragged_groups(prec, nx, ny):
     assert max(err) < TOL[prec], err
 
 
-@pytest.mark.parametrize("p,sizes", [(4, [(50, 60), (40, 50)]), (3, [(64, 78), (50, 60)]), (2, [(100, 100), (60, 70)])])
-def test_member_alone_and_in_a_union_across_the_size_rule_bitwise(p, sizes):
-    """alone the first member's group is at most 60,000 / K(p-1) elements, in the union it is more"""
+@pytest.mark.parametrize("prec,p,sizes", [(swedg.PREC_MIXED_FP32, 4, [(50, 60), (40, 50)]),
+                                          (swedg.PREC_MIXED_FP32, 3, [(64, 78), (50, 60)]),
+                                          (swedg.PREC_MIXED_FP32, 2, [(100, 100), (60, 70)]),
+                                          (swedg.PREC_FP64, 4, [(30, 50), (20, 30)]),
+                                          (swedg.PREC_FP64, 4, [(69, 70), (20, 30)])])
+def test_member_alone_and_in_a_union_across_the_size_rules_bitwise(prec, p, sizes):
+    """alone the first member's group runs one form of the element update or of the velocity solve, in the union
+    another (FP32: K(p-1) n = 60,000; FP64, order 4: 3,000 and 9,728 elements)"""
     from paper_2311_11348_gb300.ensemble import Ensemble
     members, states = [], []
     for k, (nx, ny) in enumerate(sizes):
@@ -77,9 +82,17 @@ def test_member_alone_and_in_a_union_across_the_size_rule_bitwise(p, sizes):
         states.append(c)
     out = []
     for ms, cs in ((members[:1], states[:1]), (members, states)):
-        e = Ensemble(ms, g=9.81, rk_order=3, precision=swedg.PREC_MIXED_FP32)
+        e = Ensemble(ms, g=9.81, rk_order=3, precision=prec)
         e.set_states(cs)
         e.run(2)
         out.append(e.states()[0])
         e.close()
     assert np.isfinite(out[0]).all() and np.array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("nx,ny", [(1, 4), (1, 5), (30, 50), (31, 49)])
+def test_velocity_solve_forms_meet_at_the_size_rule(nx, ny):
+    """FP64, order 4: one full block of the sixteen-lane form (8 elements), one more, its largest group (3,000)
+    and a larger one"""
+    err = rhs_errors(lambda n: np.full(n, 4, np.int8), nx, ny, swedg.PREC_FP64)
+    assert max(err) < TOL[swedg.PREC_FP64], err
