@@ -1120,9 +1120,17 @@ __global__ void __launch_bounds__(128, K == 6 ? 5 : K == 10 ? 4 : 3) k_elem_corr
   });
 }
 
-template <int K>
-__global__ void __launch_bounds__(32 * Kof(deg_of(K - 1) - 1)) k_elem_corr_split(ELEM_CORR_PARAMS) {
+// warp of mode M among W: its own, or for K = 15 on five warps a pair of a long and a short mode
+template <int K, int W>
+__host__ __device__ constexpr int warp_of(int M) {
+  constexpr int five[10] = {0, 4, 1, 1, 4, 2, 3, 0, 2, 3};
+  return W == 5 ? five[M] : M;
+}
+
+template <int K, int W>
+__global__ void __launch_bounds__(32 * W, K == 15 && W == 5 ? 2 : 1) k_elem_corr_split(ELEM_CORR_PARAMS) {
   constexpr int KL = Kof(deg_of(K - 1) - 1), KH = K - 3;
+  static_assert(W == KL || (K == 15 && W == 5), "warps of a block");
   __shared__ T B[KL][6][32];  // per mode m: the factors of D_x and D_s in the three equations
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t l = blockIdx.x * (int64_t)32 + lane;
@@ -1141,7 +1149,7 @@ __global__ void __launch_bounds__(32 * Kof(deg_of(K - 1) - 1)) k_elem_corr_split
     const T La = geo[G_JI0 * ne + e] + (T)0.5 * J2, Lb = geo[G_JI1 * ne + e] + (T)0.5 * J3;
     const T xh[3] = {xi[0] + geo[G_HB0 * ne + e], xi[1] + geo[G_HB1 * ne + e], xi[2] + geo[G_HB2 * ne + e]};
     sfor<0, KL>([&](auto M) {
-      if (w == M) {  // uniform over the warp
+      if (w == warp_of<K, W>(M)) {  // uniform over the warp
         T z[4];
         products<K, M>(z, xi, U, V, u, v, xh, (T)ph.g);
         T x[3], s[3];
@@ -1160,7 +1168,7 @@ __global__ void __launch_bounds__(32 * Kof(deg_of(K - 1) - 1)) k_elem_corr_split
   const T tau = friction(m, ph, e, rs, cbS[e], ub[e], ub[3 * ne + e]);
   const T dt = (T)stage_dt(stg, m.mem[e]);
   sfor<3, K>([&](auto q) {
-    if ((q - 3) % KL == w) {  // uniform over the warp
+    if ((q - 3) % W == w) {  // uniform over the warp
       T r[3];
 #pragma unroll
       for (int f = 0; f < 3; ++f) {
@@ -1199,7 +1207,12 @@ static int elem_group(cudaStream_t st, const DevMesh& m, const Groups& G, int p,
   T* chO = (T*)cO.ch[p];
   constexpr int KL = Kof(deg_of(K - 1) - 1);
   if (!kF32 || n * KL <= 60000) {
-    k_elem_corr_split<K><<<nblocks(n, 32), 32 * KL, 0, st>>>(m, g0, n, ph, stg, cb, chS, chN, chO, ub, uh, pe);
+    bool five = false;
+    if constexpr (K == 15 && !kF32) {
+      five = n > 9728;  // two blocks of ten warps per SM and more
+      if (five) k_elem_corr_split<K, 5><<<nblocks(n, 32), 160, 0, st>>>(m, g0, n, ph, stg, cb, chS, chN, chO, ub, uh, pe);
+    }
+    if (!five) k_elem_corr_split<K, KL><<<nblocks(n, 32), 32 * KL, 0, st>>>(m, g0, n, ph, stg, cb, chS, chN, chO, ub, uh, pe);
   } else if constexpr (kF32) {
     const int t = launch_shape().corr_threads;
     k_elem_corr<K><<<nblocks(n, t), t, 0, st>>>(m, g0, n, ph, stg, cb, chS, chN, chO, ub, uh, pe);
