@@ -108,6 +108,7 @@ struct swe_ctx {
   VelDev vel{};
   EdgeFlux fx{};
   void* rc = nullptr;
+  float* tcb = nullptr;  // tensor-core mode: the constant operands of the GEMMs
   double* d_user = nullptr;
   double* d_user2 = nullptr;
   int64_t* d_off = nullptr;  // packed caller layout: offset of each caller element's 3 K(p) values
@@ -689,6 +690,12 @@ static int build_device(swe_ctx* ctx) {
   ctx->dm.mstatus = ctx->d_mstatus;
   if ((rc = dalloc(ctx, &ctx->d_work, sizeof(unsigned) * 4))) return cuda_err(ctx, rc);
   cudaMemsetAsync(ctx->d_work, 0, sizeof(unsigned) * 4, ctx->stream);
+  if (ctx->tc) {
+    size_t bytes = 0;
+    const float* img = corrtc::tc_operand(&bytes);
+    if ((rc = dalloc(ctx, &ctx->tcb, bytes))) return cuda_err(ctx, rc);
+    CU(cudaMemcpyAsync(ctx->tcb, img, bytes, cudaMemcpyHostToDevice, ctx->stream));
+  }
   // the order-dependent part
   CU(cudaMemcpyAsync(ctx->d_newp, ctx->p_user.data(), (size_t)ne, cudaMemcpyHostToDevice, ctx->stream));
   ctx->packed_n = -1;
@@ -842,7 +849,8 @@ static int run_stage(swe_ctx* ctx, StateDev in, StateDev nst, StateDev out, cons
     }
     if (ctx->tc) {  // orders 3 and 4, beside order 2
       ProfScope ps(ctx, F_VOLTC);
-      CK(corrtc::launch_elem_tc(gs.s[1], ctx->dm, ctx->G, ph, stg, in, nst, out, ctx->vel, ctx->fx, ctx->d_status));
+      CK(corrtc::launch_elem_tc(gs.s[1], ctx->dm, ctx->G, ph, stg, in, nst, out, ctx->vel, ctx->fx, ctx->tcb,
+                                ctx->d_status));
     }
     CK(join_groups());
   }

@@ -117,8 +117,7 @@ __host__ __device__ constexpr int tc_smem(int K) { return (3 * TC_ABUF + tc_bflo
 static_assert(tc_ctas(15) * (tc_smem(15) + 1024) <= 227 * 1024 && tc_ctas(10) * (tc_smem(10) + 1024) <= 227 * 1024,
               "shared memory of an SM");
 
-__device__ __align__(128) float gTcB[TC_BTOTAL];
-static const float* g_tcb[64];  // device address of gTcB per device ordinal
+static float g_tcb[TC_BTOTAL];  // both B images (host); a context keeps its own device copy
 
 // round to the nearest value with a 10-bit mantissa (ties away from zero)
 static inline float tf32_round(float x) {
@@ -481,11 +480,7 @@ static int tc_group(cudaStream_t st, const DevMesh& m, const Groups& G, int p, c
 }
 
 int launch_elem_tc(cudaStream_t st, const DevMesh& m, const Groups& G, const Phys& ph, const Stage& stg, StateDev cS,
-                   StateDev cN, StateDev cO, VelDev u, EdgeFlux fx, unsigned* status) {
-  int dev = 0;
-  SWE_CUDA_OK(cudaGetDevice(&dev));
-  const float* bimg = (dev >= 0 && dev < 64) ? g_tcb[dev] : nullptr;
-  if (!bimg) return -1;
+                   StateDev cN, StateDev cO, VelDev u, EdgeFlux fx, const float* bimg, unsigned* status) {
   int r = tc_group<15>(st, m, G, 4, ph, stg, cS, cN, cO, u, fx, status, bimg);
   if (!r) r = tc_group<10>(st, m, G, 3, ph, stg, cS, cN, cO, u, fx, status, bimg);
   return r;
@@ -523,17 +518,17 @@ int launch_wait_selftest(cudaStream_t st, int64_t spins, unsigned* status) {
   return 0;
 }
 
-// B images and kernel attributes of the current device (once per context creation)
+const float* tc_operand(size_t* bytes) {
+  *bytes = sizeof g_tcb;
+  return g_tcb;
+}
+
+// B images (host) and kernel attributes of the current device (once per device and process)
 int upload_tc_tables() {
-  static float img[TC_BTOTAL];
-  tc_b_image<10>(img + tc_boff(10));
-  tc_b_image<15>(img + tc_boff(15));
-  SWE_CUDA_OK(cudaMemcpyToSymbol(gTcB, img, sizeof img));
+  tc_b_image<10>(g_tcb + tc_boff(10));
+  tc_b_image<15>(g_tcb + tc_boff(15));
   int dev = 0;
   SWE_CUDA_OK(cudaGetDevice(&dev));
-  void* a = nullptr;
-  SWE_CUDA_OK(cudaGetSymbolAddress(&a, gTcB));
-  if (dev >= 0 && dev < 64) g_tcb[dev] = (const float*)a;
   SWE_CUDA_OK(cudaFuncSetAttribute(k_elem_tc<10>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem(10)));
   SWE_CUDA_OK(cudaFuncSetAttribute(k_elem_tc<15>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem(15)));
   int nsm = 0;

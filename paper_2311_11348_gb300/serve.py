@@ -83,6 +83,8 @@ def device_bytes(meshes, precision):
         allocs += [ts * 2 * (KP[q] - 3) * n[q], ts * 4 * KP[q] * n[q], ts * KP[q] * n[q]]
         allocs += [ts * 3 * 3 * (KP[q] - 3) * n[q]]                                        # projected edge fluxes
     allocs += [32 * max(nrc, 1)]
+    if precision == swedg.PREC_MIXED_TF32:
+        allocs += [128 * (32 + 80)]                                                         # tensor-core operands
     b = sum(a if a > 0 else 16 for a in allocs)  # the library allocates 16 bytes for an empty array
     return b
 
