@@ -5,8 +5,8 @@
 // One RK stage (Sect. 2 time stepping, Sect. 3 order separation):
 //   usolve(base) + usolve(correction)      uH = q on every element
 //   [first stage of a CFL step: dt = cfl * min ...]
-//   edge_base -> edge_corr                 LF fluxes at Gauss points
-//   elem_corr -> elem_base                 volume/source/edge projections and
+//   edge_base + edge_corr                  LF fluxes
+//   elem_corr + elem_base                  volume/source/edge projections and
 //                                          the SSP-RK combination
 #include <algorithm>
 #include <cmath>
@@ -604,7 +604,7 @@ static int build_device(swe_ctx* ctx) {
     eLu[i] = ed[i].L; eRu[i] = ed[i].R; einfo[i] = ed[i].info;
     emem[i] = ctx->member_user[ed[i].L];
     auto E_ = [&](int row) -> double& { return egeo[(size_t)row * nE + i]; };
-    E_(E_LEN) = ed[i].len; E_(E_NX) = ed[i].nx; E_(E_NY) = ed[i].ny;
+    E_(E_NX) = ed[i].nx; E_(E_NY) = ed[i].ny;
     E_(E_HA) = ed[i].hA; E_(E_HB) = ed[i].hB;
     E_(E_HG0) = ed[i].hA + R.es[2][0] * (ed[i].hB - ed[i].hA);
     E_(E_HG1) = ed[i].hA + R.es[2][1] * (ed[i].hB - ed[i].hA);

@@ -68,8 +68,7 @@ enum {
 
 // rows of the per-edge geometry table
 enum {
-  E_LEN = 0,  // |E|
-  E_NX,       // outward unit normal of the left element
+  E_NX = 0,   // outward unit normal of the left element
   E_NY,
   E_HA,       // h_b at gamma(0) and gamma(1) of the left element's parametrisation
   E_HB,

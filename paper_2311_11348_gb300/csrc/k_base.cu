@@ -8,10 +8,11 @@
 //                  (and, in the first stage of a step, the CFL bounds of its
 //                  elements: min over elements, exact, order independent)
 //   k_edge_base    Lax-Friedrichs flux (Sect. 2) of the P1 traces at the two
-//                  Gauss points of every edge, lambda of Eq. (10) from means
+//                  Gauss points of the edges between elements of order <= 1,
+//                  lambda of Eq. (10) from means
 //   k_elem_base    volume + source terms (Eq. 13 with the degree-1 tensors in
-//                  closed form), edge projections, correction merge and the
-//                  SSP-RK stage combination of the base modes
+//                  closed form), edge projections, rc and the SSP-RK stage
+//                  combination of the base modes
 #include <cfloat>
 
 #include "base_edge.cuh"

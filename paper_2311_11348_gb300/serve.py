@@ -34,7 +34,7 @@ from .ensemble import Ensemble
 
 KMAX = swedg.KMAX
 KP = (1, 3, 6, 10, 15)
-NGEO, NEGEO = 20, 11  # rows of the element and edge geometry tables
+NGEO, NEGEO = 20, 10  # rows of the element and edge geometry tables
 
 
 def device_bytes(meshes, precision):
