@@ -39,7 +39,7 @@ TF32_OVER_BF16 = 1.1 / 2.25
 
 LEG = [0, 1, 0, 2, 1, 0, 3, 2, 1, 0, 4, 3, 2, 1, 0]  # Legendre index of each mode
 
-USOLVE_P1 = 76   # the 3 x 3 solve with the entries the orthonormal basis fixes left out
+USOLVE_P1 = 70   # the 3 x 3 solve with the entries the orthonormal basis fixes left out
 EDGE_BASE = 152
 ELEM_BASE = 208  # a stage with the full SSP-RK combination
 ELEM_BASE_EULER = 181  # the first stage (c + dt r)
@@ -156,6 +156,14 @@ def family_flops(orders, fam, nedge=None, mode="mixed"):
             tot += pr * nedge * edge_corr_flops(KP[pm], KP[max(1, pm - 1)], pm, mode == "fp64")
         return st * tot
     return None
+
+
+def edge_corr_fp64_flops(orders, nedge=None):
+    """FP64 flops per SSP-RK3 step of the base flux that the correction edge
+    kernels carry (edges with max(p_L, p_R) >= 2)"""
+    p = np.asarray(orders)
+    nedge = nedge or int(round(1.5 * len(p)))
+    return 3 * EDGE_BASE * nedge * (1.0 - float((p <= 1).mean()) ** 2)
 
 
 def pipe_of(fam, mode):
