@@ -21,7 +21,7 @@
 // but the solve's.  FP64 instructions bound these kernels (GB300: 19 cycles of
 // an SM each, 64 of the warp): about 95 per element in k_na_usolve, 97 per edge,
 // 130 per element in k_na_elem, where the modal form with its geometry formed at
-// every visit took 1,900 per element; 72 -> 40 us for 20,000 elements (GB300).
+// every visit took 1,900 per element; 72 -> 41 us for 20,000 elements (GB300).
 #include <cuda.h>
 
 #include <cmath>
