@@ -454,19 +454,18 @@ int launch_edge_base(cudaStream_t s, const DevMesh& m, const int32_t* list, int6
 // f_c U_q with bottom friction and Coriolis), and the edge terms are
 // -sum_g F_g phi_q(x_g) over the three edges (sign flipped for the right side).
 // ---------------------------------------------------------------------------
-// MINB: blocks per SM the register allocation must allow -- 4 (128 registers)
-// for uncapped grids, where the kernel's own occupancy is what counts; 3 for
-// grids capped at a few blocks per SM beside the correction kernels, where
-// the measured step is faster with the unrestricted allocation
-template <int MINB>
-__global__ void __launch_bounds__(128, MINB) k_elem_base(DevMesh m, Phys ph, Stage stg, const double* __restrict__ cbS,
-                                                   const double* __restrict__ cbN, double* __restrict__ cbO,
-                                                   float* __restrict__ cbO32, const double* __restrict__ ub,
-                                                   const double* __restrict__ Fb, const double* __restrict__ rc, int64_t rc_start, int chunk,
-                                                   unsigned* work) {
+// The update of one element.  F: the field whose three modes are computed (0 xi, 1
+// U, 2 V), or -1 for all three.  Every multiply-add is written as an fma where the
+// compiler could pick one of two contractions, so that both forms give the same bits.
+template <int F>
+__device__ __forceinline__ void elem_unit(const DevMesh& m, const Phys& ph, const Stage& stg,
+                                          const double* __restrict__ cbS, const double* __restrict__ cbN,
+                                          double* __restrict__ cbO, float* __restrict__ cbO32,
+                                          const double* __restrict__ ub, const double* __restrict__ Fb,
+                                          const double* __restrict__ rc, int64_t rc_start, int64_t e) {
+  constexpr int F0 = F < 0 ? 0 : F, F1 = F < 0 ? 3 : F + 1;
   const int64_t ne = m.ne, nE = m.nedge;
   const double* geo = m.geo;
-  for_units(ne, chunk, work, [&](int64_t e) {
   double c[3][3], u[2][3];
 #pragma unroll
   for (int f = 0; f < 3; ++f)
@@ -483,13 +482,12 @@ __global__ void __launch_bounds__(128, MINB) k_elem_base(DevMesh m, Phys ph, Sta
   double Axx = 0.0, Axy = 0.0, Ayx = 0.0, Ayy = 0.0, P = 0.0;
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    Axx += c[1][i] * u[0][i]; Axy += c[1][i] * u[1][i];
-    Ayx += c[2][i] * u[0][i]; Ayy += c[2][i] * u[1][i];
-    P += c[0][i] * (0.5 * c[0][i] + hb[i]);
+    Axx = fma(c[1][i], u[0][i], Axx); Axy = fma(c[1][i], u[1][i], Axy);
+    Ayx = fma(c[2][i], u[0][i], Ayx); Ayy = fma(c[2][i], u[1][i], Ayy);
+    P = fma(c[0][i], fma(0.5, c[0][i], hb[i]), P);
   }
-  P *= ph.g;
-  Axx += P;
-  Ayy += P;
+  Axx = fma(ph.g, P, Axx);
+  Ayy = fma(ph.g, P, Ayy);
   const double gdx = geo[G_GDHX * ne + e], gdy = geo[G_GDHY * ne + e];
   const double U0s = c[1][0] * sqa, V0s = c[2][0] * sqa;
   r[0][0] = 0.0;
@@ -498,20 +496,20 @@ __global__ void __launch_bounds__(128, MINB) k_elem_base(DevMesh m, Phys ph, Sta
 #pragma unroll
   for (int q = 1; q < 3; ++q) {
     const double gx = geo[(q == 1 ? G_GQ1X : G_GQ2X) * ne + e], gy = geo[(q == 1 ? G_GQ1Y : G_GQ2Y) * ne + e];
-    r[0][q] = gx * U0s + gy * V0s;
-    r[1][q] = gx * Axx + gy * Axy + gdx * c[0][q];
-    r[2][q] = gx * Ayx + gy * Ayy + gdy * c[0][q];
+    r[0][q] = fma(gx, U0s, gy * V0s);
+    r[1][q] = fma(gdx, c[0][q], fma(gx, Axx, gy * Axy));
+    r[2][q] = fma(gdy, c[0][q], fma(gx, Ayx, gy * Ayy));
   }
-  if (ph.src) {
+  if (F != 0 && ph.src) {
     // bottom friction and Coriolis of Eq. (5); tau from the element means of H
     // and u (Sect. 3), mean = mode 0 / sqrt|Omega| = mode 0 * sqrt 2 / s_e
     const double ra = 1.4142135623730951 * rs;
     const double Hm = (c[0][0] + hb[0]) * ra, um = u[0][0] * ra, vm = u[1][0] * ra;
-    const double tau = ph.fric_lin * Hm + ph.fric_quad * sqrt(um * um + vm * vm);
+    const double tau = fma(ph.fric_lin, Hm, ph.fric_quad * sqrt(fma(um, um, vm * vm)));
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
-      r[1][q] += ph.f_c * c[2][q] - tau * u[0][q];
-      r[2][q] -= ph.f_c * c[1][q] + tau * u[1][q];
+      r[1][q] += fma(ph.f_c, c[2][q], -(tau * u[0][q]));
+      r[2][q] -= fma(ph.f_c, c[1][q], tau * u[1][q]);
     }
   }
   // edge terms
@@ -520,12 +518,6 @@ __global__ void __launch_bounds__(128, MINB) k_elem_base(DevMesh m, Phys ph, Sta
     const int ee = m.eedge[k * ne + e];
     const int64_t ed = ee >> 1;
     const bool right = ee & 1;
-    double F[3][2];
-#pragma unroll
-    for (int f = 0; f < 3; ++f) {
-      F[f][0] = Fb[(f * 2 + 0) * nE + ed];
-      F[f][1] = Fb[(f * 2 + 1) * nE + ed];
-    }
     // the basis at the edge's two points, times -1/s_e (left side) or +1/s_e
     // (right side, whose own direction is reversed): table values with the
     // sign bit set by an integer xor, no FP64 multiply
@@ -537,41 +529,80 @@ __global__ void __launch_bounds__(128, MINB) k_elem_base(DevMesh m, Phys ph, Sta
     const double b10 = sgn(right ? p1.x : p0.x), b11 = sgn(right ? p0.x : p1.x);
     const double b20 = sgn(right ? p1.y : p0.y), b21 = sgn(right ? p0.y : p1.y);
 #pragma unroll
-    for (int f = 0; f < 3; ++f) {
+    for (int f = F0; f < F1; ++f) {
+      const double A0 = Fb[(f * 2 + 0) * nE + ed], A1 = Fb[(f * 2 + 1) * nE + ed];
       // r += x y + z w is a multiply, an FMA and an add; this way two FMAs: 113
       // FP64 instructions per element instead of 131 (GB300, 524,288 triangles, 6
       // stages: 2,800 -> 2,668 us)
-      r[f][0] = fma(s0, F[f][0] + F[f][1], r[f][0]);
-      r[f][1] = fma(F[f][1], b11, fma(F[f][0], b10, r[f][1]));
-      r[f][2] = fma(F[f][1], b21, fma(F[f][0], b20, r[f][2]));
+      r[f][0] = fma(s0, A0 + A1, r[f][0]);
+      r[f][1] = fma(A1, b11, fma(A0, b10, r[f][1]));
+      r[f][2] = fma(A1, b21, fma(A0, b20, r[f][2]));
     }
   }
   // correction of the base modes from the volume terms of p >= 2 elements
-  if (!stg.base_only && e >= rc_start) {
+  if (F != 0 && !stg.base_only && e >= rc_start) {
     const int64_t nrc = ne - rc_start, lr = e - rc_start;
-    r[1][1] += rc[0 * nrc + lr];
-    r[1][2] += rc[1 * nrc + lr];
-    r[2][1] += rc[2 * nrc + lr];
-    r[2][2] += rc[3 * nrc + lr];
+#pragma unroll
+    for (int f = F0 > 1 ? F0 : 1; f < F1; ++f)
+#pragma unroll
+      for (int q = 1; q < 3; ++q) r[f][q] += rc[((f - 1) * 2 + q - 1) * nrc + lr];
   }
   const int K = m.p[e] == 0 ? 1 : 3;
   const double dt = stage_dt(stg, m.mem[e]), a = stg.a, bb = stg.b;
   const bool euler = a == 0.0 && bb == 1.0;  // the first stage: c + dt r
 #pragma unroll
-  for (int f = 0; f < 3; ++f)
+  for (int f = F0; f < F1; ++f)
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
       const int64_t ix = (f * 3 + q) * ne + e;
       double v = 0.0;
       if (q < K) {
         if (stg.rhs_only) v = r[f][q];
-        else if (euler) v = c[f][q] + dt * r[f][q];
-        else v = (a != 0.0 ? a * cbN[ix] : 0.0) + bb * (c[f][q] + dt * r[f][q]);
+        else if (euler) v = fma(dt, r[f][q], c[f][q]);
+        else v = fma(bb, fma(dt, r[f][q], c[f][q]), a != 0.0 ? a * cbN[ix] : 0.0);
       }
       cbO[ix] = v;
       if (cbO32) cbO32[ix] = (float)v;
     }
-  });
+}
+
+// MINB: blocks per SM the register allocation must allow -- 4 (128 registers)
+// for uncapped grids, where the kernel's own occupancy is what counts; 3 for
+// grids capped at a few blocks per SM beside the correction kernels, where
+// the measured step is faster with the unrestricted allocation
+template <int MINB>
+__global__ void __launch_bounds__(128, MINB) k_elem_base(DevMesh m, Phys ph, Stage stg, const double* __restrict__ cbS,
+                                                   const double* __restrict__ cbN, double* __restrict__ cbO,
+                                                   float* __restrict__ cbO32, const double* __restrict__ ub,
+                                                   const double* __restrict__ Fb, const double* __restrict__ rc, int64_t rc_start, int chunk,
+                                                   unsigned* work) {
+  for_units(m.ne, chunk, work,
+            [&](int64_t e) { elem_unit<-1>(m, ph, stg, cbS, cbN, cbO, cbO32, ub, Fb, rc, rc_start, e); });
+}
+
+// Few elements: a block of three warps updates 32 of them, a warp to a field.  A
+// lone warp issues an FP64 instruction in 64 cycles and its SM one in 19, so the
+// longest field's about 50 instructions in a chain count instead of the 113 of all three
+// as long as an SM holds few warps.  Measured per stage (GB300, p = 1, FP64; one
+// thread per element -> this form): 512 triangles 19.1 ->
+// 17.0 us, 2,048 19.1 -> 17.1, 4,608 19.8 -> 17.7, 8,192 20.4 -> 18.4; p 1 - 4,
+// mixed: 512 43.0 -> 41.8, 2,048 44.4 -> 43.5.
+// Beside correction kernels, which share the pipe, the repeated common terms
+// cost more than the shorter chain gains from about 3,000 elements on (p 1 - 4,
+// FP64: 512 and 2,048 elements within 0.2 %, 3,200 and 4,608 0.6 and 1 % slower).
+static int64_t field_elems(bool base_only) { return base_only ? 8192 : 2048; }
+
+__global__ void __launch_bounds__(96) k_elem_base_fields(DevMesh m, Phys ph, Stage stg, const double* __restrict__ cbS,
+                                                         const double* __restrict__ cbN, double* __restrict__ cbO,
+                                                         float* __restrict__ cbO32, const double* __restrict__ ub,
+                                                         const double* __restrict__ Fb, const double* __restrict__ rc,
+                                                         int64_t rc_start) {
+  const int64_t e = blockIdx.x * (int64_t)32 + (threadIdx.x & 31);
+  if (e >= m.ne) return;
+  const int f = threadIdx.x >> 5;
+  if (f == 0) elem_unit<0>(m, ph, stg, cbS, cbN, cbO, cbO32, ub, Fb, rc, rc_start, e);
+  else if (f == 1) elem_unit<1>(m, ph, stg, cbS, cbN, cbO, cbO32, ub, Fb, rc, rc_start, e);
+  else elem_unit<2>(m, ph, stg, cbS, cbN, cbO, cbO32, ub, Fb, rc, rc_start, e);
 }
 
 int launch_elem_base(cudaStream_t s, const DevMesh& m, const Groups& G, const Phys& ph, const Stage& stg,
@@ -580,7 +611,10 @@ int launch_elem_base(cudaStream_t s, const DevMesh& m, const Groups& G, const Ph
   if (m.ne == 0) return 0;
   const LaunchShape& L = launch_shape();
   const BaseGrid g = base_grid(m.ne, L);
-  if (L.base_bpsm == 0 || L.base_bpsm >= 4)
+  if (m.ne <= field_elems(G.start[2] == m.ne))
+    k_elem_base_fields<<<nblocks(m.ne, 32), 96, 0, s>>>(m, ph, stg, cbS, cbN, cbO, cbO32, ub, fx.Fb, (const double*)rc,
+                                                        G.start[2]);
+  else if (L.base_bpsm == 0 || L.base_bpsm >= 4)
     k_elem_base<4><<<g.blocks, g.threads, 0, s>>>(m, ph, stg, cbS, cbN, cbO, cbO32, ub, fx.Fb, (const double*)rc,
                                                   G.start[2], g.chunk, work);
   else

@@ -63,10 +63,14 @@ def test_correction_kernels_on_ragged_groups(prec, nx, ny):
                                           (swedg.PREC_MIXED_FP32, 3, [(64, 78), (50, 60)]),
                                           (swedg.PREC_MIXED_FP32, 2, [(100, 100), (60, 70)]),
                                           (swedg.PREC_FP64, 4, [(30, 50), (20, 30)]),
-                                          (swedg.PREC_FP64, 4, [(69, 70), (20, 30)])])
+                                          (swedg.PREC_FP64, 4, [(69, 70), (20, 30)]),
+                                          (swedg.PREC_FP64, 1, [(60, 68), (20, 30)]),
+                                          (swedg.PREC_MIXED_FP32, 2, [(32, 32), (20, 30)]),
+                                          (swedg.PREC_FP64, 1, [(1, 1), (60, 70)])])
 def test_member_alone_and_in_a_union_across_the_size_rules_bitwise(prec, p, sizes):
     """alone the first member's group runs one form of the element update or of the velocity solve, in the union
-    another (FP32: K(p-1) n = 60,000; FP64, order 4: 3,000 and 9,728 elements)"""
+    another (FP32: K(p-1) n = 60,000; FP64, order 4: 3,000 and 9,728 elements; base
+    element update: 8,192 elements, 2,048 beside correction kernels), with all source terms"""
     from paper_2311_11348_gb300.ensemble import Ensemble
     members, states = [], []
     for k, (nx, ny) in enumerate(sizes):
@@ -82,7 +86,7 @@ def test_member_alone_and_in_a_union_across_the_size_rules_bitwise(prec, p, size
         states.append(c)
     out = []
     for ms, cs in ((members[:1], states[:1]), (members, states)):
-        e = Ensemble(ms, g=9.81, rk_order=3, precision=prec)
+        e = Ensemble(ms, g=9.81, rk_order=3, precision=prec, friction=(1e-4, 0.009), f_c=1e-2)
         e.set_states(cs)
         e.run(2)
         out.append(e.states()[0])
