@@ -866,7 +866,7 @@ def main():
 # without ncu.  None for other workloads and modes.
 MEASURED_TRAFFIC = {"usolve": 48.6e6,
                     "edge_base": 98.2e6,
-                    "edge_corr": 291.9e6,
+                    "edge_corr": 292.0e6,
                     "elem_corr": 44.9e6,
                     "elem_base": 177.6e6}
 TRAFFIC_CAPTURE = ("ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum --clock-control "
