@@ -306,6 +306,18 @@ int swe_edge_table(int npts, double* s, double* w, double* B);
  * another K or cap too small.  Host pointer; needs no device. */
 int64_t swe_tc_operand_image(int K, float* out, int64_t cap);
 
+/* The constant operand that SWE_PREC_MIXED_TF32 contexts upload, for K = 10 or 15
+ * modes (orders 3 and 4), and the pairs of modes its columns stand for (the paper
+ * has no counterpart).  out: N rows (GEMM columns; N = 32 for K = 10, 80 for K =
+ * 15) of 32 floats in the layout above; row c holds T[m][i][j] for j < K in the
+ * columns j (rounded to TF32) and 16 + j (the remainder, rounded the same way),
+ * (m, i) = (pairs[2 c], pairs[2 c + 1]), 1 <= m <= i.  pairs (may be NULL) has 3
+ * (10) more entries, the pairs summed outside the GEMM.  Every pair of a mode m >=
+ * 1 of degree below the element's and a mode i >= m with a nonzero T[m][i][j]
+ * appears once.  Returns the number of floats (out may be NULL to query it), or
+ * SWE_EINVAL for another K or cap too small.  Host pointers; needs no device. */
+int64_t swe_tc_pair_operand(int K, float* out, int64_t cap, int32_t* pairs);
+
 /* Launch shapes (the paper has no counterpart: they tune the GPU kernels to
  * the mesh, orders and device).  shape[6]:
  *   [0] resident blocks per SM of the grid-stride base edge and element

@@ -1021,8 +1021,8 @@ int swe_create(swe_ctx** out, const swe_params* params) {
       corr64::upload_tables();
       corr32::upload_tables();
       corrtc::upload_tables();
-      if (corrtc::upload_tc_tables() != 0) {
-        g_create_err = "tensor-core operand upload failed";
+      if (corrtc::set_tc_attributes() != 0) {
+        g_create_err = "tensor-core kernel attributes failed";
         e = cudaErrorUnknown;
       } else {
         e = cudaDeviceSynchronize();
@@ -1610,6 +1610,11 @@ int swe_edge_table(int npts, double* s, double* w, double* B) {
 
 int64_t swe_tc_operand_image(int K, float* out, int64_t cap) {
   const int64_t n = corrtc::tc_operand_image(K, out, cap);
+  return n < 0 ? SWE_EINVAL : n;
+}
+
+int64_t swe_tc_pair_operand(int K, float* out, int64_t cap, int32_t* pairs) {
+  const int64_t n = corrtc::tc_pair_operand(K, out, cap, pairs);
   return n < 0 ? SWE_EINVAL : n;
 }
 

@@ -118,8 +118,6 @@ __host__ __device__ constexpr int tc_smem(int K) { return (3 * TC_ABUF + tc_bflo
 static_assert(tc_ctas(15) * (tc_smem(15) + 1024) <= 227 * 1024 && tc_ctas(10) * (tc_smem(10) + 1024) <= 227 * 1024,
               "shared memory of an SM");
 
-static float g_tcb[TC_BTOTAL];  // both B images (host); a context keeps its own device copy
-
 // round to the nearest value with a 10-bit mantissa (ties away from zero)
 static inline float tf32_round(float x) {
   uint32_t u;
@@ -160,7 +158,6 @@ template <int K>
 static void tc_b_image(float* out) {
   constexpr TcPairs<K> P = tc_pairs<K>();
   const RefTables& R = tables();
-  std::fill(out, out + tc_bfloats(K), 0.0f);
   for (int c = 0; c < P.nc; ++c)
     for (int j = 0; j < K; ++j) {
       if (!tnz(P.cm[c], P.ci[c], j)) continue;
@@ -169,6 +166,39 @@ static void tc_b_image(float* out) {
       out[tc_at(c, j)] = h;
       out[tc_at(c, 16 + j)] = tf32_round((float)(t - (double)h));
     }
+}
+
+// Both B images (host).  Contexts of any device copy them to their own memory
+// without a lock, so they are written once, before the first caller gets them.
+struct TcOperand {
+  float b[TC_BTOTAL] = {};
+  TcOperand() {
+    tc_b_image<10>(b + tc_boff(10));
+    tc_b_image<15>(b + tc_boff(15));
+  }
+};
+const float* tc_operand(size_t* bytes) {
+  static const TcOperand op;
+  *bytes = sizeof op.b;
+  return op.b;
+}
+
+template <int K>
+static int64_t pair_operand(float* out, int64_t cap, int32_t* pairs) {
+  constexpr TcPairs<K> P = tc_pairs<K>();
+  constexpr int64_t need = tc_bfloats(K);
+  if (!out) return need;
+  if (cap < need) return -1;
+  size_t bytes = 0;
+  std::memcpy(out, tc_operand(&bytes) + tc_boff(K), need * sizeof(float));
+  for (int c = 0; pairs && c < P.nc + P.nt; ++c) {
+    pairs[2 * c] = c < P.nc ? P.cm[c] : P.tm[c - P.nc];
+    pairs[2 * c + 1] = c < P.nc ? P.ci[c] : P.ti[c - P.nc];
+  }
+  return need;
+}
+int64_t tc_pair_operand(int K, float* out, int64_t cap, int32_t* pairs) {
+  return K == 10 ? pair_operand<10>(out, cap, pairs) : K == 15 ? pair_operand<15>(out, cap, pairs) : -1;
 }
 
 // ------------------------------------------------------------ PTX wrappers
@@ -519,15 +549,8 @@ int launch_wait_selftest(cudaStream_t st, int64_t spins, unsigned* status) {
   return 0;
 }
 
-const float* tc_operand(size_t* bytes) {
-  *bytes = sizeof g_tcb;
-  return g_tcb;
-}
-
-// B images (host) and kernel attributes of the current device (once per device and process)
-int upload_tc_tables() {
-  tc_b_image<10>(g_tcb + tc_boff(10));
-  tc_b_image<15>(g_tcb + tc_boff(15));
+// kernel attributes of the current device (once per device and process)
+int set_tc_attributes() {
   int dev = 0;
   SWE_CUDA_OK(cudaGetDevice(&dev));
   SWE_CUDA_OK(cudaFuncSetAttribute(k_elem_tc<10>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem(10)));

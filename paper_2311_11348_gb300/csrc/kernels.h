@@ -167,11 +167,13 @@ SWE_CORR_DECL(corr32)
 // order 2, launch_elem_tc the orders 3 and 4.
 SWE_CORR_DECL(corrtc)
 namespace corrtc {
-int upload_tc_tables();
+int set_tc_attributes();
 int launch_elem_tc(cudaStream_t st, const DevMesh& m, const Groups& G, const Phys& ph, const Stage& stg, StateDev cS,
                    StateDev cN, StateDev cO, VelDev u, EdgeFlux fx, const float* bimg, unsigned* status);
-// the constant operands of launch_elem_tc (host), which a context copies to its device memory (bimg)
+// the constant operands of launch_elem_tc (host, never written again), which a context copies to its device memory (bimg)
 const float* tc_operand(size_t* bytes);
+// host: one order's operand and column pairs (swe_tc_pair_operand)
+int64_t tc_pair_operand(int K, float* out, int64_t cap, int32_t* pairs);
 // host: the operand image of swe_tc_operand_image (floats written, or needed when out is NULL)
 int64_t tc_operand_image(int K, float* out, int64_t cap);
 // a bounded wait on an mbarrier that nothing arrives on: sets ST_TIMEOUT

@@ -45,7 +45,7 @@ SYMBOLS = ("swe_default_params", "swe_create", "swe_destroy", "swe_last_error", 
            "swe_rhs_parts", "swe_rk_step", "swe_run", "swe_mass", "swe_energy", "swe_reference_tensors",
            "swe_edge_table", "swe_profile", "swe_profile_read", "swe_rhs_p1_noalloc", "swe_adapt",
            "swe_run_adaptive", "swe_set_members", "swe_set_member_times", "swe_get_member_times",
-           "swe_memory_bytes", "swe_tc_operand_image", "swe_get_launch_shape", "swe_set_launch_shape",
+           "swe_memory_bytes", "swe_tc_operand_image", "swe_tc_pair_operand", "swe_get_launch_shape", "swe_set_launch_shape",
            "swe_autotune", "swe_selftest_wait", "swe_packed_size", "swe_set_state_packed",
            "swe_get_state_packed", "swe_set_state_packed_async", "swe_run_async", "swe_get_state_packed_async",
            "swe_sync", "swe_member_status", "swe_mesh_adjacency")
@@ -108,6 +108,7 @@ def load():
         if s not in ("swe_destroy", "swe_default_params", "swe_last_error"):
             getattr(lib, s).restype = C.c_int
     lib.swe_tc_operand_image.restype = C.c_int64
+    lib.swe_tc_pair_operand.restype = C.c_int64
     lib.swe_packed_size.restype = C.c_int64
     _lib = lib
     return lib
@@ -141,6 +142,19 @@ def tc_operand_image(K: int):
     out = np.zeros(n, np.float32)
     lib.swe_tc_operand_image(int(K), out.ctypes.data_as(C.c_void_p), C.c_int64(n))
     return out
+
+
+def tc_pair_operand(K: int):
+    """the constant operand that tensor-core contexts upload for K modes (host only): (image [floats], (m, i)
+    pairs of its columns [N, 2], pairs summed outside the GEMM [3 or 10, 2])"""
+    lib = load()
+    n = lib.swe_tc_pair_operand(int(K), None, C.c_int64(0), None)
+    if n < 0:
+        raise SweError(int(n), "swe_tc_pair_operand")
+    out, cols = np.zeros(n, np.float32), n // 32
+    pairs = np.zeros((cols + (10 if K == 15 else 3), 2), np.int32)
+    lib.swe_tc_pair_operand(int(K), out.ctypes.data_as(C.c_void_p), C.c_int64(n), pairs.ctypes.data_as(C.c_void_p))
+    return out, pairs[:cols], pairs[cols:]
 
 
 def mesh_adjacency(xy, tri):

@@ -5,6 +5,8 @@ split into two TF32 parts; and the two-stage decomposition the kernel uses
 (GEMMs of per-element velocity and pressure rows against those images, then
 sums over the coefficient rows) reproduces the direct volume contraction of
 the momentum rows."""
+from concurrent.futures import ThreadPoolExecutor
+
 import numpy as np
 import pytest
 
@@ -122,3 +124,15 @@ def test_gemm_decomposition_reproduces_the_volume_contraction(lib, K):
     assert np.abs(gU - rU).max() <= tol
     assert np.abs(gV - rV).max() <= tol
     assert np.abs(rU[:, 3:]).max() > 0.1  # the test exercises nonzero higher rows
+
+
+def test_pair_operand_is_written_once(lib):
+    """contexts upload it without a lock: every caller, from any thread, gets the complete image"""
+    want = {K: swedg.tc_pair_operand(K)[0] for K in (10, 15)}
+
+    def differ(i):
+        K = (10, 15)[i % 2]
+        return sum(not np.array_equal(swedg.tc_pair_operand(K)[0], want[K]) for _ in range(2000))
+
+    with ThreadPoolExecutor(8) as ex:  # the library call runs without the interpreter's lock
+        assert sum(ex.map(differ, range(8))) == 0
