@@ -1,9 +1,14 @@
-"""Host-side checks of the tensor-core volume contraction (precision mode
-SWE_PREC_MIXED_TF32), no GPU: the library's constant operand images decode,
-by the layout the header documents, to the oracle's G tensors of Eq. (13),
-split into two TF32 parts; and the two-stage decomposition the kernel uses
-(GEMMs of per-element velocity and pressure rows against those images, then
-sums over the coefficient rows) reproduces the direct volume contraction of
+"""Host-side checks of the tensor-core operands (precision mode
+SWE_PREC_MIXED_TF32), no GPU.
+
+swe_tc_pair_operand, what the kernel contracts with: its rows decode to the
+oracle's T[m][i][j] of Eq. (13) in two TF32 parts, its pairs of modes cover every
+product once, the products formed as the kernel forms them equal the direct
+contraction with T, and it is complete and the same for every caller.
+
+swe_tc_operand_image, the layout for callers with contractions of their own with
+the G tensors: it decodes to the oracle's G in two TF32 parts, and GEMMs of
+velocity and pressure rows against it reproduce the direct volume contraction of
 the momentum rows."""
 from concurrent.futures import ThreadPoolExecutor
 
@@ -78,10 +83,10 @@ def test_operand_images_hold_G_split_into_tf32_head_and_tail(lib, K):
 
 @pytest.mark.parametrize("K", [6, 10, 15])
 def test_gemm_decomposition_reproduces_the_volume_contraction(lib, K):
-    """the kernel's two stages: GEMMs of per-element rows (2 K values: the
-    contravariant velocities, or g J^-1 xi / 2) against the image, giving W,
-    ZU, ZV [i][q]; then the sums over i with the element's U, V, xi, and the
-    bottom term's products with the higher elevation modes added apart"""
+    """GEMMs of per-element rows (2 K values: the contravariant velocities, or g
+    J^-1 xi / 2) against the image, giving W, ZU, ZV [i][q]; then the sums over i
+    with the element's U, V, xi, and the bottom term's products with the
+    higher elevation modes added apart"""
     rng = np.random.default_rng(K)
     n = 7
     xi, U, V, u, v = (rng.standard_normal((n, K)) for _ in range(5))
@@ -104,7 +109,7 @@ def test_gemm_decomposition_reproduces_the_volume_contraction(lib, K):
                         + g * (J[:, [0]] * Px + J[:, [2]] * Py))
     rV = rs[:, None] * (np.einsum("qij,ei,ej->eq", Gm[0], V, uc) + np.einsum("qij,ei,ej->eq", Gm[1], V, vc)
                         + g * (J[:, [1]] * Px + J[:, [3]] * Py))
-    # the kernel: the operand B[(i, q)][(k, j)] and three A operands of 2 K columns
+    # the operand B[(i, q)][(k, j)] and three A operands of 2 K columns
     Bop = np.zeros((16 * K, 2 * K))
     for i in range(K):
         for q in range(16):
@@ -124,6 +129,64 @@ def test_gemm_decomposition_reproduces_the_volume_contraction(lib, K):
     assert np.abs(gU - rU).max() <= tol
     assert np.abs(gV - rV).max() <= tol
     assert np.abs(rU[:, 3:]).max() > 0.1  # the test exercises nonzero higher rows
+
+
+def pair_rows(K):
+    """columns' rows of T by part [2][N][16], the columns' pairs and the others"""
+    img, cols, thin = swedg.tc_pair_operand(K)
+    B = np.array([[[img[at(c, 16 * part + j)] for j in range(16)] for c in range(len(cols))] for part in range(2)])
+    assert np.count_nonzero(img) == np.count_nonzero(B)
+    return B, cols, thin
+
+
+@pytest.mark.parametrize("K", [10, 15])
+def test_pair_operand_holds_T_split_into_tf32_head_and_tail(lib, K):
+    B, cols, _ = pair_rows(K)
+    T = O.tensors()["T"]
+    want = np.zeros((len(cols), 16))
+    want[:, :K] = T[cols[:, 0], cols[:, 1], :K]
+    floor = 1e-13 * np.abs(T).max()  # structural zeros: the oracle's quadrature noise
+    assert np.all(B.view(np.uint32) & 0x1FFF == 0)
+    assert np.all(np.abs(B[0] - want) <= 2.0 ** -11 * np.abs(want) + floor)
+    assert np.all(np.abs(B.astype(np.float64).sum(0) - want) <= 2.0 ** -22 * np.abs(want) + floor)
+    assert np.all(np.abs(want[np.abs(B[0]) == 0]) <= floor)
+
+
+@pytest.mark.parametrize("K", [10, 15])
+def test_pairs_cover_every_product_of_the_higher_modes_once(lib, K):
+    """the pairs (m, i), 1 <= m <= i, m of lower degree, with a nonzero T[m][i][j]; a constant mode needs none"""
+    _, cols, thin = pair_rows(K)
+    KL = {10: 6, 15: 10}[K]
+    T = O.tensors()["T"]
+    nz = np.abs(T) > 1e-13 * np.abs(T).max()
+    pairs = [tuple(p) for p in np.vstack([cols, thin])]
+    assert len(set(pairs)) == len(pairs)
+    assert set(pairs) == {(m, i) for m in range(1, KL) for i in range(m, K) if nz[m, i, :K].any()}
+    delta = np.sqrt(2.0) * np.eye(K)
+    assert np.abs(T[0, :K, :K] - delta).max() < 1e-13 and np.abs(T[:K, 0, :K] - delta).max() < 1e-13
+
+
+@pytest.mark.parametrize("K", [10, 15])
+def test_products_as_the_kernel_forms_them(lib, K):
+    """Z_m = sum_ij T[m][i][j] U_i u_j from the columns' GEMM, the other pairs and the constant mode, a pair of
+    two modes below the element's degree serving both"""
+    B, cols, thin = pair_rows(K)
+    KL = {10: 6, 15: 10}[K]
+    T = O.tensors()["T"]
+    rng = np.random.default_rng(K)
+    U, u = rng.standard_normal((2, 5, K))
+    W = np.hstack([u @ B.astype(np.float64).sum(0)[:, :K].T, u @ T[thin[:, 0], thin[:, 1], :K].T])
+    f0 = np.sqrt(2.0)
+    Z = f0 * U[:, :1] * u[:, :KL]
+    Z[:, 0] = f0 * (U * u).sum(1)
+    for c, (m, i) in enumerate(np.vstack([cols, thin])):
+        Z[:, m] += U[:, i] * W[:, c]
+        if i < KL and i != m:
+            Z[:, i] += U[:, m] * W[:, c]
+    want = np.einsum("mij,ei,ej->em", T[:KL, :K, :K], U, u)
+    # each entry of T to within 2^-22; the sum of the terms' magnitudes bounds the products' error
+    bound = 2.0 ** -22 * np.einsum("mij,ei,ej->em", np.abs(T[:KL, :K, :K]), np.abs(U), np.abs(u))
+    assert np.all(np.abs(Z - want) <= bound)
 
 
 def test_pair_operand_is_written_once(lib):
