@@ -56,6 +56,7 @@
 #define CORR_NS corrtc
 #define CORR_TC 1
 #include "k_corr_impl.cuh"
+#include "tc_issue.h"
 
 namespace swedg {
 namespace corrtc {
@@ -219,6 +220,10 @@ __host__ __device__ constexpr uint32_t tc_idesc(int M, int N) {
 __device__ __forceinline__ void mbar_init(uint32_t a, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(a), "r"(count) : "memory");
 }
+__device__ __forceinline__ void mbar_arrive(uint32_t a) {
+  uint64_t state;
+  asm volatile("mbarrier.arrive.shared::cta.b64 %0, [%1];" : "=l"(state) : "r"(a) : "memory");
+}
 __device__ __forceinline__ bool mbar_wait(uint32_t a, uint32_t parity) {
   for (uint32_t it = 0; it < TC_SPIN; ++it) {
     uint32_t ok;
@@ -332,7 +337,7 @@ __global__ void __launch_bounds__(TC_M, tc_ctas(K)) k_elem_tc(ELEM_CORR_PARAMS, 
   }
   // the swizzle XOR acts on address bits 4-9: operands must start on 1024 bytes
   bool ok = (smem_u32(sA) & 1023u) == 0 && (smem_u32(sB) & 1023u) == 0;
-  bool bready = false;
+  bool blanded = false;
   uint32_t commits = 0;
   const uint32_t idesc = tc_idesc(TC_M, N);
   const uint32_t lane_base = tmem + ((uint32_t)(32 * w) << 16);
@@ -369,25 +374,26 @@ __global__ void __launch_bounds__(TC_M, tc_ctas(K)) k_elem_tc(ELEM_CORR_PARAMS, 
       tc_fence_before();
       __syncthreads();
       if (t == 0) {
-        if (!bready) {
-          ok &= mbar_wait(bfull, 0);
-          bready = true;
-        }
-        tc_fence_after();
-        const uint32_t b = smem_u32(sB);
+        ok = tc_issue(
+            ok, blanded, [&] { return mbar_wait(bfull, 0); },
+            [&] {
+              tc_fence_after();
+              const uint32_t b = smem_u32(sB);
 #pragma unroll
-        for (int gi = 0; gi < 3; ++gi) {
-          const uint32_t a = smem_u32(sA + gi * TC_ABUF), d = tmem + (uint32_t)(gi * N);
+              for (int gi = 0; gi < 3; ++gi) {
+                const uint32_t a = smem_u32(sA + gi * TC_ABUF), d = tmem + (uint32_t)(gi * N);
 #pragma unroll
-          for (int st = 0; st < 2; ++st) {  // two steps of 8 columns: 32 bytes further into the rows; tails 64 on
-            const uint32_t o = 32u * st;
-            tc_mma(d, tc_desc(a + o), tc_desc(b + o), idesc, st > 0 ? 1u : 0u);  // h h
-            tc_mma(d, tc_desc(a + o), tc_desc(b + 64u + o), idesc, 1u);           // h t
-            tc_mma(d, tc_desc(a + 64u + o), tc_desc(b + o), idesc, 1u);           // t h
-          }
-        }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mdone)
-                     : "memory");
+                for (int st = 0; st < 2; ++st) {  // two steps of 8 columns: 32 bytes further into the rows; tails 64 on
+                  const uint32_t o = 32u * st;
+                  tc_mma(d, tc_desc(a + o), tc_desc(b + o), idesc, st > 0 ? 1u : 0u);  // h h
+                  tc_mma(d, tc_desc(a + o), tc_desc(b + 64u + o), idesc, 1u);           // h t
+                  tc_mma(d, tc_desc(a + 64u + o), tc_desc(b + o), idesc, 1u);           // t h
+                }
+              }
+              asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mdone)
+                           : "memory");
+            },
+            [&] { mbar_arrive(mdone); });
       }
       // while the MMAs run: what needs no GEMM.  The constant mode on either side ...
       Prod z0{0.f, 0.f, 0.f, 0.f, 0.f};
@@ -484,7 +490,7 @@ __global__ void __launch_bounds__(TC_M, tc_ctas(K)) k_elem_tc(ELEM_CORR_PARAMS, 
   if (!ok && t == 0) atomicOr(status, (unsigned)ST_TIMEOUT);
   // a commit still in flight (a wait that gave up) completes before TMEM is freed
   if (!ok && commits > 0) mbar_wait(mdone, (commits - 1) & 1u);
-  if (!bready && t == 0) mbar_wait(bfull, 0);  // the B copy lands before the CTA exits
+  if (t == 0) tc_drain(blanded, [&] { return mbar_wait(bfull, 0); });  // the B copy lands before the CTA exits
   tc_fence_before();
   __syncthreads();
   if (w == 0) {
