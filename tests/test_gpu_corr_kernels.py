@@ -100,3 +100,29 @@ def test_velocity_solve_forms_meet_at_the_size_rule(nx, ny):
     and a larger one"""
     err = rhs_errors(lambda n: np.full(n, 4, np.int8), nx, ny, swedg.PREC_FP64)
     assert max(err) < TOL[swedg.PREC_FP64], err
+
+
+@pytest.mark.parametrize("prec,eps", [(swedg.PREC_FP64, 2.0**-53), (swedg.PREC_MIXED_FP32, 2.0**-24),
+                                      (swedg.PREC_MIXED_TF32, 2.0**-24)])
+def test_uniform_current_over_deep_water_keeps_the_jump_term_out_of_the_products(prec, eps):
+    """A uniform current over a flat bottom has a zero right-hand side away from the walls.  On equal squares both
+    sides of an edge have the same traces to the bit, so lambda (U_L - U_R) vanishes and what is left are the
+    roundings of the terms U w, about 100 each: 100 eps |U| |u| perimeter / s.  Products of U with w +- lambda would
+    leave eps |U| lambda |E| / s, here 9,000 eps |U| |u| |E| / s."""
+    n, h, u = 16, 2000.0, (0.013, 0.007)
+    xy, tri = inputs.split_square_mesh(n, 1024.0, jitter=0.0, seed=1)
+    nbr, _ = swedg.mesh_adjacency(xy, tri)
+    orders = (np.arange(len(tri)) % 3 + 2).astype(np.int8)
+    s = swedg.Solver(g=9.81, precision=prec)
+    s.set_mesh(xy, tri)
+    s.set_bathymetry(np.full(len(xy), h))
+    s.set_orders(orders)
+    se = 64.0  # sqrt det J
+    c = np.zeros((3, swedg.KMAX, len(tri)))
+    c[1, 0], c[2, 0] = (h * ui * se / np.sqrt(2.0) for ui in u)
+    r = s.rhs(c)[1:, 3:, (nbr >= 0).all(axis=1)]
+    s.close()
+    speed = float(np.hypot(*u))
+    bound = 100 * eps * h * speed * speed * (2 + np.sqrt(2.0)) * 64.0 / se
+    print(prec, float(np.abs(r).max()) / bound)
+    assert np.abs(r).max() <= bound
