@@ -19,9 +19,9 @@
 // the areas cancel, so that the only square roots are one per element (the scale
 // of its orthonormal basis) and one per edge (lambda), and there is no division
 // but the solve's.  FP64 instructions bound these kernels (GB300: 19 cycles of
-// an SM each, 64 of the warp): about 95 per element in k_na_usolve, 97 per edge,
+// an SM each, 64 of the warp): about 95 per element in k_na_usolve, 106 per edge,
 // 130 per element in k_na_elem, where the modal form with its geometry formed at
-// every visit took 1,900 per element; 72 -> 41 us for 20,000 elements (GB300).
+// every visit took 1,900 per element; 72 -> 42 us for 20,000 elements (GB300).
 #include <cuda.h>
 
 #include <cmath>
@@ -296,12 +296,12 @@ __global__ void __launch_bounds__(BT) k_na_edge(int64_t ne, const double* __rest
     double FB = (a.U[1] + b.U[1]) * Nx + (a.V[1] + b.V[1]) * Ny + lam * (a.x[1] - b.x[1]);
     F[(0 * 3 + k) * NMAX] = 2.0 * fma(2.0, FA, FB);
     F[(1 * 3 + k) * NMAX] = 2.0 * fma(2.0, FB, FA);
-    // momentum rows: U (w + lambda) + U+ (w+ - lambda) + (P + P+) N
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      a.w[q] += lam;
-      b.w[q] -= lam;
-    }
+    // momentum rows: U w + U+ w+ + (P + P+) N, and lambda (U - U+) as a linear
+    // term: w +- lambda in the products would drop the low bits of w, which is
+    // orders of magnitude below lambda (40 us instead of 42, and noise of
+    // lambda |U| instead of |w U| in the momentum rows)
+    const double lam2 = 2.0 * lam;
+    const double UA = a.U[0] - b.U[0], UB = a.U[1] - b.U[1], VA = a.V[0] - b.V[0], VB = a.V[1] - b.V[1];
     const double wa = a.w[0] + a.w[1], wb = b.w[0] + b.w[1];
     const double xa = a.x[0] + a.x[1], xb = b.x[0] + b.x[1];
     const double gNx = g * Nx, gNy = g * Ny, hs = hA + hB;
@@ -310,12 +310,12 @@ __global__ void __launch_bounds__(BT) k_na_edge(int64_t ne, const double* __rest
     const double PS = xa * fma(0.5, xa, hs) + xb * fma(0.5, xb, hs);
     const double XA = a.U[0] * a.w[0] + b.U[0] * b.w[0] + PA * gNx, XB = a.U[1] * a.w[1] + b.U[1] * b.w[1] + PB * gNx;
     const double XS = (a.U[0] + a.U[1]) * wa + (b.U[0] + b.U[1]) * wb + PS * gNx;
-    F[(2 * 3 + k) * NMAX] = fma(2.0, XA, XS);
-    F[(3 * 3 + k) * NMAX] = fma(2.0, XB, XS);
+    F[(2 * 3 + k) * NMAX] = fma(lam2, fma(2.0, UA, UB), fma(2.0, XA, XS));
+    F[(3 * 3 + k) * NMAX] = fma(lam2, fma(2.0, UB, UA), fma(2.0, XB, XS));
     const double YA = a.V[0] * a.w[0] + b.V[0] * b.w[0] + PA * gNy, YB = a.V[1] * a.w[1] + b.V[1] * b.w[1] + PB * gNy;
     const double YS = (a.V[0] + a.V[1]) * wa + (b.V[0] + b.V[1]) * wb + PS * gNy;
-    F[(4 * 3 + k) * NMAX] = fma(2.0, YA, YS);
-    F[(5 * 3 + k) * NMAX] = fma(2.0, YB, YS);
+    F[(4 * 3 + k) * NMAX] = fma(lam2, fma(2.0, VA, VB), fma(2.0, YA, YS));
+    F[(5 * 3 + k) * NMAX] = fma(lam2, fma(2.0, VB, VA), fma(2.0, YB, YS));
   }
 }
 

@@ -201,3 +201,25 @@ def test_noalloc_rejects_a_non_positive_or_non_finite_g():
         with pytest.raises(swedg.SweError) as ei:
             _noalloc(xy, hv, tri, neighbours(tri), c[:, :3], g=g)
         assert ei.value.code == -1
+
+
+def test_noalloc_uniform_current_over_deep_water():
+    """A uniform current over a flat bottom has a zero right-hand side away from the walls.  On equal squares both
+    sides of an edge have the same traces to the bit, so lambda (U_L - U_R) vanishes and what is left are the
+    roundings of the terms U w, about 100 each: 100 eps |U| |u| perimeter / s.  Products of U with w +- lambda would
+    leave eps |U| lambda |E| / s, here 9,000 eps |U| |u| |E| / s."""
+    import torch
+    n, h, u, side, se = 16, 2000.0, (0.013, 0.007), 64.0, 64.0  # se = sqrt det J
+    xy, tri = inputs.split_square_mesh(n, n * side, jitter=0.0, seed=1)
+    nbr = neighbours(tri)
+    c = np.zeros((3, 3, len(tri)))
+    c[1, 0], c[2, 0] = (h * ui * se / np.sqrt(2.0) for ui in u)
+    put = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()  # noqa: E731
+    out = torch.empty((3, 3, len(tri)), dtype=torch.float64, device="cuda")
+    args = [put(a) for a in (xy, np.full(len(xy), h), np.ascontiguousarray(tri, dtype=np.int32), nbr, c)]
+    torch.cuda.synchronize()
+    swedg.rhs_p1_noalloc(*args, 9.81, out)
+    torch.cuda.synchronize()
+    r = out.cpu().numpy()[1:, :, (nbr >= 0).all(axis=1)]
+    speed = float(np.hypot(*u))
+    assert np.abs(r).max() <= 100 * 2.0**-53 * h * speed * speed * (2 + np.sqrt(2.0)) * side / se
