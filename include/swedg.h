@@ -194,7 +194,9 @@ int swe_rhs(swe_ctx* ctx, const double* c_in, double* rhs_out);
 
 /* The two parts of the order separation (Sect. 3, Eq. 13 and the text after
  * it): base_out holds every term whose test index and coefficient indices are
- * all modes of degree <= 1; corr_out holds the rest.  base + corr = rhs. */
+ * all modes of degree <= 1; corr_out holds the rest.  base + corr = rhs.  The
+ * elevation rows of the modes 1..3 in corr_out are exact zeros where the
+ * element and its neighbours have no coefficient of degree >= 2. */
 int swe_rhs_parts(swe_ctx* ctx, const double* c_in, double* base_out, double* corr_out);
 
 /* One SSP Runge-Kutta step of the context state (Sect. 2).  dt > 0 is used as

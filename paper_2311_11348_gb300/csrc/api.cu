@@ -733,6 +733,21 @@ static int usolve_all(swe_ctx* ctx, StateDev in) {
   return 0;
 }
 
+// The trace records without their modes of degree >= 2, for a stage of the base
+// part alone: the correction edge kernels then form the flux of the P1 parts
+// with the operations of the whole flux, so that the difference of the two is
+// zero where the higher modes are.
+static int p1_traces(swe_ctx* ctx, cudaStream_t st) {
+  const size_t ts = ctx->corr32 ? sizeof(float) : sizeof(double);
+  for (int p = 2; p < 5; ++p) {
+    const size_t n = (size_t)(ctx->G.start[p + 1] - ctx->G.start[p]), K = (size_t)Kof(p);
+    if (n == 0) continue;
+    CU(cudaMemset2DAsync((char*)ctx->vel.tr[p] + 12 * ts, 4 * K * ts, 0, 4 * (K - 3) * ts, n, st));
+    CU(cudaMemset2DAsync((char*)ctx->vel.trv[p] + 3 * ts, K * ts, 0, (K - 3) * ts, n, st));
+  }
+  return 0;
+}
+
 // One stage: out = a n + b (in + dt L(in)), or out = L(in) (rhs_only).
 //
 // The base kernels (FP64 pipe bound) run on stream A, the correction kernels
@@ -787,14 +802,11 @@ static int run_stage(swe_ctx* ctx, StateDev in, StateDev nst, StateDev out, cons
       CK(corr32::launch_usolve_corr(gs, ctx->dm, ctx->G, ph, in, ctx->vel, ctx->d_status, dmin, ctx->rc));
     else CK(corr64::launch_usolve_corr(gs, ctx->dm, ctx->G, ph, in, ctx->vel, ctx->d_status, dmin, ctx->rc));
     CK(join_groups());
+    if (stg.base_only) CK(p1_traces(ctx, B));
   }
-  // the correction edge kernel computes the whole flux of its edges; both
-  // elements of the others have order <= 1, so they need usolve_base alone
-  const bool part = !stg.base_only && ctx->ce.n[1] < ctx->nedge;
   if (conc) {
     CU(cudaEventRecord(ctx->ev_u1, A));
     CU(cudaEventRecord(ctx->ev_u2, B));
-    if (!part) CU(cudaStreamWaitEvent(A, ctx->ev_u2, 0));
     CU(cudaStreamWaitEvent(B, ctx->ev_u1, 0));
   }
   Stage es = stg;  // of the edge kernels
@@ -810,20 +822,21 @@ static int run_stage(swe_ctx* ctx, StateDev in, StateDev nst, StateDev out, cons
     es.dt_host = 0.0;
   }
   {
+    // the correction edge kernel computes the whole flux of its edges; both
+    // elements of the others have order <= 1, so they need usolve_base alone
     ProfScope ps(ctx, F_EDGEB);
-    CK(launch_edge_base(A, ctx->dm, part ? ctx->ce.list[1] : nullptr, part ? ctx->ce.n[1] : ctx->nedge, ph, es, in.cb,
-                        ctx->vel.ub, ctx->fx, ctx->d_work));
+    const bool all = ctx->ce.n[1] == ctx->nedge;
+    CK(launch_edge_base(A, ctx->dm, all ? nullptr : ctx->ce.list[1], ctx->ce.n[1], ph, es, in.cb, ctx->vel.ub, ctx->fx,
+                        ctx->d_work));
   }
   if (conc && last) CU(cudaEventRecord(ctx->ev_e1, A));
-  if (!stg.base_only) {
-    {
-      ProfScope ps(ctx, F_EDGEC);
-      CK(fork_groups());
-      if (ctx->tc) CK(corrtc::launch_edge_corr(gs, ctx->dm, ctx->ce, ctx->G, ph, es, in, ctx->vel, ctx->fx));
-      else if (ctx->corr32) CK(corr32::launch_edge_corr(gs, ctx->dm, ctx->ce, ctx->G, ph, es, in, ctx->vel, ctx->fx));
-      else CK(corr64::launch_edge_corr(gs, ctx->dm, ctx->ce, ctx->G, ph, es, in, ctx->vel, ctx->fx));
-      CK(join_groups());
-    }
+  {
+    ProfScope ps(ctx, F_EDGEC);
+    CK(fork_groups());
+    if (ctx->tc) CK(corrtc::launch_edge_corr(gs, ctx->dm, ctx->ce, ctx->G, ph, es, in, ctx->vel, ctx->fx));
+    else if (ctx->corr32) CK(corr32::launch_edge_corr(gs, ctx->dm, ctx->ce, ctx->G, ph, es, in, ctx->vel, ctx->fx));
+    else CK(corr64::launch_edge_corr(gs, ctx->dm, ctx->ce, ctx->G, ph, es, in, ctx->vel, ctx->fx));
+    CK(join_groups());
   }
   if (conc) {  // the fluxes of edge_corr's edges
     CU(cudaEventRecord(ctx->ev_c, B));

@@ -126,3 +126,23 @@ def test_uniform_current_over_deep_water_keeps_the_jump_term_out_of_the_products
     bound = 100 * eps * h * speed * speed * (2 + np.sqrt(2.0)) * 64.0 / se
     print(prec, float(np.abs(r).max()) / bound)
     assert np.abs(r).max() <= bound
+
+
+@pytest.mark.parametrize("prec", [swedg.PREC_FP64, swedg.PREC_MIXED_FP32, swedg.PREC_MIXED_TF32])
+def test_rhs_parts_without_higher_coefficients_has_no_correction_of_the_base_elevation(prec):
+    """the elevation flux is linear, so with every coefficient of degree >= 2 zero both parts form the same base rows"""
+    xy, tri = inputs.split_square_mesh(12, 1e3, jitter=0.2, seed=7)
+    orders = (np.arange(len(tri)) % 5).astype(np.int8)
+    s = swedg.Solver(g=9.81, precision=prec)
+    s.set_mesh(xy, tri)
+    s.set_bathymetry(inputs.fourier_bathymetry(xy, 1e3, lo=10.0, hi=50.0, seed=2))
+    s.set_orders(orders)
+    rng = np.random.default_rng(1)
+    c = np.zeros((3, swedg.KMAX, len(tri)))
+    c[:, 0] = rng.standard_normal((3, len(tri)))
+    c[:, 1:3, orders > 0] = rng.standard_normal((3, 2, int((orders > 0).sum())))
+    base, corr = s.rhs_parts(c)
+    whole = s.rhs(c)
+    s.close()
+    assert not corr[0, :3].any()
+    assert np.array_equal(base[0, :3], whole[0, :3])
