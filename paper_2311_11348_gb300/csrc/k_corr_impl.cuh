@@ -134,13 +134,6 @@ static void usolve_terms(UsolveTerms* U) {
 }
 #endif
 
-// P_0 .. P_4 at t
-static void legendre5(double t, double (&P)[5]) {
-  P[0] = 1.0;
-  P[1] = t;
-  for (int l = 1; l < 4; ++l) P[l + 1] = ((2 * l + 1) * t * P[l] - l * P[l - 1]) / (l + 1);
-}
-
 void upload_tables() {
   const RefTables& R = tables();
   static T t[KMAX][120], dx[KMAX][10], ds[KMAX][10], el[3][KMAX][5], gp[3][4][5], gw[3][4];
@@ -150,26 +143,17 @@ void upload_tables() {
   for (int q = 0; q < KMAX; ++q)
     for (int m = 0; m < 10; ++m) {
       dx[q][m] = (T)R.D[0][q][m];
-      ds[q][m] = (T)(R.D[1][q][m] - 0.5 * R.D[0][q][m]);
+      ds[q][m] = (T)R.Ds[q][m];
     }
   for (int k = 0; k < 3; ++k)
     for (int i = 0; i < KMAX; ++i)
-      for (int l = 0; l < 5; ++l) {  // (2 l + 1) int_0^1 phihat_i(gamma_k(s)) P_l(2 s - 1) ds, exact with 8 points
-        double acc = 0.0, P[5];
-        for (int gg = 0; gg < 8; ++gg) {
-          legendre5(2.0 * R.es[8][gg] - 1.0, P);
-          acc += R.ew[8][gg] * R.EB[8][k][i][gg] * P[l];
-        }
-        el[k][i][l] = (T)((2 * l + 1) * acc);
-      }
+      for (int l = 0; l < 5; ++l) el[k][i][l] = (T)R.EL[k][i][l];
   for (int pm = 2; pm <= 4; ++pm) {
     const int N = npts_for(pm), H = N / 2;
     for (int j = 0; j < 4; ++j) {
-      double P[5] = {0, 0, 0, 0, 0};
-      const bool mid = j == H && N % 2;
-      if (j < H || mid) legendre5(mid ? 0.0 : 2.0 * R.es[N][N - 1 - j] - 1.0, P);
-      for (int l = 0; l < 5; ++l) gp[pm - 2][j][l] = (T)P[l];
-      gw[pm - 2][j] = j < H || mid ? (T)R.ew[N][N - 1 - j] : (T)0;
+      const bool in = j < H || (j == H && N % 2);  // points t > 0, then the middle one
+      for (int l = 0; l < 5; ++l) gp[pm - 2][j][l] = in ? (T)R.GL[N][N - 1 - j][l] : (T)0;
+      gw[pm - 2][j] = in ? (T)R.ew[N][N - 1 - j] : (T)0;
     }
   }
 #ifdef CORR_LANES

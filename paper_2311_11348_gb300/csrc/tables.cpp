@@ -7,13 +7,20 @@
 //     and Sect. 3, integrated with a 14 x 14 collapsed rule (exact for the
 //     degree <= 12 integrands);
 //   - edge trace tables B_k[i][g] = phihat_i(gamma_k(s_g)), which apply the
-//     edge tensors of the quadrature-free scheme in factored form.
+//     edge tensors of the quadrature-free scheme in factored form, and the
+//     Legendre coefficients of the same traces.
+// Everything is formed in long double and rounded once, so that the tables are
+// good to the last bit of FP64: summed in FP64 their entries carried up to 450
+// roundings (1e-13 of T), which every right-hand side inherited.
 #include "tables.h"
 
 #include <cmath>
 #include <cstring>
+#include <limits>
 
 namespace swedg {
+
+typedef long double real;
 
 // Dubiner basis (Sect. 2: hierarchical and orthonormal on the element).  In
 // collapsed coordinates eta1 = (2x + y - 1)/(1 - y), eta2 = 2y - 1 the mode
@@ -21,40 +28,40 @@ namespace swedg {
 // R_a = P_a(eta1) (1-y)^a is evaluated without the singular division through
 // (a+1) R_{a+1} = (2a+1) l R_a - a m^2 R_{a-1},  l = 2x + y - 1, m = 1 - y.
 // Modes are ordered by total degree a + b, then by b.
-void dubiner(double x, double y, double* v, double* vx, double* vy) {
-  const double l = 2.0 * x + y - 1.0, m = 1.0 - y;
-  double R[5], Rx[5], Ry[5];
+static void dubiner(real x, real y, real* v, real* vx, real* vy) {
+  const real l = 2.0 * x + y - 1.0, m = 1.0 - y;
+  real R[5], Rx[5], Ry[5];
   R[0] = 1.0; Rx[0] = 0.0; Ry[0] = 0.0;
   R[1] = l;   Rx[1] = 2.0; Ry[1] = 1.0;
   for (int a = 1; a < 4; ++a) {
-    const double c1 = (2.0 * a + 1.0) / (a + 1.0), c2 = (double)a / (a + 1.0);
+    const real c1 = (2 * a + (real)1) / (a + 1), c2 = (real)a / (a + 1.0);
     R[a + 1] = c1 * l * R[a] - c2 * m * m * R[a - 1];
     Rx[a + 1] = c1 * (2.0 * R[a] + l * Rx[a]) - c2 * m * m * Rx[a - 1];
     Ry[a + 1] = c1 * (R[a] + l * Ry[a]) - c2 * (m * m * Ry[a - 1] - 2.0 * m * R[a - 1]);
   }
-  const double t = 2.0 * y - 1.0;
+  const real t = 2.0 * y - 1.0;
   int idx = 0;
   for (int d = 0; d <= 4; ++d) {
     for (int b = 0; b <= d; ++b) {
       const int a = d - b;
-      const double al = 2.0 * a + 1.0;
+      const real al = 2.0 * a + 1.0;
       // Jacobi P_n^(al,0)(t) and its t-derivative by the three-term recurrence
-      double P0 = 1.0, dP0 = 0.0;
-      double P1 = 0.5 * ((al + 2.0) * t + al), dP1 = 0.5 * (al + 2.0);
-      double P = P0, dP = dP0;
+      real P0 = 1.0, dP0 = 0.0;
+      real P1 = 0.5 * ((al + 2.0) * t + al), dP1 = 0.5 * (al + 2.0);
+      real P = P0, dP = dP0;
       if (b >= 1) { P = P1; dP = dP1; }
       for (int n = 1; n < b; ++n) {
-        const double s = 2.0 * n + al;
-        const double A1 = 2.0 * (n + 1) * (n + al + 1) * s;
-        const double A2 = (s + 1) * al * al;
-        const double A3 = s * (s + 1) * (s + 2);
-        const double A4 = 2.0 * (n + al) * n * (s + 2);
-        const double P2 = ((A2 + A3 * t) * P1 - A4 * P0) / A1;
-        const double dP2 = (A3 * P1 + (A2 + A3 * t) * dP1 - A4 * dP0) / A1;
+        const real s = 2.0 * n + al;
+        const real A1 = 2.0 * (n + 1) * (n + al + 1) * s;
+        const real A2 = (s + 1) * al * al;
+        const real A3 = s * (s + 1) * (s + 2);
+        const real A4 = 2.0 * (n + al) * n * (s + 2);
+        const real P2 = ((A2 + A3 * t) * P1 - A4 * P0) / A1;
+        const real dP2 = (A3 * P1 + (A2 + A3 * t) * dP1 - A4 * dP0) / A1;
         P0 = P1; dP0 = dP1; P1 = P2; dP1 = dP2;
         P = P2; dP = dP2;
       }
-      const double N = std::sqrt(2.0 * (2.0 * a + 1.0) * (a + b + 1.0));
+      const real N = std::sqrt((real)(2 * (2 * a + 1) * (a + b + 1)));
       v[idx] = N * R[a] * P;
       if (vx) vx[idx] = N * Rx[a] * P;
       if (vy) vy[idx] = N * (Ry[a] * P + R[a] * 2.0 * dP);
@@ -64,25 +71,25 @@ void dubiner(double x, double y, double* v, double* vx, double* vy) {
 }
 
 // Gauss-Legendre nodes and weights on [0,1], by Newton's method on P_n.
-void gauss01(int n, double* s, double* w) {
+static void gauss01(int n, real* s, real* w) {
   for (int i = 0; i < n; ++i) {
-    double z = -std::cos(M_PI * (i + 0.75) / (n + 0.5));  // ascending
-    double dp = 1.0;
+    real z = -std::cos(std::acos((real)-1) * (i + (real)0.75) / (n + (real)0.5));  // ascending
+    real dp = 1.0;
     for (int it = 0; it < 60; ++it) {
-      double p0 = 1.0, p1 = z;
+      real p0 = 1.0, p1 = z;
       for (int k = 1; k < n; ++k) {
-        const double p2 = ((2.0 * k + 1.0) * z * p1 - k * p0) / (k + 1.0);
+        const real p2 = ((2.0 * k + 1.0) * z * p1 - k * p0) / (k + 1.0);
         p0 = p1; p1 = p2;
       }
-      const double pn = n == 0 ? 1.0 : p1, pm = n == 1 ? 1.0 : p0;
+      const real pn = n == 0 ? 1.0 : p1, pm = n == 1 ? 1.0 : p0;
       dp = n * (pm - z * pn) / (1.0 - z * z);
-      const double step = pn / dp;
+      const real step = pn / dp;
       z -= step;
-      if (std::fabs(step) < 1e-17) break;
+      if (std::fabs(step) < std::numeric_limits<real>::epsilon()) break;
     }
-    double p0 = 1.0, p1 = z;
+    real p0 = 1.0, p1 = z;
     for (int k = 1; k < n; ++k) {
-      const double p2 = ((2.0 * k + 1.0) * z * p1 - k * p0) / (k + 1.0);
+      const real p2 = ((2.0 * k + 1.0) * z * p1 - k * p0) / (k + 1.0);
       p0 = p1; p1 = p2;
     }
     dp = n * (p0 - z * p1) / (1.0 - z * z);
@@ -91,54 +98,64 @@ void gauss01(int n, double* s, double* w) {
   }
 }
 
-void edge_point(int k, double s, double* x, double* y) {
+static void edge_point(int k, real s, real* x, real* y) {
   // gamma_0(s) = (1-s, s), gamma_1(s) = (0, 1-s), gamma_2(s) = (s, 0)
   if (k == 0) { *x = 1.0 - s; *y = s; }
   else if (k == 1) { *x = 0.0; *y = 1.0 - s; }
   else { *x = s; *y = 0.0; }
 }
 
-void build_tables(RefTables* R) {
+static void build_tables(RefTablesOf<real>* R) {
   std::memset(R, 0, sizeof(*R));
   const int n = 14;
-  double s[32], w[32];
+  real s[32], w[32];
   gauss01(n, s, w);
   for (int a = 0; a < n; ++a) {
     for (int b = 0; b < n; ++b) {
       // Duffy map of the unit square onto T: x = u (1 - v), y = v, dx dy = (1 - v) du dv
-      const double u = s[a], v = s[b];
-      const double x = u * (1.0 - v), y = v, wt = w[a] * w[b] * (1.0 - v);
-      double ph[KMAX], px[KMAX], py[KMAX];
+      const real u = s[a], v = s[b];
+      const real x = u * (1.0 - v), y = v, wt = w[a] * w[b] * (1.0 - v);
+      real ph[KMAX], px[KMAX], py[KMAX];
       dubiner(x, y, ph, px, py);
-      const double* dk[2] = {px, py};
+      const real* dk[2] = {px, py};
       for (int i = 0; i < KMAX; ++i) {
         for (int q = 0; q < KMAX; ++q) {
           R->M[q][i] += wt * ph[q] * ph[i];
           for (int k = 0; k < 2; ++k) R->D[k][q][i] += wt * ph[i] * dk[k][q];
         }
-        for (int j = 0; j < KMAX; ++j) {
-          const double pij = wt * ph[i] * ph[j];
-          for (int q = 0; q < KMAX; ++q) {
-            R->T[q][i][j] += pij * ph[q];
-            R->G[0][q][i][j] += pij * px[q];
-            R->G[1][q][i][j] += pij * py[q];
-          }
+        for (int j = 0; j <= i; ++j) {
+          const real pij = wt * ph[i] * ph[j];
+          for (int q = 0; q <= j; ++q) R->T[q][j][i] += pij * ph[q];
         }
       }
     }
   }
+  for (int i = 0; i < KMAX; ++i)  // T is symmetric
+    for (int j = 0; j <= i; ++j)
+      for (int q = 0; q <= j; ++q) {
+        const real t = R->T[q][j][i];
+        R->T[q][i][j] = R->T[i][q][j] = R->T[i][j][q] = R->T[j][q][i] = R->T[j][i][q] = t;
+      }
+  // d_k phi_q = sum_m D_k[q][m] phi_m
+  for (int k = 0; k < 2; ++k)
+    for (int q = 0; q < KMAX; ++q)
+      for (int m = 0; m < KMAX; ++m)
+        for (int i = 0; i < KMAX; ++i)
+          for (int j = 0; j < KMAX; ++j) R->G[k][q][i][j] += R->D[k][q][m] * R->T[m][i][j];
+  for (int q = 0; q < KMAX; ++q)
+    for (int m = 0; m < KMAX; ++m) R->Ds[q][m] = R->D[1][q][m] - R->D[0][q][m] / 2;
   // gradients of the degree-1 modes (constant)
-  double ph[KMAX], px[KMAX], py[KMAX];
+  real ph[KMAX], px[KMAX], py[KMAX];
   dubiner(0.25, 0.25, ph, px, py);
   for (int q = 0; q < 3; ++q) { R->grad1[q][0] = px[q]; R->grad1[q][1] = py[q]; }
   R->phi0 = ph[0];
   // barycentric hat functions against the basis: Lv[v][i] = int lambda_v phihat_i
   for (int a = 0; a < n; ++a)
     for (int b = 0; b < n; ++b) {
-      const double u = s[a], v = s[b];
-      const double x = u * (1.0 - v), y = v, wt = w[a] * w[b] * (1.0 - v);
+      const real u = s[a], v = s[b];
+      const real x = u * (1.0 - v), y = v, wt = w[a] * w[b] * (1.0 - v);
       dubiner(x, y, ph, nullptr, nullptr);
-      const double lam[3] = {1.0 - x - y, x, y};
+      const real lam[3] = {1.0 - x - y, x, y};
       for (int vv = 0; vv < 3; ++vv)
         for (int i = 0; i < 3; ++i) R->Lv[vv][i] += wt * lam[vv] * ph[i];
     }
@@ -147,21 +164,38 @@ void build_tables(RefTables* R) {
     gauss01(np, R->es[np], R->ew[np]);
     for (int k = 0; k < 3; ++k)
       for (int g = 0; g < np; ++g) {
-        double x, y;
+        real x, y;
         edge_point(k, R->es[np][g], &x, &y);
         dubiner(x, y, ph, nullptr, nullptr);
         for (int i = 0; i < KMAX; ++i) R->EB[np][k][i][g] = ph[i];
       }
+    for (int g = 0; g < np; ++g) {
+      real* P = R->GL[np][g];
+      const real t = 2 * R->es[np][g] - 1;
+      P[0] = 1;
+      P[1] = t;
+      for (int l = 1; l < 4; ++l) P[l + 1] = ((2 * l + 1) * t * P[l] - l * P[l - 1]) / (l + 1);
+    }
   }
+  for (int k = 0; k < 3; ++k)
+    for (int i = 0; i < KMAX; ++i)
+      for (int l = 0; l < 5; ++l)  // exact with 8 points
+        for (int g = 0; g < 8; ++g) R->EL[k][i][l] += (2 * l + 1) * R->ew[8][g] * R->EB[8][k][i][g] * R->GL[8][g][l];
+}
+
+static const RefTables* rounded_tables() {
+  RefTablesOf<real>* x = new RefTablesOf<real>;
+  build_tables(x);
+  RefTables* t = new RefTables;
+  constexpr size_t n = sizeof(RefTables) / sizeof(double);
+  static_assert(sizeof(RefTables) == n * sizeof(double) && sizeof *x == n * sizeof(real), "tables of one type");
+  for (size_t i = 0; i < n; ++i) reinterpret_cast<double*>(t)[i] = (double)reinterpret_cast<const real*>(x)[i];
+  delete x;
+  return t;
 }
 
 const RefTables& tables() {
-  static RefTables* R = nullptr;
-  if (!R) {
-    RefTables* t = new RefTables;
-    build_tables(t);
-    R = t;
-  }
+  static const RefTables* const R = rounded_tables();
   return *R;
 }
 

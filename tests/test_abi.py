@@ -40,6 +40,17 @@ def test_library_tensors_match_oracle(lib):
         assert np.abs(a - b).max() <= 1e-14 * np.abs(b).max()
 
 
+def test_library_tensors_are_rounded_once(lib):
+    """the library's entries and the oracle's (summed in double-double), each an FP64 rounding of the exact value:
+    one unit in the last place apart at most; structural zeros below the last place of the largest terms"""
+    D, G, T = swedg.reference_tensors()
+    t = O.tensors()
+    for a, b in ((D, t["D"]), (G, t["G"]), (T, t["T"])):
+        zero = np.abs(b) < 1e-12
+        assert np.all(np.abs(a - b)[~zero] <= 2.0**-52 * np.abs(b)[~zero])
+        assert np.abs(a[zero]).max() <= 2.0**-53 * np.abs(b).max()
+
+
 def test_p1_mass_tensor_structure_the_velocity_solve_uses(lib):
     """the P1 velocity solve drops T[0][i][j] = T[i][0][j] = phihat_1 delta_ij
     (orthonormal basis, constant phihat_1 = sqrt 2) from its arithmetic"""
