@@ -635,8 +635,9 @@ int launch_usolve_corr(GroupStreams gs, const DevMesh& m, const Groups& G, const
 // ---------------------------------------------------------------------------
 template <int PM>
 struct SideC {
-  T x[PM + 1], U[PM + 1], V[PM + 1], w[PM + 1];  // FP64: the whole trace; FP32: its higher part
-  T xl[2], Ul[2], Vl[2], wl[2];                  // the P1 part (FP64: only xl is kept apart)
+  T x[PM + 1];                       // the higher part of the elevation
+  T U[PM + 1], V[PM + 1], w[PM + 1];  // FP64: the whole trace; FP32: its higher part
+  T xl[2], Ul[2], Vl[2], wl[2];      // the P1 part (FP64: only xl is kept apart)
   T un, xm;                                      // mean normal velocity and mean elevation
 };
 
@@ -689,7 +690,7 @@ __device__ __forceinline__ void side_coefs(const DevMesh& m, const Groups& G, co
   });
   const T rso = reverse ? -rs : rs;  // odd coefficients change sign on the reversed edge
   if constexpr (!kF32) {
-    sfor<0, 2>([&](auto l) { S.x[l] += S.xl[l]; S.U[l] += S.Ul[l]; S.V[l] += S.Vl[l]; S.w[l] += S.wl[l]; });
+    sfor<0, 2>([&](auto l) { S.U[l] += S.Ul[l]; S.V[l] += S.Vl[l]; S.w[l] += S.wl[l]; });
   }
   sfor<0, PM + 1>([&](auto l) {
     const T f = l % 2 ? rso : rs;
@@ -767,7 +768,6 @@ __device__ __forceinline__ void edge_corr_body(const DevMesh& m, const int32_t* 
     sfor<0, PM + 1>([&](auto l) { b.x[l] = 0; });
     b.xl[0] = xh;
     b.xl[1] = 0;
-    if constexpr (!kF32) b.x[0] = xh;
     b.xm = xh;
   } else {
     const T nx = eg[E_NX * nE + ed], ny = eg[E_NY * nE + ed];
@@ -801,11 +801,18 @@ __device__ __forceinline__ void edge_corr_body(const DevMesh& m, const int32_t* 
   // of pmax = 2 (0.5 % of an FP64 step, nothing in FP32) and costs accuracy: error
   // of a mixed step of p 1 - 3 over deep water 7.4e-10 instead of 5.6e-10, of the
   // FP64 momentum rows of p 0 - 4 3.6e-15 instead of 3.3e-15 (against 80 bits).
+  T ax[PM + 1], bx[PM + 1];  // FP64: the whole elevation; FP32: its higher part, as U, V, w
   T m0[PM + 1], m1[PM + 1], m2[PM + 1], lc[PM + 1];
   sfor<0, PM + 1>([&](auto l) {
     constexpr T c = (T)(1.0 / (2 * l + 1));
     lc[l] = lam * c;
-    m0[l] = ((a.U[l] + b.U[l]) * nxw + (a.V[l] + b.V[l]) * nyw) * c + lc[l] * (a.x[l] - b.x[l]);
+    ax[l] = a.x[l];
+    bx[l] = b.x[l];
+    if constexpr (!kF32 && l < 2) {
+      ax[l] += a.xl[l];
+      bx[l] += b.xl[l];
+    }
+    m0[l] = ((a.U[l] + b.U[l]) * nxw + (a.V[l] + b.V[l]) * nyw) * c + lc[l] * (ax[l] - bx[l]);
     m1[l] = lc[l] * (a.U[l] - b.U[l]);
     m2[l] = lc[l] * (a.V[l] - b.V[l]);
   });
@@ -824,9 +831,9 @@ __device__ __forceinline__ void edge_corr_body(const DevMesh& m, const int32_t* 
   sfor<0, (N + 1) / 2>([&](auto J) {
     constexpr bool mid = 2 * J + 1 == N;
     T f1[2] = {0, 0}, f2[2] = {0, 0}, pp[2] = {0, 0};
-    auto side = [&](const SideC<PM>& S) {
+    auto side = [&](const SideC<PM>& S, const T (&sx)[PM + 1]) {
       T x[2], U[2], V[2], w[2];
-      at_pair<PM, J>(S.x, x[0], x[1]);
+      at_pair<PM, J>(sx, x[0], x[1]);
       at_pair<PM, J>(S.U, U[0], U[1]);
       at_pair<PM, J>(S.V, V[0], V[1]);
       at_pair<PM, J>(S.w, w[0], w[1]);
@@ -845,8 +852,8 @@ __device__ __forceinline__ void edge_corr_body(const DevMesh& m, const int32_t* 
         }
       });
     };
-    side(a);
-    side(b);
+    side(a, ax);
+    side(b, bx);
     sfor<0, mid ? 1 : 2>([&](auto s) {
       const T P = kF32 ? pp[s] : (T)0.5 * pp[s];
       f1[s] += P * gnx;
@@ -872,12 +879,11 @@ __device__ __forceinline__ void edge_corr_body(const DevMesh& m, const int32_t* 
     }
   });
   // h_b (xi_h,L + xi_h,R): the product with the linear h_b shifts the moments by one
+  // (the higher part is held apart: whole minus P1 part would carry the rounding
+  // of the whole times g h_b into the higher momentum modes)
   {
     T S[PM + 1];
-    sfor<0, PM + 1>([&](auto l) {
-      S[l] = a.x[l] + b.x[l];
-      if constexpr (!kF32 && l < 2) S[l] -= a.xl[l] + b.xl[l];
-    });
+    sfor<0, PM + 1>([&](auto l) { S[l] = a.x[l] + b.x[l]; });
     sfor<0, PM + 1>([&](auto l) {
       T s1 = 0;
       if constexpr (l > 0) s1 += S[l > 0 ? l - 1 : 0] * (T)((double)l / (2 * l - 1));

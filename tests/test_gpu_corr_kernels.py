@@ -128,6 +128,35 @@ def test_uniform_current_over_deep_water_keeps_the_jump_term_out_of_the_products
     assert np.abs(r).max() <= bound
 
 
+@pytest.mark.parametrize("prec,eps", [(swedg.PREC_FP64, 2.0**-53), (swedg.PREC_MIXED_FP32, 2.0**-24),
+                                      (swedg.PREC_MIXED_TF32, 2.0**-24)])
+def test_small_higher_elevation_modes_over_deep_water_keep_their_digits(prec, eps):
+    """Still water over a flat bottom with a constant elevation a and tiny higher modes: the higher momentum rows are
+    linear in those modes with the factor g (h + a), so the rows for a = 1 and a = 0 differ by (h + a) / h.  On equal
+    squares the jump of a vanishes to the bit and the roundings left are those of g a^2 / 2, about 100 of them:
+    100 eps g a^2 perimeter / s.  Higher modes taken as whole minus constant would leave eps g h a |E| / s."""
+    n, h, se = 16, 8192.0, 64.0  # se = sqrt det J
+    xy, tri = inputs.split_square_mesh(n, 1024.0, jitter=0.0, seed=1)
+    orders = (np.arange(len(tri)) % 3 + 2).astype(np.int8)
+    s = swedg.Solver(g=9.81, precision=prec)
+    s.set_mesh(xy, tri)
+    s.set_bathymetry(np.full(len(xy), h))
+    s.set_orders(orders)
+    K = (orders + 1) * (orders + 2) // 2
+    c = np.zeros((3, swedg.KMAX, len(tri)))
+    c[0, 3:] = 2.0**-20 * np.random.default_rng(4).uniform(-1, 1, (12, len(tri))) * se
+    c[0] *= np.arange(swedg.KMAX)[:, None] < K[None]
+    c[0] = c[0].astype(np.float32)  # held exactly in every mode
+    r0 = s.rhs(c)[1:, 3:]
+    c[0, 0] = se / np.sqrt(2.0)
+    r1 = s.rhs(c)[1:, 3:]
+    s.close()
+    bound = 100 * eps * 9.81 * (2 + np.sqrt(2.0)) * 64.0 / se
+    d = np.abs(r1 - r0 * (1.0 + 1.0 / h)).max()
+    print(prec, d / bound, np.abs(r0).max() / bound)
+    assert d <= bound
+
+
 @pytest.mark.parametrize("prec", [swedg.PREC_FP64, swedg.PREC_MIXED_FP32, swedg.PREC_MIXED_TF32])
 def test_rhs_parts_without_higher_coefficients_has_no_correction_of_the_base_elevation(prec):
     """the elevation flux is linear, so with every coefficient of degree >= 2 zero both parts form the same base rows"""
