@@ -595,7 +595,7 @@ static int build_device(swe_ctx* ctx) {
   });
   const int64_t nE = (int64_t)ed.size();
   ctx->nedge = nE;
-  if (nE >= (1ll << 27) || ne >= (1ll << 30)) return fail(ctx, SWE_EINVAL, "mesh too large for 27-bit edge slots");
+  if (nE >= (1ll << 27) || ne >= (1ll << 30)) return fail(ctx, SWE_EINVAL, "mesh too large: 2^27 edges or 2^30 elements");
   std::vector<int32_t> eLu(nE), eRu(nE), einfo(nE), eedge_u(3 * ne, -1), emem(nE);
   std::vector<double> egeo((size_t)NEGEO * nE);
   const int64_t nint = nI;
@@ -635,7 +635,7 @@ static int build_device(swe_ctx* ctx) {
       (rc = dalloc(ctx, &D.geo32, 4 * (size_t)NGEO * ne)) || (rc = dalloc(ctx, &D.etb, 96 * (size_t)ne)) ||
       (rc = dalloc(ctx, &D.mem, 4 * (size_t)ne)) || (rc = dalloc(ctx, &D.eedge, 12 * (size_t)ne)) ||
       (rc = dalloc(ctx, &D.eL, 4 * (size_t)nE)) || (rc = dalloc(ctx, &D.eR, 4 * (size_t)nE)) ||
-      (rc = dalloc(ctx, &D.slot, 4 * (size_t)nE)) || (rc = dalloc(ctx, &D.lists, 16 * (size_t)nE)) ||
+      (rc = dalloc(ctx, &D.lists, 16 * (size_t)nE)) ||
       (rc = dalloc(ctx, &D.off, 8 * (size_t)ne)))
     return cuda_err(ctx, rc);
   {
@@ -652,7 +652,6 @@ static int build_device(swe_ctx* ctx) {
   ctx->d_off = D.off;
   ctx->dm = DevMesh{ne, nE, nint, D.geo, D.p, D.eedge, D.eL, D.eR, d_einfo, d_egeo, D.geo32, d_egeo32, D.etb,
                     D.mem, d_emem, ctx->nmem, nullptr};
-  ctx->ce.slot = D.slot;
   for (int pm = 2; pm <= 4; ++pm) ctx->ce.list[pm] = D.lists + (size_t)(pm - 2) * nE;
   ctx->ce.list[1] = D.lists + (size_t)3 * nE;
   // base state, velocity and fluxes (sized by the mesh)

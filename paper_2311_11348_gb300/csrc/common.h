@@ -127,7 +127,6 @@ struct DevMesh {
 struct CorrEdges {
   int64_t n[5];           // per pmax
   const int32_t* list[5]; // edge ids
-  const int32_t* slot;    // [nedge]: (pmax << 28) | slot within group, or -1
 };
 
 __device__ __forceinline__ double stage_dt(const Stage& st, int mem) { return st.dt ? st.dt[mem] : st.dt_host; }

@@ -34,6 +34,7 @@ static inline int nblocks(int64_t n, int t) { return (int)((n + t - 1) / t); }
 
 static int g_sm_count = 152;
 void set_sm_count(int n) { g_sm_count = n > 0 ? n : 152; }
+int sm_count() { return g_sm_count; }
 
 // Threads per block of a kernel over n units: t, halved (down to a warp) while the
 // blocks would not cover the SMs twice.  An FP64 instruction takes a warp 64 cycles and

@@ -414,9 +414,10 @@ __device__ __forceinline__ void usolve_corr_body(const DevMesh& m, int64_t g0, i
   }
 }
 
-// The compiler's register allocation (FP32: 80, 127, 255 registers for K =
+// The compiler's register allocation (FP32: 72, 128, 233 registers for K =
 // 6, 10, 15), and for K = 15 in FP32 a second build in 168 registers (3
-// blocks per SM) for launch shapes that cap the base grids (see k_edge_corr).
+// blocks per SM) for launch shapes that cap the base grids: the few base blocks
+// leave room for more of its warps.
 template <int K>
 __global__ void __launch_bounds__(128) k_usolve_corr(DevMesh m, int64_t g0, int64_t n, Phys ph, StateDev c,
                                                      const T* __restrict__ ch, double* __restrict__ ub,
@@ -426,13 +427,14 @@ __global__ void __launch_bounds__(128) k_usolve_corr(DevMesh m, int64_t g0, int6
                                                      double* __restrict__ rc, int64_t rc_off, int64_t nrc) {
   usolve_corr_body<K>(m, g0, n, ph, c, ch, ub, ub32, uh, tr, trv, status, dmin, rc, rc_off, nrc);
 }
+template <int K>
 __global__ void __launch_bounds__(128, 3) k_usolve_corr15(DevMesh m, int64_t g0, int64_t n, Phys ph, StateDev c,
                                                          const T* __restrict__ ch, double* __restrict__ ub,
                                                          float* __restrict__ ub32, T* __restrict__ uh,
                                                          T* __restrict__ tr, T* __restrict__ trv,
                                                          unsigned* status, unsigned long long* dmin,
                                                          double* __restrict__ rc, int64_t rc_off, int64_t nrc) {
-  usolve_corr_body<15>(m, g0, n, ph, c, ch, ub, ub32, uh, tr, trv, status, dmin, rc, rc_off, nrc);
+  usolve_corr_body<K>(m, g0, n, ph, c, ch, ub, ub32, uh, tr, trv, status, dmin, rc, rc_off, nrc);
 }
 
 // The solve of FP64 groups of order 4 with 16 lanes per element, for small groups:
@@ -578,11 +580,15 @@ static int usolve_group(cudaStream_t st, const DevMesh& m, const Groups& G, int 
     return 0;
   }
 #endif
-  if (K == 15 && kF32 && launch_shape().base_bpsm > 0)
-    k_usolve_corr15<<<nblocks(n, ct), ct, 0, st>>>(m, g0, n, ph, c, (const T*)c.ch[p], u.ub, u.ub32,
-                                                   (T*)u.uh[p], (T*)u.tr[p], (T*)u.trv[p], status, dmin,
-                                                   (double*)rc, rc_off, nrc);
-  else
+  bool capped = false;
+  if constexpr (K == 15 && kF32) {
+    capped = launch_shape().base_bpsm > 0;
+    if (capped)
+      k_usolve_corr15<K><<<nblocks(n, ct), ct, 0, st>>>(m, g0, n, ph, c, (const T*)c.ch[p], u.ub, u.ub32,
+                                                        (T*)u.uh[p], (T*)u.tr[p], (T*)u.trv[p], status, dmin,
+                                                        (double*)rc, rc_off, nrc);
+  }
+  if (!capped)
     k_usolve_corr<K><<<nblocks(n, ct), ct, 0, st>>>(m, g0, n, ph, c, (const T*)c.ch[p], u.ub, u.ub32,
                                                       (T*)u.uh[p], (T*)u.tr[p], (T*)u.trv[p], status, dmin,
                                                       (double*)rc, rc_off, nrc);
@@ -1205,7 +1211,7 @@ static int elem_group(cudaStream_t st, const DevMesh& m, const Groups& G, int p,
   if (!kF32 || n * KL <= 60000) {
     bool five = false;
     if constexpr (K == 15 && !kF32) {
-      five = n > 9728;  // two blocks of ten warps per SM and more
+      five = n > 64 * (int64_t)sm_count();  // two blocks of ten warps per SM and more
       if (five) k_elem_corr_split<K, 5><<<nblocks(n, 32), 160, 0, st>>>(m, g0, n, ph, stg, cb, chS, chN, chO, ub, uh, pe);
     }
     if (!five) k_elem_corr_split<K, KL><<<nblocks(n, 32), 32 * KL, 0, st>>>(m, g0, n, ph, stg, cb, chS, chN, chO, ub, uh, pe);

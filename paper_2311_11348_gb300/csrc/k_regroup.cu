@@ -132,18 +132,16 @@ __global__ void __launch_bounds__(RG_T) k_elem_scatter(const int8_t* p_user, int
   }
 }
 
-// edges: slot[i] = (pmax << 28) | position in its correction group, or -1;
-// lists[category * nedge + position] = i.  off includes the group starts
+// edges: lists[category * nedge + position in its group] = i.  off includes the group starts
 // (start), which the positions are taken relative to.
 __global__ void __launch_bounds__(RG_T) k_edge_scatter(EdgeCat cat, int64_t nedge, const int64_t* off,
-                                                      const int64_t* start, int32_t* slot, int32_t* lists) {
+                                                      const int64_t* start, int32_t* lists) {
   __shared__ int cnt_s[RG_W][RG_MAXC];
   const int64_t i = blockIdx.x * (int64_t)RG_T + threadIdx.x;
   const int c = i < nedge ? cat(i) : -1;
   const int r = block_rank<4>(c, cnt_s);
   if (i < nedge) {
     const int64_t pos = off[(int64_t)blockIdx.x * 4 + c] + r - start[c];
-    slot[i] = c < 3 ? ((c + 2) << 28) | (int32_t)pos : -1;
     lists[(int64_t)c * nedge + pos] = (int32_t)i;
   }
 }
@@ -250,7 +248,7 @@ int launch_regroup(cudaStream_t s, const MeshStatic& S, const int8_t* p_user, De
     const EdgeCat ec{p_user, S.eLu, S.eRu};
     k_part_counts<4><<<(unsigned)bg, RG_T, 0, s>>>(ec, nE, W.gcnt);
     k_part_scan<4><<<1, 1024, 0, s>>>(W.gcnt, bg, W.goff, W.info + 6);
-    k_edge_scatter<<<(unsigned)bg, RG_T, 0, s>>>(ec, nE, W.goff, W.info + 6, D.slot, D.lists);
+    k_edge_scatter<<<(unsigned)bg, RG_T, 0, s>>>(ec, nE, W.goff, W.info + 6, D.lists);
     k_gather_edges<<<nb(nE, 256), 256, 0, s>>>(S, D.inv, D);
     count_launch(4);
   }

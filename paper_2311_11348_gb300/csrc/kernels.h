@@ -62,7 +62,6 @@ struct DevMeshOut {
   int32_t* eedge;  // [3][ne]
   int32_t* eL;     // [nedge] internal index of the left element
   int32_t* eR;     // [nedge] internal index of the right element or -1
-  int32_t* slot;   // [nedge] (pmax << 28) | position in the correction group, or -1
   int32_t* lists;  // [4][nedge] edge ids per pmax = 2, 3, 4 (correction edges), then those with pmax <= 1
   int64_t* off;    // [ne] packed caller layout offsets (caller order)
 };
@@ -103,6 +102,7 @@ const LaunchShape& launch_shape();
 // base-path tables (host -> constant memory of the base kernels)
 void upload_base_tables();
 void set_sm_count(int n);
+int sm_count();
 int spread_threads(int64_t n, int t);  // threads per block (at most t) so that n units cover the SMs
 
 // off == nullptr: the caller layout c[3][15][ne]; else packed, element u's

@@ -71,7 +71,7 @@ def device_bytes(meshes, precision):
     allocs = [NGEO * 8 * ne, 96 * ne, 12 * ne, 4 * nE, 4 * nE, 4 * ne,                    # mesh in caller order
               4 * nE, NEGEO * 8 * nE, NEGEO * 4 * nE, 4 * nE,                                # edge info, geometry, members
               4 * ne, 4 * ne, ne, NGEO * 8 * ne, NGEO * 4 * ne, 96 * ne, 4 * ne, 12 * ne,    # regrouped elements
-              4 * nE, 4 * nE, 4 * nE, 16 * nE, 8 * ne,                                       # regrouped edges, offsets
+              4 * nE, 4 * nE, 16 * nE, 8 * ne,                                               # regrouped edges, offsets
               20 * be, 40 * be, 16 * bg, 32 * bg, 8 * be, 8 * (be + 1), 128]                # partition scratch
     allocs += [72 * ne] * 3 + ([36 * ne] * 3 if corr32 else [])                             # base RK states
     allocs += [48 * ne] + ([24 * ne] if corr32 else [])                                     # base velocity
