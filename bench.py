@@ -860,18 +860,20 @@ def main():
 
 
 # DRAM bytes (read + write) per SSP-RK3 step of each kernel family of the mixed
-# mode on the 131,072-triangle ocean workload with the autotuned ocean shape
-# (uncapped base grids: the 128-register element kernel), from one ncu capture
-# (cold cache), TRAFFIC_CAPTURE below, run after the same command exited 0
-# without ncu.  None for other workloads and modes.
+# mode on the 131,072-triangle ocean workload, from one ncu capture (cold cache)
+# with the launch shape TRAFFIC_SHAPE, TRAFFIC_CAPTURE below, run after the same
+# command exited 0 without ncu.  The line's own autotuned shape may be another
+# one; the bytes of two of its choices agree within 1 % per family.  None for other
+# workloads and modes.
 MEASURED_TRAFFIC = {"usolve": 48.6e6,
-                    "edge_base": 98.2e6,
-                    "edge_corr": 292.0e6,
+                    "edge_base": 98.3e6,
+                    "edge_corr": 292.5e6,
                     "elem_corr": 44.9e6,
-                    "elem_base": 177.6e6}
+                    "elem_base": 177.5e6}
+TRAFFIC_SHAPE = "4,128,128,64,0,2"
 TRAFFIC_CAPTURE = ("ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum --clock-control "
                    "none -k regex:'k_edge_base|k_elem_base|k_elem_corr|k_edge_corr|k_usolve' -s 27 -c 27 python bench.py "
-                   "--steps 2 --warmup 3 --no-oracle --no-serving --no-adaptive --shape 0,64,128,64,0,2")
+                   f"--steps 2 --warmup 3 --no-oracle --no-serving --no-adaptive --shape {TRAFFIC_SHAPE}")
 
 
 def roofline(w, r, dom, steps, pk, head):

@@ -56,9 +56,11 @@ extern "C" {
 #define SWE_PREC_FP64 0       /* correction in FP64 as well                          */
 #define SWE_PREC_MIXED_FP32 1 /* correction arithmetic and storage in FP32           */
 #define SWE_PREC_MIXED_TF32 2 /* as MIXED_FP32, but the momentum volume terms of the
-                               * correction (the G contractions of Eq. 13) run on the
-                               * tensor cores for the orders 3 and 4: every FP32 operand split into two TF32
-                               * parts, three partial products, FP32 accumulation   */
+                               * correction (Eq. 13; the contractions with T[m][i][j],
+                               * G_k[q] = sum_m D_k[q][m] T[m]) run on the tensor
+                               * cores for the orders 3 and 4: every FP32 operand split
+                               * into two TF32 parts, three partial products, FP32
+                               * accumulation                                       */
 
 typedef struct swe_ctx swe_ctx; /* opaque */
 
@@ -339,9 +341,8 @@ int64_t swe_tc_pair_operand(int K, float* out, int64_t cap, int32_t* pairs);
  *       block takes up to c * [1] consecutive edges (elements) at a time from
  *       a ticket counter until none are left, so blocks that share their SM
  *       with the concurrent correction kernels take fewer tiles
- * Defaults {2, 128, 256, 128, 0, 2}.  Results do not depend on the shape (every
- * unit of work is computed by one thread in the same order).  SWE_EINVAL for
- * a shape out of range. */
+ * Defaults {2, 128, 256, 128, 0, 2}.  Results do not depend on the shape: every
+ * kernel form gives the same bits.  SWE_EINVAL for a shape out of range. */
 int swe_get_launch_shape(swe_ctx* ctx, int32_t* shape);
 int swe_set_launch_shape(swe_ctx* ctx, const int32_t* shape);
 

@@ -3,7 +3,7 @@
 // in FP64.  Plus the layout conversions, the CFL reduction, the time update
 // and the diagnostics.
 //
-// Kernels (one thread per element or per edge, FP64-pipe bound on GB300):
+// Kernels (one thread per element or per edge, on few elements a warp per field; FP64-pipe bound on GB300):
 //   k_usolve_base  auxiliary system uH = q (Sect. 3) for p <= 1 elements
 //                  (and, in the first stage of a step, the CFL bounds of its
 //                  elements: min over elements, exact, order independent)
@@ -419,8 +419,8 @@ int launch_advance_time(cudaStream_t s, double* t_dev, unsigned long long* dmin,
 
 // ---------------------------------------------------------------------------
 // Base edge flux (base_edge.cuh) of the edges of list[n], or of all of them
-// (list == nullptr, n = nedge).  A step leaves the correction edges out: their
-// kernel adds its own flux to the base flux in the same thread.
+// (list == nullptr, n = nedge).  The correction edges are left out: their kernel
+// writes the whole flux.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(128) k_edge_base(DevMesh m, Phys ph, Stage stg, const int32_t* __restrict__ list,
                                                    int64_t n, const double* __restrict__ cb,

@@ -443,9 +443,9 @@ __global__ void __launch_bounds__(128, 3) k_usolve_corr15(DevMesh m, int64_t g0,
 // length and the elimination broadcasts L_kj d_j from lane to lane, about 300
 // instructions per warp of two elements (twice the total).  Every operation on an
 // element is the same, in the same order, as in the one-thread form, so the
-// results are too.  77 us for any group up to 10,000 elements on one thread; 24 us
-// here for 512, 70 for 5,000 (GB300); beside the other groups' kernels, which share
-// the FP64 pipe, it pays up to about 3,000.
+// results are too.  74 to 76 us for any group up to 10,000 elements on one thread;
+// here 24 us for 512, 74 for 5,000, 115 for 10,000 (GB300, alone); beside the other groups'
+// kernels, which share the FP64 pipe, it pays up to about 3,000.
 #ifdef CORR_LANES
 constexpr int64_t UL_MAX = 3000;
 constexpr int UL_BLOCK = 128, UL_EL = UL_BLOCK / 16;
@@ -631,13 +631,14 @@ int launch_usolve_corr(GroupStreams gs, const DevMesh& m, const Groups& G, const
 // FP64 additions and 18 loads per element.
 // All fluxes are weighted by |E| / 4 (the weight of the two-point base rule)
 // through the normal.
-// FP64 is bound by its instruction count (about 340, 620, 1,080 per edge of
+// FP64 is bound by its instruction count (about 350, 640, 1,100 per edge of
 // pmax = 2, 3, 4 with one side an order lower, against 700, 1,450, 3,000 and the base
-// flux for traces and projections mode by mode at every point): 226, 371, 601 us for
-// 249,000 edges between elements of order 2, 3, 4 (GB300, alone), 0.9, 1.5, 2.4 ns
+// flux for traces and projections mode by mode at every point): 229, 379, 620 us for
+// 249,000 edges between elements of order 2, 3, 4 (GB300, alone), 0.9, 1.5, 2.5 ns
 // per edge where the other form took 1.6, 2.9, 5.8.  FP32 waits on the gathers of
-// the two trace records; 37, 50, 79 us for the same edges, and 106, 115, 123
-// registers instead of 124, 168, 210, so that every pmax runs 4 blocks per SM.
+// the two trace records and of the FP64 base state: 70, 82, 108 us for the same
+// edges with the FP64 base flux; 117, 128, 128 registers, so that every pmax
+// runs 4 blocks per SM.
 // ---------------------------------------------------------------------------
 template <int PM>
 struct SideC {
@@ -1017,13 +1018,13 @@ int launch_edge_corr(GroupStreams gs, const DevMesh& m, const CorrEdges& ce, con
 // 64 cycles whatever its parallelism inside the warp and four warps fill an
 // SM's pipe (19 cycles each), so what counts is the instruction count and
 // that few elements still give every scheduler a warp.  FP64, 165,888 elements
-// alone: K = 6, 10, 15 118, 382, 1131 us (GB300), 75 - 85 % of what the pipe
+// alone: K = 6, 10, 15 117, 389, 1045 us (GB300), 75 - 85 % of what the pipe
 // can issue; the contraction per test mode took about 250, 1260, 4450.
 // k_elem_corr (FP32, large groups): one thread per element, each coefficient
 // loaded once, the 3 (K - 3) results in registers.  It is straight-line code (55
-// KB for K = 15) and waits for instruction fetches: 19, 42, 90 us for 165,888
-// elements of K = 6, 10, 15 (the split form 20, 52, 319: ten code bodies at once
-// on an SM), but 20 us for 512 of K = 15 (split 10).  The forms cross where the
+// KB for K = 15) and waits for instruction fetches: 19, 48, 108 us for 165,888
+// elements of K = 6, 10, 15 (the split form 23, 108, 316: ten code bodies at once
+// on an SM), but 20 us for 512 of K = 15 (split 11).  The forms cross where the
 // split form's threads fill the device about once (n KL = 60,000: K = 15
 // between 5,000 and 10,000 elements, K = 10 between 10,000 and 20,000).
 // ---------------------------------------------------------------------------

@@ -6,10 +6,9 @@
 // hands the solver fixed buffers and forbids cudaMalloc/cudaFree on its
 // streams), or a host process that must not grow its device footprint after
 // start-up.  For them the intermediate arrays of this one computation -- the
-// auxiliary velocity u and the Lax-Friedrichs flux of every edge at its two
-// Gauss points -- live in a file-scope __device__ array of fixed size,
-// g_na_scratch, which every GPU that loads the library holds until the
-// process exits.  The caller passes inputs and outputs; nothing else is
+// auxiliary velocity u and the moments of every edge's Lax-Friedrichs flux --
+// live in file-scope __device__ arrays of fixed size, g_na_scratch and g_na_ok,
+// which every GPU that loads the library holds until the process exits.  The caller passes inputs and outputs; nothing else is
 // allocated, by this file or by any library it calls.
 //
 // Sect. 2-3 of the paper for p = 1 with land walls, in the vertex values of the

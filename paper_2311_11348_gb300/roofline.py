@@ -114,8 +114,8 @@ def vol_tc_flops(K):
 
 
 def edge_corr_flops(KL, KR, pm, fp64):
-    """Legendre coefficients of both sides (xi, U, V, w), the linear row and the
-    products with h_b by coefficients, the products at npts(pm) points, their
+    """Legendre coefficients of both sides (xi, U, V, w), the linear row, the jump
+    terms and the products with h_b by coefficients, the products at npts(pm) points, their
     moments, and the projections onto the higher test modes of each side"""
     N, L = npts(pm), pm + 1
     f = 60
@@ -124,8 +124,8 @@ def edge_corr_flops(KL, KR, pm, fp64):
         if K >= 6:
             f += 9 * L + 6 * sum(DEG[q] + 1 for q in range(3, K))
     ev = 6 if pm == 2 else 9 if pm == 3 else 10  # a field at a pair of points
-    f += L * (9 + 10) + (N // 2) * (8 * ev) + N * (14 if fp64 else 34) + 4 * L * ((N + 1) // 2)
-    return f + (0 if fp64 else 60)
+    f += L * (14 + 10) + (N // 2) * (8 * ev) + N * (14 if fp64 else 34) + 4 * L * ((N + 1) // 2)
+    return f + (0 if fp64 else 68)
 
 
 def family_flops(orders, fam, nedge=None, mode="mixed"):
