@@ -637,7 +637,7 @@ int launch_usolve_corr(GroupStreams gs, const DevMesh& m, const Groups& G, const
 // 249,000 edges between elements of order 2, 3, 4 (GB300, alone), 0.9, 1.5, 2.5 ns
 // per edge where the other form took 1.6, 2.9, 5.8.  FP32 waits on the gathers of
 // the two trace records and of the FP64 base state: 70, 82, 108 us for the same
-// edges with the FP64 base flux; 117, 128, 128 registers, so that every pmax
+// edges with the FP64 base flux; 117, 126, 128 registers, so that every pmax
 // runs 4 blocks per SM.
 // ---------------------------------------------------------------------------
 template <int PM>
@@ -755,7 +755,9 @@ __device__ __forceinline__ void edge_corr_body(const DevMesh& m, const int32_t* 
   const T g = (T)ph.g;
   // jump of the degree-1 elevation along the edge, j0 + j1 t (zero on land): it
   // carries the volume term g xi_lin h_b of the higher test modes (moved here,
-  // see products)
+  // see products), and in FP32 lambda (xi_L - xi_R) of the P1 parts too, whose FP32
+  // traces would leave the rounding of xi times lambda (smooth state over deep
+  // water: elevation rows of degree 2 - 4 2.9e-4 that way, 5.0e-5 with this jump)
   T j0 = 0, j1 = 0;
   double F[6];
   if constexpr (kF32) {
@@ -827,7 +829,7 @@ __device__ __forceinline__ void edge_corr_body(const DevMesh& m, const int32_t* 
   if constexpr (kF32) {
     sfor<0, 2>([&](auto l) {
       constexpr T c = (T)(1.0 / (2 * l + 1));
-      z0[l] = ((a.Ul[l] + b.Ul[l]) * nxw + (a.Vl[l] + b.Vl[l]) * nyw) * c + lc[l] * (a.xl[l] - b.xl[l]);
+      z0[l] = ((a.Ul[l] + b.Ul[l]) * nxw + (a.Vl[l] + b.Vl[l]) * nyw) * c - lc[l] * (l == 0 ? j0 : j1);
       z1[l] = lc[l] * (a.Ul[l] - b.Ul[l]);
       z2[l] = lc[l] * (a.Vl[l] - b.Vl[l]);
     });

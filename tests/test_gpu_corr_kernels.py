@@ -158,6 +158,27 @@ def test_small_higher_elevation_modes_over_deep_water_keep_their_digits(prec, ep
 
 
 @pytest.mark.parametrize("prec", [swedg.PREC_FP64, swedg.PREC_MIXED_FP32, swedg.PREC_MIXED_TF32])
+def test_still_water_has_elevation_rows_of_fp64_rounding(prec):
+    """still water with a constant elevation a over a varying bottom: the elevation flux is lambda times the jump of
+    a, whose P1 part every mode forms in FP64: about 100 roundings, 100 2^-53 lambda a perimeter / s"""
+    xy, tri = inputs.split_square_mesh(16, 1024.0, jitter=0.2, seed=7)
+    hv = inputs.fourier_bathymetry(xy, 1024.0, lo=500.0, hi=4000.0, seed=2)
+    orders = (np.arange(len(tri)) % 5).astype(np.int8)
+    a, b = xy[tri[:, 1]] - xy[tri[:, 0]], xy[tri[:, 2]] - xy[tri[:, 0]]
+    se = np.sqrt(a[:, 0] * b[:, 1] - a[:, 1] * b[:, 0])
+    s = swedg.Solver(g=9.81, precision=prec)
+    s.set_mesh(xy, tri)
+    s.set_bathymetry(hv)
+    s.set_orders(orders)
+    c = np.zeros((3, swedg.KMAX, len(tri)))
+    c[0, 0] = se / np.sqrt(2.0)
+    r = np.abs(s.rhs(c)[0]).max(axis=0)
+    s.close()
+    perimeter = sum(np.linalg.norm(xy[tri[:, (k + 1) % 3]] - xy[tri[:, k]], axis=1) for k in range(3))
+    assert np.all(r <= 100 * 2.0**-53 * np.sqrt(9.81 * 4001.0) * perimeter / se)
+
+
+@pytest.mark.parametrize("prec", [swedg.PREC_FP64, swedg.PREC_MIXED_FP32, swedg.PREC_MIXED_TF32])
 def test_rhs_parts_without_higher_coefficients_has_no_correction_of_the_base_elevation(prec):
     """the elevation flux is linear, so with every coefficient of degree >= 2 zero both parts form the same base rows"""
     xy, tri = inputs.split_square_mesh(12, 1e3, jitter=0.2, seed=7)
